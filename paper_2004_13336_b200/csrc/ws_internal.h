@@ -88,6 +88,36 @@ struct WsItemSeg {
     int count;
 };
 
+// Adafactor's all-shard update as one kernel (ws_af_onelaunch.cu).  A work item is a block of a tensor's
+// rows x cols matrix: 256 threads as rp rows of tpr threads, a thread owning 8 columns (4 where the row
+// length is no multiple of 8) and walking down the rows, so that its column sums live in registers for the
+// whole block.
+enum { WS_AF_VEC8 = 0, WS_AF_VEC4 = 1, WS_AF_SCALAR = 2, WS_AF_FULL = 3 };
+__host__ __device__ constexpr int ws_af_width(int mode) { return mode == WS_AF_VEC8 ? 8 : 4; }   // columns per thread
+constexpr int kWsAfChunk = 1024;      // state entries per moments entry
+// One record per schedule entry, in execution order, so that a CTA reads its work with one access.
+struct __align__(16) WsAfItem {
+    int seg;               // tensor index
+    int row0, col0;        // first row and column of the block
+    unsigned goff32;       // where the block's summed gradients are kept, in units of 32 floats
+    unsigned short nr;     // rows of the block
+    unsigned short nc;     // columns of the block, <= 8 tpr (4 tpr)
+    unsigned short tpr;    // threads per row
+    unsigned short rp;     // rows in parallel
+    unsigned item;         // index of the block (partial sums)
+    int phase;             // 0: sums, 1: moments (row0, col0: first state entry, low and high half; goff32: entries), 2: U^2, 3: apply
+};
+static_assert(sizeof(WsAfItem) == 32, "WsAfItem is read as two 16-byte words");
+struct __align__(16) WsAfTensor {
+    long long numel, ncol, nrow;      // WS_AF_FULL: ncol is the length of the virtual rows the items walk
+    long long foff, irow, icol;       // factored state and its padded workspace layout, as in WsSegAf
+    long long piece, off;             // packed position of element e: (e / piece) S + off + e % piece
+    long long pad_end;                // concatenated layout: its pads are elements [numel, pad_end)
+    int item_first, item_count, chunk_count, mode;
+    long long unused;
+};
+static_assert(sizeof(WsAfTensor) == 96, "WsAfTensor is read as six 16-byte words");
+
 struct ws_plan {
     int T = 0, R = 0, A = 0, K = 0;
     int layout = 0;                           // ws_layout
@@ -114,6 +144,12 @@ struct ws_plan {
     std::vector<WsItem> items;
     std::vector<WsItemSeg> itemsegs;          // [T]
     std::vector<unsigned> sched;              // [2 n_items]: item index * 2 + phase, in execution order
+    // the same for Adafactor (0 items: the plan has none)
+    long long n_afitems = 0, n_afsched = 0, af_ghat = 0;   // items, schedule entries, floats of kept gradient sums
+    std::vector<WsAfTensor> aftensors;
+    std::vector<WsAfItem> afsched;
+    const WsAfTensor* d_aftensors = nullptr;
+    const WsAfItem* d_afsched = nullptr;
     const WsItem* d_items = nullptr;
     const WsItemSeg* d_itemsegs = nullptr;
     const unsigned* d_sched = nullptr;
@@ -143,6 +179,13 @@ struct WsLambWs {
     float* acc;        // Adafactor: [Fi] this step's row / column sums (padded layout)
     double* rsum;      // Adafactor: [T] sum of the new row accumulators, directly after acc
     size_t acc_bytes;  // acc and rsum together: cleared at the start of every step
+    // one-kernel Adafactor: arrival counters, ready words and the ticket, directly after rsum and cleared
+    // with it (af_sync_bytes from acc on); the status word is the one above
+    int *af_count1, *af_countm, *af_count2;        // [T] each
+    unsigned long long *af_flagm, *af_flag2;       // [T] each
+    unsigned long long* af_ticket;
+    size_t af_sync_bytes;
+    float2* af_ipart;  // [n_afitems] partial sums of w^2 and U^2
     float* fac;        // Adafactor: [Fi] 1/sqrt factors of V (padded layout)
     float* alpha;      // Adafactor: [T] step sizes
     size_t bytes_af;   // through alpha: what Adafactor needs

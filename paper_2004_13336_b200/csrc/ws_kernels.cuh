@@ -742,4 +742,39 @@ bool one_launch_supports(int pair, int R);
 ws_status launch_one_launch(int pair, bool gbf, int out, bool fused, bool wide, const UpdParams& P,
                             const void* const* gptrs, const OneLaunch& Q, cudaStream_t st);
 
+// The one-kernel Adafactor update (ws_af_onelaunch.cu).
+struct AfLaunch {
+    const WsAfItem* sched;       // [nsched] in execution order
+    unsigned nsched;
+    int T, R;
+    int wide;                    // every fp32 buffer allows 256-bit accesses
+    int fused, master, out;      // formatting fused in; fp32 weight tensors are the master copy; O_* next to the state
+    int nshards;
+    const WsAfTensor* tensors;
+    long long S;
+    const void* const* gtab;     // fused: [T][R] gradient tensors
+    void* const* wtab;           // fused: [T] weight tensors
+    float* w;                    // packed weights (null with master)
+    void* gathered;
+    float* state;                // factored second moments
+    float* kept;                 // summed gradients, block by block
+    float *acc, *fac;            // row / column sums, 1/sqrt factors (padded layout)
+    double* rsum;                // [T] sum of the new row accumulators
+    float2* ipart;               // [items] sums of w^2 and U^2
+    int *count1, *countm, *count2;               // [T] finished P1, M and P2 entries
+    unsigned long long *flagm, *flag2;           // ready words: (float bits << 32) | 1
+    unsigned long long* ticket;
+    int* status;
+    float *alpha, *rho;
+    double* norms;
+    float gscale, eps;
+    double beta, eps2, rho_step, clip;
+#ifdef WS_DEBUG_BOUNDS
+    unsigned* bounds;
+    long long state_elems, kept_elems;
+#endif
+};
+// Clears `clear_bytes` from `clear` on and runs the update; gptrs: packed gradient buffers (not fused).
+ws_status launch_af(const AfLaunch& P, bool gbf, const void* const* gptrs, void* clear, size_t clear_bytes, cudaStream_t st);
+
 }  // namespace wsk

@@ -66,16 +66,73 @@ static void ws_matrix_views(ws_plan* p, const ws_tensor_desc* descs) {
         a.icol = ioff;
         ioff += (a.ncol + 7) / 8 * 8;
         p->segaf[t] = a;
-        for (long long b = 0; b < a.nrow + a.ncol; b += 1024) {
+        for (long long b = 0; b < a.nrow + a.ncol; b += kWsAfChunk) {
             WsAfChunk c;
             c.begin = b;
-            c.count = (int)((a.nrow + a.ncol - b) < 1024 ? (a.nrow + a.ncol - b) : 1024);
+            c.count = (int)((a.nrow + a.ncol - b) < kWsAfChunk ? (a.nrow + a.ncol - b) : kWsAfChunk);
             c.seg = t;
             p->afchunks.push_back(c);
         }
     }
     p->F = foff;
     p->Fi = ioff;
+}
+
+// Adafactor's blocks (see WsAfItem).  The strips of a row are chosen so that rp rows of tpr threads fill the
+// CTA best (a 1200-column matrix: two strips of 75 threads in three rows, 88 % busy, instead of one of 150,
+// 59 %).  A block holds up to 65536 elements, fewer where that would leave less than 750 blocks (1.7 waves of
+// CTAs): every entry pays a chain of dependent table reads and a barrier.  Measured (Transformer set, 4 copies):
+// 16384 elements 1305 us, 32768 1255 us, 65536 1245 us; 22.7 M parameters in ragged tensors, 2 copies: at least
+// 3000 blocks 255 us, 1500 194 us, 750 176 us.
+template <typename F>
+static void ws_af_blocks(const ws_plan* p, F&& emit) {
+    long long block = 65536;
+    while (block > 1024 && p->N / block < 750) block >>= 1;
+    for (int t = 0; t < p->T; ++t) {
+        const WsSegAf& a = p->segaf[t];
+        if (a.numel <= 0) continue;
+        const bool full = a.nrow == 0;
+        const long long ncol = full ? (a.numel < 1024 ? a.numel : 1024) : a.ncol;
+        const long long nrow = full ? (a.numel + ncol - 1) / ncol : a.nrow;
+        const int mode = full ? WS_AF_FULL : ncol % 8 == 0 ? WS_AF_VEC8 : ncol % 4 == 0 ? WS_AF_VEC4 : WS_AF_SCALAR;
+        const long long W = ws_af_width(mode);
+        const long long units = (ncol + W - 1) / W, s0 = (units + 255) / 256;
+        long long best_s = s0, best = -1;              // (busy threads of 256) / strips, compared as fractions
+        for (long long s = s0; s < s0 + 8 && s <= units; ++s) {
+            const long long tpr = (units + s - 1) / s, score = units * (256 / tpr) * 4096 / s;
+            if (score > best) { best = score; best_s = s; }
+        }
+        const long long tpr = (units + best_s - 1) / best_s;
+        long long rp = 256 / tpr;
+        if (rp > nrow) rp = nrow;
+        const long long step = rp * (block < 256 * W ? 1 : block / (256 * W));
+        for (long long r0 = 0; r0 < nrow; r0 += step)
+            for (long long c0 = 0; c0 < ncol; c0 += W * tpr) {
+                const long long nc = ncol - c0 < W * tpr ? ncol - c0 : W * tpr;
+                const long long nr = nrow - r0 < step ? nrow - r0 : step;
+                emit(t, mode, r0, c0, nr, nc, (nc + W - 1) / W, rp);
+            }
+    }
+}
+
+// Block and schedule-entry counts and the floats of kept gradient sums; a tensor beyond the block fields'
+// ranges leaves the plan without Adafactor blocks.
+static void ws_count_af(ws_plan* p) {
+    p->n_afitems = p->n_afsched = p->af_ghat = 0;
+    if (p->R > 65535) return;
+    long long n = 0, m = 0, g = 0;
+    for (const WsSegAf& a : p->segaf) {
+        if (a.nrow > 0x7fffffffLL || a.ncol > 0x7fffffffLL) return;
+        if (a.nrow > 0) m += (a.nrow + a.ncol + kWsAfChunk - 1) / kWsAfChunk;
+    }
+    ws_af_blocks(p, [&](int, int mode, long long, long long, long long nr, long long, long long tpr, long long rp) {
+        ++n;
+        g += ((nr + rp - 1) / rp * rp * tpr * ws_af_width(mode) + 31) / 32 * 32;
+    });
+    if (n > 0x0fffffffLL || m > 0x0fffffffLL || g / 32 > 0xffffffffLL) return;
+    p->n_afitems = n;
+    p->n_afsched = 3 * n + m;
+    p->af_ghat = g;
 }
 
 // Work items of the one-launch schedule: every tile cut into runs of kWsItemElems elements, for every
@@ -200,6 +257,7 @@ extern "C" ws_status ws_plan_create_layout(const ws_tensor_desc* descs, int32_t 
                     p->segtiles[k].tile_begin = k > 0 ? p->segtiles[k - 1].tile_begin + p->segtiles[k - 1].tile_count : 0;
             ws_matrix_views(p, descs);
             ws_count_items(p);
+            ws_count_af(p);
             *out = p;
             return WS_OK;
         }
@@ -242,6 +300,7 @@ extern "C" ws_status ws_plan_create_layout(const ws_tensor_desc* descs, int32_t 
         p->ntiles = (long long)p->tiles.size();
         ws_matrix_views(p, descs);
         ws_count_items(p);
+        ws_count_af(p);
     } catch (...) {
         delete p;
         return WS_ERR_INVALID_ARG;
@@ -286,30 +345,39 @@ extern "C" ws_status ws_plan_factored_layout(const ws_plan* p, int64_t* layout) 
     return WS_OK;
 }
 
+// Copies `n` tables to their offsets in one device buffer with one copy.
+static ws_status upload_image(char* dev, const void* const* src, const size_t* nb, const size_t* off, int n, size_t total,
+                              cudaStream_t st, const char* what) {
+    std::vector<char> host;
+    try {
+        host.resize(total);
+    } catch (...) {
+        return WS_ERR_INVALID_ARG;
+    }
+    for (int i = 0; i < n; ++i)
+        if (nb[i]) memcpy(host.data() + off[i], src[i], nb[i]);
+    // (pageable memory: the runtime has staged it before cudaMemcpyAsync returns)
+    const cudaError_t e = total ? cudaMemcpyAsync(dev, host.data(), total, cudaMemcpyHostToDevice, st) : cudaSuccess;
+    return e == cudaSuccess ? WS_OK : ws_cuda_fail(e, what);
+}
+
 extern "C" ws_status ws_plan_upload(ws_plan* p, void* dev_buf, size_t bytes, void* stream) {
     if (!p || !dev_buf) return WS_ERR_INVALID_ARG;
     if (!ws_aligned16(dev_buf)) return WS_ERR_ALIGNMENT;
     if (bytes < ws_plan_device_bytes(p)) return WS_ERR_WORKSPACE;
-    cudaStream_t st = (cudaStream_t)stream;
-    size_t tb = p->tiles.size() * sizeof(WsTile);
+    // one image, one copy: every cudaMemcpyAsync from pageable memory costs the host some 10 us
     char* base = (char*)dev_buf;
-    cudaError_t e = cudaMemcpyAsync(base, p->tiles.data(), tb, cudaMemcpyHostToDevice, st);
-    if (e != cudaSuccess) return ws_cuda_fail(e, "ws_plan_upload(tiles)");
-    e = cudaMemcpyAsync(base + round16(tb), p->segtiles.data(), p->segtiles.size() * sizeof(WsSegTiles),
-                        cudaMemcpyHostToDevice, st);
-    if (e != cudaSuccess) return ws_cuda_fail(e, "ws_plan_upload(segments)");
-    const size_t ab = round16(tb) + round16(p->segtiles.size() * sizeof(WsSegTiles));
-    e = cudaMemcpyAsync(base + ab, p->segaf.data(), p->segaf.size() * sizeof(WsSegAf), cudaMemcpyHostToDevice, st);
-    if (e != cudaSuccess) return ws_cuda_fail(e, "ws_plan_upload(matrix views)");
-    p->d_tiles = (const WsTile*)base;
-    p->d_segtiles = (const WsSegTiles*)(base + round16(tb));
-    p->d_segaf = (const WsSegAf*)(base + ab);
-    const size_t cb = ab + round16(p->segaf.size() * sizeof(WsSegAf));
-    if (!p->afchunks.empty()) {
-        e = cudaMemcpyAsync(base + cb, p->afchunks.data(), p->afchunks.size() * sizeof(WsAfChunk), cudaMemcpyHostToDevice, st);
-        if (e != cudaSuccess) return ws_cuda_fail(e, "ws_plan_upload(state chunks)");
-    }
-    p->d_afchunks = (const WsAfChunk*)(base + cb);
+    size_t o[4], at = 0;
+    const size_t nb[4] = {p->tiles.size() * sizeof(WsTile), p->segtiles.size() * sizeof(WsSegTiles),
+                          p->segaf.size() * sizeof(WsSegAf), p->afchunks.size() * sizeof(WsAfChunk)};
+    const void* src[4] = {p->tiles.data(), p->segtiles.data(), p->segaf.data(), p->afchunks.data()};
+    for (int i = 0; i < 4; ++i) { o[i] = at; at += round16(nb[i]); }
+    const ws_status s = upload_image(base, src, nb, o, 4, at, (cudaStream_t)stream, "ws_plan_upload");
+    if (s != WS_OK) return s;
+    p->d_tiles = (const WsTile*)(base + o[0]);
+    p->d_segtiles = (const WsSegTiles*)(base + o[1]);
+    p->d_segaf = (const WsSegAf*)(base + o[2]);
+    p->d_afchunks = (const WsAfChunk*)(base + o[3]);
     return WS_OK;
 }
 
@@ -339,13 +407,27 @@ WsLambWs ws_lamb_layout(const ws_plan* p, void* workspace) {
     o = (o + 255) & ~(size_t)255;
     L.ghat = (float*)(b + o);
     L.bytes_lars = o + sizeof(float) * (size_t)p->R * (size_t)p->S;
-    o = (L.bytes_lars + 255) & ~(size_t)255;
+    // (the one-kernel Adafactor keeps the sums block by block, a few floats more than [R][S] may hold)
+    const size_t ghat_af = (size_t)p->af_ghat > (size_t)p->R * (size_t)p->S ? (size_t)p->af_ghat : (size_t)p->R * (size_t)p->S;
+    o = ((size_t)((char*)L.ghat - b) + sizeof(float) * ghat_af + 255) & ~(size_t)255;
     L.acc = (float*)(b + o);
     const size_t acc0 = o;
     o = (o + sizeof(float) * (size_t)p->Fi + 15) & ~(size_t)15;
     L.rsum = (double*)(b + o);
     o += sizeof(double) * (size_t)p->T;
     L.acc_bytes = o - acc0;
+    const size_t T = (size_t)p->T;
+    L.af_flagm = (unsigned long long*)(b + o);
+    L.af_flag2 = L.af_flagm + T;
+    L.af_ticket = L.af_flag2 + T;
+    o += sizeof(unsigned long long) * (2 * T + 1);
+    L.af_count1 = (int*)(b + o);
+    L.af_countm = L.af_count1 + T;
+    L.af_count2 = L.af_countm + T;
+    o = round16(o + sizeof(int) * 3 * T);
+    L.af_sync_bytes = o - acc0;
+    L.af_ipart = (float2*)(b + o);
+    o += sizeof(float2) * (size_t)p->n_afitems;
     o = (o + 255) & ~(size_t)255;
     L.fac = (float*)(b + o);
     o = (o + sizeof(float) * (size_t)p->Fi + 255) & ~(size_t)255;
@@ -489,10 +571,152 @@ void ws_build_schedule(ws_plan* p) {
     }
 }
 
-size_t schedule_bytes(const ws_plan* p) {
+// Adafactor: sums (P1) -> moments of every 1024-entry chunk (M) -> U^2 (P2) -> apply (P3).  Groups of tensors
+// as above; a phase of a group starts at least kLag entries after its previous one ended, and the phases of
+// different groups alternate, so that P1 (and P2's weights) stream from DRAM while the others work from L2.
+// P2 walks a group back to front and P3 front to back, each starting with what the one before touched last.
+constexpr long long kAfGroupElems = 512 << 10;
+
+void ws_build_af_schedule(ws_plan* p) {
+    const int T = p->T;
+    std::vector<WsAfItem> items;
+    items.reserve((size_t)p->n_afitems);
+    p->aftensors.resize(T);
+    for (int t = 0; t < T; ++t) {
+        const WsSegAf& a = p->segaf[t];
+        WsAfTensor& d = p->aftensors[t];
+        memset(&d, 0, sizeof(d));
+        d.numel = a.numel; d.ncol = a.ncol; d.nrow = a.nrow;
+        d.foff = a.foff; d.irow = a.irow; d.icol = a.icol;
+        d.piece = p->layout == WS_LAYOUT_CONCAT ? (1LL << 62) : p->segs[t].piece;
+        d.off = p->segs[t].shard_off;
+        d.pad_end = (t + 1 < T ? p->segs[t + 1].shard_off : (long long)p->R * p->S) - d.off;
+        d.chunk_count = a.nrow > 0 ? (int)((a.nrow + a.ncol + kWsAfChunk - 1) / kWsAfChunk) : 0;
+        d.mode = a.nrow > 0 ? WS_AF_VEC4 : WS_AF_FULL;
+        if (d.mode == WS_AF_FULL) d.ncol = a.numel < 1024 ? a.numel : 1024;
+    }
+    long long goff = 0;
+    ws_af_blocks(p, [&](int t, int mode, long long r0, long long c0, long long nr, long long nc, long long tpr, long long rp) {
+        WsAfTensor& d = p->aftensors[t];
+        if (d.item_count++ == 0) d.item_first = (int)items.size();
+        d.mode = mode;
+        WsAfItem it;
+        memset(&it, 0, sizeof(it));
+        it.seg = t;
+        it.row0 = (int)r0; it.col0 = (int)c0;
+        it.nr = (unsigned short)nr; it.nc = (unsigned short)nc;
+        it.tpr = (unsigned short)tpr; it.rp = (unsigned short)rp;
+        it.goff32 = (unsigned)goff;
+        it.item = (unsigned)items.size();
+        goff += ((nr + rp - 1) / rp * rp * tpr * ws_af_width(mode) + 31) / 32;
+        items.push_back(it);
+    });
+    struct Group { int i0, i1; std::vector<int> tensors; long long m; };
+    std::vector<Group> groups;
+    {
+        Group g{0, 0, {}, 0};
+        long long acc = 0;
+        for (int t = 0; t < T; ++t) {
+            const WsAfTensor& d = p->aftensors[t];
+            if (d.item_count == 0) continue;
+            g.tensors.push_back(t);
+            g.m += d.chunk_count;
+            g.i1 = d.item_first + d.item_count;
+            acc += d.numel;
+            if (acc >= kAfGroupElems) {
+                const int next = g.i1;
+                groups.push_back(std::move(g));
+                g = Group{next, next, {}, 0};
+                acc = 0;
+            }
+        }
+        if (g.i1 > g.i0) groups.push_back(std::move(g));
+    }
+    std::vector<int> chunk0(T, 0);                    // first entry of every tensor in the plan's chunk list
+    {
+        long long c = 0;
+        for (int t = 0; t < T; ++t) {
+            chunk0[t] = (int)c;
+            c += (p->segaf[t].nrow + p->segaf[t].ncol + kWsAfChunk - 1) / kWsAfChunk;
+        }
+    }
+    std::vector<WsAfItem>& out = p->afsched;
+    out.clear();
+    out.reserve((size_t)p->n_afsched);
+    const int G = (int)groups.size();
+    // next[ph]: group of phase ph's next entry, at[ph]: entries of it already out, done[ph][g]: where it ended
+    int next[4] = {0, 0, 0, 0};
+    long long at[4] = {0, 0, 0, 0};
+    std::vector<long long> done[4];
+    for (auto& d : done) d.assign(G, -1);
+    std::vector<int> mchunks;                         // chunk indexes of the group phase M works on
+    int mgroup = -1;
+    auto size_of = [&](int ph, int g) { return ph == 1 ? groups[g].m : (long long)(groups[g].i1 - groups[g].i0); };
+    auto emit = [&](int ph) {
+        const int g = next[ph];
+        const Group& gr = groups[g];
+        if (size_of(ph, g) > 0) {
+            WsAfItem rec;
+            if (ph == 1) {
+                if (mgroup != g) {
+                    mgroup = g;
+                    mchunks.clear();
+                    for (int t : gr.tensors)
+                        for (int k = 0; k < p->aftensors[t].chunk_count; ++k) mchunks.push_back(chunk0[t] + k);
+                }
+                const WsAfChunk& c = p->afchunks[(size_t)mchunks[(size_t)at[1]]];
+                memset(&rec, 0, sizeof(rec));
+                rec.seg = c.seg;
+                rec.row0 = (int)(unsigned)((unsigned long long)c.begin & 0xffffffffu);
+                rec.col0 = (int)(c.begin >> 32);
+                rec.goff32 = (unsigned)c.count;
+            } else {
+                rec = items[(size_t)(ph == 2 ? gr.i1 - 1 - at[ph] : gr.i0 + at[ph])];
+            }
+            rec.phase = ph;
+            out.push_back(rec);
+        }
+        if (++at[ph] >= size_of(ph, g)) {
+            done[ph][g] = (long long)out.size() - 1;
+            at[ph] = 0;
+            ++next[ph];
+        }
+    };
+    int last = 3;
+    while (next[3] < G) {
+        const long long pos = (long long)out.size();
+        // phase ph may go on with group g once phase ph-1 of g has ended (lag entries ago)
+        auto ready = [&](int ph, long long lag) {
+            if (next[ph] >= G) return false;
+            if (ph == 0 || at[ph] > 0) return true;
+            const long long d = done[ph - 1][next[ph]];
+            return next[ph - 1] > next[ph] && pos - d >= lag;
+        };
+        int ph = -1;
+        if (ready(1, kLag)) {
+            ph = 1;
+        } else {
+            for (int k = 1; k <= 4 && ph < 0; ++k) {
+                const int c = (last + k) & 3;
+                if (c != 1 && ready(c, kLag)) ph = c;
+            }
+        }
+        for (int c = 1; c < 4 && ph < 0; ++c)          // the tail: nothing is far enough behind
+            if (ready(c, 0)) ph = c;
+        emit(ph);
+        if (ph != 1) last = ph;
+    }
+}
+
+size_t af_schedule_bytes(const ws_plan* p) {
+    if (p->n_afitems <= 0) return 0;
+    return round16((size_t)p->T * sizeof(WsAfTensor)) + (size_t)p->n_afsched * sizeof(WsAfItem);
+}
+size_t lamb_schedule_bytes(const ws_plan* p) {
     return round16((size_t)p->n_items * sizeof(WsItem)) + round16((size_t)p->T * sizeof(WsItemSeg)) +
            round16((size_t)p->n_items * 2 * sizeof(unsigned));
 }
+size_t schedule_bytes(const ws_plan* p) { return lamb_schedule_bytes(p) + af_schedule_bytes(p); }
 }  // namespace
 
 extern "C" size_t ws_plan_schedule_bytes(const ws_plan* p) {
@@ -507,23 +731,28 @@ extern "C" ws_status ws_plan_upload_schedule(ws_plan* p, void* dev_buf, size_t b
     if (bytes < schedule_bytes(p)) return WS_ERR_WORKSPACE;
     try {
         if (p->sched.empty()) ws_build_schedule(p);
+        if (p->afsched.empty() && p->n_afitems > 0) ws_build_af_schedule(p);
     } catch (...) {
         return WS_ERR_INVALID_ARG;
     }
-    if ((long long)p->items.size() != p->n_items) return WS_ERR_INVALID_ARG;
-    cudaStream_t st = (cudaStream_t)stream;
+    if ((long long)p->items.size() != p->n_items || (long long)p->afsched.size() != p->n_afsched) return WS_ERR_INVALID_ARG;
     char* base = (char*)dev_buf;
-    const size_t ib = (size_t)p->n_items * sizeof(WsItem), sb = (size_t)p->T * sizeof(WsItemSeg);
-    cudaError_t e = cudaMemcpyAsync(base, p->items.data(), ib, cudaMemcpyHostToDevice, st);
-    if (e != cudaSuccess) return ws_cuda_fail(e, "ws_plan_upload_schedule(items)");
-    e = cudaMemcpyAsync(base + round16(ib), p->itemsegs.data(), sb, cudaMemcpyHostToDevice, st);
-    if (e != cudaSuccess) return ws_cuda_fail(e, "ws_plan_upload_schedule(tensor ranges)");
-    e = cudaMemcpyAsync(base + round16(ib) + round16(sb), p->sched.data(), p->sched.size() * sizeof(unsigned),
-                        cudaMemcpyHostToDevice, st);
-    if (e != cudaSuccess) return ws_cuda_fail(e, "ws_plan_upload_schedule(order)");
-    p->d_items = (const WsItem*)base;
-    p->d_itemsegs = (const WsItemSeg*)(base + round16(ib));
-    p->d_sched = (const unsigned*)(base + round16(ib) + round16(sb));
+    const bool af = p->n_afitems > 0;
+    size_t o[5], at = 0;
+    const size_t nb[5] = {p->items.size() * sizeof(WsItem), p->itemsegs.size() * sizeof(WsItemSeg),
+                          p->sched.size() * sizeof(unsigned), p->aftensors.size() * sizeof(WsAfTensor),
+                          p->afsched.size() * sizeof(WsAfItem)};
+    const void* src[5] = {p->items.data(), p->itemsegs.data(), p->sched.data(), p->aftensors.data(), p->afsched.data()};
+    for (int i = 0; i < (af ? 5 : 3); ++i) { o[i] = at; at += round16(nb[i]); }
+    const ws_status s = upload_image(base, src, nb, o, af ? 5 : 3, at, (cudaStream_t)stream, "ws_plan_upload_schedule");
+    if (s != WS_OK) return s;
+    p->d_items = (const WsItem*)(base + o[0]);
+    p->d_itemsegs = (const WsItemSeg*)(base + o[1]);
+    p->d_sched = (const unsigned*)(base + o[2]);
+    if (af) {
+        p->d_aftensors = (const WsAfTensor*)(base + o[3]);
+        p->d_afsched = (const WsAfItem*)(base + o[4]);
+    }
     return WS_OK;
 }
 

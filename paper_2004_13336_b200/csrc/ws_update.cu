@@ -858,6 +858,20 @@ ws_status fused_phase(const ws_plan* plan, int32_t r, const ws_tensor_table* gra
     return launch_f<true>(phase, gbf, out_kind, P, nullptr, wide, st);
 }
 
+// Checks that every Adafactor call shares.
+ws_status af_check(const ws_plan* plan, int32_t r, const ws_hyper* hyper, void* workspace, size_t workspace_bytes) {
+    if (!plan || !hyper) return WS_ERR_INVALID_ARG;
+    if (!plan->d_tiles) return WS_ERR_NOT_UPLOADED;
+    if (r < -1 || r >= plan->R) return WS_ERR_INVALID_ARG;
+    if (hyper->opt != WS_ADAFACTOR || hyper->weight_decay != 0.0 || !(hyper->clip_threshold > 0.0) ||
+        !(hyper->decay_exponent > 0.0) || !(hyper->eps >= 0.0) || !(hyper->eps2 >= 0.0) || hyper->step < 1)
+        return WS_ERR_INVALID_ARG;
+    const ws_status s = check_ws(plan, workspace, workspace_bytes, WS_ADAFACTOR);
+    if (s != WS_OK) return s;
+    // pass 2 reads the stored gradient sum (256 bytes into the workspace and onwards) with 256-bit loads
+    return aligned32(workspace) ? WS_OK : WS_ERR_ALIGNMENT;
+}
+
 // Adafactor, all shards: zero the row / column sums, pass 1 (reduce, keep the sum, partial row and
 // column sums), moments + step size, pass 2 (sum U^2), clipping, pass 3 (apply).  Either the
 // packed-buffer arguments (grads, out) or the tensor tables (gtab, wtab) are given.
@@ -866,16 +880,8 @@ ws_status fused_phase(const ws_plan* plan, int32_t r, const ws_tensor_table* gra
 ws_status af_stage(const ws_plan* plan, int stage, int32_t r, const ws_grads* grads, const ws_tensor_table* gtab,
                    const ws_state* state, const ws_hyper* hyper, const ws_out* out, const ws_tensor_table* wtab,
                    void* workspace, size_t workspace_bytes, cudaStream_t st) {
-    if (!plan || !hyper) return WS_ERR_INVALID_ARG;
-    if (!plan->d_tiles) return WS_ERR_NOT_UPLOADED;
-    if (r < -1 || r >= plan->R) return WS_ERR_INVALID_ARG;
-    if (hyper->opt != WS_ADAFACTOR || hyper->weight_decay != 0.0 || !(hyper->clip_threshold > 0.0) ||
-        !(hyper->decay_exponent > 0.0) || !(hyper->eps >= 0.0) || !(hyper->eps2 >= 0.0) || hyper->step < 1)
-        return WS_ERR_INVALID_ARG;
-    ws_status s = check_ws(plan, workspace, workspace_bytes, WS_ADAFACTOR);
+    ws_status s = af_check(plan, r, hyper, workspace, workspace_bytes);
     if (s != WS_OK) return s;
-    // pass 2 reads the stored gradient sum (256 bytes into the workspace and onwards) with 256-bit loads
-    if (!aligned32(workspace)) return WS_ERR_ALIGNMENT;
     const WsLambWs L = ws_lamb_layout(plan, workspace);
     const bool fused = gtab != nullptr;
     UpdParams P;
@@ -942,11 +948,91 @@ ws_status af_stage(const ws_plan* plan, int stage, int32_t r, const ws_grads* gr
     }
 }
 
-// Adafactor, all shards: the six stages in order.
+// Adafactor for all shards as one kernel, when the plan's blocks are on the device; `done` as above.
+ws_status try_af_one_launch(const ws_plan* plan, const ws_grads* grads, const ws_tensor_table* gtab, const ws_state* state,
+                            const ws_hyper* hyper, const ws_out* out, const ws_tensor_table* wtab, void* workspace,
+                            size_t workspace_bytes, cudaStream_t st, bool& done) {
+    done = false;
+    if (!plan || !hyper || !plan->d_afsched) return WS_OK;
+    const bool fused = gtab != nullptr;
+    ws_status s = af_check(plan, -1, hyper, workspace, workspace_bytes);
+    if (s != WS_OK) return s;
+    UpdParams U;
+    int out_kind;
+    bool gbf;
+    s = prepare(plan, -1, grads, state, hyper, fused ? nullptr : out, K_AF1, U, out_kind, gbf, fused);
+    if (s != WS_OK) return s;
+    if (!state->v) return WS_ERR_INVALID_ARG;
+    if (!ws_aligned16(state->v)) return WS_ERR_ALIGNMENT;
+    const WsLambWs L = ws_lamb_layout(plan, workspace);
+    AfLaunch P = {};
+    P.sched = plan->d_afsched;
+    P.nsched = (unsigned)plan->n_afsched;
+    P.T = plan->T;
+    P.R = fused ? gtab->nsets : grads->R;
+    P.fused = fused;
+    P.master = fused && state->w == nullptr;
+    if (fused) {
+        if (P.master && wtab->dtype != WS_F32) return WS_ERR_INVALID_ARG;
+        gbf = gtab->dtype == WS_BF16;
+        out_kind = P.master ? O_F32M : (wtab->dtype == WS_F32 ? O_F32 : O_BF16);
+        P.gtab = (const void* const*)gtab->dev;
+        P.wtab = (void* const*)wtab->dev;
+    }
+    P.out = out_kind;
+    bool wide = aligned32(U.w) && aligned32(U.gathered);
+    if (fused) {
+        wide = wide && (gbf || gtab->min_align >= 32) && (wtab->dtype == WS_BF16 || wtab->min_align >= 32);
+    } else {
+        for (int k = 0; k < P.R && wide; ++k) wide = gbf || aligned32(grads->ptrs[k]);
+    }
+    P.wide = wide;
+    P.nshards = plan->R;
+    P.tensors = plan->d_aftensors;
+    P.S = plan->S;
+    P.w = U.w;
+    P.gathered = U.gathered;
+    P.state = (float*)state->v;
+    P.kept = L.ghat;
+    P.acc = L.acc;
+    P.fac = L.fac;
+    P.rsum = L.rsum;
+    P.ipart = L.af_ipart;
+    P.count1 = L.af_count1;
+    P.countm = L.af_countm;
+    P.count2 = L.af_count2;
+    P.flagm = L.af_flagm;
+    P.flag2 = L.af_flag2;
+    P.ticket = L.af_ticket;
+    P.status = L.status;
+    P.alpha = L.alpha;
+    P.rho = L.rho;
+    P.norms = L.norms;
+    P.gscale = U.c.gscale;
+    P.eps = U.c.eps;
+    P.beta = 1.0 - pow((double)hyper->step, -hyper->decay_exponent);
+    P.eps2 = hyper->eps2;
+    const double inv_sqrt_t = 1.0 / sqrt((double)hyper->step);
+    P.rho_step = hyper->lr < inv_sqrt_t ? hyper->lr : inv_sqrt_t;
+    P.clip = hyper->clip_threshold;
+#ifdef WS_DEBUG_BOUNDS
+    P.bounds = U.bounds;
+    P.state_elems = (long long)plan->R * plan->S;
+    P.kept_elems = (long long)((L.acc - L.ghat));
+#endif
+    s = launch_af(P, gbf, fused ? nullptr : grads->ptrs, L.acc, L.af_sync_bytes, st);
+    if (s == WS_OK) done = true;
+    return s;
+}
+
+// Adafactor, all shards: one kernel where the plan has its blocks on the device, else the six stages in order.
 ws_status af_update(const ws_plan* plan, int32_t r, const ws_grads* grads, const ws_tensor_table* gtab,
                     const ws_state* state, const ws_hyper* hyper, const ws_out* out, const ws_tensor_table* wtab,
                     void* workspace, size_t workspace_bytes, cudaStream_t st) {
     if (r != -1 || !state) return WS_ERR_INVALID_ARG;
+    bool done = false;
+    const ws_status one = try_af_one_launch(plan, grads, gtab, state, hyper, out, wtab, workspace, workspace_bytes, st, done);
+    if (one != WS_OK || done) return one;
     for (int stage = WS_AF_BEGIN; stage <= WS_AF_APPLY; ++stage) {
         const ws_status s = af_stage(plan, stage, -1, grads, gtab, state, hyper, out, wtab, workspace, workspace_bytes, st);
         if (s != WS_OK) return s;
