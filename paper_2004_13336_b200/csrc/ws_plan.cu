@@ -345,19 +345,26 @@ extern "C" ws_status ws_plan_factored_layout(const ws_plan* p, int64_t* layout) 
     return WS_OK;
 }
 
-// Copies `n` tables to their offsets in one device buffer with one copy.
+// Copies `n` tables to their offsets in one device buffer.  Small plans: as one image, one copy (every
+// cudaMemcpyAsync from pageable memory costs the host some 10 us); from 128 KB on gathering the image costs more.
 static ws_status upload_image(char* dev, const void* const* src, const size_t* nb, const size_t* off, int n, size_t total,
                               cudaStream_t st, const char* what) {
-    std::vector<char> host;
-    try {
-        host.resize(total);
-    } catch (...) {
-        return WS_ERR_INVALID_ARG;
-    }
-    for (int i = 0; i < n; ++i)
-        if (nb[i]) memcpy(host.data() + off[i], src[i], nb[i]);
     // (pageable memory: the runtime has staged it before cudaMemcpyAsync returns)
-    const cudaError_t e = total ? cudaMemcpyAsync(dev, host.data(), total, cudaMemcpyHostToDevice, st) : cudaSuccess;
+    cudaError_t e = cudaSuccess;
+    if (total <= (128u << 10)) {
+        std::vector<char> host;
+        try {
+            host.resize(total);
+        } catch (...) {
+            return WS_ERR_INVALID_ARG;
+        }
+        for (int i = 0; i < n; ++i)
+            if (nb[i]) memcpy(host.data() + off[i], src[i], nb[i]);
+        if (total) e = cudaMemcpyAsync(dev, host.data(), total, cudaMemcpyHostToDevice, st);
+    } else {
+        for (int i = 0; i < n && e == cudaSuccess; ++i)
+            if (nb[i]) e = cudaMemcpyAsync(dev + off[i], src[i], nb[i], cudaMemcpyHostToDevice, st);
+    }
     return e == cudaSuccess ? WS_OK : ws_cuda_fail(e, what);
 }
 
@@ -365,7 +372,6 @@ extern "C" ws_status ws_plan_upload(ws_plan* p, void* dev_buf, size_t bytes, voi
     if (!p || !dev_buf) return WS_ERR_INVALID_ARG;
     if (!ws_aligned16(dev_buf)) return WS_ERR_ALIGNMENT;
     if (bytes < ws_plan_device_bytes(p)) return WS_ERR_WORKSPACE;
-    // one image, one copy: every cudaMemcpyAsync from pageable memory costs the host some 10 us
     char* base = (char*)dev_buf;
     size_t o[4], at = 0;
     const size_t nb[4] = {p->tiles.size() * sizeof(WsTile), p->segtiles.size() * sizeof(WsSegTiles),
@@ -611,100 +617,89 @@ void ws_build_af_schedule(ws_plan* p) {
         goff += ((nr + rp - 1) / rp * rp * tpr * ws_af_width(mode) + 31) / 32;
         items.push_back(it);
     });
-    struct Group { int i0, i1; std::vector<int> tensors; long long m; };
+    // groups of consecutive tensors; a group's chunks are consecutive too, once the unfactored tensors' are left out
+    struct Group { int i0, i1, m0, m1; };
     std::vector<Group> groups;
+    std::vector<int> chunks;
+    chunks.reserve((size_t)(p->n_afsched - 3 * p->n_afitems));
     {
-        Group g{0, 0, {}, 0};
+        Group g{0, 0, 0, 0};
         long long acc = 0;
+        int c = 0;
         for (int t = 0; t < T; ++t) {
             const WsAfTensor& d = p->aftensors[t];
+            for (int k = 0; k < d.chunk_count; ++k) chunks.push_back(c + k);
+            c += (int)((p->segaf[t].nrow + p->segaf[t].ncol + kWsAfChunk - 1) / kWsAfChunk);
             if (d.item_count == 0) continue;
-            g.tensors.push_back(t);
-            g.m += d.chunk_count;
             g.i1 = d.item_first + d.item_count;
+            g.m1 = (int)chunks.size();
             acc += d.numel;
             if (acc >= kAfGroupElems) {
-                const int next = g.i1;
-                groups.push_back(std::move(g));
-                g = Group{next, next, {}, 0};
+                groups.push_back(g);
+                g = Group{g.i1, g.i1, g.m1, g.m1};
                 acc = 0;
             }
         }
-        if (g.i1 > g.i0) groups.push_back(std::move(g));
-    }
-    std::vector<int> chunk0(T, 0);                    // first entry of every tensor in the plan's chunk list
-    {
-        long long c = 0;
-        for (int t = 0; t < T; ++t) {
-            chunk0[t] = (int)c;
-            c += (p->segaf[t].nrow + p->segaf[t].ncol + kWsAfChunk - 1) / kWsAfChunk;
-        }
+        if (g.i1 > g.i0) groups.push_back(g);
     }
     std::vector<WsAfItem>& out = p->afsched;
-    out.clear();
-    out.reserve((size_t)p->n_afsched);
+    out.resize((size_t)p->n_afsched);
     const int G = (int)groups.size();
-    // next[ph]: group of phase ph's next entry, at[ph]: entries of it already out, done[ph][g]: where it ended
-    int next[4] = {0, 0, 0, 0};
-    long long at[4] = {0, 0, 0, 0};
-    std::vector<long long> done[4];
-    for (auto& d : done) d.assign(G, -1);
-    std::vector<int> mchunks;                         // chunk indexes of the group phase M works on
-    int mgroup = -1;
-    auto size_of = [&](int ph, int g) { return ph == 1 ? groups[g].m : (long long)(groups[g].i1 - groups[g].i0); };
-    auto emit = [&](int ph) {
-        const int g = next[ph];
-        const Group& gr = groups[g];
-        if (size_of(ph, g) > 0) {
-            WsAfItem rec;
-            if (ph == 1) {
-                if (mgroup != g) {
-                    mgroup = g;
-                    mchunks.clear();
-                    for (int t : gr.tensors)
-                        for (int k = 0; k < p->aftensors[t].chunk_count; ++k) mchunks.push_back(chunk0[t] + k);
-                }
-                const WsAfChunk& c = p->afchunks[(size_t)mchunks[(size_t)at[1]]];
+    constexpr long long kNever = 1LL << 62;
+    // phase ph works on group next[ph], of which `left` entries are to come, and may go on from position from[ph]
+    // (kNever: the phase before has not ended the group yet)
+    struct Phase { int next; int left; long long from; } ph[4];
+    std::vector<long long> done[4];                   // position after a group's last entry of the phase
+    for (auto& d : done) d.assign(G, kNever);
+    auto size_of = [&](int c, int g) { return c == 1 ? groups[g].m1 - groups[g].m0 : groups[g].i1 - groups[g].i0; };
+    auto open = [&](int c) {                          // phase c turns to group next[c]
+        Phase& f = ph[c];
+        if (f.next >= G) { f.from = kNever; return; }
+        f.left = size_of(c, f.next);
+        f.from = c == 0 ? 0 : done[c - 1][f.next] == kNever ? kNever : done[c - 1][f.next] + kLag - 1;
+    };
+    for (int c = 0; c < 4; ++c) { ph[c].next = 0; open(c); }
+    long long pos = 0;
+    auto emit = [&](int c) {
+        Phase& f = ph[c];
+        const Group& g = groups[f.next];
+        if (f.left > 0) {
+            WsAfItem& rec = out[(size_t)pos++];
+            if (c == 1) {
+                const WsAfChunk& k = p->afchunks[(size_t)chunks[(size_t)(g.m1 - f.left)]];
                 memset(&rec, 0, sizeof(rec));
-                rec.seg = c.seg;
-                rec.row0 = (int)(unsigned)((unsigned long long)c.begin & 0xffffffffu);
-                rec.col0 = (int)(c.begin >> 32);
-                rec.goff32 = (unsigned)c.count;
+                rec.seg = k.seg;
+                rec.row0 = (int)(unsigned)((unsigned long long)k.begin & 0xffffffffu);
+                rec.col0 = (int)(k.begin >> 32);
+                rec.goff32 = (unsigned)k.count;
             } else {
-                rec = items[(size_t)(ph == 2 ? gr.i1 - 1 - at[ph] : gr.i0 + at[ph])];
+                rec = items[(size_t)(c == 2 ? g.i0 + f.left - 1 : g.i1 - f.left)];
             }
-            rec.phase = ph;
-            out.push_back(rec);
+            rec.phase = c;
+            --f.left;
+            f.from = 0;
         }
-        if (++at[ph] >= size_of(ph, g)) {
-            done[ph][g] = (long long)out.size() - 1;
-            at[ph] = 0;
-            ++next[ph];
-        }
+        if (f.left > 0) return;
+        const int g_done = f.next++;
+        done[c][g_done] = pos;
+        open(c);
+        if (c < 3 && ph[c + 1].next == g_done) open(c + 1);
     };
     int last = 3;
-    while (next[3] < G) {
-        const long long pos = (long long)out.size();
-        // phase ph may go on with group g once phase ph-1 of g has ended (lag entries ago)
-        auto ready = [&](int ph, long long lag) {
-            if (next[ph] >= G) return false;
-            if (ph == 0 || at[ph] > 0) return true;
-            const long long d = done[ph - 1][next[ph]];
-            return next[ph - 1] > next[ph] && pos - d >= lag;
-        };
-        int ph = -1;
-        if (ready(1, kLag)) {
-            ph = 1;
+    while (ph[3].next < G) {
+        int c = -1;
+        if (ph[1].from <= pos) {
+            c = 1;
         } else {
-            for (int k = 1; k <= 4 && ph < 0; ++k) {
-                const int c = (last + k) & 3;
-                if (c != 1 && ready(c, kLag)) ph = c;
+            for (int k = 1; k <= 4 && c < 0; ++k) {
+                const int t = (last + k) & 3;
+                if (t != 1 && ph[t].from <= pos) c = t;
             }
         }
-        for (int c = 1; c < 4 && ph < 0; ++c)          // the tail: nothing is far enough behind
-            if (ready(c, 0)) ph = c;
-        emit(ph);
-        if (ph != 1) last = ph;
+        for (int t = 1; t < 4 && c < 0; ++t)           // the tail: nothing is far enough behind
+            if (ph[t].from != kNever) c = t;
+        emit(c);
+        if (c != 1) last = c;
     }
 }
 
