@@ -161,8 +161,9 @@ ws_status ws_plan_upload(ws_plan* plan, void* dev_buf, size_t bytes, void* strea
  *                            cudaMemcpyAsync on `stream`; call once, before the plan is shared
  *                            between threads
  * Afterwards ws_shard_update / ws_fused_update with r == -1 and WS_LAMB (and
- * ws_lamb_update_static_scratch) take the one-kernel route when there are 8 to 32 gradient copies -
- * where it measured faster on a B200; other cases, WS_LARS and the shard-by-shard calls run as
+ * ws_lamb_update_static_scratch) take the one-kernel route when there are 8 to 32 gradient copies, WS_LARS
+ * when there are 4 to 32 and WS_ADAFACTOR always - where it measured faster on a B200 (Adafactor's blocks and
+ * their order are part of the same upload); other cases and the shard-by-shard calls run as
  * before.  The kernel's waits (a phase-2 item waits for its tensor's ratio) are bounded: if one
  * ever runs out, the kernel leaves the update incomplete and sets the 32-bit status word inside
  * the workspace (ws_workspace_sync_status gives its byte offset; 0 = completed) - a caller that

@@ -666,29 +666,6 @@ __global__ void __launch_bounds__(kBlock, kMinBlocks) af_kernel(const AfLaunch P
     if (!P.master) zero_pads(P, T);
 }
 
-// Clears the sums, counters and words in front of the kernel (a 16-byte aligned range, a multiple of 16 bytes).
-__global__ void __launch_bounds__(kBlock) af_clear_kernel(uint4* a, long long na, int* status) {
-    asm volatile("griddepcontrol.launch_dependents;");
-    asm volatile("griddepcontrol.wait;" ::: "memory");     // an earlier step may still be using them
-    const long long n = (long long)gridDim.x * kBlock;
-    for (long long i = (long long)blockIdx.x * kBlock + threadIdx.x; i < na; i += n) a[i] = make_uint4(0u, 0u, 0u, 0u);
-    if (blockIdx.x == 0 && threadIdx.x == 0) *status = 0;
-}
-
-template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(void (*kernel)(KArgs...), long long grid, cudaStream_t st, const Args&... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3(kBlock);
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
-}
-
 template <bool GBF, int RB, int U, bool LOOPK, int NP>
 ws_status launch(const AfLaunch& P, const void* const* gptrs, cudaStream_t st) {
     GradPtrs<NP> gp;
@@ -712,11 +689,7 @@ ws_status launch_r(const AfLaunch& P, const void* const* gptrs, cudaStream_t st)
 }  // namespace
 
 ws_status launch_af(const AfLaunch& P, bool gbf, const void* const* gptrs, void* clear, size_t clear_bytes, cudaStream_t st) {
-    const long long n16 = (long long)(clear_bytes / 16);
-    long long grid = (n16 + kBlock - 1) / kBlock;
-    if (grid > 296) grid = 296;
-    launch_pdl(af_clear_kernel, grid < 1 ? 1 : grid, st, (uint4*)clear, n16, P.status);
-    const ws_status s = ws_check_launch("one-kernel Adafactor (clear)");
+    const ws_status s = launch_clear(clear, clear_bytes, P.status, st);
     if (s != WS_OK) return s;
     return gbf ? launch_r<true>(P, gptrs, st) : launch_r<false>(P, gptrs, st);
 }

@@ -719,6 +719,25 @@ __device__ __forceinline__ void process_item(const UpdParams& P, const GradPtrs<
 }
 
 
+// Programmatic dependent launch: the grid may become resident while the previous kernel of the stream drains;
+// a kernel launched this way touches nothing that kernel may write before its griddepcontrol.wait.
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl(void (*kernel)(KArgs...), long long grid, cudaStream_t st, const Args&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3(kBlock);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+}
+// Clears the counters and words of a one-kernel update (a 16-byte aligned range, a multiple of 16 bytes) and its
+// status word.  A kernel and not a memset, so that it and the update chain by programmatic dependent launch.
+ws_status launch_clear(void* p, size_t bytes, int* status, cudaStream_t st);
+
 // ---------------------------------------------------------- one-launch update ---
 // What the one-kernel LAMB / LARS update (ws_onelaunch.cu) needs beyond UpdParams: the plan's
 // schedule and the synchronisation scratch inside the workspace.

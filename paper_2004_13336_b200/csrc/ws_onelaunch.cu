@@ -73,6 +73,8 @@ two_phase_kernel(const UpdParams P, const __grid_constant__ GradPtrs<NP> gp, con
     __shared__ double fin_a[kBlock / 32], fin_b[kBlock / 32];   // (small on purpose: shared memory comes out of the L1)
     __shared__ int s_last;
     const int tid = threadIdx.x;
+    asm volatile("griddepcontrol.launch_dependents;");
+    asm volatile("griddepcontrol.wait;" ::: "memory");     // the counters are cleared by the kernel in front
 
     if (tid == 0) s_word = atomicAdd(Q.ticket, 1ULL);
     __syncthreads();
@@ -192,7 +194,7 @@ ws_status launch(const UpdParams& P, const void* const* gptrs, const OneLaunch& 
     auto kern = two_phase_kernel<PAIR, GBF, OUT, VEC1, U1, RB, NP, VEC2, FUSED>;
     const long long grid = Q.nsched;            // one CTA per schedule entry
     if (grid < 1) return WS_OK;
-    kern<<<(unsigned)grid, kBlock, 0, st>>>(P, gp, Q);
+    launch_pdl(kern, grid, st, P, gp, Q);
     return ws_check_launch("one-launch update");
 }
 
@@ -230,19 +232,37 @@ ws_status launch_o(const UpdParams& P, const void* const* gptrs, const OneLaunch
     }
 }
 
+__global__ void __launch_bounds__(kBlock) clear_kernel(uint4* a, long long n16, int* status) {
+    asm volatile("griddepcontrol.launch_dependents;");
+    asm volatile("griddepcontrol.wait;" ::: "memory");     // an earlier step may still be using them
+    const long long n = (long long)gridDim.x * kBlock;
+    for (long long i = (long long)blockIdx.x * kBlock + threadIdx.x; i < n16; i += n) a[i] = make_uint4(0u, 0u, 0u, 0u);
+    if (blockIdx.x == 0 && threadIdx.x == 0) *status = 0;
+}
+
 }  // namespace
 
-// Where the one-kernel route measured faster than the three launches on a B200: LAMB with 8 to 32
-// gradient copies (BERT-large set, R = 16: 4.87 ms against 5.13 ms, R = 8: 3.27 against 3.46 ms;
-// Transformer set under LAMB: 5 % faster at R = 8, 3.6 % at R = 32).  With few copies phase 1 is as
-// short as phase 2 and the three launches win (Transformer set, R = 4: 1.64 ms against 1.67 ms, R = 2:
-// 1.38 against 1.49 ms), and so they do for LARS on the ResNet-50 set, whose 161 mostly tiny tensors
-// make a step of 0.24 ms.
-bool one_launch_supports(int pair, int R) { return pair == 0 && R >= 8 && R <= 32; }
+ws_status launch_clear(void* p, size_t bytes, int* status, cudaStream_t st) {
+    const long long n16 = (long long)(bytes / 16);
+    long long grid = (n16 + kBlock - 1) / kBlock;
+    if (grid > 296) grid = 296;
+    launch_pdl(clear_kernel, grid < 1 ? 1 : grid, st, (uint4*)p, n16, status);
+    return ws_check_launch("one-kernel update (clear)");
+}
+
+// Where the one-kernel route measured faster than the three launches on a B200.  LAMB with 8 to 32 gradient
+// copies (BERT-large set, R = 16: 4.85 ms against 5.13 ms; with items of their own size instead of the plan's
+// tiles: ResNet-50 set 324 -> 253 us, a 37.6 M parameter Transformer 463 -> 361 us, a 1.7 M parameter one 40 ->
+// 28 us, R = 8 each); with few copies phase 1 is as short as phase 2 and the three launches win (Transformer
+// set, R = 4: 1.64 ms against 1.67 ms, R = 2: 1.38 against 1.49 ms).  LARS with 4 to 32 copies (ResNet-50 set,
+// R = 8: 234 -> 226 us; Transformer set, R = 4: 1418 -> 1386 us, R = 16 bf16: 2036 -> 1845 us; 45 792 parameters:
+// 14.6 -> 8.7 us); at R = 2 the three launches win by 1 % (152 against 154 us).
+bool one_launch_supports(int pair, int R) { return R <= 32 && R >= (pair == 0 ? 8 : 4); }
 
 ws_status launch_one_launch(int pair, bool gbf, int out, bool fused, bool wide, const UpdParams& P,
                             const void* const* gptrs, const OneLaunch& Q, cudaStream_t st) {
-    if (pair != 0) return WS_ERR_INVALID_ARG;
+    if (pair == 1)
+        return gbf ? launch_o<1, true>(P, gptrs, Q, out, fused, wide, st) : launch_o<1, false>(P, gptrs, Q, out, fused, wide, st);
     return gbf ? launch_o<0, true>(P, gptrs, Q, out, fused, wide, st) : launch_o<0, false>(P, gptrs, Q, out, fused, wide, st);
 }
 

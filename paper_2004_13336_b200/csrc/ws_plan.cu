@@ -135,14 +135,40 @@ static void ws_count_af(ws_plan* p) {
     p->af_ghat = g;
 }
 
-// Work items of the one-launch schedule: every tile cut into runs of kWsItemElems elements, for every
-// shard it serves.  Plans beyond the item fields' ranges get no schedule (n_items stays 0).
+// Work items of the one-launch schedule: every run of consecutive positions of one tensor in one shard (a piece;
+// in the concatenated layout what lies of the tensor in the shard), cut into items.  8192 elements per item - a
+// CTA pays its chain of table reads per item - and fewer where that would leave less than 750 items (1.7 waves).
+template <typename F>
+static void ws_lamb_items(const ws_plan* p, F&& emit) {
+    const bool concat = p->layout == WS_LAYOUT_CONCAT;
+    long long item = kWsItemElems;
+    while (item > 1024 && p->N / item < 750) item >>= 1;
+    auto cut = [&](int t, int shard, long long pos, long long toff, long long len, long long valid) {
+        for (long long so = 0; so < len; so += item)
+            emit(t, shard, pos + so, toff + so, len - so < item ? len - so : item, valid - so);
+    };
+    for (int t = 0; t < p->T; ++t) {
+        const ws_segment& g = p->segs[t];
+        if (!concat) {
+            for (int r = 0; r < p->R; ++r) cut(t, r, g.shard_off, r * g.piece, g.piece, g.numel - r * g.piece);
+            continue;
+        }
+        const WsSegTiles st = p->segtiles[t];
+        for (int k = 0; k < st.tile_count;) {          // a tensor's tiles of one shard are neighbours
+            const WsTile& first = p->tiles[st.tile_begin + k];
+            long long len = 0;
+            for (; k < st.tile_count && p->tiles[st.tile_begin + k].shard == first.shard; ++k) len += p->tiles[st.tile_begin + k].len;
+            cut(t, first.shard, first.pos, first.poff, len, first.vt);
+        }
+    }
+}
+
+// Plans beyond the item fields' ranges get no schedule (n_items stays 0).
 static void ws_count_items(ws_plan* p) {
     p->n_items = 0;
     if (p->R > 65535) return;
-    long long per_shard = 0;
-    for (const WsTile& tl : p->tiles) per_shard += (tl.len + kWsItemElems - 1) / kWsItemElems;
-    const long long n = p->layout == WS_LAYOUT_CONCAT ? per_shard : per_shard * p->R;
+    long long n = 0;
+    ws_lamb_items(p, [&](int, int, long long, long long, long long, long long) { ++n; });
     if (n > 0x3fffffffLL) return;
     p->n_items = n;
 }
@@ -479,37 +505,25 @@ constexpr long long kGroupBytes = 6LL << 20;    // state bytes (12 per element) 
 constexpr int kLag = 512;
 
 void ws_build_schedule(ws_plan* p) {
-    const int T = p->T, R = p->R;
-    const bool concat = p->layout == WS_LAYOUT_CONCAT;
+    const int T = p->T;
     p->items.clear();
     p->items.reserve((size_t)p->n_items);
     p->itemsegs.assign(T, WsItemSeg{0, 0});
     std::vector<long long> seg_bytes(T, 0);
-    for (int t = 0; t < T; ++t) {
-        p->itemsegs[t].first = (int)p->items.size();
-        const WsSegTiles st = p->segtiles[t];
-        for (int r = 0; r < (concat ? 1 : R); ++r)
-            for (int k = 0; k < st.tile_count; ++k) {
-                const WsTile& tl = p->tiles[st.tile_begin + k];
-                const long long toff0 = concat ? tl.poff : (long long)r * tl.piece + tl.poff;
-                const long long valid0 = concat ? tl.vt : tl.vt - (long long)r * tl.piece;
-                for (int so = 0; so < tl.len; so += kWsItemElems) {
-                    WsItem it;
-                    memset(&it, 0, sizeof(it));
-                    const int len = tl.len - so < kWsItemElems ? tl.len - so : kWsItemElems;
-                    long long nv = valid0 - so;
-                    it.pos = tl.pos + so;
-                    it.toff = toff0 + so;
-                    it.seg = t;
-                    it.nvalid = (int)(nv < 0 ? 0 : (nv > len ? len : nv));
-                    it.len = (unsigned short)len;
-                    it.shard = (unsigned short)(concat ? tl.shard : r);
-                    p->items.push_back(it);
-                    seg_bytes[t] += 12LL * len;
-                }
-            }
-        p->itemsegs[t].count = (int)p->items.size() - p->itemsegs[t].first;
-    }
+    ws_lamb_items(p, [&](int t, int shard, long long pos, long long toff, long long len, long long valid) {
+        WsItem it;
+        it.pos = pos;
+        it.toff = toff;
+        it.seg = t;
+        it.nvalid = (int)(valid < 0 ? 0 : (valid > len ? len : valid));
+        it.len = (unsigned short)len;
+        it.shard = (unsigned short)shard;
+        it.flags = 0;
+        p->items.push_back(it);
+        ++p->itemsegs[t].count;
+        seg_bytes[t] += 12LL * len;
+    });
+    for (int t = 1; t < T; ++t) p->itemsegs[t].first = p->itemsegs[t - 1].first + p->itemsegs[t - 1].count;
     // groups of consecutive tensors
     struct Group { int first, end; };     // item range
     std::vector<Group> groups;

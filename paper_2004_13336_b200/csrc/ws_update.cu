@@ -714,8 +714,7 @@ ws_status try_one_launch(const ws_plan* plan, int pair, const ws_grads* grads, c
     Q.norms = L.norms;
     Q.eta = hyper->trust_coeff;
     Q.beta = hyper->weight_decay;
-    cudaError_t e = cudaMemsetAsync(L.count, 0, L.sync_bytes, st);     // counters, ready words, ticket, status
-    if (e != cudaSuccess) return ws_cuda_fail(e, "one-launch update (clear counters)");
+    if ((s = launch_clear(L.count, L.sync_bytes, L.status, st)) != WS_OK) return s;     // counters, ready words, ticket, status
     s = launch_one_launch(pair, gbf, out_kind, fused, wide, P, fused ? nullptr : gp.data(), Q, st);
     if (s == WS_OK) done = true;
     return s;
