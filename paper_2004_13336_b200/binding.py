@@ -9,6 +9,7 @@ from __future__ import annotations
 
 import ctypes as C
 import os
+import struct
 from typing import List, Optional, Sequence
 
 import torch
@@ -213,6 +214,28 @@ def lib() -> C.CDLL:
     return L
 
 
+_step_lib = None
+
+
+def _step():
+    """The entry points of a training step on a second handle of the library whose prototypes take plain
+    addresses: converting a ctypes pointer per struct argument cost more than the rest of a small call."""
+    global _step_lib
+    if _step_lib is None:
+        lib()
+        S = C.CDLL(LIB_PATH)
+        vp, i32, size = C.c_void_p, C.c_int32, C.c_size_t
+        for name, args in (("ws_pack", [vp, vp, C.c_int, vp, vp]), ("ws_unpack", [vp, vp, C.c_int, vp, vp]),
+                           ("ws_pack_sets", [vp, vp, vp, vp]),
+                           ("ws_shard_update", [vp, i32, vp, vp, vp, vp, vp, size, vp]),
+                           ("ws_fused_update", [vp, i32, vp, vp, vp, vp, vp, size, vp])):
+            f = getattr(S, name)
+            f.restype = C.c_int
+            f.argtypes = args
+        _step_lib = S
+    return _step_lib
+
+
 def debug_bounds_read(clear: bool = True) -> int:
     """Bits of the bounds-checking debug build's status word (synchronises the device)."""
     bits = C.c_uint32()
@@ -227,6 +250,14 @@ def _check(status: int, what: str):
 
 def _stream() -> int:
     return torch.cuda.current_stream().cuda_stream
+
+
+# the same from torch's own accessors, without a Stream object per call, where this torch has them
+if hasattr(torch._C, "_cuda_getCurrentRawStream") and hasattr(torch._C, "_cuda_getDevice"):
+    def _stream() -> int:  # noqa: F811
+        if not torch.cuda.is_initialized():
+            return torch.cuda.current_stream().cuda_stream
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _dtype_code(dt: torch.dtype) -> int:
@@ -262,12 +293,17 @@ def _ptr_array(tensors):
     return arr
 
 
+_HYPER = struct.Struct("@i4x7dq4d")          # ws_hyper as the C compiler lays it out
+assert _HYPER.size == C.sizeof(ws_hyper)
+
+
 def make_hyper(opt, hyper: dict) -> ws_hyper:
     code = OPT_CODE[opt] if isinstance(opt, str) else int(opt)
-    return ws_hyper(code, hyper["lr"], hyper["beta1"], hyper["beta2"], hyper["eps"],
-                    hyper["weight_decay"], hyper["momentum"], hyper["grad_scale"], int(hyper["step"]),
-                    float(hyper.get("trust_coeff", 0.001)), float(hyper.get("eps2", 1e-3)),
-                    float(hyper.get("clip_threshold", 1.0)), float(hyper.get("decay_exponent", 0.8)))
+    get = hyper.get
+    return ws_hyper.from_buffer_copy(_HYPER.pack(
+        code, hyper["lr"], hyper["beta1"], hyper["beta2"], hyper["eps"], hyper["weight_decay"], hyper["momentum"],
+        hyper["grad_scale"], int(hyper["step"]), get("trust_coeff", 0.001), get("eps2", 1e-3),
+        get("clip_threshold", 1.0), get("decay_exponent", 0.8)))
 
 
 class Plan:
@@ -383,12 +419,16 @@ class Plan:
 
 def ws_pack(plan: Plan, tensors: Sequence[torch.Tensor], flat: torch.Tensor):
     dt = _dtype_code(flat.dtype)
-    _check(lib().ws_pack(plan.handle, _ptr_array(tensors), dt, flat.data_ptr(), _stream()), "ws_pack")
+    st = _step().ws_pack(plan.handle, _ptr_array(tensors), dt, flat.data_ptr(), _stream())
+    if st:
+        raise WsError(st, "ws_pack")
 
 
 def ws_unpack(plan: Plan, flat: torch.Tensor, tensors: Sequence[torch.Tensor]):
     dt = _dtype_code(flat.dtype)
-    _check(lib().ws_unpack(plan.handle, flat.data_ptr(), dt, _ptr_array(tensors), _stream()), "ws_unpack")
+    st = _step().ws_unpack(plan.handle, flat.data_ptr(), dt, _ptr_array(tensors), _stream())
+    if st:
+        raise WsError(st, "ws_unpack")
 
 
 def _grads(gbufs: Sequence[torch.Tensor], slice_mode: int):
@@ -403,6 +443,17 @@ def _state(w, m, v):
                     v.data_ptr() if v is not None else None)
 
 
+# ws_state and ws_out as the C compiler lays them out; a bytes object is passed by its address
+_STATE = struct.Struct("@PPP")
+_OUT = struct.Struct("@Pi4x")
+assert _STATE.size == C.sizeof(ws_state) and _OUT.size == C.sizeof(ws_out)
+
+
+def _state_bytes(w, m, v):
+    return _STATE.pack(w.data_ptr() if w is not None else 0, m.data_ptr() if m is not None else 0,
+                       v.data_ptr() if v is not None else 0)
+
+
 def _out(gathered):
     if gathered is None:
         return None
@@ -412,12 +463,14 @@ def _out(gathered):
 def ws_shard_update(plan: Plan, r: int, gbufs: Sequence[torch.Tensor], w, m, v, hyper: ws_hyper,
                     gathered: Optional[torch.Tensor] = None, workspace: Optional[torch.Tensor] = None,
                     slice_mode: int = 0):
-    g, s, o = _grads(gbufs, slice_mode), _state(w, m, v), _out(gathered)
-    _check(lib().ws_shard_update(plan.handle, r, C.byref(g), C.byref(s), C.byref(hyper),
-                                 C.byref(o) if o is not None else None,
-                                 workspace.data_ptr() if workspace is not None else None,
-                                 workspace.numel() * workspace.element_size() if workspace is not None else 0,
-                                 _stream()), "ws_shard_update")
+    g = _grads(gbufs, slice_mode)
+    st = _step().ws_shard_update(
+        plan.handle, r, C.addressof(g), _state_bytes(w, m, v), C.addressof(hyper),
+        _OUT.pack(gathered.data_ptr(), _dtype_code(gathered.dtype)) if gathered is not None else None,
+        workspace.data_ptr() if workspace is not None else None,
+        workspace.numel() * workspace.element_size() if workspace is not None else 0, _stream())
+    if st:
+        raise WsError(st, "ws_shard_update")
 
 
 def ws_lamb_partial(plan: Plan, r: int, gbufs, w, m, v, hyper: ws_hyper, workspace: torch.Tensor,
@@ -558,13 +611,16 @@ class TensorTable:
 
 def ws_fused_update(plan: Plan, r: int, grads: TensorTable, w, m, v, hyper: ws_hyper, weights: TensorTable,
                     workspace: Optional[torch.Tensor] = None):
-    s = _state(w, m, v)
-    _check(lib().ws_fused_update(plan.handle, r, C.byref(grads.c), C.byref(s), C.byref(hyper), C.byref(weights.c),
-                                 workspace.data_ptr() if workspace is not None else None,
-                                 workspace.numel() * workspace.element_size() if workspace is not None else 0,
-                                 _stream()), "ws_fused_update")
+    st = _step().ws_fused_update(
+        plan.handle, r, C.addressof(grads.c), _state_bytes(w, m, v), C.addressof(hyper), C.addressof(weights.c),
+        workspace.data_ptr() if workspace is not None else None,
+        workspace.numel() * workspace.element_size() if workspace is not None else 0, _stream())
+    if st:
+        raise WsError(st, "ws_fused_update")
 
 
 def ws_pack_sets(plan: Plan, table: TensorTable, flats):
     """All sets of a tensor table packed in one launch (set k -> flats[k])."""
-    _check(lib().ws_pack_sets(plan.handle, C.byref(table.c), _ptr_array(flats), _stream()), "ws_pack_sets")
+    st = _step().ws_pack_sets(plan.handle, C.addressof(table.c), _ptr_array(flats), _stream())
+    if st:
+        raise WsError(st, "ws_pack_sets")
