@@ -1,4 +1,4 @@
-// LAMB (and, by the same scheme, LARS) for all shards as ONE kernel.
+// LAMB and LARS for all shards as ONE kernel.
 //
 // Both optimizers need a per-tensor norm ratio before any element of the tensor can take its
 // step (paper Section 4.1, "Non-elementwise operators": the shards' partial reduce results are
