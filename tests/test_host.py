@@ -8,6 +8,7 @@ import re
 
 import numpy as np
 import pytest
+import torch
 
 from oracle import ws_oracle as O
 from paper_2004_13336_b200 import binding as B
@@ -163,6 +164,41 @@ def test_header_is_plain_c_and_links_from_c(tmp_path):
     r = subprocess.run([str(exe)], capture_output=True, text=True)
     assert r.returncode == 0, r.stdout + r.stderr
     assert "piece 73728" in r.stdout and "piece 9216" in r.stdout
+
+
+def test_step_calls_refuse_another_struct():
+    """The step calls hand plain addresses to the library: what is not the expected struct is refused before that
+    (a smaller one would be read past its end), and no call is made."""
+    plan = B.Plan([(64,)], 2, 32, upload=False)
+
+    class Table:
+        c = B.ws_tensor_table()
+
+    class Other:
+        c = B.ws_sched_item()
+
+    for bad, kind in ((B.ws_state(), C.ArgumentError), (C.c_int32(3), C.ArgumentError), ({"lr": 1.0}, TypeError), (None, TypeError)):
+        with pytest.raises(kind):
+            B.ws_shard_update(plan, -1, B.PtrList([torch.zeros(1)]), None, None, None, bad)
+        with pytest.raises(kind):
+            B.ws_fused_update(plan, -1, Table, None, None, None, bad, Table)
+    hy = B.make_hyper("adam", dict(lr=1, beta1=0.9, beta2=0.999, eps=1e-8, weight_decay=0, momentum=0, grad_scale=1, step=1))
+    for tables in ((Other, Table), (Table, Other)):
+        with pytest.raises(C.ArgumentError):
+            B.ws_fused_update(plan, -1, tables[0], None, None, None, hy, tables[1])
+    with pytest.raises(C.ArgumentError):
+        B.ws_pack_sets(plan, Other, B.PtrList([torch.zeros(1)]))
+
+
+def test_make_hyper_takes_what_ctypes_takes():
+    base = dict(lr=1, beta1=0.9, beta2=np.float32(0.5), eps=1e-8, weight_decay=torch.tensor(0.25), momentum=0,
+                grad_scale=1, step=np.int64(7), trust_coeff="0.5", decay_exponent="0.75")
+    h = B.make_hyper("lars", base)
+    assert (h.opt, h.lr, h.beta2, h.weight_decay, h.step) == (B.WS_LARS, 1.0, 0.5, 0.25, 7)
+    assert (h.trust_coeff, h.eps2, h.clip_threshold, h.decay_exponent) == (0.5, 1e-3, 1.0, 0.75)
+    with pytest.raises(TypeError):
+        B.make_hyper("lars", dict(base, lr="0.1"))
+    assert B.make_hyper(2 ** 32 + 1, base).opt == 1                    # a ctypes integer wraps
 
 
 def test_factored_layout_matches_oracle_view():
