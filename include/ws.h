@@ -148,12 +148,11 @@ ws_status ws_plan_upload(ws_plan* plan, void* dev_buf, size_t bytes, void* strea
  * of a tensor before any shard can apply the step (Section 4.1), so their all-shard update is
  * phase 1, a combination step, phase 2.  As three launches, phase 2 reads the weight and the new
  * moments from DRAM again.  A plan whose schedule has been uploaded runs WS_LAMB's all-shard update
- * as ONE kernel instead: the two phases of every tensor are work items (runs of up to 8192 shard
- * positions) ordered so that a tensor's phase 2 follows its phase 1 at a short distance, while other
+ * as ONE kernel instead: the two phases of every tensor are work items (one or several whole work
+ * tiles, several up to 8192 shard positions) ordered so that a tensor's phase 2 follows its phase 1 at a short distance, while other
  * tensors' phase 1 streams from DRAM, and phase 2 finds part of its operands in L2 (toward the
- * update of Section 2.2, where every operand crosses HBM once).  Results: the same as the
- * three-launch form up to the order of the norm sums (the ratios agree to rounding; they are
- * bit-stable from run to run).
+ * update of Section 2.2, where every operand crosses HBM once).  Results: bit for bit those of the
+ * three-launch form (the partial norms are the tiles' and are summed in the same order).
  *   ws_plan_schedule_bytes   device bytes of the schedule (0: this plan has none - more than
  *                            65535 shards or 2^30 work items)
  *   ws_plan_upload_schedule  builds the schedule on first use and copies it into the caller's
@@ -304,8 +303,8 @@ ws_status ws_plan_factored_layout(const ws_plan* plan, int64_t* layout);
  *   double norms[T][2]       squared norms (sum w^2, sum u^2) per tensor
  *   float  partials[R][tiles][2]   per-tile partial sums from phase 1
  *                                  ([tiles][2] for the concatenated layout)
- *   (scratch of the one-launch route: per-item partial sums, per-tensor
- *    counters and flags, a ticket counter and the status word)
+ *   (scratch of the one-launch route: per-tensor counters and flags, a
+ *    ticket counter and the status word)
  * so a caller can read rho and the norms back for logging.  WS_LARS uses the
  * same arrays (rho holds the local rates, norms sum w^2 and sum g^2)
  * followed, at the next 256-byte boundary, by

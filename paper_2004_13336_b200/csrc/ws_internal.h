@@ -67,25 +67,26 @@ struct WsAfChunk {
 };
 
 // One-launch schedule of the norm-based optimizers (LAMB, LARS): the update of all shards as ONE
-// kernel.  A work item is a run of at most kWsItemElems consecutive shard positions inside
-// one tile; every item appears twice in the schedule, once for phase 1 (reduce, moments, partial
-// norm sums) and once for phase 2 (apply the step with the tensor's ratio).
-constexpr int kWsItemElems = 8192;
+// kernel.  A work item is one or several consecutive whole tiles of a tensor in one shard; every item
+// appears twice in the schedule, once for phase 1 (reduce, moments, partial norm sums of every tile)
+// and once for phase 2 (apply the step with the tensor's ratio).
+constexpr int kWsItemElems = 8192;    // an item of several tiles has at most this many elements
+constexpr int kWsItemTiles = 8;       // ... and tiles
 struct __align__(16) WsItem {
-    long long pos;        // start inside the shard, multiple of 8
+    unsigned long long pos_shard;   // (start inside the shard, multiple of 8) << 16 | shard
     long long toff;       // element index of the first element inside tensor `seg`
     int seg;              // tensor index
     int nvalid;           // elements of the item that exist in the tensor (the rest is padding)
-    unsigned short len;   // elements, multiple of 8
-    unsigned short shard;
-    unsigned flags;       // bit 0: the tensor group is small enough to stay in L2 between its phases
+    int len;              // elements, multiple of 8
+    int tile;             // its first tile (per-tensor layout: of the shard's; concatenated: of all)
 };
 static_assert(sizeof(WsItem) == 32, "WsItem is read as two 16-byte words");
-// Items are numbered tensor by tensor (then shard by shard), so a tensor's items - and with them its
-// partial norm sums - are one contiguous range.
-struct WsItemSeg {
+// Items are numbered tensor by tensor (then shard by shard): a tensor's items are one contiguous range.
+struct __align__(16) WsItemSeg {
     int first;
     int count;
+    int tile_begin;       // its tiles, as in WsSegTiles
+    int tile_count;
 };
 
 // Adafactor's all-shard update as one kernel (ws_af_onelaunch.cu).  A work item is a block of a tensor's
@@ -165,9 +166,8 @@ struct WsLambWs {
     float* rho;        // [T]
     double* norms;     // [T][2]
     float2* partials;  // [R][ntiles]
-    // one-launch update: per-item partial sums, per-tensor arrival counters and ready flags, the
-    // ticket counter and the status word (sync_bytes from `count` on are cleared before every launch)
-    float2* ipart;     // [n_items]
+    // one-launch update: per-tensor arrival counters and ready flags, the ticket counter and the
+    // status word (sync_bytes from `count` on are cleared before every launch)
     int* count;        // [T]
     unsigned long long* flag;   // [T] ready words
     unsigned long long* ticket;

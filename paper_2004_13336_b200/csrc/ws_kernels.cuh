@@ -286,9 +286,60 @@ struct ItemCtx {
     long long sbase;     // ... inside w / m / v
     long long obase;     // ... inside the gathered buffer and the stored gradient sum
     long long toff;      // ... inside tensor `seg` (fused formatting, Adafactor's rows and columns)
-    float2* partial;     // where a phase-1 item leaves its two partial sums
+    float2* partial;     // where a phase-1 item leaves its two partial sums (TILES: those of its first tile)
     bool keep;           // HINT only: the state this item touches is read again soon (keep it in L2)
+    int unit;            // TILES only: elements of a tile
 };
+
+// Sums a tensor's per-tile partials over all shards in a fixed order, in double (stands where the paper combines
+// per-replica reduce results with one batched scalar all-reduce, Section 4.1 / 5.2); the totals are valid in
+// thread 0.  One function for the finalize step and for the one-kernel routes, so that both give the same bits.
+// R: strided repetitions of the tensor's tile run; sa, sb: kBlock/32 doubles of shared memory each.
+__device__ __forceinline__ void sum_partials(const WsSegTiles st, const float2* partials, long long ntiles, int R,
+                                             double* sa, double* sb, double& a, double& b) {
+    const long long n = (long long)R * st.tile_count;
+    a = 0.0;
+    b = 0.0;
+    constexpr int U = 8;                                  // loads in flight per thread
+    // partial i is tile i % tile_count of repetition i / tile_count; a thread takes every kBlock-th one
+    const int tc = st.tile_count > 0 ? st.tile_count : 1, dr = kBlock / tc, dk = kBlock - dr * tc;
+    int r = (int)threadIdx.x / tc, k = (int)threadIdx.x - r * tc;
+    for (long long i0 = threadIdx.x; i0 < n; i0 += U * kBlock) {
+        float2 p[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            p[u] = make_float2(0.f, 0.f);
+            if (i0 + u * kBlock < n) p[u] = __ldcg(partials + r * ntiles + st.tile_begin + k);
+            r += dr;
+            k += dk;
+            if (k >= tc) {
+                k -= tc;
+                ++r;
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            a += (double)p[u].x;
+            b += (double)p[u].y;
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {                    // fixed tree inside the warp ...
+        a += __shfl_xor_sync(0xffffffffu, a, o);
+        b += __shfl_xor_sync(0xffffffffu, b, o);
+    }
+    if ((threadIdx.x & 31) == 0) {
+        sa[threadIdx.x >> 5] = a;
+        sb[threadIdx.x >> 5] = b;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int i = 1; i < kBlock / 32; ++i) {           // ... and the warps in order
+            a += sa[i];
+            b += sb[i];
+        }
+    }
+}
 
 // Sums two values over the CTA at once (one pair of barriers for both); the totals are valid in
 // thread 0.  The order of the additions is fixed, so the result is run-to-run bit-stable.
@@ -361,10 +412,14 @@ __device__ __forceinline__ Fv<VEC> load_f32_partial(const float* p, int n) {
 // OUT == O_F32M the fp32 weight tensors are the master copy themselves: the weight is read
 // from its tensor and written back there, and no sharded copy of w exists.
 // HINT: see ItemCtx::keep.
+// TILES: a phase-1 item of up to kWsItemTiles whole tiles that leaves every tile's partial sums, each formed in
+// the order in which an item of that one tile forms it (the two forms of the update then have the same norms bit
+// for bit): a tile's sums leave the registers with the pass that ends it, without a barrier, and are put together
+// at the end of the item.  red then has 8 * kWsItemTiles entries, and the totals are written by warp 0.
 // sgp: this item's R gradient tensor pointers (FUSED), swp: its weight tensor pointers when the
 // result goes to several weight lists, wt: its first weight tensor; red: kBlock/32 float2 of
 // shared memory.
-template <int OPT, bool GBF, int OUT, int VEC, int U, int RB, int NP, bool FUSED, bool HINT>
+template <int OPT, bool GBF, int OUT, int VEC, int U, int RB, int NP, bool FUSED, bool HINT, bool TILES = false>
 __device__ __forceinline__ void process_item(const UpdParams& P, const GradPtrs<NP>& gp, const ItemCtx& it,
                                              const void* const* sgp, void* const* swp, char* wt, float lr_rho,
                                              float2* red) {
@@ -441,6 +496,25 @@ __device__ __forceinline__ void process_item(const UpdParams& P, const GradPtrs<
             sub_col = (unsigned)(kBlock * VEC) - sub_rl * (unsigned)af.ncol;
         }
     }
+    static_assert(!TILES || U == 1, "a pass ends at most one tile per warp");
+    // (a pass of 8-element vectors over tiles of 1024 has one tile in each half of the CTA)
+    const bool halves = TILES && VEC == 8 && it.unit == 1024;
+    int tile_left = TILES ? it.unit : 0, tile_no = 0;
+    // the sums of the tile that the pass before ended: put together while this pass's loads are in flight
+    float ended_w = 0.f, ended_u = 0.f;
+    bool ended = false;
+    auto flush = [&]() {
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+        // the tree of block_sum2 for both sums at once: the halves of the warp exchange and keep one sum each
+        float x = lane < 16 ? ended_w : ended_u, y = lane < 16 ? ended_u : ended_w;
+        x += __shfl_xor_sync(0xffffffffu, y, 16);
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        float2& slot = red[halves ? (tile_no + (warp >> 2)) * 8 + (warp & 3) : tile_no * 8 + warp];
+        if (lane == 0) slot.x = x;
+        if (lane == 16) slot.y = x;
+        tile_no += halves ? 2 : 1;
+    };
     float cacc[OPT == K_AF1 ? VEC : 1];
     long long cbase = -1;
 #pragma unroll
@@ -502,6 +576,12 @@ __device__ __forceinline__ void process_item(const UpdParams& P, const GradPtrs<
                                 raw[u][j] = load_grad<GBF, VEC>(gp.p[k0 + j], gbase + e0[u]);
                             }
                         }
+                }
+                if constexpr (TILES) {
+                    if (k0 == 0 && ended) {
+                        flush();
+                        ended = false;
+                    }
                 }
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
@@ -705,6 +785,38 @@ __device__ __forceinline__ void process_item(const UpdParams& P, const GradPtrs<
                 store_bf16<VEC>(reinterpret_cast<unsigned short*>(P.gathered) + obase + e0[u], wv[u]);
             }
         }
+        if constexpr (TILES) {
+            tile_left -= kBlock * VEC;
+            if (tile_left <= 0 || q0 + kBlock >= nvec) {
+                ended_w = sw;
+                ended_u = su;
+                ended = true;
+                sw = 0.f;
+                su = 0.f;
+                tile_left = it.unit;
+            }
+        }
+    }
+    if constexpr (TILES) {
+        static_assert(kBlock == 256, "eight warps: a tile's sums are one group of eight lanes");
+        if (ended) flush();
+        __syncthreads();
+        if (threadIdx.x < 32) {
+            const int ntile = (it.len + it.unit - 1) / it.unit, lane = threadIdx.x;
+            for (int b = 0; b < ntile; b += 4) {       // the tree of block_sum2, four tiles at a time
+                const int k = b + (lane >> 3);
+                float2 t = make_float2(0.f, 0.f);
+                if (k < ntile && !(halves && (lane & 7) >= 4)) t = red[k * 8 + (lane & 7)];
+#pragma unroll
+                for (int o = 4; o > 0; o >>= 1) {
+                    t.x += __shfl_xor_sync(0xffffffffu, t.x, o);
+                    t.y += __shfl_xor_sync(0xffffffffu, t.y, o);
+                }
+                if (k < ntile && (lane & 7) == 0) it.partial[k] = t;
+            }
+            __syncwarp();
+        }
+        return;
     }
     if constexpr (OPT == K_AF1) {
         // (these adds of partial reduce results across tiles and shards stand where the paper
@@ -747,7 +859,8 @@ struct OneLaunch {
     const WsItem* items;
     const WsItemSeg* segs;       // [T] item range of every tensor
     int T;
-    float2* ipart;               // [items] partial norm sums of every item's phase 1
+    int reps;                    // strided repetitions of a tensor's tile run in P.partials (see sum_partials)
+    int unit;                    // elements of a tile
     int* count;                  // [T] finished phase-1 items per tensor        (cleared before the launch)
     unsigned long long* flag;    // [T] (ratio bits << 32) | 1 once the ratio is known (cleared before the launch)
     unsigned long long* ticket;  // next schedule entry to hand out              (cleared before the launch)

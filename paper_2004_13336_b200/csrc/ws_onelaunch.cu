@@ -11,7 +11,9 @@
 // One CTA per schedule entry.  A CTA draws a ticket from a global counter when it starts running and
 // takes the schedule entry of that number, so entries are started in schedule order whatever order the
 // hardware launches CTAs in.  The CTA that completes a tensor's last phase-1 item sums the tensor's
-// partial norms in a fixed order in double (run-to-run bit-stable) and publishes the ratio.
+// partial norms in a fixed order in double and publishes the ratio.  The partial norms are those of the plan's
+// tiles, formed and summed as the separate launches form and sum them: the update has the same bits in both forms,
+// and a replica that runs its own shard's phases has the bits of the all-shard call.
 //
 // Progress: a phase-2 entry waits only for phase-1 entries that come earlier in the schedule.  Tickets
 // are drawn by running CTAs, so every earlier entry belongs to a CTA that is running or has finished,
@@ -61,15 +63,16 @@ __device__ __forceinline__ const void* ld_ptr(const void* const* p) {
 // PAIR 0: LAMB, 1: LARS.  VEC1, U1, RB, NP: phase 1's vector width, accesses per pass, tree block and
 // pointer capacity; VEC2: phase 2's vector width.  Other parameters as for process_item.
 // One CTA per schedule entry; the CTA's entry is the ticket it draws when it starts running.
-template <int PAIR, bool GBF, int OUT, int VEC1, int U1, int RB, int NP, int VEC2, bool FUSED>
-__global__ void __launch_bounds__(kBlock, RB > 8 ? kMinBlocksWide : kMinBlocks)
+// TILES: items of several tiles (see process_item).
+template <int PAIR, bool GBF, int OUT, int VEC1, int U1, int RB, int NP, int VEC2, bool FUSED, bool TILES>
+__global__ void __launch_bounds__(kBlock, kMinBlocks)
 two_phase_kernel(const UpdParams P, const __grid_constant__ GradPtrs<NP> gp, const OneLaunch Q) {
     constexpr int OPT1 = PAIR == 0 ? K_LAMB1 : K_LARS1;
     constexpr int OPT2 = PAIR == 0 ? K_LAMB2 : K_LARS2;
     constexpr int OUT1 = (FUSED && OUT == O_F32M) ? O_F32M : O_NONE;
     __shared__ unsigned long long s_word;      // the ticket, later the tensor's ready word
     __shared__ const void* sgp[FUSED ? NP : 1];
-    __shared__ float2 red[kBlock / 32];
+    __shared__ float2 red[kBlock / 32 * (TILES ? kWsItemTiles : 1)];
     __shared__ double fin_a[kBlock / 32], fin_b[kBlock / 32];   // (small on purpose: shared memory comes out of the L1)
     __shared__ int s_last;
     const int tid = threadIdx.x;
@@ -95,18 +98,20 @@ two_phase_kernel(const UpdParams P, const __grid_constant__ GradPtrs<NP> gp, con
     const char* src = reinterpret_cast<const char*>(Q.items + pidx);
     const uint4 da = ld_u128(src), db = ld_u128(src + 16);
     ItemCtx it;
-    const long long pos = (long long)(((unsigned long long)da.y << 32) | da.x);
-    const int shard = (int)(db.z >> 16);
+    const long long pos = (long long)((((unsigned long long)da.y << 32) | da.x) >> 16);
+    const int shard = (int)(da.x & 0xffffu);
     const long long base = (long long)shard * P.S + pos;
-    it.len = (int)(db.z & 0xffffu);
+    it.len = (int)db.z;
     it.nvalid = (int)db.y;
     it.seg = (int)db.x;
     it.gbase = base;
     it.sbase = base;
     it.obase = base;
     it.toff = (long long)(((unsigned long long)da.w << 32) | da.z);
-    it.partial = Q.ipart + pidx;
-    it.keep = kind == 0 && (db.w & 1u) != 0;
+    it.partial = P.partials + (P.concat ? 0 : (long long)shard * P.ntiles) + (int)db.w;
+    it.keep = kind == 0;      // (phase 2 follows closely, and reads a group back to front: also a tensor many
+                              // times the L2 finds its last-written part there)
+    it.unit = Q.unit;
     char* wt = nullptr;
     if constexpr (FUSED) {
         if (kind == 1 || OUT == O_F32M)
@@ -118,41 +123,20 @@ two_phase_kernel(const UpdParams P, const __grid_constant__ GradPtrs<NP> gp, con
             for (int k = tid; k < P.R; k += kBlock) sgp[k] = ld_ptr(P.gtab + (long long)it.seg * P.R + k);
             __syncthreads();
         }
-        process_item<OPT1, GBF, OUT1, VEC1, U1, RB, NP, FUSED, true>(P, gp, it, sgp, nullptr, wt, 0.f, red);
-        // thread 0 has stored the item's partial sums; count the item, and the CTA that counts a tensor's
-        // last one forms the ratio
+        process_item<OPT1, GBF, OUT1, VEC1, U1, RB, NP, FUSED, true, TILES>(P, gp, it, sgp, nullptr, wt, 0.f, red);
+        // warp 0 has stored the partial sums of the item's tiles; count the item, and the CTA that counts a
+        // tensor's last one forms the ratio
+        const uint4 sg = ld_u128(Q.segs + it.seg);
         if (tid == 0) {
             __threadfence();
-            const WsItemSeg sg = Q.segs[it.seg];
-            s_last = (atomicAdd(Q.count + it.seg, 1) + 1 == sg.count) ? 1 : 0;
+            s_last = (atomicAdd(Q.count + it.seg, 1) + 1 == (int)sg.y) ? 1 : 0;
         }
         __syncthreads();
         if (!s_last) return;
         __threadfence();
-        const WsItemSeg sg = Q.segs[it.seg];
-        double a = 0.0, b = 0.0;
-        for (int i = tid; i < sg.count; i += kBlock) {        // fixed order: bit-stable
-            const float2 p = __ldcg(Q.ipart + sg.first + i);
-            a += (double)p.x;
-            b += (double)p.y;
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {                    // fixed tree inside the warp ...
-            a += __shfl_xor_sync(0xffffffffu, a, o);
-            b += __shfl_xor_sync(0xffffffffu, b, o);
-        }
-        if ((tid & 31) == 0) {
-            fin_a[tid >> 5] = a;
-            fin_b[tid >> 5] = b;
-        }
-        __syncthreads();
+        double a, b;
+        sum_partials(WsSegTiles{(int)sg.z, (int)sg.w}, P.partials, P.ntiles, Q.reps, fin_a, fin_b, a, b);
         if (tid == 0) {
-            a = 0.0;
-            b = 0.0;
-            for (int i = 0; i < kBlock / 32; ++i) {           // ... and the warps in order
-                a += fin_a[i];
-                b += fin_b[i];
-            }
             Q.norms[2 * it.seg] = a;
             Q.norms[2 * it.seg + 1] = b;
             float ratio = 1.0f;
@@ -187,15 +171,21 @@ two_phase_kernel(const UpdParams P, const __grid_constant__ GradPtrs<NP> gp, con
     process_item<OPT2, false, OUT, VEC2, kU2, 1, 1, FUSED, true>(P, none, it, nullptr, nullptr, wt, P.c.lr * rho, red);
 }
 
-template <int PAIR, bool GBF, int OUT, int VEC1, int U1, int RB, int NP, int VEC2, bool FUSED>
-ws_status launch(const UpdParams& P, const void* const* gptrs, const OneLaunch& Q, cudaStream_t st) {
+template <int PAIR, bool GBF, int OUT, int VEC1, int U1, int RB, int NP, int VEC2, bool FUSED, bool TILES>
+ws_status launch_t(const UpdParams& P, const void* const* gptrs, const OneLaunch& Q, cudaStream_t st) {
     GradPtrs<NP> gp;
     for (int k = 0; k < NP; ++k) gp.p[k] = (!FUSED && gptrs && k < P.R) ? gptrs[k] : nullptr;
-    auto kern = two_phase_kernel<PAIR, GBF, OUT, VEC1, U1, RB, NP, VEC2, FUSED>;
+    auto kern = two_phase_kernel<PAIR, GBF, OUT, VEC1, U1, RB, NP, VEC2, FUSED, TILES>;
     const long long grid = Q.nsched;            // one CTA per schedule entry
     if (grid < 1) return WS_OK;
     launch_pdl(kern, grid, st, P, gp, Q);
     return ws_check_launch("one-launch update");
+}
+
+template <int PAIR, bool GBF, int OUT, int VEC1, int U1, int RB, int NP, int VEC2, bool FUSED>
+ws_status launch(const UpdParams& P, const void* const* gptrs, const OneLaunch& Q, cudaStream_t st) {
+    if (Q.unit < kWsItemElems) return launch_t<PAIR, GBF, OUT, VEC1, U1, RB, NP, VEC2, FUSED, true>(P, gptrs, Q, st);
+    return launch_t<PAIR, GBF, OUT, VEC1, U1, RB, NP, VEC2, FUSED, false>(P, gptrs, Q, st);   // (an item is one tile)
 }
 
 // Phase 1's flavour follows the separate-launch kernels: 256-bit accesses when the gradients are

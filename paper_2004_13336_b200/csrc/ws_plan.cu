@@ -136,29 +136,33 @@ static void ws_count_af(ws_plan* p) {
 }
 
 // Work items of the one-launch schedule: every run of consecutive positions of one tensor in one shard (a piece;
-// in the concatenated layout what lies of the tensor in the shard), cut into items.  8192 elements per item - a
-// CTA pays its chain of table reads per item - and fewer where that would leave less than 750 items (1.7 waves).
+// in the concatenated layout what lies of the tensor in the shard), cut into items of whole tiles (the partial
+// norms are the tiles').  Up to 8192 elements per item - a CTA pays its chain of table reads per item - and fewer
+// where that would leave less than 750 items (1.7 waves).  A kernel's pass over an item is 1024 or 2048 elements;
+// several tiles share an item only where a pass ends with a tile, or two tiles of 1024 fill one.
 template <typename F>
 static void ws_lamb_items(const ws_plan* p, F&& emit) {
     const bool concat = p->layout == WS_LAYOUT_CONCAT;
     long long item = kWsItemElems;
     while (item > 1024 && p->N / item < 750) item >>= 1;
-    auto cut = [&](int t, int shard, long long pos, long long toff, long long len, long long valid) {
+    item = (p->K == 1024 || p->K % 2048 == 0) && item > p->K ? item / p->K * p->K : p->K;
+    auto cut = [&](int t, int shard, long long pos, long long toff, long long len, long long valid, int tile) {
         for (long long so = 0; so < len; so += item)
-            emit(t, shard, pos + so, toff + so, len - so < item ? len - so : item, valid - so);
+            emit(t, shard, pos + so, toff + so, len - so < item ? len - so : item, valid - so, tile + (int)(so / p->K));
     };
     for (int t = 0; t < p->T; ++t) {
         const ws_segment& g = p->segs[t];
+        const WsSegTiles st = p->segtiles[t];
         if (!concat) {
-            for (int r = 0; r < p->R; ++r) cut(t, r, g.shard_off, r * g.piece, g.piece, g.numel - r * g.piece);
+            for (int r = 0; r < p->R; ++r) cut(t, r, g.shard_off, r * g.piece, g.piece, g.numel - r * g.piece, st.tile_begin);
             continue;
         }
-        const WsSegTiles st = p->segtiles[t];
         for (int k = 0; k < st.tile_count;) {          // a tensor's tiles of one shard are neighbours
-            const WsTile& first = p->tiles[st.tile_begin + k];
+            const int k0 = st.tile_begin + k;
+            const WsTile& first = p->tiles[k0];
             long long len = 0;
             for (; k < st.tile_count && p->tiles[st.tile_begin + k].shard == first.shard; ++k) len += p->tiles[st.tile_begin + k].len;
-            cut(t, first.shard, first.pos, first.poff, len, first.vt);
+            cut(t, first.shard, first.pos, first.poff, len, first.vt, k0);
         }
     }
 }
@@ -166,9 +170,9 @@ static void ws_lamb_items(const ws_plan* p, F&& emit) {
 // Plans beyond the item fields' ranges get no schedule (n_items stays 0).
 static void ws_count_items(ws_plan* p) {
     p->n_items = 0;
-    if (p->R > 65535) return;
+    if (p->R > 65535 || p->S >= (1LL << 47)) return;
     long long n = 0;
-    ws_lamb_items(p, [&](int, int, long long, long long, long long, long long) { ++n; });
+    ws_lamb_items(p, [&](int, int, long long, long long, long long, long long, int) { ++n; });
     if (n > 0x3fffffffLL) return;
     p->n_items = n;
 }
@@ -423,8 +427,6 @@ WsLambWs ws_lamb_layout(const ws_plan* p, void* workspace) {
     o = round16(o + sizeof(double) * 2 * (size_t)p->T);
     L.partials = (float2*)(b + o);
     o = round16(o + sizeof(float2) * (size_t)(p->layout == WS_LAYOUT_CONCAT ? 1 : p->R) * (size_t)p->ntiles);
-    L.ipart = (float2*)(b + o);
-    o = round16(o + sizeof(float2) * (size_t)p->n_items);
     const size_t sync0 = o;
     L.count = (int*)(b + o);
     o = (o + sizeof(int) * (size_t)p->T + 7) & ~(size_t)7;
@@ -508,17 +510,20 @@ void ws_build_schedule(ws_plan* p) {
     const int T = p->T;
     p->items.clear();
     p->items.reserve((size_t)p->n_items);
-    p->itemsegs.assign(T, WsItemSeg{0, 0});
+    p->itemsegs.assign(T, WsItemSeg{0, 0, 0, 0});
+    for (int t = 0; t < T; ++t) {
+        p->itemsegs[t].tile_begin = p->segtiles[t].tile_begin;
+        p->itemsegs[t].tile_count = p->segtiles[t].tile_count;
+    }
     std::vector<long long> seg_bytes(T, 0);
-    ws_lamb_items(p, [&](int t, int shard, long long pos, long long toff, long long len, long long valid) {
+    ws_lamb_items(p, [&](int t, int shard, long long pos, long long toff, long long len, long long valid, int tile) {
         WsItem it;
-        it.pos = pos;
+        it.pos_shard = (unsigned long long)pos << 16 | (unsigned)shard;
         it.toff = toff;
         it.seg = t;
         it.nvalid = (int)(valid < 0 ? 0 : (valid > len ? len : valid));
-        it.len = (unsigned short)len;
-        it.shard = (unsigned short)shard;
-        it.flags = 0;
+        it.len = (int)len;
+        it.tile = tile;
         p->items.push_back(it);
         ++p->itemsegs[t].count;
         seg_bytes[t] += 12LL * len;
@@ -529,25 +534,17 @@ void ws_build_schedule(ws_plan* p) {
     std::vector<Group> groups;
     {
         long long acc = 0;
-        int gfirst = 0, t0 = 0;
+        int gfirst = 0;
         for (int t = 0; t < T; ++t) {
             acc += seg_bytes[t];
             const bool last = t == T - 1;
             if (acc >= kGroupBytes || last) {
                 const int gend = p->itemsegs[t].first + p->itemsegs[t].count;
-                if (gend > gfirst) {
-                    groups.push_back(Group{gfirst, gend});
-                    // (every group leaves its state in L2 at normal priority: phase 2 reads a group back to
-                    // front, so even a tensor many times the L2 finds its last-written part there)
-                    const unsigned keep = 1u;
-                    for (int i = gfirst; i < gend; ++i) p->items[i].flags = keep;
-                }
+                if (gend > gfirst) groups.push_back(Group{gfirst, gend});
                 gfirst = gend;
                 acc = 0;
-                t0 = t + 1;
             }
         }
-        (void)t0;
     }
     // merge the phase-1 stream and the phase-2 stream
     const long long n = (long long)p->items.size();
@@ -789,8 +786,8 @@ extern "C" ws_status ws_plan_schedule_item(ws_plan* p, int64_t item, ws_sched_it
     if (item < 0 || item >= p->n_items) return WS_ERR_INVALID_ARG;
     const WsItem& it = p->items[(size_t)item];
     out->tensor = it.seg;
-    out->shard = it.shard;
-    out->pos = it.pos;
+    out->shard = (int32_t)(it.pos_shard & 0xffffu);
+    out->pos = (int64_t)(it.pos_shard >> 16);
     out->tensor_off = it.toff;
     out->len = it.len;
     out->nvalid = it.nvalid;

@@ -90,48 +90,19 @@ __global__ void __launch_bounds__(kBlock, ((VEC == 8 && GBF && !FUSED) || RB > 8
     }
 }
 
-// Sum every shard's per-tile partials of tensor t in a fixed order, in double
-// (stands where the paper combines per-replica reduce results with one batched
-// scalar all-reduce, Section 4.1 / 5.2), then rho_t = sqrt(a)/sqrt(b).
+// Sum every shard's per-tile partials of tensor t (sum_partials), then rho_t = sqrt(a)/sqrt(b).
 // With lars != 0 the ratio is the LARS local rate eta sqrt(a) / (sqrt(b) + beta sqrt(a)).
-// Sums tensor t's per-tile partials over all shards in a fixed order, in double; the totals
-// are valid in thread 0.
-__device__ __forceinline__ void sum_partials(const WsSegTiles st, const float2* partials, long long ntiles, int R,
-                                             double& a, double& b) {
-    __shared__ double sa[kBlock], sb[kBlock];
-    const long long n = (long long)R * st.tile_count;
-    a = 0.0;
-    b = 0.0;
-    for (long long i = threadIdx.x; i < n; i += kBlock) {
-        const long long r = i / st.tile_count, k = i - r * st.tile_count;
-        const float2 p = partials[r * ntiles + st.tile_begin + k];
-        a += (double)p.x;
-        b += (double)p.y;
-    }
-    sa[threadIdx.x] = a;
-    sb[threadIdx.x] = b;
-    __syncthreads();
-    for (int s = kBlock / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s) {
-            sa[threadIdx.x] += sa[threadIdx.x + s];
-            sb[threadIdx.x] += sb[threadIdx.x + s];
-        }
-        __syncthreads();
-    }
-    a = sa[0];
-    b = sb[0];
-}
-
 __global__ void __launch_bounds__(kBlock) lamb_finalize_kernel(const WsSegTiles* segtiles, const float2* partials,
                                                                long long ntiles, int R, float* rho, double* norms,
                                                                int lars, double eta, double beta) {
     // R == 1 with the concatenated layout: a tensor's tiles of all shards are one contiguous run
+    __shared__ double sa[kBlock / 32], sb[kBlock / 32];
     const int t = blockIdx.x;
     double a, b;
     const WsSegTiles mine = segtiles[t];
     asm volatile("griddepcontrol.launch_dependents;");
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    sum_partials(mine, partials, ntiles, R, a, b);
+    sum_partials(mine, partials, ntiles, R, sa, sb, a, b);
     if (threadIdx.x == 0) {
         norms[2 * t] = a;
         norms[2 * t + 1] = b;
@@ -190,9 +161,10 @@ __global__ void __launch_bounds__(kBlock) af_finalize_clip_kernel(const WsSegTil
                                                                   const float2* partials, long long ntiles, int R,
                                                                   float* alpha, float* rho, double* norms, double eps2,
                                                                   double rho_step, double d) {
+    __shared__ double sa[kBlock / 32], sb[kBlock / 32];
     const int t = blockIdx.x;
     double sw, su;
-    sum_partials(segtiles[t], partials, ntiles, R, sw, su);
+    sum_partials(segtiles[t], partials, ntiles, R, sa, sb, sw, su);
     if (threadIdx.x == 0) {
         const long long n = segaf[t].numel;
         const double rms_w = n > 0 ? sqrt(sw / (double)n) : 0.0;
@@ -705,7 +677,9 @@ ws_status try_one_launch(const ws_plan* plan, int pair, const ws_grads* grads, c
     Q.items = plan->d_items;
     Q.segs = plan->d_itemsegs;
     Q.T = plan->T;
-    Q.ipart = L.ipart;
+    Q.reps = finalize_reps(plan);
+    Q.unit = plan->K;
+    P.partials = L.partials;
     Q.count = L.count;
     Q.flag = L.flag;
     Q.ticket = L.ticket;

@@ -797,6 +797,44 @@ def test_lars_shard_by_shard_phases(R):
     assert e.value.status == 1
 
 
+@pytest.mark.parametrize("opt,R", [("lamb", 8), ("lamb", 32), ("lars", 5), ("lars", 8)])
+@pytest.mark.parametrize("gdtype,layout,tile", [(torch.float32, "per_tensor", 0), (torch.bfloat16, "per_tensor", 1024),
+                                                (torch.bfloat16, "concat", 2048), (torch.float32, "concat", 3072),
+                                                (torch.bfloat16, "per_tensor", 3072), (torch.float32, "per_tensor", 16384)])
+def test_one_kernel_has_the_bits_of_the_shard_by_shard_calls(opt, R, gdtype, layout, tile):
+    # the one kernel's items are several tiles (tiles of 1024 share a pass of 8-element vectors, in tiles of 3072
+    # a pass does not end with the tile, 16384 is more than an item of several tiles has); the partial norms are the
+    # tiles' in both forms, so norms, ratios, state and emitted weights agree bit for bit
+    shapes = SHAPES + [(1500, 4099), (0,), (1500, 307)]
+    wl, w, m, v, g = _model(shapes, R, gdtype, seed=R, gstd=1e-3)
+    plan = B.Plan(shapes, 8, 32, tile, layout=layout)
+    assert plan.sched_buf is not None
+    h = B.make_hyper(opt, _lars_hyper() if opt == "lars" else _hyper("lamb"))
+    pw, pm, pv, pg = _pack_all(plan, w, m, v, g)
+    state = lambda x: [x[0].clone(), x[1].clone(), x[2].clone() if opt == "lamb" else None]  # noqa: E731
+    one, per = state((pw, pm, pv)), state((pw, pm, pv))
+    wsa = torch.zeros(plan.workspace_bytes(opt), dtype=torch.uint8, device=DEV)
+    off = plan.sync_status_offset()
+    wsa[off:off + 4] = 0xFF                        # the one kernel clears the status word, nothing else writes it
+    wsb = torch.zeros_like(wsa)
+    ga, gb = torch.zeros(plan.G, dtype=torch.bfloat16, device=DEV), torch.zeros(plan.G, dtype=torch.bfloat16, device=DEV)
+    B.ws_shard_update(plan, -1, pg, *one, h, ga, wsa)
+    assert int(wsa[off:off + 4].view(torch.int32).item()) == 0
+    S = plan.S
+    cut = lambda r: [None if x is None else x[r * S:(r + 1) * S] for x in per]  # noqa: E731
+    for r in range(plan.R):
+        sw, sm, sv = cut(r)
+        B.ws_lamb_partial(plan, r, pg, sw, sm, sv, h, wsb) if opt == "lamb" else B.ws_lars_partial(plan, r, pg, sw, sm, h, wsb)
+    B.ws_lamb_finalize(plan, wsb) if opt == "lamb" else B.ws_lars_finalize(plan, h, wsb)
+    for r in range(plan.R):
+        sw, sm, sv = cut(r)
+        B.ws_lamb_apply(plan, r, sw, sm, sv, h, wsb, gb) if opt == "lamb" else B.ws_lars_apply(plan, r, sw, sm, h, wsb, gb)
+    up = lambda x: (x + 15) // 16 * 16  # noqa: E731
+    head = up(4 * plan.T) + 16 * plan.T           # ratios and squared norms
+    assert torch.equal(wsa[:head], wsb[:head])
+    assert all(x is None or torch.equal(x, y) for x, y in zip(one, per)) and torch.equal(ga, gb)
+
+
 def test_lars_poisoned_pads_and_error_codes():
     import ctypes as C
     R = 5

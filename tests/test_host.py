@@ -273,6 +273,22 @@ def test_one_launch_schedule_invariants(layout, R, tile):
     assert all(p > end1 for i, p in pos2.items() if p - last1[tens[i]] < 512)
 
 
+@pytest.mark.parametrize("layout", ["per_tensor", "concat"])
+@pytest.mark.parametrize("tile", [0, 1024, 2048, 3072, 16384])
+def test_one_launch_items_are_whole_tiles(layout, tile):
+    """The partial norms of the one-kernel update are the tiles', so an item is one or several whole tiles."""
+    shapes = [(7,), (1500, 4099), (0,), (300, 301), (1024, 512), (9,)]
+    plan = B.Plan(shapes, 4, 32, tile, upload=False, layout=layout)
+    K = tile or 1024                                    # (the default of a model of this size)
+    _, items = plan.schedule()
+    starts = {}
+    for it in items:                                    # the run of a tensor in a shard starts at its first item
+        first = starts.setdefault((it.tensor, it.shard), it.pos)
+        assert (it.pos - first) % K == 0 and it.len <= max(K, 8192) and -(-it.len // K) <= 8
+        assert it.len <= K or K == 1024 or K % 2048 == 0
+    assert max(it.len for it in items) == {1024: 8192, 2048: 8192, 3072: 3072, 16384: 16384}[K]
+
+
 def test_one_launch_schedule_on_bert_large_keeps_phase_two_close():
     """On the BERT-large set (R = 16) the state a phase-2 item reads was written a bounded distance earlier:
     except for the embedding (larger than L2) and the few tensors whose phase 2 queues behind the
