@@ -315,8 +315,8 @@ ws_status ws_plan_factored_layout(const ws_plan* plan, int64_t* layout);
  *   double rsum[T]           sum of the new row accumulators per tensor
  *   float  fac[F']           1/sqrt factors of V for the two elementwise passes
  *   float  alpha[T]          max(eps2, RMS(w_t)) min(lr, 1/sqrt(step))
- *   (with rsum: scratch of the one-kernel route, counters, ready words and a ticket; before alpha: its
- *    partial sums.  There ghat holds the sums in another order and rsum, fac are its own)
+ *   (after rsum: scratch of the one-kernel route, counters, ready words, a ticket, its partial sums and
+ *    row factors, both in 64 bits.  There ghat holds the sums in another order and rsum, fac are its own)
  * where F' is F = ws_plan_factored_elems() with every tensor's row part and
  * column part padded to a multiple of 8 floats.  The WS_ADAFACTOR workspace
  * must be 32-byte aligned (its second pass reads ghat with 256-bit loads);

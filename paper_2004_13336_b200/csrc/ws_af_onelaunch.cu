@@ -381,8 +381,8 @@ __device__ __forceinline__ void sums_block(const AfLaunch& P, const WsAfTensor& 
 
 // ------------------------------------------------------------------ P2 and P3
 template <bool APPLY, int MODE>
-__device__ __forceinline__ void second_block(const AfLaunch& P, const WsAfTensor& T, const WsAfItem& it, float rscale,
-                                             float rate, char* wt, float& sw, float& su) {
+__device__ __forceinline__ void second_block(const AfLaunch& P, const WsAfTensor& T, const WsAfItem& it, double rscale,
+                                             float rate, char* wt, double& sw, double& su) {
     constexpr int W = Idx<MODE>::W;
     constexpr int U = MODE == WS_AF_VEC4 ? 4 : 2;
     const bool wide = P.wide != 0;
@@ -405,14 +405,16 @@ __device__ __forceinline__ void second_block(const AfLaunch& P, const WsAfTensor
             for (int j = 0; j < 4; ++j) fc[j] = (k.cmask >> j) & 1u ? __ldcg(c + j * it.tpr) : 0.f;
         }
     }
-    const float* rowfac = P.fac + T.irow + it.row0 + k.rr;
+    // a row's factor sqrt(sum(Rv') / Rv'_i) is formed in 64 bits and rounded once, like the stages'
+    const double* rowfac = P.rfac + T.rfac + it.row0 + k.rr;
     long long e = k.e0;
     for (int v0 = 0; v0 < k.passes; v0 += U, e += U * k.estep) {
         unsigned m[U];
         Idx<MODE> x[U];
         Fv<W> g[U], w[U];
         float4 fv[MODE == WS_AF_FULL ? U : 1];
-        float fr[U];
+        double fr[U];
+        float tw = 0.f, tu = 0.f;      // of up to 16 elements; a block's thread walks over 256, which are summed in 64 bits
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             m[u] = mask_of<MODE>(T, k, v0 + u, e + u * k.estep);
@@ -429,7 +431,7 @@ __device__ __forceinline__ void second_block(const AfLaunch& P, const WsAfTensor
             if (!m[u]) continue;
             float frs = 1.f;
             if constexpr (MODE == WS_AF_FULL) { fc[0] = fv[u].x; fc[1] = fv[u].y; fc[2] = fv[u].z; fc[3] = fv[u].w; }
-            else frs = fr[u] * rscale;
+            else frs = (float)(fr[u] * rscale);
 #pragma unroll
             for (int j = 0; j < W; ++j) {
                 if ((MODE == WS_AF_SCALAR || MODE == WS_AF_FULL) && !((m[u] >> j) & 1u)) continue;
@@ -437,8 +439,8 @@ __device__ __forceinline__ void second_block(const AfLaunch& P, const WsAfTensor
                 if (APPLY) {
                     w[u].f[j] = fmaf(-rate, uu, w[u].f[j]);
                 } else {
-                    sw = fmaf(w[u].f[j], w[u].f[j], sw);
-                    su = fmaf(uu, uu, su);
+                    tw = fmaf(w[u].f[j], w[u].f[j], tw);
+                    tu = fmaf(uu, uu, tu);
                 }
             }
             if constexpr (APPLY) {
@@ -451,6 +453,10 @@ __device__ __forceinline__ void second_block(const AfLaunch& P, const WsAfTensor
                 }
             }
         }
+        if constexpr (!APPLY) {
+            sw += (double)tw;
+            su += (double)tu;
+        }
     }
 }
 
@@ -459,7 +465,7 @@ __device__ __forceinline__ unsigned long long wait_word(const AfLaunch& P, const
     unsigned long long word = 0;
     for (int tries = 0; tries < kSpinLimitAf; ++tries) {
         word = ld_acquire64(p);
-        if (word & 1ULL) return word;
+        if (word != 0) return word;
         if ((tries & 255) == 255 && ld_volatile_int(P.status) != 0) break;
         __nanosleep(50);
     }
@@ -496,7 +502,7 @@ template <bool GBF, int RB, int U, bool LOOPK, int NP>
 __global__ void __launch_bounds__(kBlock, kMinBlocks) af_kernel(const AfLaunch P, const __grid_constant__ GradPtrs<NP> gp) {
     __shared__ unsigned long long s_word;
     __shared__ const void* sgp[NP];
-    __shared__ float2 red[kBlock / 32];
+    __shared__ float s_rate;
     __shared__ double da[kBlock / 32], db[kBlock / 32];
     __shared__ int s_last;
     const int tid = threadIdx.x;
@@ -551,7 +557,9 @@ __global__ void __launch_bounds__(kBlock, kMinBlocks) af_kernel(const AfLaunch P
             const long long k = isrow ? T.irow + e : T.icol + (e - T.nrow);
             const double v = P.beta * (double)P.state[T.foff + e] + (1.0 - P.beta) * (double)__ldcg(P.acc + k);
             P.state[T.foff + e] = (float)v;
-            P.fac[k] = (float)(1.0 / sqrt((double)(float)v));
+            const double f = 1.0 / sqrt((double)(float)v);
+            if (isrow) P.rfac[T.rfac + e] = f;
+            else P.fac[k] = (float)f;
             if (isrow) rs += v;
         }
 #pragma unroll
@@ -565,8 +573,9 @@ __global__ void __launch_bounds__(kBlock, kMinBlocks) af_kernel(const AfLaunch P
             if (atomicAdd(P.countm + it.seg, 1) + 1 == T.chunk_count) {
                 __threadfence();
                 // the row factors still lack sqrt(sum(Rv')), which goes with the word
-                const float r = (float)sqrt(__ldcg(P.rsum + it.seg));
-                st_release64(P.flagm + it.seg, ((unsigned long long)__float_as_uint(r) << 32) | 1ULL);
+                // (its bits inverted: no square root gives the word 0)
+                const double r = sqrt(__ldcg(P.rsum + it.seg));
+                st_release64(P.flagm + it.seg, ~(unsigned long long)__double_as_longlong(r));
             }
         }
         return;
@@ -599,19 +608,20 @@ __global__ void __launch_bounds__(kBlock, kMinBlocks) af_kernel(const AfLaunch P
 
     // a factored tensor's row factors lack sqrt(sum(Rv')), which comes with M's ready word; P3 also needs the rate
     if (tid == 0) {
-        unsigned long long a = 1ULL | ((unsigned long long)__float_as_uint(1.f) << 32), b = 1ULL;
+        unsigned long long a = ~(unsigned long long)__double_as_longlong(1.0), b = 1ULL;
         if (kind == 3) b = wait_word(P, P.flag2 + it.seg);
         if (T.chunk_count > 0) a = wait_word(P, P.flagm + it.seg);
         else if (kind == 2 && !wait_count(P, P.count1 + it.seg, T.item_count)) a = 0;
-        s_word = (a && b) ? (a & 0xffffffff00000000ULL) | (b >> 32) : 0;
+        s_word = ~a;
+        s_rate = __uint_as_float((unsigned)(b >> 32));
         s_last = (a && b) ? 1 : 0;
     }
     __syncthreads();
     if (!s_last) return;
-    const float rscale = __uint_as_float((unsigned)(s_word >> 32));
-    float sw = 0.f, su = 0.f;
+    const double rscale = __longlong_as_double((long long)s_word);
+    double sw = 0.0, su = 0.0;
     if (kind == 3) {
-        const float rate = __uint_as_float((unsigned)s_word);
+        const float rate = s_rate;
         if (T.mode == WS_AF_VEC8) second_block<true, WS_AF_VEC8>(P, T, it, rscale, rate, wt, sw, su);
         else if (T.mode == WS_AF_VEC4) second_block<true, WS_AF_VEC4>(P, T, it, rscale, rate, wt, sw, su);
         else if (T.mode == WS_AF_SCALAR) second_block<true, WS_AF_SCALAR>(P, T, it, rscale, rate, wt, sw, su);
@@ -622,36 +632,25 @@ __global__ void __launch_bounds__(kBlock, kMinBlocks) af_kernel(const AfLaunch P
     else if (T.mode == WS_AF_VEC4) second_block<false, WS_AF_VEC4>(P, T, it, rscale, 0.f, wt, sw, su);
     else if (T.mode == WS_AF_SCALAR) second_block<false, WS_AF_SCALAR>(P, T, it, rscale, 0.f, wt, sw, su);
     else second_block<false, WS_AF_FULL>(P, T, it, rscale, 0.f, wt, sw, su);
-    const float2 ab = block_sum2(sw, su, red);
+    double a = sw, b = su;
+    sum_block(a, b, da, db);
     if (tid == 0) {
-        P.ipart[it.item] = ab;
+        P.ipart[it.item] = make_double2(a, b);
         __threadfence();
         s_last = (atomicAdd(P.count2 + it.seg, 1) + 1 == T.item_count) ? 1 : 0;
     }
     __syncthreads();
     if (!s_last) return;
     __threadfence();
-    double a = 0.0, b = 0.0;
+    a = 0.0;
+    b = 0.0;
     for (int i = tid; i < T.item_count; i += kBlock) {     // fixed order
-        const float2 p = __ldcg(P.ipart + T.item_first + i);
-        a += (double)p.x;
-        b += (double)p.y;
+        const double2 p = __ldcg(P.ipart + T.item_first + i);
+        a += p.x;
+        b += p.y;
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        a += __shfl_xor_sync(0xffffffffu, a, o);
-        b += __shfl_xor_sync(0xffffffffu, b, o);
-    }
-    if ((tid & 31) == 0) {
-        da[tid >> 5] = a;
-        db[tid >> 5] = b;
-    }
-    __syncthreads();
+    sum_block(a, b, da, db);
     if (tid == 0) {
-        for (int i = 1; i < kBlock / 32; ++i) {
-            a += da[i];
-            b += db[i];
-        }
         const double rms_w = sqrt(a / (double)T.numel), rms_u = sqrt(b / (double)T.numel);
         const double al = (P.eps2 > rms_w ? P.eps2 : rms_w) * P.rho_step;
         const double clip = rms_u / P.clip > 1.0 ? rms_u / P.clip : 1.0;

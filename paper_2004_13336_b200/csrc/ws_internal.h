@@ -115,7 +115,7 @@ struct __align__(16) WsAfTensor {
     long long piece, off;             // packed position of element e: (e / piece) S + off + e % piece
     long long pad_end;                // concatenated layout: its pads are elements [numel, pad_end)
     int item_first, item_count, chunk_count, mode;
-    long long unused;
+    long long rfac;                   // start of its 64-bit row factors
 };
 static_assert(sizeof(WsAfTensor) == 96, "WsAfTensor is read as six 16-byte words");
 
@@ -146,7 +146,7 @@ struct ws_plan {
     std::vector<WsItemSeg> itemsegs;          // [T]
     std::vector<unsigned> sched;              // [2 n_items]: item index * 2 + phase, in execution order
     // the same for Adafactor (0 items: the plan has none)
-    long long n_afitems = 0, n_afsched = 0, af_ghat = 0;   // items, schedule entries, floats of kept gradient sums
+    long long n_afitems = 0, n_afsched = 0, af_ghat = 0, af_rows = 0;   // items, schedule entries, floats of kept gradient sums, rows
     std::vector<WsAfTensor> aftensors;
     std::vector<WsAfItem> afsched;
     const WsAfTensor* d_aftensors = nullptr;
@@ -185,7 +185,8 @@ struct WsLambWs {
     unsigned long long *af_flagm, *af_flag2;       // [T] each
     unsigned long long* af_ticket;
     size_t af_sync_bytes;
-    float2* af_ipart;  // [n_afitems] partial sums of w^2 and U^2
+    double2* af_ipart; // [n_afitems] partial sums of w^2 and U^2
+    double* af_rfac;   // [af_rows] 1/sqrt(Rv') of the factored tensors' rows
     float* fac;        // Adafactor: [Fi] 1/sqrt factors of V (padded layout)
     float* alpha;      // Adafactor: [T] step sizes
     size_t bytes_af;   // through alpha: what Adafactor needs

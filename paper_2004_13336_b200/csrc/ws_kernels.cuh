@@ -291,6 +291,27 @@ struct ItemCtx {
     int unit;            // TILES only: elements of a tile
 };
 
+// Sums two values over the CTA in 64 bits, in a fixed order; the totals are valid in thread 0.  sa, sb: kBlock/32
+// doubles of shared memory each.
+__device__ __forceinline__ void sum_block(double& a, double& b, double* sa, double* sb) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {                    // fixed tree inside the warp ...
+        a += __shfl_xor_sync(0xffffffffu, a, o);
+        b += __shfl_xor_sync(0xffffffffu, b, o);
+    }
+    if ((threadIdx.x & 31) == 0) {
+        sa[threadIdx.x >> 5] = a;
+        sb[threadIdx.x >> 5] = b;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int i = 1; i < kBlock / 32; ++i) {           // ... and the warps in order
+            a += sa[i];
+            b += sb[i];
+        }
+    }
+}
+
 // Sums a tensor's per-tile partials over all shards in a fixed order, in double (stands where the paper combines
 // per-replica reduce results with one batched scalar all-reduce, Section 4.1 / 5.2); the totals are valid in
 // thread 0.  One function for the finalize step and for the one-kernel routes, so that both give the same bits.
@@ -323,22 +344,7 @@ __device__ __forceinline__ void sum_partials(const WsSegTiles st, const float2* 
             b += (double)p[u].y;
         }
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {                    // fixed tree inside the warp ...
-        a += __shfl_xor_sync(0xffffffffu, a, o);
-        b += __shfl_xor_sync(0xffffffffu, b, o);
-    }
-    if ((threadIdx.x & 31) == 0) {
-        sa[threadIdx.x >> 5] = a;
-        sb[threadIdx.x >> 5] = b;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int i = 1; i < kBlock / 32; ++i) {           // ... and the warps in order
-            a += sa[i];
-            b += sb[i];
-        }
-    }
+    sum_block(a, b, sa, sb);
 }
 
 // Sums two values over the CTA at once (one pair of barriers for both); the totals are valid in
@@ -890,11 +896,13 @@ struct AfLaunch {
     void* gathered;
     float* state;                // factored second moments
     float* kept;                 // summed gradients, block by block
-    float *acc, *fac;            // row / column sums, 1/sqrt factors (padded layout)
+    float *acc, *fac;            // row / column sums, 1/sqrt factors (padded layout; rows: rfac)
+    double* rfac;                // 1/sqrt(Rv') of the factored tensors' rows
     double* rsum;                // [T] sum of the new row accumulators
-    float2* ipart;               // [items] sums of w^2 and U^2
+    double2* ipart;              // [items] sums of w^2 and U^2
     int *count1, *countm, *count2;               // [T] finished P1, M and P2 entries
-    unsigned long long *flagm, *flag2;           // ready words: (float bits << 32) | 1
+    unsigned long long* flagm;                   // ready words: ~bits of sqrt(sum(Rv')) in 64 bits
+    unsigned long long* flag2;                   // ... (float bits of the step size << 32) | 1
     unsigned long long* ticket;
     int* status;
     float *alpha, *rho;

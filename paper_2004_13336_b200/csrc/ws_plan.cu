@@ -118,12 +118,13 @@ static void ws_af_blocks(const ws_plan* p, F&& emit) {
 // Block and schedule-entry counts and the floats of kept gradient sums; a tensor beyond the block fields'
 // ranges leaves the plan without Adafactor blocks.
 static void ws_count_af(ws_plan* p) {
-    p->n_afitems = p->n_afsched = p->af_ghat = 0;
+    p->n_afitems = p->n_afsched = p->af_ghat = p->af_rows = 0;
     if (p->R > 65535) return;
-    long long n = 0, m = 0, g = 0;
+    long long n = 0, m = 0, g = 0, rows = 0;
     for (const WsSegAf& a : p->segaf) {
         if (a.nrow > 0x7fffffffLL || a.ncol > 0x7fffffffLL) return;
         if (a.nrow > 0) m += (a.nrow + a.ncol + kWsAfChunk - 1) / kWsAfChunk;
+        rows += a.nrow;
     }
     ws_af_blocks(p, [&](int, int mode, long long, long long, long long nr, long long, long long tpr, long long rp) {
         ++n;
@@ -133,6 +134,7 @@ static void ws_count_af(ws_plan* p) {
     p->n_afitems = n;
     p->n_afsched = 3 * n + m;
     p->af_ghat = g;
+    p->af_rows = rows;
 }
 
 // Work items of the one-launch schedule: every run of consecutive positions of one tensor in one shard (a piece;
@@ -460,8 +462,10 @@ WsLambWs ws_lamb_layout(const ws_plan* p, void* workspace) {
     L.af_count2 = L.af_countm + T;
     o = round16(o + sizeof(int) * 3 * T);
     L.af_sync_bytes = o - acc0;
-    L.af_ipart = (float2*)(b + o);
-    o += sizeof(float2) * (size_t)p->n_afitems;
+    L.af_ipart = (double2*)(b + o);
+    o += sizeof(double2) * (size_t)p->n_afitems;
+    L.af_rfac = (double*)(b + o);
+    o += sizeof(double) * (size_t)p->af_rows;
     o = (o + 255) & ~(size_t)255;
     L.fac = (float*)(b + o);
     o = (o + sizeof(float) * (size_t)p->Fi + 255) & ~(size_t)255;
@@ -599,12 +603,15 @@ void ws_build_af_schedule(ws_plan* p) {
     std::vector<WsAfItem> items;
     items.reserve((size_t)p->n_afitems);
     p->aftensors.resize(T);
+    long long rows = 0;
     for (int t = 0; t < T; ++t) {
         const WsSegAf& a = p->segaf[t];
         WsAfTensor& d = p->aftensors[t];
         memset(&d, 0, sizeof(d));
         d.numel = a.numel; d.ncol = a.ncol; d.nrow = a.nrow;
         d.foff = a.foff; d.irow = a.irow; d.icol = a.icol;
+        d.rfac = rows;
+        rows += a.nrow;
         d.piece = p->layout == WS_LAYOUT_CONCAT ? (1LL << 62) : p->segs[t].piece;
         d.off = p->segs[t].shard_off;
         d.pad_end = (t + 1 < T ? p->segs[t + 1].shard_off : (long long)p->R * p->S) - d.off;

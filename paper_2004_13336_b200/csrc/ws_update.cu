@@ -969,6 +969,7 @@ ws_status try_af_one_launch(const ws_plan* plan, const ws_grads* grads, const ws
     P.kept = L.ghat;
     P.acc = L.acc;
     P.fac = L.fac;
+    P.rfac = L.af_rfac;
     P.rsum = L.rsum;
     P.ipart = L.af_ipart;
     P.count1 = L.af_count1;

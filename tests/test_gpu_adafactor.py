@@ -412,3 +412,45 @@ def test_one_kernel_equals_the_stages(R, gdtype, shift, layout):
             assert err(x, y) <= TOL_LAMB
         np.testing.assert_allclose(a[1], b[1], rtol=TOL_LAMB)
         np.testing.assert_allclose(a[2], b[2], rtol=TOL_LAMB)
+
+
+@pytest.mark.parametrize("layout", ["per_tensor", "concat"])
+def test_one_kernel_forms_the_row_factors_like_the_stages(layout):
+    # gradients of +-1 and +-2 with eps1 = 0: every row and column sum is a whole number below 2^24, the same in any
+    # order, so both forms have the same Rv', Cv'; with eps2 above RMS(w) and no clipping the step size is the same
+    # number too.  The row factor sqrt(sum(Rv') / Rv'_i) rounded once then gives the same weights bit for bit.
+    shapes = [(257, 2056), (3, 2060), (129, 12), (70, 9), (513, 1), (1, 513), (4097,), (1100, 8), (40, 2049)]
+    numels = [int(torch.Size(s).numel()) for s in shapes]
+    gen = torch.Generator(device=DEV).manual_seed(5)
+    vals = torch.tensor([-2.0, -1.0, 1.0, 2.0], device=DEV)
+    g = [vals[torch.randint(0, 4, (n,), generator=gen, device=DEV)] for n in numels]
+    w = [torch.randn(n, generator=gen, device=DEV) * 0.02 for n in numels]
+    hy = B.make_hyper("adafactor", _hyper(eps=0.0, eps2=1.0, clip_threshold=1e30))
+    got = []
+    for one in (True, False):
+        plan = B.Plan(shapes, 3, 8, layout=layout, one_launch=one)
+        f = torch.rand(plan.factored_elems, generator=torch.Generator(device=DEV).manual_seed(9), device=DEV) + 0.5
+        wt = [x.clone() for x in w]
+        ws = torch.zeros(plan.workspace_bytes("adafactor"), dtype=torch.uint8, device=DEV)
+        B.ws_fused_update(plan, -1, B.TensorTable(plan, [g]), None, None, f, hy, B.TensorTable(plan, [wt]), ws)
+        got.append((f, wt))
+    assert torch.equal(got[0][0], got[1][0])
+    for t, (a, b) in enumerate(zip(got[0][1], got[1][1])):
+        assert torch.equal(a, b), t
+
+
+def test_one_kernel_sums_norms_in_short_chains():
+    # blocks of 65536 elements (50 M parameters): a thread adds 256 squares.  The weight is one whose square, added
+    # 256 times in fp32, is off by 64 x 2^-24; 32 fp32 additions and a tree of 8 levels, what the stages do, are off by
+    # at most 39 x 2^-24
+    n, val = 49152 * 1024, 0.02189512364566326
+    plan = B.Plan([(49152, 1024)], 1, 32)
+    w = torch.full((n,), val, device=DEV)
+    g = torch.full((n,), 1e-3, device=DEV)
+    f = torch.full((plan.factored_elems,), 1e-6, device=DEV)
+    ws = torch.zeros(plan.workspace_bytes("adafactor"), dtype=torch.uint8, device=DEV)
+    B.ws_fused_update(plan, -1, B.TensorTable(plan, [[g]]), None, None, f, B.make_hyper("adafactor", _hyper()),
+                      B.TensorTable(plan, [[w]]), ws)
+    got = float(ws[16:24].view(torch.float64).item())         # norms[0]: sum w^2
+    exact = n * float(np.float32(val)) ** 2
+    assert abs(got / exact - 1.0) <= 39 * 2.0 ** -24
