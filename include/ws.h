@@ -139,8 +139,10 @@ ws_status ws_plan_segments(const ws_plan* plan, const ws_segment** segs, int32_t
 /* The kernels read the plan from device memory.  The caller provides a buffer
  * of at least ws_plan_device_bytes(plan) bytes (16-byte aligned) that must
  * stay alive and unmodified while the plan is in use; ws_plan_upload copies
- * the tables into it with one cudaMemcpyAsync on `stream`.  Upload once per
- * plan; afterwards the plan is immutable and may be shared between threads. */
+ * the tables into it with cudaMemcpyAsync on `stream`, from host memory of the
+ * plan (a captured upload can be replayed as long as the plan lives).  Upload
+ * once per plan; afterwards the plan is immutable and may be shared between
+ * threads. */
 size_t ws_plan_device_bytes(const ws_plan* plan);
 ws_status ws_plan_upload(ws_plan* plan, void* dev_buf, size_t bytes, void* stream);
 

@@ -131,6 +131,8 @@ struct ws_plan {
     // tensor arena: tensors back to back, each start rounded up to 8 elements
     std::vector<long long> arena_off;
     long long arena_elems = 0;
+    // images of small uploads; they live as long as the plan, since a captured copy reads its source at every replay
+    std::vector<char> table_image, sched_image;
     // device copies (caller-owned memory, set by ws_plan_upload)
     const WsTile* d_tiles = nullptr;
     const WsSegTiles* d_segtiles = nullptr;

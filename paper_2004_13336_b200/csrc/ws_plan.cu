@@ -379,20 +379,21 @@ extern "C" ws_status ws_plan_factored_layout(const ws_plan* p, int64_t* layout) 
 
 // Copies `n` tables to their offsets in one device buffer.  Small plans: as one image, one copy (every
 // cudaMemcpyAsync from pageable memory costs the host some 10 us); from 128 KB on gathering the image costs more.
+// The image and the tables are the plan's: under stream capture the copy becomes a node that reads them at replay.
 static ws_status upload_image(char* dev, const void* const* src, const size_t* nb, const size_t* off, int n, size_t total,
-                              cudaStream_t st, const char* what) {
-    // (pageable memory: the runtime has staged it before cudaMemcpyAsync returns)
+                              std::vector<char>& image, cudaStream_t st, const char* what) {
     cudaError_t e = cudaSuccess;
     if (total <= (128u << 10)) {
-        std::vector<char> host;
-        try {
-            host.resize(total);
-        } catch (...) {
-            return WS_ERR_INVALID_ARG;
+        if (image.empty()) {                 // (a plan's tables never change once they are built)
+            try {
+                image.resize(total);
+            } catch (...) {
+                return WS_ERR_INVALID_ARG;
+            }
+            for (int i = 0; i < n; ++i)
+                if (nb[i]) memcpy(image.data() + off[i], src[i], nb[i]);
         }
-        for (int i = 0; i < n; ++i)
-            if (nb[i]) memcpy(host.data() + off[i], src[i], nb[i]);
-        if (total) e = cudaMemcpyAsync(dev, host.data(), total, cudaMemcpyHostToDevice, st);
+        if (total) e = cudaMemcpyAsync(dev, image.data(), total, cudaMemcpyHostToDevice, st);
     } else {
         for (int i = 0; i < n && e == cudaSuccess; ++i)
             if (nb[i]) e = cudaMemcpyAsync(dev + off[i], src[i], nb[i], cudaMemcpyHostToDevice, st);
@@ -410,7 +411,7 @@ extern "C" ws_status ws_plan_upload(ws_plan* p, void* dev_buf, size_t bytes, voi
                           p->segaf.size() * sizeof(WsSegAf), p->afchunks.size() * sizeof(WsAfChunk)};
     const void* src[4] = {p->tiles.data(), p->segtiles.data(), p->segaf.data(), p->afchunks.data()};
     for (int i = 0; i < 4; ++i) { o[i] = at; at += round16(nb[i]); }
-    const ws_status s = upload_image(base, src, nb, o, 4, at, (cudaStream_t)stream, "ws_plan_upload");
+    const ws_status s = upload_image(base, src, nb, o, 4, at, p->table_image, (cudaStream_t)stream, "ws_plan_upload");
     if (s != WS_OK) return s;
     p->d_tiles = (const WsTile*)(base + o[0]);
     p->d_segtiles = (const WsSegTiles*)(base + o[1]);
@@ -757,7 +758,7 @@ extern "C" ws_status ws_plan_upload_schedule(ws_plan* p, void* dev_buf, size_t b
                           p->afsched.size() * sizeof(WsAfItem)};
     const void* src[5] = {p->items.data(), p->itemsegs.data(), p->sched.data(), p->aftensors.data(), p->afsched.data()};
     for (int i = 0; i < (af ? 5 : 3); ++i) { o[i] = at; at += round16(nb[i]); }
-    const ws_status s = upload_image(base, src, nb, o, af ? 5 : 3, at, (cudaStream_t)stream, "ws_plan_upload_schedule");
+    const ws_status s = upload_image(base, src, nb, o, af ? 5 : 3, at, p->sched_image, (cudaStream_t)stream, "ws_plan_upload_schedule");
     if (s != WS_OK) return s;
     p->d_items = (const WsItem*)(base + o[0]);
     p->d_itemsegs = (const WsItemSeg*)(base + o[1]);

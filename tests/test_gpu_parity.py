@@ -1216,3 +1216,33 @@ def test_replica_kernels_over_all_replicas_tensors(opt, gdtype, odtype, R):
     with pytest.raises(B.WsError) as e:
         B.ws_fused_update(plan, 0, B.TensorTable(plan, g[:1]), pw[:S], pm[:S], pv[:S], hy, wtab, None)
     assert e.value.status == 1
+
+
+@pytest.mark.parametrize("shapes", [SHAPES, SHAPES + [(n % 7 + 1, 64) for n in range(3000)]])
+def test_plan_uploads_can_be_captured_and_replayed(shapes):
+    # a captured copy reads its host source at every replay: the source has to be the plan's own memory, for small
+    # plans (tables gathered into one image) as for large ones (copied table by table)
+    plan = B.Plan(shapes, 3, 8, upload=False)
+    sizes = [B.lib().ws_plan_device_bytes(plan.handle), B.lib().ws_plan_schedule_bytes(plan.handle)]
+    calls = [B.lib().ws_plan_upload, B.lib().ws_plan_upload_schedule]
+    want = [torch.zeros(n, dtype=torch.uint8, device=DEV) for n in sizes]
+    got = [torch.full((n,), 0xEE, dtype=torch.uint8, device=DEV) for n in sizes]
+    for call, b in zip(calls, want):
+        assert call(plan.handle, b.data_ptr(), b.numel(), torch.cuda.current_stream().cuda_stream) == 0
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        with torch.cuda.graph(graph, stream=side):
+            for call, b in zip(calls, got):
+                assert call(plan.handle, b.data_ptr(), b.numel(), side.cuda_stream) == 0
+    junk = [bytearray(b"\x55" * n) for n in sizes for _ in range(64)]      # what a freed source would be overwritten with
+    for _ in range(2):
+        for b in got:
+            b.fill_(0xEE)
+        graph.replay()
+        torch.cuda.synchronize()
+        for b, w in zip(got, want):                                        # (bytes that pad a table are never written)
+            known = w != 0
+            assert torch.equal(b[known], w[known])
+    del junk
