@@ -63,13 +63,13 @@ __device__ __forceinline__ long long packed_pos(const WsAfTensor& T, long long e
 
 // A thread's W elements of one row.  WS_AF_VEC8: 8 consecutive ones as one 256-bit access, or (P.wide == 0) two
 // quads 4 tpr columns apart, so that a warp's 128-bit accesses stay contiguous.  WS_AF_VEC4, WS_AF_FULL: 4
-// consecutive ones.  WS_AF_SCALAR: 4, tpr columns apart.  `mask` says which exist: all, or what the end of the
-// row (WS_AF_SCALAR) or of the tensor (WS_AF_FULL) leaves.  Idx: their element offsets in a tensor (flat) or in a
+// consecutive ones.  WS_AF_SCALAR, WS_AF_NARROW: 4, tpr columns apart.  `mask` says which exist: all, or what the end of the
+// row (scalar) or of the tensor (WS_AF_FULL) leaves.  Idx: their element offsets in a tensor (flat) or in a
 // packed buffer.
 template <int MODE>
 struct Idx {
     static constexpr int W = ws_af_width(MODE);
-    static constexpr int N = MODE == WS_AF_SCALAR ? 4 : MODE == WS_AF_VEC8 ? 2 : 1;
+    static constexpr int N = ws_af_scalar(MODE) ? 4 : MODE == WS_AF_VEC8 ? 2 : 1;
     long long i[N];
 };
 template <int MODE>
@@ -79,7 +79,7 @@ __device__ __forceinline__ Idx<MODE> index_of(const AfLaunch& P, const WsAfTenso
     if constexpr (MODE == WS_AF_VEC8) {
         if (P.wide) x.i[1] = x.i[0] + 4;
         else x.i[1] = flat ? e + 4 * tpr : packed_pos(T, e + 4 * tpr, P.S);
-    } else if constexpr (MODE == WS_AF_SCALAR) {
+    } else if constexpr (ws_af_scalar(MODE)) {
 #pragma unroll
         for (int j = 1; j < 4; ++j) {
             const long long ej = e + (long long)j * tpr;
@@ -95,7 +95,7 @@ __device__ __forceinline__ bool whole(unsigned mask) {
 }
 template <int MODE>
 __device__ __forceinline__ long long at_of(const Idx<MODE>& x, int j) {
-    return MODE == WS_AF_SCALAR ? x.i[j % Idx<MODE>::N] : x.i[0] + j;
+    return ws_af_scalar(MODE) ? x.i[j % Idx<MODE>::N] : x.i[0] + j;
 }
 
 template <bool GBF, int MODE>
@@ -111,7 +111,7 @@ __device__ __forceinline__ GradRaw<GBF, Idx<MODE>::W> load_grads(const void* bas
             for (int j = 0; j < 4; ++j) { g.f[j] = a.f[j]; g.f[4 + j] = b.f[j]; }
         }
         return g;
-    } else if constexpr (MODE != WS_AF_SCALAR) {
+    } else if constexpr (!ws_af_scalar(MODE)) {
         if (whole<MODE>(mask)) return load_grad<GBF, 4>(base, x.i[0]);
         return load_grad_partial<GBF, 4>(base, x.i[0], __popc(mask));
     } else {
@@ -141,21 +141,34 @@ __device__ __forceinline__ Fv<8> load8_keep(const float* p) {
     for (int i = 0; i < 8; ++i) o.f[i] = __uint_as_float(r[i]);
     return o;
 }
-template <int W>
-__device__ __forceinline__ Fv<W> load_kept(const float* p) {
-    if constexpr (W == 8) {
+// A thread's kept sums of one row (tpr: distance of its columns where they are kept element by element).
+template <int MODE>
+__device__ __forceinline__ Fv<Idx<MODE>::W> load_kept(const float* p, unsigned mask, int tpr) {
+    if constexpr (MODE == WS_AF_VEC8) {
         return load8_keep(p);
     } else {
-        const float4 v = __ldcg(reinterpret_cast<const float4*>(p));
-        Fv<W> o;
-        o.f[0] = v.x; o.f[1] = v.y; o.f[2] = v.z; o.f[3] = v.w;
+        Fv<4> o;
+        if constexpr (MODE == WS_AF_NARROW) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) o.f[j] = (mask >> j) & 1u ? __ldcg(p + j * tpr) : 0.f;
+        } else {
+            const float4 v = __ldcg(reinterpret_cast<const float4*>(p));
+            o.f[0] = v.x; o.f[1] = v.y; o.f[2] = v.z; o.f[3] = v.w;
+        }
         return o;
     }
 }
-template <int W>
-__device__ __forceinline__ void store_kept(float* p, const Fv<W>& x) {
-    if constexpr (W == 8) store_f32<8>(p, x);
-    else __stcg(reinterpret_cast<float4*>(p), make_float4(x.f[0], x.f[1], x.f[2], x.f[3]));
+template <int MODE>
+__device__ __forceinline__ void store_kept(float* p, const Fv<Idx<MODE>::W>& x, unsigned mask, int tpr) {
+    if constexpr (MODE == WS_AF_VEC8) {
+        store_f32<8>(p, x);
+    } else if constexpr (MODE == WS_AF_NARROW) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if ((mask >> j) & 1u) __stcg(p + j * tpr, x.f[j]);
+    } else {
+        __stcg(reinterpret_cast<float4*>(p), make_float4(x.f[0], x.f[1], x.f[2], x.f[3]));
+    }
 }
 
 // Weights: read at normal priority in P2 (P3 reads them again), streaming in P3.
@@ -233,12 +246,12 @@ __device__ __forceinline__ Walk walk_of(const AfLaunch& P, const WsAfTensor& T, 
     Walk k;
     k.rr = (int)threadIdx.x / it.tpr;
     const int cc = (int)threadIdx.x - k.rr * it.tpr;
-    k.c0 = MODE == WS_AF_SCALAR ? cc : (MODE == WS_AF_VEC8 && P.wide) ? 8 * cc : 4 * cc;
+    k.c0 = ws_af_scalar(MODE) ? cc : (MODE == WS_AF_VEC8 && P.wide) ? 8 * cc : 4 * cc;
     k.passes = (it.nr + it.rp - 1) / it.rp;
     k.nv = (k.rr < it.rp && k.rr < it.nr) ? (it.nr - k.rr + it.rp - 1) / it.rp : 0;
-    k.kstep = it.rp * it.tpr * W;
+    k.kstep = it.rp * ws_af_kept_row(MODE, it.nc, it.tpr);
     k.cmask = 15u;
-    if (MODE == WS_AF_SCALAR) {
+    if (ws_af_scalar(MODE)) {
         k.cmask = 0;
 #pragma unroll
         for (int j = 0; j < 4; ++j)
@@ -246,7 +259,7 @@ __device__ __forceinline__ Walk walk_of(const AfLaunch& P, const WsAfTensor& T, 
     }
     k.e0 = ((long long)it.row0 + k.rr) * T.ncol + it.col0 + k.c0;
     k.estep = it.rp * T.ncol;
-    k.kept = P.kept + (long long)it.goff32 * 32 + threadIdx.x * W;
+    k.kept = P.kept + (long long)it.goff32 * 32 + (MODE == WS_AF_NARROW ? k.rr * it.nc + cc : (int)threadIdx.x * W);
     return k;
 }
 template <int MODE>
@@ -346,7 +359,7 @@ __device__ __forceinline__ void sums_block(const AfLaunch& P, const WsAfTensor& 
                         cacc[j] += q[j];
                     }
                 }
-                store_kept<W>(k.kept + (long long)(v0 + u) * k.kstep, g[u]);
+                store_kept<MODE>(k.kept + (long long)(v0 + u) * k.kstep, g[u], m[u], it.tpr);
                 if (MODE == WS_AF_FULL) {
                     // unfactored: the element's own second moment, final here
                     const long long eu = e + u * k.estep;
@@ -380,7 +393,7 @@ __device__ __forceinline__ void sums_block(const AfLaunch& P, const WsAfTensor& 
         if (rows > 1) {
             float* mine = colsum + k.rr * width + k.c0;
             if (k.nv > 0) {
-                if constexpr (MODE != WS_AF_SCALAR) {
+                if constexpr (!ws_af_scalar(MODE)) {
                     *reinterpret_cast<float4*>(mine) = make_float4(cacc[0], cacc[1], cacc[2], cacc[3]);
                     if constexpr (W == 8) *reinterpret_cast<float4*>(mine + h) = make_float4(cacc[4], cacc[5], cacc[6], cacc[7]);
                 } else {
@@ -402,7 +415,7 @@ __device__ __forceinline__ void sums_block(const AfLaunch& P, const WsAfTensor& 
             }
             __syncthreads();
             if (k.rr == 0 && k.nv > 0) {
-                if constexpr (MODE != WS_AF_SCALAR) {
+                if constexpr (!ws_af_scalar(MODE)) {
                     const float4 a = *reinterpret_cast<const float4*>(mine);
                     cacc[0] = a.x; cacc[1] = a.y; cacc[2] = a.z; cacc[3] = a.w;
                     if constexpr (W == 8) {
@@ -417,7 +430,7 @@ __device__ __forceinline__ void sums_block(const AfLaunch& P, const WsAfTensor& 
         }
         if (k.rr == 0 && k.nv > 0) {
             float* c = P.acc + T.icol + it.col0 + k.c0;
-            if constexpr (MODE != WS_AF_SCALAR) {
+            if constexpr (!ws_af_scalar(MODE)) {
                 red_add_vec<4>(c, cacc);
                 if constexpr (W == 8) red_add_vec<4>(c + h, cacc + 4);
             } else {
@@ -444,7 +457,7 @@ __device__ __forceinline__ void second_block(const AfLaunch& P, const WsAfTensor
     for (int j = 0; j < W; ++j) fc[j] = 0.f;
     if (MODE != WS_AF_FULL && k.nv > 0) {
         const float* c = P.fac + T.icol + it.col0 + k.c0;
-        if constexpr (MODE != WS_AF_SCALAR) {
+        if constexpr (!ws_af_scalar(MODE)) {
 #pragma unroll
             for (int h = 0; h < W / 4; ++h) {
                 const float4 t = __ldcg(reinterpret_cast<const float4*>(c + (h == 0 ? 0 : wide ? 4 : 4 * it.tpr)));
@@ -470,7 +483,7 @@ __device__ __forceinline__ void second_block(const AfLaunch& P, const WsAfTensor
             m[u] = mask_of<MODE>(T, k, v0 + u, e + u * k.estep);
             if (m[u]) {
                 x[u] = index_of<MODE>(P, T, e + u * k.estep, m[u], it.tpr, P.master != 0);
-                g[u] = load_kept<W>(k.kept + (long long)(v0 + u) * k.kstep);
+                g[u] = load_kept<MODE>(k.kept + (long long)(v0 + u) * k.kstep, m[u], it.tpr);
                 w[u] = load_weights<MODE, !APPLY>(wbase, x[u], m[u], wide);
                 if constexpr (MODE == WS_AF_FULL) fv[u] = __ldcg(reinterpret_cast<const float4*>(P.fac + T.icol + e + u * k.estep));
                 else fr[u] = __ldcg(rowfac + (v0 + u) * it.rp);
@@ -484,7 +497,7 @@ __device__ __forceinline__ void second_block(const AfLaunch& P, const WsAfTensor
             else frs = (float)(fr[u] * rscale);
 #pragma unroll
             for (int j = 0; j < W; ++j) {
-                if ((MODE == WS_AF_SCALAR || MODE == WS_AF_FULL) && !((m[u] >> j) & 1u)) continue;
+                if ((ws_af_scalar(MODE) || MODE == WS_AF_FULL) && !((m[u] >> j) & 1u)) continue;
                 const float uu = (g[u].f[j] * frs) * fc[j];
                 if (APPLY) {
                     w[u].f[j] = fmaf(-rate, uu, w[u].f[j]);
@@ -638,7 +651,7 @@ __global__ void __launch_bounds__(kBlock, kMinBlocks) af_kernel(const AfLaunch P
         if (last >= T.numel || it.col0 < 0 || it.row0 < 0) bits |= WS_BOUNDS_STATE;
         if (!P.master && packed_pos(T, last, P.S) >= P.state_elems) bits |= WS_BOUNDS_STATE;
         if (!P.fused && packed_pos(T, last, P.S) >= P.state_elems) bits |= WS_BOUNDS_GRAD;
-        if ((long long)it.goff32 * 32 + (long long)(it.nr + it.rp - 1) / it.rp * it.rp * it.tpr * ws_af_width(T.mode) > P.kept_elems)
+        if ((long long)it.goff32 * 32 + (long long)it.nr * ws_af_kept_row(T.mode, it.nc, it.tpr) > P.kept_elems)
             bits |= WS_BOUNDS_OUT;
         if (bits && tid == 0 && P.bounds) atomicOr(P.bounds, bits);
         if (bits) return;
@@ -650,6 +663,7 @@ __global__ void __launch_bounds__(kBlock, kMinBlocks) af_kernel(const AfLaunch P
         if (T.mode == WS_AF_VEC8) sums_block<GBF, RB, U, LOOPK, WS_AF_VEC8>(P, T, it, sgp, colsum);
         else if (T.mode == WS_AF_VEC4) sums_block<GBF, RB, U, LOOPK, WS_AF_VEC4>(P, T, it, sgp, colsum);
         else if (T.mode == WS_AF_SCALAR) sums_block<GBF, RB, U, LOOPK, WS_AF_SCALAR>(P, T, it, sgp, colsum);
+        else if (T.mode == WS_AF_NARROW) sums_block<GBF, RB, U, LOOPK, WS_AF_NARROW>(P, T, it, sgp, colsum);
         else sums_block<GBF, RB, 1, LOOPK, WS_AF_FULL>(P, T, it, sgp, colsum);
         __syncthreads();
         // (no CTA looks whether it was the last one: M waits for the count, and this CTA is done at once)
@@ -676,12 +690,14 @@ __global__ void __launch_bounds__(kBlock, kMinBlocks) af_kernel(const AfLaunch P
         if (T.mode == WS_AF_VEC8) second_block<true, WS_AF_VEC8>(P, T, it, rscale, rate, wt, sw, su);
         else if (T.mode == WS_AF_VEC4) second_block<true, WS_AF_VEC4>(P, T, it, rscale, rate, wt, sw, su);
         else if (T.mode == WS_AF_SCALAR) second_block<true, WS_AF_SCALAR>(P, T, it, rscale, rate, wt, sw, su);
+        else if (T.mode == WS_AF_NARROW) second_block<true, WS_AF_NARROW>(P, T, it, rscale, rate, wt, sw, su);
         else second_block<true, WS_AF_FULL>(P, T, it, rscale, rate, wt, sw, su);
         return;
     }
     if (T.mode == WS_AF_VEC8) second_block<false, WS_AF_VEC8>(P, T, it, rscale, 0.f, wt, sw, su);
     else if (T.mode == WS_AF_VEC4) second_block<false, WS_AF_VEC4>(P, T, it, rscale, 0.f, wt, sw, su);
     else if (T.mode == WS_AF_SCALAR) second_block<false, WS_AF_SCALAR>(P, T, it, rscale, 0.f, wt, sw, su);
+    else if (T.mode == WS_AF_NARROW) second_block<false, WS_AF_NARROW>(P, T, it, rscale, 0.f, wt, sw, su);
     else second_block<false, WS_AF_FULL>(P, T, it, rscale, 0.f, wt, sw, su);
     double a = sw, b = su;
     sum_block(a, b, da, db);

@@ -93,8 +93,16 @@ struct __align__(16) WsItemSeg {
 // rows x cols matrix: 256 threads as rp rows of tpr threads, a thread owning 8 columns (4 where the row
 // length is no multiple of 8) and walking down the rows, so that its column sums live in registers for the
 // whole block.
-enum { WS_AF_VEC8 = 0, WS_AF_VEC4 = 1, WS_AF_SCALAR = 2, WS_AF_FULL = 3 };
+enum { WS_AF_VEC8 = 0, WS_AF_VEC4 = 1, WS_AF_SCALAR = 2, WS_AF_FULL = 3, WS_AF_NARROW = 4 };
 __host__ __device__ constexpr int ws_af_width(int mode) { return mode == WS_AF_VEC8 ? 8 : 4; }   // columns per thread
+// Rows that 4 does not divide: a thread's 4 columns are scalar accesses, but one vector in the kept sums, whose places
+// beyond the row stay empty.  Where those would be more than an eighth of the row (a row of one column would take four
+// times its size) the sums are kept element by element too: WS_AF_NARROW.
+__host__ __device__ constexpr bool ws_af_scalar(int mode) { return mode == WS_AF_SCALAR || mode == WS_AF_NARROW; }
+// Floats that a row of a block takes in the kept sums.
+__host__ __device__ constexpr int ws_af_kept_row(int mode, int nc, int tpr) {
+    return mode == WS_AF_NARROW ? nc : tpr * ws_af_width(mode);
+}
 constexpr int kWsAfChunk = 1024;      // state entries per moments entry
 // One record per schedule entry, in execution order, so that a CTA reads its work with one access.
 struct __align__(16) WsAfItem {

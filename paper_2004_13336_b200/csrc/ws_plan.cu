@@ -94,7 +94,8 @@ static void ws_af_blocks(const ws_plan* p, F&& emit) {
         const bool full = a.nrow == 0;
         const long long ncol = full ? (a.numel < 1024 ? a.numel : 1024) : a.ncol;
         const long long nrow = full ? (a.numel + ncol - 1) / ncol : a.nrow;
-        const int mode = full ? WS_AF_FULL : ncol % 8 == 0 ? WS_AF_VEC8 : ncol % 4 == 0 ? WS_AF_VEC4 : WS_AF_SCALAR;
+        const int mode = full ? WS_AF_FULL : ncol % 8 == 0 ? WS_AF_VEC8 : ncol % 4 == 0 ? WS_AF_VEC4 :
+                         (4 - ncol % 4) * 8 > ncol ? WS_AF_NARROW : WS_AF_SCALAR;
         const long long W = ws_af_width(mode);
         const long long units = (ncol + W - 1) / W, s0 = (units + 255) / 256;
         long long best_s = s0, best = -1;              // (busy threads of 256) / strips, compared as fractions
@@ -126,9 +127,9 @@ static void ws_count_af(ws_plan* p) {
         if (a.nrow > 0) m += (a.nrow + a.ncol + kWsAfChunk - 1) / kWsAfChunk;
         rows += a.nrow;
     }
-    ws_af_blocks(p, [&](int, int mode, long long, long long, long long nr, long long, long long tpr, long long rp) {
+    ws_af_blocks(p, [&](int, int mode, long long, long long, long long nr, long long nc, long long tpr, long long) {
         ++n;
-        g += ((nr + rp - 1) / rp * rp * tpr * ws_af_width(mode) + 31) / 32 * 32;
+        g += (nr * ws_af_kept_row(mode, (int)nc, (int)tpr) + 31) / 32 * 32;
     });
     if (n > 0x0fffffffLL || m > 0x0fffffffLL || g / 32 > 0xffffffffLL) return;
     p->n_afitems = n;
@@ -444,7 +445,8 @@ WsLambWs ws_lamb_layout(const ws_plan* p, void* workspace) {
     o = (o + 255) & ~(size_t)255;
     L.ghat = (float*)(b + o);
     L.bytes_lars = o + sizeof(float) * (size_t)p->R * (size_t)p->S;
-    // (the one-kernel Adafactor keeps the sums block by block, a few floats more than [R][S] may hold)
+    // (the one-kernel Adafactor keeps the sums block by block, which may be more than [R][S] by an eighth and by
+    // less than 128 bytes a block)
     const size_t ghat_af = (size_t)p->af_ghat > (size_t)p->R * (size_t)p->S ? (size_t)p->af_ghat : (size_t)p->R * (size_t)p->S;
     o = ((size_t)((char*)L.ghat - b) + sizeof(float) * ghat_af + 255) & ~(size_t)255;
     L.acc = (float*)(b + o);
@@ -633,7 +635,7 @@ void ws_build_af_schedule(ws_plan* p) {
         it.tpr = (unsigned short)tpr; it.rp = (unsigned short)rp;
         it.goff32 = (unsigned)goff;
         it.item = (unsigned)items.size();
-        goff += ((nr + rp - 1) / rp * rp * tpr * ws_af_width(mode) + 31) / 32;
+        goff += (nr * ws_af_kept_row(mode, (int)nc, (int)tpr) + 31) / 32;
         items.push_back(it);
     });
     // groups of consecutive tensors; a group's chunks are consecutive too, once the unfactored tensors' are left out

@@ -289,6 +289,16 @@ def test_one_launch_items_are_whole_tiles(layout, tile):
     assert max(it.len for it in items) == {1024: 8192, 2048: 8192, 3072: 3072, 16384: 16384}[K]
 
 
+@pytest.mark.parametrize("shapes", [[(100000, 1)], [(100000, 5)], [(50000, 3)], [(30000, 17)], [(257, 2056), (70, 9), (513, 1)]])
+def test_adafactor_workspace_keeps_narrow_rows_dense(shapes):
+    """The kept gradient sums take at most an eighth more than a float per parameter, also where a row is shorter
+    than a thread's four columns (a row of one column took four floats)."""
+    plan = B.Plan(shapes, 1, 32, upload=False)
+    rows, F, N = sum(s[0] for s in shapes), plan.factored_elems, plan.N
+    rest = 8 * (F + 16 * plan.T) + 8 * rows + 200 * (N // 1024 + 8) + 4096     # sums, factors, blocks, rounding
+    assert plan.workspace_bytes("adafactor") <= plan.workspace_bytes("lars") + N // 2 + rest
+
+
 def test_one_launch_schedule_on_bert_large_keeps_phase_two_close():
     """On the BERT-large set (R = 16) the state a phase-2 item reads was written a bounded distance earlier:
     except for the embedding (larger than L2) and the few tensors whose phase 2 queues behind the
