@@ -100,7 +100,8 @@ static void ws_af_blocks(const ws_plan* p, F&& emit) {
         const long long units = (ncol + W - 1) / W, s0 = (units + 255) / 256;
         long long best_s = s0, best = -1;              // (busy threads of 256) / strips, compared as fractions
         for (long long s = s0; s < s0 + 8 && s <= units; ++s) {
-            const long long tpr = (units + s - 1) / s, score = units * (256 / tpr) * 4096 / s;
+            const long long tpr = (units + s - 1) / s, rows = 256 / tpr < nrow ? 256 / tpr : nrow;
+            const long long score = units * rows * 4096 / s;     // (a vector is one row: the fewest strips)
             if (score > best) { best = score; best_s = s; }
         }
         const long long tpr = (units + best_s - 1) / best_s;

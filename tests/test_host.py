@@ -299,6 +299,21 @@ def test_adafactor_workspace_keeps_narrow_rows_dense(shapes):
     assert plan.workspace_bytes("adafactor") <= plan.workspace_bytes("lars") + N // 2 + rest
 
 
+def _adafactor_entries(shapes):
+    plan = B.Plan(shapes, 1, 32, upload=False)
+    n, up = len(plan.schedule()[1]), lambda x: (x + 15) // 16 * 16  # noqa: E731
+    lamb = up(32 * n) + up(16 * plan.T) + up(8 * n)
+    return (B.lib().ws_plan_schedule_bytes(plan.handle) - lamb - 96 * plan.T) // 32
+
+
+@pytest.mark.parametrize("shape,blocks,chunks", [((768,), 1, 0), ((640,), 1, 0), ((1023,), 1, 0), ((1, 513), 1, 1), ((2, 640), 1, 1),
+                                                 ((1,), 1, 0), ((3, 8), 1, 1), ((64, 24), 1, 1)])
+def test_adafactor_short_tensors_are_one_block(shape, blocks, chunks):
+    """Strips that a row is cut into only pay where the tensor has rows for the threads that they leave: a vector of
+    768 elements was three blocks of 64 threads, each three schedule entries."""
+    assert _adafactor_entries([shape]) == 3 * blocks + chunks
+
+
 def test_one_launch_schedule_on_bert_large_keeps_phase_two_close():
     """On the BERT-large set (R = 16) the state a phase-2 item reads was written a bounded distance earlier:
     except for the embedding (larger than L2) and the few tensors whose phase 2 queues behind the
