@@ -167,8 +167,8 @@ ws_status ws_plan_upload(ws_plan* plan, void* dev_buf, size_t bytes, void* strea
  * their order are part of the same upload); other cases and the shard-by-shard calls run as
  * before.  The kernel's waits (a phase-2 item waits for its tensor's ratio) are bounded: if one
  * ever runs out, the kernel leaves the update incomplete and sets the 32-bit status word inside
- * the workspace (ws_workspace_sync_status gives its byte offset; 0 = completed) - a caller that
- * wants to detect this reads the word after synchronising the stream.
+ * the workspace (ws_workspace_sync_status gives its byte offset; 0 = completed, also after the
+ * separate launches) - a caller that wants to detect this reads the word after synchronising the stream.
  * ws_plan_schedule_view / ws_plan_schedule_item expose the order for inspection (host only):
  * entry i of `order` is item index * 2 + phase (0: phase 1, 1: phase 2). */
 size_t ws_plan_schedule_bytes(const ws_plan* plan);

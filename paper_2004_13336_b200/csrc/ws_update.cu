@@ -94,7 +94,7 @@ __global__ void __launch_bounds__(kBlock, ((VEC == 8 && GBF && !FUSED) || RB > 8
 // With lars != 0 the ratio is the LARS local rate eta sqrt(a) / (sqrt(b) + beta sqrt(a)).
 __global__ void __launch_bounds__(kBlock) lamb_finalize_kernel(const WsSegTiles* segtiles, const float2* partials,
                                                                long long ntiles, int R, float* rho, double* norms,
-                                                               int lars, double eta, double beta) {
+                                                               int lars, double eta, double beta, int* status) {
     // R == 1 with the concatenated layout: a tensor's tiles of all shards are one contiguous run
     __shared__ double sa[kBlock / 32], sb[kBlock / 32];
     const int t = blockIdx.x;
@@ -104,6 +104,7 @@ __global__ void __launch_bounds__(kBlock) lamb_finalize_kernel(const WsSegTiles*
     asm volatile("griddepcontrol.wait;" ::: "memory");
     sum_partials(mine, partials, ntiles, R, sa, sb, a, b);
     if (threadIdx.x == 0) {
+        if (t == 0) *status = 0;      // (nothing waits in this form: the update is complete)
         norms[2 * t] = a;
         norms[2 * t + 1] = b;
         if (!(a > 0.0 && b > 0.0)) rho[t] = 1.0f;
@@ -160,12 +161,13 @@ __global__ void __launch_bounds__(kBlock) af_factors_kernel(const WsAfChunk* chu
 __global__ void __launch_bounds__(kBlock) af_finalize_clip_kernel(const WsSegTiles* segtiles, const WsSegAf* segaf,
                                                                   const float2* partials, long long ntiles, int R,
                                                                   float* alpha, float* rho, double* norms, double eps2,
-                                                                  double rho_step, double d) {
+                                                                  double rho_step, double d, int* status) {
     __shared__ double sa[kBlock / 32], sb[kBlock / 32];
     const int t = blockIdx.x;
     double sw, su;
     sum_partials(segtiles[t], partials, ntiles, R, sa, sb, sw, su);
     if (threadIdx.x == 0) {
+        if (t == 0) *status = 0;
         const long long n = segaf[t].numel;
         const double rms_w = n > 0 ? sqrt(sw / (double)n) : 0.0;
         const double rms_u = n > 0 ? sqrt(su / (double)n) : 0.0;
@@ -291,7 +293,7 @@ __global__ void __launch_bounds__(kBlock, kAf2Ctas) af_sumsq_kernel(const UpdPar
 
 // -------------------------------------------------------------- dispatch ---
 void launch_lamb_finalize(int T, cudaStream_t st, const WsSegTiles* segtiles, const float2* partials, long long ntiles,
-                          int R, float* rho, double* norms, int lars, double eta, double beta) {
+                          int R, float* rho, double* norms, int lars, double eta, double beta, int* status) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)T);
     cfg.blockDim = dim3(kBlock);
@@ -301,7 +303,7 @@ void launch_lamb_finalize(int T, cudaStream_t st, const WsSegTiles* segtiles, co
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, lamb_finalize_kernel, segtiles, partials, ntiles, R, rho, norms, lars, eta, beta);
+    cudaLaunchKernelEx(&cfg, lamb_finalize_kernel, segtiles, partials, ntiles, R, rho, norms, lars, eta, beta, status);
 }
 
 template <int OPT, bool GBF, int OUT, int VEC, int U, int RB, int NP, bool FUSED>
@@ -558,7 +560,7 @@ extern "C" ws_status ws_lamb_finalize(const ws_plan* plan, void* workspace, size
     if (s != WS_OK) return s;
     WsLambWs L = ws_lamb_layout(plan, workspace);
     launch_lamb_finalize(plan->T, (cudaStream_t)stream, plan->d_segtiles, L.partials, plan->ntiles,
-                                                                      finalize_reps(plan), L.rho, L.norms, 0, 0.0, 0.0);
+                                                                      finalize_reps(plan), L.rho, L.norms, 0, 0.0, 0.0, L.status);
     return ws_check_launch("ws_lamb_finalize");
 }
 
@@ -604,7 +606,7 @@ extern "C" ws_status ws_lars_finalize(const ws_plan* plan, const ws_hyper* hyper
     const WsLambWs L = ws_lamb_layout(plan, workspace);
     launch_lamb_finalize(plan->T, (cudaStream_t)stream, plan->d_segtiles, L.partials, plan->ntiles,
                                                                       finalize_reps(plan), L.rho, L.norms, 1,
-                                                                      hyper->trust_coeff, hyper->weight_decay);
+                                                                      hyper->trust_coeff, hyper->weight_decay, L.status);
     return ws_check_launch("ws_lars_finalize");
 }
 
@@ -906,7 +908,7 @@ ws_status af_stage(const ws_plan* plan, int stage, int32_t r, const ws_grads* gr
             const double rho_step = hyper->lr < inv_sqrt_t ? hyper->lr : inv_sqrt_t;
             af_finalize_clip_kernel<<<plan->T, kBlock, 0, st>>>(plan->d_segtiles, plan->d_segaf, L.partials, plan->ntiles,
                                                                finalize_reps(plan), L.alpha, L.rho, L.norms, hyper->eps2,
-                                                               rho_step, hyper->clip_threshold);
+                                                               rho_step, hyper->clip_threshold, L.status);
             return ws_check_launch("adafactor(clipping)");
         }
         case WS_AF_APPLY: {
@@ -1061,7 +1063,7 @@ extern "C" ws_status ws_fused_update(const ws_plan* plan, int32_t r, const ws_te
         if ((s = fused_phase(plan, -1, grads, state, hyper, weights, K_LARS1, workspace, st)) != WS_OK) return s;
         const WsLambWs L = ws_lamb_layout(plan, workspace);
         launch_lamb_finalize(plan->T, st, plan->d_segtiles, L.partials, plan->ntiles, finalize_reps(plan), L.rho,
-                                                        L.norms, 1, hyper->trust_coeff, hyper->weight_decay);
+                                                        L.norms, 1, hyper->trust_coeff, hyper->weight_decay, L.status);
         if ((s = ws_check_launch("ws_fused_update(LARS finalize)")) != WS_OK) return s;
         return fused_phase(plan, -1, grads, state, hyper, weights, K_LARS2, workspace, st);
     }

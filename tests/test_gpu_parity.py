@@ -835,6 +835,23 @@ def test_one_kernel_has_the_bits_of_the_shard_by_shard_calls(opt, R, gdtype, lay
     assert all(x is None or torch.equal(x, y) for x, y in zip(one, per)) and torch.equal(ga, gb)
 
 
+@pytest.mark.parametrize("opt,slots", [("lamb", 2), ("lars", 1), ("adafactor", 0)])
+@pytest.mark.parametrize("R", [1, 8])
+def test_status_word_is_valid_after_every_all_shard_update(opt, slots, R):
+    # whichever route a call takes, the word says 0 (completed) afterwards, also on a workspace that held anything
+    wl, w, m, v, g = _model(SHAPES, R, seed=3, gstd=1e-3)
+    h = dict(_hyper("sgdm"), weight_decay=0.0, trust_coeff=0.001, lr=1e-3)
+    for one_launch in (True, False):
+        plan = B.Plan(SHAPES, 2, 32, one_launch=one_launch)
+        pw, pm, pv, pg = _pack_all(plan, w, m, v, g)
+        if opt == "adafactor":
+            pv = torch.full((plan.factored_elems,), 1e-6, device=DEV)
+        ws = torch.full((plan.workspace_bytes(opt),), 0xA5, dtype=torch.uint8, device=DEV)
+        B.ws_shard_update(plan, -1, pg, pw, pm if slots else None, pv if slots != 1 else None, B.make_hyper(opt, h), None, ws)
+        off = plan.sync_status_offset()
+        assert int(ws[off:off + 4].view(torch.int32).item()) == 0
+
+
 def test_lars_poisoned_pads_and_error_codes():
     import ctypes as C
     R = 5
