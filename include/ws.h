@@ -162,17 +162,20 @@ ws_status ws_plan_upload(ws_plan* plan, void* dev_buf, size_t bytes, void* strea
  *                            cudaMemcpyAsync on `stream`; call once, before the plan is shared
  *                            between threads
  * Afterwards ws_shard_update / ws_fused_update with r == -1 and WS_LAMB (and
- * ws_lamb_update_static_scratch) take the one-kernel route when there are 8 to 32 gradient copies, WS_LARS
- * when there are 4 to 32 and WS_ADAFACTOR always - where it measured faster on a B200 (Adafactor's blocks and
- * their order are part of the same upload); other cases and the shard-by-shard calls run as
- * before.  The kernel's waits (a phase-2 item waits for its tensor's ratio) are bounded: if one
+ * ws_lamb_update_static_scratch), WS_LARS or WS_ADAFACTOR (whose blocks and their order are part of the
+ * same upload) take the one-kernel route where it measured no slower on a B200; ws_plan_one_kernel says
+ * for which number and type of gradient copies that is.  Other cases and the shard-by-shard calls run as
+ * separate launches.  The kernel's waits (a phase-2 item waits for its tensor's ratio) are bounded: if one
  * ever runs out, the kernel leaves the update incomplete and sets the 32-bit status word inside
  * the workspace (ws_workspace_sync_status gives its byte offset; 0 = completed, also after the
  * separate launches) - a caller that wants to detect this reads the word after synchronising the stream.
+ *   ws_plan_one_kernel       1 where the all-shard update of `opt` from `copies` gradient copies of
+ *                            `grad_dtype` runs as one kernel once the schedule is uploaded, else 0 (host only)
  * ws_plan_schedule_view / ws_plan_schedule_item expose the order for inspection (host only):
  * entry i of `order` is item index * 2 + phase (0: phase 1, 1: phase 2). */
 size_t ws_plan_schedule_bytes(const ws_plan* plan);
 ws_status ws_plan_upload_schedule(ws_plan* plan, void* dev_buf, size_t bytes, void* stream);
+int32_t ws_plan_one_kernel(const ws_plan* plan, ws_opt opt, int32_t copies, ws_dtype grad_dtype);
 typedef struct {
     int32_t tensor, shard;
     int64_t pos;        /* start inside the shard                     */

@@ -94,7 +94,7 @@ EXPORTS = [
     "ws_lars_partial", "ws_lars_finalize", "ws_lars_apply",
     "ws_adafactor_stage", "ws_workspace_adafactor_sums",
     "ws_plan_schedule_bytes", "ws_plan_upload_schedule", "ws_plan_schedule_view", "ws_plan_schedule_item",
-    "ws_workspace_sync_status",
+    "ws_workspace_sync_status", "ws_plan_one_kernel",
     "ws_debug_bounds_enabled", "ws_debug_bounds_read", "ws_debug_bounds_selftest",
 ]
 
@@ -198,6 +198,8 @@ def lib() -> C.CDLL:
     L.ws_plan_schedule_view.argtypes = [vp, C.POINTER(C.POINTER(C.c_uint32)), C.POINTER(C.c_int64)]
     L.ws_plan_schedule_item.restype = C.c_int
     L.ws_plan_schedule_item.argtypes = [vp, C.c_int64, C.POINTER(ws_sched_item)]
+    L.ws_plan_one_kernel.restype = C.c_int32
+    L.ws_plan_one_kernel.argtypes = [vp, C.c_int, C.c_int32, C.c_int]
     L.ws_workspace_sync_status.restype = C.c_int
     L.ws_workspace_sync_status.argtypes = [vp, C.POINTER(C.c_size_t)]
     L.ws_debug_bounds_enabled.restype = C.c_int32
@@ -315,8 +317,8 @@ class Plan:
     def __init__(self, shapes: Sequence[Sequence[int]], R: int, align_elems: int = 32, tile_elems: int = 0,
                  device: Optional[torch.device] = None, upload: bool = True, layout: str = "per_tensor",
                  one_launch: bool = True):
-        """``one_launch``: also upload the plan's one-launch schedule, so that the all-shard LAMB and LARS
-        updates run as one kernel (with ``False`` they run as three launches)."""
+        """``one_launch``: also upload the plan's one-launch schedule, so that the all-shard LAMB, LARS and
+        Adafactor updates run as one kernel where that is no slower (with ``False`` always as separate launches)."""
         T = len(shapes)
         descs = (ws_tensor_desc * max(1, T))()
         for i, s in enumerate(shapes):
@@ -377,6 +379,11 @@ class Plan:
             _check(lib().ws_plan_schedule_item(self._h, i, C.byref(it)), "ws_plan_schedule_item")
             items.append(it)
         return [(int(e) >> 1, int(e) & 1) for e in arr], items
+
+    def one_kernel(self, opt, copies: int, grad_dtype: torch.dtype = torch.float32) -> bool:
+        """Whether the all-shard update of ``opt`` from ``copies`` gradient copies runs as one kernel on this plan."""
+        code = OPT_CODE[opt] if isinstance(opt, str) else int(opt)
+        return self.sched_buf is not None and bool(lib().ws_plan_one_kernel(self._h, code, copies, _dtype_code(grad_dtype)))
 
     def sync_status_offset(self) -> int:
         off = C.c_size_t()

@@ -157,6 +157,7 @@ struct ws_plan {
     std::vector<unsigned> sched;              // [2 n_items]: item index * 2 + phase, in execution order
     // the same for Adafactor (0 items: the plan has none)
     long long n_afitems = 0, n_afsched = 0, af_ghat = 0, af_rows = 0;   // items, schedule entries, floats of kept gradient sums, rows
+    long long af_scalar = 0;                  // elements in rows that 4 does not divide
     std::vector<WsAfTensor> aftensors;
     std::vector<WsAfItem> afsched;
     const WsAfTensor* d_aftensors = nullptr;

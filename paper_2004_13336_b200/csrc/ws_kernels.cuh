@@ -875,7 +875,6 @@ struct OneLaunch {
     double* norms;               // [T][2]
     double eta, beta;            // LARS: trust coefficient and weight decay
 };
-bool one_launch_supports(int pair, int R);
 // pair 0: LAMB, 1: LARS.  P carries the arguments of both phases (gradient sources, state, outputs).
 ws_status launch_one_launch(int pair, bool gbf, int out, bool fused, bool wide, const UpdParams& P,
                             const void* const* gptrs, const OneLaunch& Q, cudaStream_t st);

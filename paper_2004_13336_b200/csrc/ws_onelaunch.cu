@@ -240,15 +240,6 @@ ws_status launch_clear(void* p, size_t bytes, int* status, cudaStream_t st) {
     return ws_check_launch("one-kernel update (clear)");
 }
 
-// Where the one-kernel route measured faster than the three launches on a B200.  LAMB with 8 to 32 gradient
-// copies (BERT-large set, R = 16: 4.85 ms against 5.13 ms; with items of their own size instead of the plan's
-// tiles: ResNet-50 set 324 -> 253 us, a 37.6 M parameter Transformer 463 -> 361 us, a 1.7 M parameter one 40 ->
-// 28 us, R = 8 each); with few copies phase 1 is as short as phase 2 and the three launches win (Transformer
-// set, R = 4: 1.64 ms against 1.67 ms, R = 2: 1.38 against 1.49 ms).  LARS with 4 to 32 copies (ResNet-50 set,
-// R = 8: 234 -> 226 us; Transformer set, R = 4: 1418 -> 1386 us, R = 16 bf16: 2036 -> 1845 us; 45 792 parameters:
-// 14.6 -> 8.7 us); at R = 2 the three launches win by 1 % (152 against 154 us).
-bool one_launch_supports(int pair, int R) { return R <= 32 && R >= (pair == 0 ? 8 : 4); }
-
 ws_status launch_one_launch(int pair, bool gbf, int out, bool fused, bool wide, const UpdParams& P,
                             const void* const* gptrs, const OneLaunch& Q, cudaStream_t st) {
     if (pair == 1)

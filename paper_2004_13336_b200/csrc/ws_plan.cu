@@ -120,13 +120,14 @@ static void ws_af_blocks(const ws_plan* p, F&& emit) {
 // Block and schedule-entry counts and the floats of kept gradient sums; a tensor beyond the block fields'
 // ranges leaves the plan without Adafactor blocks.
 static void ws_count_af(ws_plan* p) {
-    p->n_afitems = p->n_afsched = p->af_ghat = p->af_rows = 0;
+    p->n_afitems = p->n_afsched = p->af_ghat = p->af_rows = p->af_scalar = 0;
     if (p->R > 65535) return;
     long long n = 0, m = 0, g = 0, rows = 0;
     for (const WsSegAf& a : p->segaf) {
         if (a.nrow > 0x7fffffffLL || a.ncol > 0x7fffffffLL) return;
         if (a.nrow > 0) m += (a.nrow + a.ncol + kWsAfChunk - 1) / kWsAfChunk;
         rows += a.nrow;
+        if (a.nrow > 0 && a.ncol % 4 != 0) p->af_scalar += a.numel;
     }
     ws_af_blocks(p, [&](int, int mode, long long, long long, long long nr, long long nc, long long tpr, long long) {
         ++n;

@@ -528,6 +528,43 @@ void offset_grad_ptrs(const ws_plan* p, int32_t r, const ws_grads* g, std::vecto
 // shard, ntiles apart) for the per-tensor layout, 1 for the concatenated layout.
 int finalize_reps(const ws_plan* p) { return p->layout == WS_LAYOUT_CONCAT ? 1 : p->R; }
 
+// Parameters from which the one kernel of LAMB / LARS is not slower than the three launches (-1: never); both give
+// the same bits.  Its two phases are the waves of one grid, each behind a chain of table reads, and a small model has
+// two or three of them; what it saves, phase 2's second read, grows with the model.  More copies shorten that saving's
+// share, and fp32 gradients leave the three launches closer to the copy bandwidth than bf16 ones, whose wide phase 1
+// spills in both forms - but not with 4 copies, where the separate kernel has a variant of its own.  Device time one
+// kernel / three launches, state and gradients not in L2 (encoder-decoder and image sets of M parameters, us):
+//   LAMB fp32   8 copies   1.7 M 30.2/28.2   2.4 M 40.1/36.3   4.6 M 62.4/63.1   7.6 M 81.8/93.7     26 M 257/279
+//              16 copies   4.6 M 86.0/83.1   7.6 M 130/128     26 M 389/411      32 copies 7.6 M 227/204  26 M 644/686
+//        bf16   8 copies  0.37 M 16.2/14.0   1.7 M 42.4/48.9   7.6 M 120/181     32 copies 1.7 M 78.9/85.7
+//   LARS fp32   4 copies   4.6 M 44.1/45.8   6.9 M 58.9/53.3   26 M 178/190      8 copies 2.4 M 37.4/31.9  4.6 M 55.4/53.5
+//               8 copies   6.9 M 76.9/77.4   7.6 M 75.6/81.7   26 M 229/234     16 copies 26 M 359/356  56 M 748/772
+//        bf16   4 copies   7.6 M 76.0/47.9   56 M 459/350        8 copies 2.0 M 50.5/46.6  4.1 M 67.9/78.5  26 M 243/299
+// LAMB with 2 to 7 copies and LARS with 2 or 3 run as three launches (211 M, LAMB: 4 copies 1.64 ms against 1.67).
+long long pair_min_params(bool lars, bool gbf, int copies) {
+    constexpr long long M = 1 << 20;
+    if (copies < (lars ? 4 : 8) || copies > 32) return -1;
+    if (lars) return gbf ? (copies == 4 ? -1 : 3 * M) : (copies == 4 ? 8 * M : copies <= 8 ? 4 * M : 32 * M);
+    return gbf ? M : (copies <= 8 ? 4 * M : copies <= 16 ? 8 * M : 16 * M);
+}
+
+// Whether an all-shard update of `opt` runs as one kernel where the plan's schedule is on the device.
+// Adafactor's kernel has every model size and copy count as long as rows are vectors.  Rows that 4 does not divide are
+// read element by element there, while the stages read runs of the flat tensor, so that many copies are faster by
+// stages (ragged tensors, one kernel / stages, us: 13.6 M fp32 32 copies 468/525, 64 copies 940/730; bf16 16 copies
+// 383/415, 32 copies 684/454; 30 M fp32 16 copies 539/566, 32 copies 965/932; bf16 12 copies 523/477; with vector rows
+// 26 M, 128 copies: fp32 2068/2291, bf16 1305/1773).  At 1.5 to 2 times the time for those against 0.7 to 0.9 for
+// the others the two even out where an eighth of the elements lies in such rows.
+bool one_kernel(const ws_plan* p, int opt, int copies, bool gbf) {
+    if (copies < 1) return false;
+    if (opt == WS_LAMB || opt == WS_LARS) {
+        const long long n = pair_min_params(opt == WS_LARS, gbf, copies);
+        return p->n_items > 0 && n >= 0 && p->N >= n;
+    }
+    if (opt != WS_ADAFACTOR || p->n_afitems <= 0) return false;
+    return p->af_scalar <= p->N / 8 || copies <= (gbf ? 16 : 32) / (p->N > (24LL << 20) ? 2 : 1);
+}
+
 ws_status check_ws(const ws_plan* p, void* workspace, size_t bytes, ws_opt opt = WS_LAMB) {
     if (!workspace || bytes < ws_workspace_bytes(p, opt)) return WS_ERR_WORKSPACE;
     if (!ws_aligned16(workspace)) return WS_ERR_ALIGNMENT;
@@ -535,6 +572,10 @@ ws_status check_ws(const ws_plan* p, void* workspace, size_t bytes, ws_opt opt =
 }
 
 }  // namespace
+
+extern "C" int32_t ws_plan_one_kernel(const ws_plan* plan, ws_opt opt, int32_t copies, ws_dtype grad_dtype) {
+    return plan && one_kernel(plan, (int)opt, copies, grad_dtype == WS_BF16) ? 1 : 0;
+}
 
 extern "C" ws_status ws_lamb_partial(const ws_plan* plan, int32_t r, const ws_grads* grads, const ws_state* state,
                                      const ws_hyper* hyper, void* workspace, size_t workspace_bytes, void* stream) {
@@ -642,7 +683,8 @@ ws_status try_one_launch(const ws_plan* plan, int pair, const ws_grads* grads, c
     if (!plan || !plan->d_sched) return WS_OK;
     const bool fused = gtab != nullptr;
     const int copies = fused ? gtab->nsets : (grads ? grads->R : 0);
-    if (!one_launch_supports(pair, copies)) return WS_OK;
+    if (!one_kernel(plan, pair == 0 ? WS_LAMB : WS_LARS, copies, (fused ? gtab->dtype : grads ? grads->dtype : WS_F32) == WS_BF16))
+        return WS_OK;
     UpdParams P;
     int out_kind;
     bool gbf;
@@ -930,6 +972,8 @@ ws_status try_af_one_launch(const ws_plan* plan, const ws_grads* grads, const ws
     done = false;
     if (!plan || !hyper || !plan->d_afsched) return WS_OK;
     const bool fused = gtab != nullptr;
+    const int copies = fused ? gtab->nsets : (grads ? grads->R : 0);
+    if (!one_kernel(plan, WS_ADAFACTOR, copies, (fused ? gtab->dtype : grads ? grads->dtype : WS_F32) == WS_BF16)) return WS_OK;
     ws_status s = af_check(plan, -1, hyper, workspace, workspace_bytes);
     if (s != WS_OK) return s;
     UpdParams U;

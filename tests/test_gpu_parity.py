@@ -797,7 +797,7 @@ def test_lars_shard_by_shard_phases(R):
     assert e.value.status == 1
 
 
-@pytest.mark.parametrize("opt,R", [("lamb", 8), ("lamb", 32), ("lars", 5), ("lars", 8)])
+@pytest.mark.parametrize("opt,R", [("lamb", 8), ("lamb", 16), ("lars", 5), ("lars", 8), ("lars", 32)])
 @pytest.mark.parametrize("gdtype,layout,tile", [(torch.float32, "per_tensor", 0), (torch.bfloat16, "per_tensor", 1024),
                                                 (torch.bfloat16, "concat", 2048), (torch.float32, "concat", 3072),
                                                 (torch.bfloat16, "per_tensor", 3072), (torch.float32, "per_tensor", 16384)])
@@ -805,17 +805,17 @@ def test_one_kernel_has_the_bits_of_the_shard_by_shard_calls(opt, R, gdtype, lay
     # the one kernel's items are several tiles (tiles of 1024 share a pass of 8-element vectors, in tiles of 3072
     # a pass does not end with the tile, 16384 is more than an item of several tiles has); the partial norms are the
     # tiles' in both forms, so norms, ratios, state and emitted weights agree bit for bit
-    shapes = SHAPES + [(1500, 4099), (0,), (1500, 307)]
+    shapes = SHAPES + [(2000, 4099), (0,), (1500, 307)]
     wl, w, m, v, g = _model(shapes, R, gdtype, seed=R, gstd=1e-3)
     plan = B.Plan(shapes, 8, 32, tile, layout=layout)
-    assert plan.sched_buf is not None
+    assert plan.one_kernel(opt, R, gdtype) or (opt, R, gdtype) == ("lars", 32, torch.float32)    # (that needs 32 M parameters)
     h = B.make_hyper(opt, _lars_hyper() if opt == "lars" else _hyper("lamb"))
     pw, pm, pv, pg = _pack_all(plan, w, m, v, g)
     state = lambda x: [x[0].clone(), x[1].clone(), x[2].clone() if opt == "lamb" else None]  # noqa: E731
     one, per = state((pw, pm, pv)), state((pw, pm, pv))
     wsa = torch.zeros(plan.workspace_bytes(opt), dtype=torch.uint8, device=DEV)
     off = plan.sync_status_offset()
-    wsa[off:off + 4] = 0xFF                        # the one kernel clears the status word, nothing else writes it
+    wsa[off:off + 4] = 0xFF
     wsb = torch.zeros_like(wsa)
     ga, gb = torch.zeros(plan.G, dtype=torch.bfloat16, device=DEV), torch.zeros(plan.G, dtype=torch.bfloat16, device=DEV)
     B.ws_shard_update(plan, -1, pg, *one, h, ga, wsa)
@@ -833,6 +833,21 @@ def test_one_kernel_has_the_bits_of_the_shard_by_shard_calls(opt, R, gdtype, lay
     head = up(4 * plan.T) + 16 * plan.T           # ratios and squared norms
     assert torch.equal(wsa[:head], wsb[:head])
     assert all(x is None or torch.equal(x, y) for x, y in zip(one, per)) and torch.equal(ga, gb)
+    # formatting fused in, bf16 weights next to the state and fp32 weights as the master copy, two steps in a row:
+    # against the three launches
+    plans = (plan, B.Plan(shapes, 8, 32, tile, layout=layout, one_launch=False))
+    for master in (False, True):
+        got = []
+        for p in plans:
+            sw, sm, sv = state((pw, pm, pv))
+            outs = [x.clone() if master else x.to(torch.bfloat16) for x in w]
+            gt, wt = B.TensorTable(p, g), B.TensorTable(p, [outs])
+            ws = torch.full((p.workspace_bytes(opt),), 0xA5, dtype=torch.uint8, device=DEV)
+            for _ in range(2):
+                B.ws_fused_update(p, -1, gt, None if master else sw, sm, sv, h, wt, ws)
+            assert int(ws[off:off + 4].view(torch.int32).item()) == 0
+            got.append([sw, sm] + ([sv] if sv is not None else []) + outs + [ws[:head]])
+        assert all(torch.equal(a, b) for a, b in zip(*got))
 
 
 @pytest.mark.parametrize("opt,slots", [("lamb", 2), ("lars", 1), ("adafactor", 0)])

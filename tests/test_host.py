@@ -314,6 +314,33 @@ def test_adafactor_short_tensors_are_one_block(shape, blocks, chunks):
     assert _adafactor_entries([shape]) == 3 * blocks + chunks
 
 
+@pytest.mark.parametrize("opt,gdtype,copies,least", [
+    ("lamb", torch.float32, 8, 4 << 20), ("lamb", torch.float32, 9, 8 << 20), ("lamb", torch.float32, 32, 16 << 20),
+    ("lamb", torch.bfloat16, 8, 1 << 20), ("lamb", torch.bfloat16, 7, None), ("lamb", torch.float32, 33, None),
+    ("lars", torch.float32, 4, 8 << 20), ("lars", torch.float32, 5, 4 << 20), ("lars", torch.float32, 9, 32 << 20),
+    ("lars", torch.bfloat16, 5, 3 << 20), ("lars", torch.bfloat16, 4, None), ("lars", torch.float32, 3, None),
+    ("lars", torch.bfloat16, 33, None), ("sgdm", torch.float32, 8, None), ("adam", torch.float32, 8, None)])
+def test_one_kernel_route_by_size_and_copies(opt, gdtype, copies, least):
+    route = lambda n: B.lib().ws_plan_one_kernel(  # noqa: E731
+        B.Plan([(n // 1024, 1024)], 2, 32, upload=False).handle, B.OPT_CODE[opt], copies, B._dtype_code(gdtype))
+    assert route(64 << 20) == (least is not None)
+    if least is not None:
+        assert route(least) == 1 and route(least - 1024) == 0
+
+
+def test_one_kernel_route_of_adafactor_by_odd_rows():
+    def route(shapes, copies, gdtype=torch.float32):
+        plan = B.Plan(shapes, 2, 32, upload=False)
+        assert not plan.one_kernel("adafactor", 1)            # (nothing uploaded)
+        return B.lib().ws_plan_one_kernel(plan.handle, B.WS_ADAFACTOR, copies, B._dtype_code(gdtype))
+    even, odd, some = [(1000, 1024), (7,)], [(1000, 1025)], [(1000, 1024), (100, 1025)]
+    large = [(25000, 1025)]
+    assert all(route(s, c, d) for s in (even, some) for c in (1, 1024) for d in (torch.float32, torch.bfloat16))
+    assert route(odd, 32) and not route(odd, 33) and route(odd, 16, torch.bfloat16) and not route(odd, 17, torch.bfloat16)
+    assert route(large, 16) and not route(large, 17) and route(large, 8, torch.bfloat16) and not route(large, 9, torch.bfloat16)
+    assert not route(even, 0)
+
+
 def test_one_launch_schedule_on_bert_large_keeps_phase_two_close():
     """On the BERT-large set (R = 16) the state a phase-2 item reads was written a bounded distance earlier:
     except for the embedding (larger than L2) and the few tensors whose phase 2 queues behind the
