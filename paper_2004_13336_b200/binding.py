@@ -302,13 +302,15 @@ assert _HYPER.size == C.sizeof(ws_hyper)
 def make_hyper(opt, hyper: dict) -> ws_hyper:
     code = OPT_CODE[opt] if isinstance(opt, str) else int(opt)
     get = hyper.get
-    fields = (code, hyper["lr"], hyper["beta1"], hyper["beta2"], hyper["eps"], hyper["weight_decay"], hyper["momentum"],
-              hyper["grad_scale"], int(hyper["step"]), float(get("trust_coeff", 0.001)), float(get("eps2", 1e-3)),
-              float(get("clip_threshold", 1.0)), float(get("decay_exponent", 0.8)))
     try:
-        return ws_hyper.from_buffer_copy(_HYPER.pack(*fields))
+        return ws_hyper.from_buffer_copy(_HYPER.pack(
+            code, hyper["lr"], hyper["beta1"], hyper["beta2"], hyper["eps"], hyper["weight_decay"], hyper["momentum"],
+            hyper["grad_scale"], int(hyper["step"]), get("trust_coeff", 0.001), get("eps2", 1e-3),
+            get("clip_threshold", 1.0), get("decay_exponent", 0.8)))
     except struct.error:         # what struct refuses goes by ctypes' rules
-        return ws_hyper(*fields)
+        return ws_hyper(code, hyper["lr"], hyper["beta1"], hyper["beta2"], hyper["eps"], hyper["weight_decay"],
+                        hyper["momentum"], hyper["grad_scale"], int(hyper["step"]), float(get("trust_coeff", 0.001)),
+                        float(get("eps2", 1e-3)), float(get("clip_threshold", 1.0)), float(get("decay_exponent", 0.8)))
 
 
 class Plan:
@@ -459,12 +461,12 @@ _OUT = struct.Struct("@Pi4x")
 assert _STATE.size == C.sizeof(ws_state) and _OUT.size == C.sizeof(ws_out)
 
 
-def _address(x, cls):
-    """Address of a ctypes object that has to be a `cls` (the plain-address prototypes cannot tell)."""
+def _refuse(x, cls):
+    """For an object that is not exactly a `cls`: raises unless it is one by inheritance (the plain-address
+    prototypes cannot tell)."""
     if not isinstance(x, cls):
         C.byref(x)               # a TypeError where x is no ctypes object at all
         raise C.ArgumentError(f"expected {cls.__name__} instead of {type(x).__name__}")
-    return C.addressof(x)
 
 
 def _state_bytes(w, m, v):
@@ -481,9 +483,11 @@ def _out(gathered):
 def ws_shard_update(plan: Plan, r: int, gbufs: Sequence[torch.Tensor], w, m, v, hyper: ws_hyper,
                     gathered: Optional[torch.Tensor] = None, workspace: Optional[torch.Tensor] = None,
                     slice_mode: int = 0):
+    if type(hyper) is not ws_hyper:
+        _refuse(hyper, ws_hyper)
     g = _grads(gbufs, slice_mode)
     st = _step().ws_shard_update(
-        plan.handle, r, C.addressof(g), _state_bytes(w, m, v), _address(hyper, ws_hyper),
+        plan.handle, r, C.addressof(g), _state_bytes(w, m, v), C.addressof(hyper),
         _OUT.pack(gathered.data_ptr(), _dtype_code(gathered.dtype)) if gathered is not None else None,
         workspace.data_ptr() if workspace is not None else None,
         workspace.numel() * workspace.element_size() if workspace is not None else 0, _stream())
@@ -629,8 +633,12 @@ class TensorTable:
 
 def ws_fused_update(plan: Plan, r: int, grads: TensorTable, w, m, v, hyper: ws_hyper, weights: TensorTable,
                     workspace: Optional[torch.Tensor] = None):
+    gc, wc = grads.c, weights.c
+    if type(hyper) is not ws_hyper or type(gc) is not ws_tensor_table or type(wc) is not ws_tensor_table:
+        for x, cls in ((gc, ws_tensor_table), (hyper, ws_hyper), (wc, ws_tensor_table)):
+            _refuse(x, cls)
     st = _step().ws_fused_update(
-        plan.handle, r, _address(grads.c, ws_tensor_table), _state_bytes(w, m, v), _address(hyper, ws_hyper), _address(weights.c, ws_tensor_table),
+        plan.handle, r, C.addressof(gc), _state_bytes(w, m, v), C.addressof(hyper), C.addressof(wc),
         workspace.data_ptr() if workspace is not None else None,
         workspace.numel() * workspace.element_size() if workspace is not None else 0, _stream())
     if st:
@@ -639,6 +647,8 @@ def ws_fused_update(plan: Plan, r: int, grads: TensorTable, w, m, v, hyper: ws_h
 
 def ws_pack_sets(plan: Plan, table: TensorTable, flats):
     """All sets of a tensor table packed in one launch (set k -> flats[k])."""
-    st = _step().ws_pack_sets(plan.handle, _address(table.c, ws_tensor_table), _ptr_array(flats), _stream())
+    if type(table.c) is not ws_tensor_table:
+        _refuse(table.c, ws_tensor_table)
+    st = _step().ws_pack_sets(plan.handle, C.addressof(table.c), _ptr_array(flats), _stream())
     if st:
         raise WsError(st, "ws_pack_sets")
