@@ -1,5 +1,5 @@
 #!/usr/bin/env python
-"""Benchmark of the sharded weight update (one JSON line on stdout).
+"""Benchmark of the sharded weight update (one JSON line on stdout; the side records as a second one on stderr).
 
 A step is one pass of the whole hot path over one model-shaped set of synthetic
 tensors: the R replicas' gradients are reduced shard by shard, the optimizer
@@ -14,10 +14,12 @@ box's host cores.
     python bench.py [--gpus N] [--steps K] [--warmup W] [--workload NAME] [--impl reference]
 
 Without --workload the line is the largest single-GPU workload (decoder_1p5b:
-1.56 G parameters, bf16 gradients, R = 4) and carries, under `configs`, one full
-record for each of the other named workloads, under `transformer_r_sweep` the
-Transformer set at R = 1 ... 1024 and alignments 8 and 32, and under
-`next_workloads` the LARS, Adafactor, concatenated-layout and partial-sharding runs.
+1.56 G parameters, bf16 gradients, R = 4).  The side records of that run go to
+stderr as one JSON line of their own, which keeps the result line short: under
+`configs` one full record for each of the other named workloads, under
+`transformer_r_sweep` the Transformer set at R = 1 ... 1024 and alignments 8 and
+32, and under `next_workloads` the LARS, Adafactor, concatenated-layout and
+partial-sharding runs.
 
 Whatever K is, the timed region lasts at least half a second: it covers
 K x `inner_repeats` back-to-back steps and `ms_per_step` is their mean.
@@ -60,8 +62,8 @@ NCU_DRAM_BYTES_PER_PARAM = {
     ("bert_large", 16, "fused"): (88.9, "profiles/lamb_one_kernel_bert_large_R16.md (six layers at full size: 88.2; the "
                                         "embeddings, a tenth of the parameters, captured by themselves: 96.0; weighted by "
                                         "parameters)"),
-    ("resnet50_lars", 8, "fused"): (56.5, "profiles/fused_lars_kernels_resnet50_R8.md (full size, no cache flush between the launches)"),
-    ("transformer_adafactor", 8, "fused"): (55.5, "profiles/fused_adafactor_kernels_transformer.md (dimensions clipped to 1024)"),
+    ("resnet50_lars", 8, "fused"): (51.2, "profiles/fused_lars_kernels_resnet50_R8.md (the one kernel, full size)"),
+    ("transformer_adafactor", 8, "fused"): (55.9, "profiles/fused_adafactor_kernels_transformer.md (the one kernel, dimensions clipped to 1024)"),
 }
 
 
@@ -101,7 +103,7 @@ def parse_args():
                          "nccl: ONE model over the ranks, NCCL reduce-scatter / all-gather around the single-shard "
                          "kernels; peer: ONE model, one kernel per rank over symmetric-memory tensors")
     ap.add_argument("--three-launch", action="store_true",
-                    help="LAMB as three launches (phase 1, combination, phase 2) instead of the one kernel")
+                    help="LAMB, LARS and Adafactor as separate launches instead of the one kernel")
     ap.add_argument("--no-e2e", action="store_true")
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--no-side-rows", action="store_true",
@@ -156,7 +158,8 @@ def bytes_per_param(wl):
     copies, the weight and the auxiliaries; write the weight and the auxiliaries): SGD-momentum
     g R + 16, Adam g R + 24 (+2 for a bf16 copy next to the fp32 master), LAMB g R + 24 (its phase 2
     re-reads are not algorithmic), LARS g R + 16, Adafactor g R + 8, with g = gradient element bytes.
-    `update` / `fused`: what the separate-kernel update and the fused-formatting update move by design.
+    `update` / `fused`: what the separate-kernel update and the fused-formatting update move by design (LAMB, LARS and
+    Adafactor: what their phases access; the one-kernel routes find a part of the second accesses in L2).
     `pack` / `unpack`: one formatting launch."""
     gb = 2 if str(wl.grad_dtype).endswith("bfloat16") else 4
     slots = {"sgdm": 1, "lars": 1, "adafactor": 0}.get(wl.opt, 2)
@@ -834,10 +837,14 @@ def measure(ctx, wl, align=32, layout="per_tensor", shards=0, tile=0, path="both
     # ---- per-kernel rates and the roofline of the dominant kernel
     peak, peak_src = measured_peak()
     bpp = bytes_per_param(wl)
-    one_kernel = wl.opt == "lamb" and plan.sched_buf is not None and 8 <= R <= 32
-    n_upd_launch = 1 if one_kernel else {"lamb": 3, "lars": 3, "adafactor": 6}.get(wl.opt, 1)
+    one_kernel = plan.one_kernel(wl.opt, R, gdt)
+    # (the one-kernel routes clear their counters with a kernel in front)
+    n_upd_launch = 2 if one_kernel else {"lamb": 3, "lars": 3, "adafactor": 6}.get(wl.opt, 1)
     chunks = -(-T // 1024)
-    upd_name = ("two_phase_kernel (phase 1 and phase 2 of every tensor as work items of one kernel)" if one_kernel else
+    upd_name = ("clear_kernel + af_kernel (sums, moments, U^2 and apply of every tensor as work items of one kernel)"
+                if one_kernel and wl.opt == "adafactor" else
+                "clear_kernel + two_phase_kernel (phase 1 and phase 2 of every tensor as work items of one kernel)"
+                if one_kernel else
                 "update_kernel" if n_upd_launch == 1 else
                 "update_kernel pass 1 + af_moments_kernel + af_factors_kernel + pass 2 + af_finalize_clip_kernel + pass 3"
                 if n_upd_launch == 6 else
@@ -872,7 +879,7 @@ def measure(ctx, wl, align=32, layout="per_tensor", shards=0, tile=0, path="both
     dom = max(kernels, key=lambda z: z["ms_per_step"])
     # the multi-launch optimizers' update is reported as one unit (its launches depend on one another)
     traffic_pp, traffic_src = NCU_DRAM_BYTES_PER_PARAM.get((wl.name, wl.R, primary), (None, None))
-    if layout != "per_tensor" or shards != R or (wl.opt == "lamb" and not one_kernel):
+    if layout != "per_tensor" or shards != R or (wl.opt in ("lamb", "lars", "adafactor") and not one_kernel):
         traffic_pp, traffic_src = None, None
     roofline = {"bound": "hbm", "kernel": dom["kernel"], "achieved": dom["achieved_gbs"], "peak": peak,
                 "peak_source": f"{peak_src} copy bandwidth", "unit": "GB/s", "frac": dom["frac"],
@@ -914,7 +921,7 @@ def measure(ctx, wl, align=32, layout="per_tensor", shards=0, tile=0, path="both
         off = plan.sync_status_offset()
         rec["config"]["one_kernel_wait_status"] = int(ws[off:off + 4].view(torch.int32).item())
         if rec["config"]["one_kernel_wait_status"] != 0:
-            raise RuntimeError("one-kernel LAMB: a bounded wait ran out (status word set); the update is incomplete")
+            raise RuntimeError("one-kernel update: a bounded wait ran out (status word set); the update is incomplete")
     if unfused_skipped:
         rec["unfused_path"] = {"skipped": unfused_skipped}
     if e2e_rec is not None:
@@ -1025,13 +1032,14 @@ def run_ours(args):
     head = measure(ctx, workload_from_args(args), align=args.align, layout=args.layout, shards=args.shards,
                    tile=args.tile, path=args.path, e2e=not args.no_e2e, cpu=not args.no_cpu_baseline, **common)
     release()
+    detail = {}
     side = (args.workload == "all" and ctx.world == 1 and not args.no_side_rows
             and not (args.R or args.opt or args.clip or args.tensors))
     if side:
         # one full record for each of the other named workloads
-        head["configs"] = []
+        detail["configs"] = []
         for name in ("tiny", "resnet50", "transformer", "bert_large"):
-            head["configs"].append(guarded(lambda: measure(
+            detail["configs"].append(guarded(lambda: measure(
                 ctx, get_workload(name), align=args.align, e2e=not args.no_e2e, cpu=not args.no_cpu_baseline,
                 cpu_seconds=4.0, **common), name))
             release()
@@ -1042,10 +1050,10 @@ def run_ours(args):
                 ctx, get_workload("transformer", R=R), align=A, path="fused", e2e=False, cpu=False, **common)),
                 f"transformer R={R} A={A}"))
             release()
-        for r_ in head["configs"]:          # the R = 8, A = 32 point is the full record above
+        for r_ in detail["configs"]:        # the R = 8, A = 32 point is the full record above
             if isinstance(r_, dict) and r_.get("config", {}).get("workload", "").startswith("transformer"):
                 sweep.insert(2, short_row(r_))
-        head["transformer_r_sweep"] = sweep
+        detail["transformer_r_sweep"] = sweep
         nxt = []
         for name, kw in (("resnet50_lars", {}), ("transformer_adafactor", {}),
                          ("bert_large", {"layout": "concat"}), ("decoder_1p5b", {"layout": "concat"}),
@@ -1057,9 +1065,11 @@ def run_ours(args):
                 ctx, get_workload(name, R=R_), align=args.align, path="fused", e2e=False, cpu=False, **kw, **common)),
                 name))
             release()
-        head["next_workloads"] = nxt
+        detail["next_workloads"] = nxt
     if ctx.rank == 0:
-        print(json.dumps(head))
+        if detail:
+            print(json.dumps(detail), file=sys.stderr, flush=True)
+        print(json.dumps(head), flush=True)
     ctx.close()
 
 
