@@ -363,10 +363,10 @@ def test_one_kernel_equals_the_stages(R, gdtype, shift, layout):
     # vectors around the 1024-element rows they are walked in, empty tensors; `shift` moves the tensors off
     # their 32-byte boundaries (16-byte aligned), where a thread's 8 columns become two quads
     shapes = [(257, 2056), (3, 2060), (129, 12), (70, 9), (513, 1), (1, 513), (0, 8), (1023,), (1024,), (4097,), (2, 3, 4, 8),
-              (), (1100, 8), (40, 2049), (0,)]
+              (), (1100, 8), (40, 2049), (0,), (60, 2000)]
     numels = [int(torch.Size(s).numel()) for s in shapes]
     gen = torch.Generator(device=DEV).manual_seed(R)
-    hy = B.make_hyper("adafactor", _hyper(grad_scale=1.0 / R))
+    steps = [B.make_hyper("adafactor", _hyper(grad_scale=1.0 / R, step=t)) for t in (10, 11)]
 
     def draw(std, dtype):
         out = []
@@ -379,35 +379,44 @@ def test_one_kernel_equals_the_stages(R, gdtype, shift, layout):
     got = []
     for one in (True, False):
         plan = B.Plan(shapes, 3, 8, layout=layout, one_launch=one)
+        assert plan.one_kernel("adafactor", R, gdtype) == one
+        off = plan.sync_status_offset()
         f = torch.rand(plan.factored_elems, generator=torch.Generator(device=DEV).manual_seed(9), device=DEV) * 1e-3 + 1e-6
         ws = torch.full((plan.workspace_bytes("adafactor"),), 0xFF, dtype=torch.uint8, device=DEV)
         table = B.TensorTable(plan, g)
-        for form in ("master", "state", "packed"):
+        for form in ("master", "state", "bf16", "packed"):
             fs = f.clone()
-            wt = [torch.empty(n + 64, device=DEV)[shift:shift + n].copy_(x) for n, x in zip(numels, w)]
+            odt = torch.bfloat16 if form == "bf16" else torch.float32
+            at = 8 if shift and form == "bf16" else shift          # (tensors start on 16 bytes)
+            wt = [torch.empty(n + 64, dtype=odt, device=DEV)[at:at + n].copy_(x) for n, x in zip(numels, w)]
             pw = torch.full((plan.G,), 7.0, device=DEV)
             B.ws_pack(plan, w, pw)
             if form == "packed":
                 flats = [torch.full((plan.G,), float("nan"), dtype=gdtype, device=DEV) for _ in range(R)]
                 B.ws_pack_sets(plan, table, flats)
                 gathered = torch.full((plan.G,), 7.0, dtype=torch.bfloat16, device=DEV)
-                B.ws_shard_update(plan, -1, flats, pw, None, fs, hy, gathered, ws)
+                for hy in steps:
+                    B.ws_shard_update(plan, -1, flats, pw, None, fs, hy, gathered, ws)
                 assert torch.equal(gathered, pw.to(torch.bfloat16))
                 B.ws_unpack(plan, pw, wt)
             else:
-                B.ws_fused_update(plan, -1, table, pw if form == "state" else None, None, fs, hy, B.TensorTable(plan, [wt]), ws)
+                out = B.TensorTable(plan, [wt])
+                for hy in steps:               # (the second step finds the first one's counters and words)
+                    B.ws_fused_update(plan, -1, table, None if form == "master" else pw, None, fs, hy, out, ws)
+            assert int(ws[off:off + 4].view(torch.int32).item()) == 0
             back = [torch.empty(n, device=DEV) for n in numels]
             if form != "master":
                 B.ws_unpack(plan, pw, back)
-                assert all(torch.equal(a, b) for a, b in zip(back, wt))
+                assert all(torch.equal(a.to(odt), b) for a, b in zip(back, wt))
                 pads = pw.clone()
-                B.ws_pack(plan, wt, pads)
+                B.ws_pack(plan, back, pads)
                 assert torch.equal(pads, pw)                        # (ws_pack writes +0 pads)
+                wt = back
             rho = ws[:4 * plan.T].view(torch.float32).clone()
             got.append(([to_np(x) for x in wt], to_np(fs), to_np(rho)))
     # the same sums in another order: a few fp32 roundings of sums of squares, far inside the bar that either
     # form is held to against the oracle
-    for a, b in zip(got[:3], got[3:]):
+    for a, b in zip(got[:4], got[4:]):
         for x, y in zip(a[0], b[0]):
             assert err(x, y) <= TOL_LAMB
         np.testing.assert_allclose(a[1], b[1], rtol=TOL_LAMB)

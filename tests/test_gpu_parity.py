@@ -628,13 +628,16 @@ def test_step_can_be_captured_in_a_cuda_graph():
         assert torch.equal(a, b)
 
 
-@pytest.mark.parametrize("opt,R", [("lamb", 3), ("lamb", 8), ("lars", 3)])
-def test_multi_launch_steps_can_be_captured_in_a_cuda_graph(opt, R):
-    # the norm-based optimizers are three launches joined by programmatic dependent launch - or, for LAMB
-    # with 8 copies, a clear of the counters and the one kernel: the captured graph replays to the same
-    # bits as the eager calls (fixed-order sums)
-    wl, w, m, v, g = _model(SHAPES, R, seed=14, gstd=1e-3)
-    plan = B.Plan(SHAPES, R, 32)
+@pytest.mark.parametrize("opt,R,gdtype", [("lamb", 3, torch.float32), ("lamb", 8, torch.float32), ("lars", 3, torch.float32),
+                                          ("lamb", 8, torch.bfloat16), ("lars", 8, torch.bfloat16)])
+def test_multi_launch_steps_can_be_captured_in_a_cuda_graph(opt, R, gdtype):
+    # the norm-based optimizers are three launches joined by programmatic dependent launch - or, on a model of
+    # 3.4 M parameters with 8 bf16 copies, a clear of the counters and the one kernel: the captured graph replays
+    # to the same bits as the eager calls (fixed-order sums)
+    shapes = SHAPES if gdtype == torch.float32 else SHAPES + [(1500, 2200)]
+    wl, w, m, v, g = _model(shapes, R, gdtype, seed=14, gstd=1e-3)
+    plan = B.Plan(shapes, R, 32)
+    assert plan.one_kernel(opt, R, gdtype) == (gdtype == torch.bfloat16)
     h = _lars_hyper() if opt == "lars" else _hyper(opt)
     hy = B.make_hyper(opt, h)
     pw, pm, pv, pg = _pack_all(plan, w, m, v, g)
@@ -655,9 +658,8 @@ def test_multi_launch_steps_can_be_captured_in_a_cuda_graph(opt, R):
     graph.replay()
     torch.cuda.synchronize()
     assert torch.equal(pw, ew) and torch.equal(pm, em)
-    if opt == "lamb" and R == 8:
-        off = plan.sync_status_offset()
-        assert int(ws[off:off + 4].view(torch.int32).item()) == 0
+    off = plan.sync_status_offset()
+    assert int(ws[off:off + 4].view(torch.int32).item()) == 0
 
 
 @pytest.mark.parametrize("opt", ["sgdm", "adam", "lamb"])
@@ -724,11 +726,10 @@ def test_lars_matches_oracle_and_fused_equals_unfused(R, gdtype):
 @pytest.mark.parametrize("gdtype,layout,fused", [(torch.float32, "per_tensor", False), (torch.bfloat16, "per_tensor", True),
                                                  (torch.float32, "concat", True), (torch.bfloat16, "concat", False)])
 def test_one_launch_update_equals_three_launches(opt, R, gdtype, layout, fused):
-    # The all-shard LAMB / LARS update as ONE kernel (plan with its one-launch schedule) against
-    # the three launches (phase 1, combination, phase 2): same elementwise arithmetic, the norm sums grouped
-    # by work item instead of by tile, so ratios agree to rounding; the status word stays 0; two steps in
-    # a row (the second finds the first's counters and flags in the workspace).  The one-kernel route is
-    # taken for LAMB with 8 to 32 gradient copies; every other case runs the three launches on both plans.
+    # A plan with its one-launch schedule against one without, on a model of 0.6 M parameters: the status word
+    # is 0; two steps in a row (the second finds the first's counters and flags in the workspace).  At this size
+    # both plans run the three launches (phase 1, combination, phase 2); the one kernel, which the larger models of
+    # test_one_kernel_has_the_bits_of_the_shard_by_shard_calls take, has the same bits.
     shapes = SHAPES + [(1024, 512), (0,), (70001,)]
     wl, w, m, v, g = _model(shapes, R, gdtype, seed=R + 31, gstd=1e-3 if opt == "lars" else 1e-2)
     p1 = B.Plan(shapes, R, 32, layout=layout)
@@ -754,9 +755,8 @@ def test_one_launch_update_equals_three_launches(opt, R, gdtype, layout, fused):
         if not fused:
             B.ws_unpack(plan, gathered, outs)
         bufs[name] = (pw, pm, pv, outs, B.lamb_ratios(plan, ws).clone(), ws)
-    if opt == "lamb" and 8 <= R <= 32:         # (otherwise both plans run the three launches)
-        off = p1.sync_status_offset()
-        assert int(bufs["one"][5][off:off + 4].view(torch.int32).item()) == 0
+    off = p1.sync_status_offset()
+    assert all(int(b[5][off:off + 4].view(torch.int32).item()) == 0 for b in bufs.values())
     a, b = bufs["one"], bufs["three"]
     tol = 3e-7
     assert err(to_np(a[0]), to_np(b[0])) <= tol and err(to_np(a[1]), to_np(b[1])) <= tol
@@ -797,7 +797,7 @@ def test_lars_shard_by_shard_phases(R):
     assert e.value.status == 1
 
 
-@pytest.mark.parametrize("opt,R", [("lamb", 8), ("lamb", 16), ("lars", 5), ("lars", 8), ("lars", 32)])
+@pytest.mark.parametrize("opt,R", [("lamb", 8), ("lamb", 16), ("lars", 4), ("lars", 5), ("lars", 7), ("lars", 8), ("lars", 32)])
 @pytest.mark.parametrize("gdtype,layout,tile", [(torch.float32, "per_tensor", 0), (torch.bfloat16, "per_tensor", 1024),
                                                 (torch.bfloat16, "concat", 2048), (torch.float32, "concat", 3072),
                                                 (torch.bfloat16, "per_tensor", 3072), (torch.float32, "per_tensor", 16384)])
@@ -808,7 +808,8 @@ def test_one_kernel_has_the_bits_of_the_shard_by_shard_calls(opt, R, gdtype, lay
     shapes = SHAPES + [(2000, 4099), (0,), (1500, 307)]
     wl, w, m, v, g = _model(shapes, R, gdtype, seed=R, gstd=1e-3)
     plan = B.Plan(shapes, 8, 32, tile, layout=layout)
-    assert plan.one_kernel(opt, R, gdtype) or (opt, R, gdtype) == ("lars", 32, torch.float32)    # (that needs 32 M parameters)
+    # (LARS with 32 fp32 copies takes the one kernel from 32 M parameters on, with 4 bf16 copies never)
+    assert plan.one_kernel(opt, R, gdtype) == ((opt, R, gdtype) not in (("lars", 32, torch.float32), ("lars", 4, torch.bfloat16)))
     h = B.make_hyper(opt, _lars_hyper() if opt == "lars" else _hyper("lamb"))
     pw, pm, pv, pg = _pack_all(plan, w, m, v, g)
     state = lambda x: [x[0].clone(), x[1].clone(), x[2].clone() if opt == "lamb" else None]  # noqa: E731
