@@ -151,8 +151,9 @@ ws_status ws_plan_upload(ws_plan* plan, void* dev_buf, size_t bytes, void* strea
  * phase 1, a combination step, phase 2.  As three launches, phase 2 reads the weight and the new
  * moments from DRAM again.  A plan whose schedule has been uploaded runs WS_LAMB's all-shard update
  * as ONE kernel instead: the two phases of every tensor are work items (one or several whole work
- * tiles, several up to 8192 shard positions) ordered so that a tensor's phase 2 follows its phase 1 at a short distance, while other
- * tensors' phase 1 streams from DRAM, and phase 2 finds part of its operands in L2 (toward the
+ * tiles, several up to 8192 shard positions) ordered so that a tensor's phase 2 follows its phase 1 at a
+ * short distance, while other tensors' phase 1 streams from DRAM, and phase 2 finds part of its operands
+ * in L2 (toward the
  * update of Section 2.2, where every operand crosses HBM once).  Results: bit for bit those of the
  * three-launch form (the partial norms are the tiles' and are summed in the same order).
  *   ws_plan_schedule_bytes   device bytes of the schedule (0: this plan has none - more than
@@ -344,10 +345,11 @@ ws_status ws_workspace_partials(const ws_plan* plan, size_t* offset_bytes, size_
  * once, writes w/m/v (and the gathered slot) once (Section 2.2: the update is
  * memory bound - read gradient, weight, auxiliaries; write weight,
  * auxiliaries).  With opt == WS_LAMB or WS_LARS only r == -1 is accepted here
- * (phase 1 over all shards, finalize, phase 2 over all shards): the per-tensor
+ * (phase 1 over all shards, finalize, phase 2 over all shards, as three
+ * launches or one kernel with the same bits): the per-tensor
  * ratio needs every shard's partial norms before any shard can apply
  * (Section 4.1).
- * WS_ADAFACTOR (r == -1 only) runs three passes: (1) reduce the gradients, keep
+ * WS_ADAFACTOR (r == -1 only) runs three passes, as one kernel or as stages: (1) reduce the gradients, keep
  * the sum, and add every tile's partial row sums and column sums of g^2 + eps
  * (pads masked by location) into acc - the sharding cuts rows and columns, so
  * this stands where the paper combines the shards' partial reduce results with
@@ -402,7 +404,8 @@ ws_status ws_lars_apply(const ws_plan* plan, int32_t r, const ws_state* state,
                         size_t workspace_bytes, void* stream);
 
 /* Adafactor stage by stage, for one shard r >= 0 or all shards (r == -1): what
- * ws_shard_update(WS_ADAFACTOR) runs in this order.  On real replicas each
+ * ws_shard_update(WS_ADAFACTOR) runs in this order where it does not run as one
+ * kernel (which has the same sums in another order).  On real replicas each
  * runs the per-shard stages for its own shard and exchanges the reduce results
  * between them - the case of Section 4.1 where "sharding affects the collapsed
  * dimensions": every replica reduces what its shard holds, then the replicas

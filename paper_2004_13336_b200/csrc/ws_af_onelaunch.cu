@@ -2,10 +2,9 @@
 //
 // Adafactor needs every row and column sum of g^2 before any element's update direction exists, and the
 // direction's norm before any element can take its step (paper Section 4.1, reduces over sharded dimensions):
-// three passes over a tensor.  As separate launches over the whole model each pass goes to DRAM (4R + 24 bytes
-// per parameter) and six launches drain the GPU in turn.  Here the passes of every tensor are entries of one
-// schedule, ordered so that a tensor's later passes run while its summed gradients (and, in the last pass, its
-// weights) are still in L2 and other tensors' first passes stream from DRAM.
+// three passes over a tensor.  As separate launches six kernels drain the GPU in turn.  Here the passes of every
+// tensor are entries of one schedule, ordered so that a tensor's later passes run behind its first one while other
+// tensors' first passes stream from DRAM.
 //
 //   P1  sum the R gradient copies of a block, keep the sum, add g^2 + eps to the row and column sums
 //   M   the moving averages Rv', Cv' of a chunk of the factored state, 1/sqrt factors, sum of Rv'
@@ -13,19 +12,22 @@
 //   P3  w' = w - step size * U
 //
 // A block is a piece of the tensor's rows x cols matrix and not a run of its elements: a thread owns 8 columns
-// and walks down the rows, the block's rows in parallel are summed in shared memory, and a column's sum takes one add
-// to memory per block whatever the row length.  (One add per thread put all adds of a tall narrow matrix on a few
-// addresses, where they follow one another: an encoder-decoder of 2.4 M parameters, 128 wide, took 118 us with one
-// copy where the stages take 47, now 41; 0.86 M, 64 wide: 105, 56, 25 us.)  A row's
-// sum needs one warp-wide reduction and one add per 256 columns.  Row lengths that 8 does not divide have 4
-// columns per thread, and those that 4 does not divide 4 scalar accesses in place of a vector one.
+// and walks down the rows, the block's rows in parallel are summed in shared memory, and a column's sum takes one
+// add to memory per block whatever the row length.  (One add per thread put all adds of a tall narrow matrix on a
+// few addresses, where they follow one another: an encoder-decoder of 2.4 M parameters, 128 wide, took 118 us with
+// one copy where the stages take 47, now 41; 0.86 M, 64 wide: 105, 56, 25 us.)  A row's sum needs one warp-wide
+// reduction and one add per 256 columns.  Row lengths that 8 does not divide have 4 columns per thread, and those
+// that 4 does not divide 4 scalar accesses in place of a vector one.
 //
-// What bounds it: the latency of an entry (ticket -> record -> tables and ready word -> data, then the arrival),
-// not bytes - leaving the kept sums in L2 more firmly (evict-last hints, discarding them after P3) changed
-// nothing, while blocks of 65536 elements instead of 8192 and one record per entry instead of two hops did.
-// Measured against the six launches it replaces: Transformer set (211 M), R = 4 fp32 1405 -> 1245 us, R = 1
-// 1174 -> 886, R = 8 1888 -> 1765; 22.7 M parameters in ragged tensors, R = 2: 837 -> 173 us (there a
-// scalar reduction per element went to memory); 45 792 parameters 26 -> 19 us.
+// What bounds it: on large models the bytes of three passes through DRAM, 4R + 24 per parameter, at the copy
+// bandwidth (102 M parameters: 27.8, 39.7 and 55.9 bytes at R = 1, 4, 8, L2 hit rate 5 to 9 %).  The kept sums of
+// the blocks in flight, 256 KB each on 444 resident CTAs, and the weights that P2 reads take the whole L2 before a
+// later pass comes back to them, so that leaving them in L2 more firmly (evict-last hints, discarding them after
+// P3) changed nothing.  On small models an entry's chain of dependent reads (ticket -> record -> tables and ready
+// word -> data, then the arrival): hence large blocks and one record per entry.
+// Measured against the six launches it replaces (us): Transformer set (211 M), fp32, R = 1 1148 -> 877, R = 4 1376 ->
+// 1245, R = 8 1862 -> 1760; ResNet-50 set (25.6 M), R = 4 269 -> 164; 22.7 M parameters in ragged tensors, R = 2:
+// 749 -> 172 (there a scalar reduction per element went to memory); 45 792 parameters, called from the host, 27 -> 17.
 //
 // Tickets, waits and their progress argument are those of ws_onelaunch.cu: an entry waits only for entries with
 // smaller tickets, which belong to CTAs that are running or have finished; every wait has an iteration limit.

@@ -294,16 +294,7 @@ __global__ void __launch_bounds__(kBlock, kAf2Ctas) af_sumsq_kernel(const UpdPar
 // -------------------------------------------------------------- dispatch ---
 void launch_lamb_finalize(int T, cudaStream_t st, const WsSegTiles* segtiles, const float2* partials, long long ntiles,
                           int R, float* rho, double* norms, int lars, double eta, double beta, int* status) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)T);
-    cfg.blockDim = dim3(kBlock);
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, lamb_finalize_kernel, segtiles, partials, ntiles, R, rho, norms, lars, eta, beta, status);
+    launch_pdl(lamb_finalize_kernel, T, st, segtiles, partials, ntiles, R, rho, norms, lars, eta, beta, status);
 }
 
 template <int OPT, bool GBF, int OUT, int VEC, int U, int RB, int NP, bool FUSED>
@@ -313,18 +304,8 @@ ws_status launch(const UpdParams& P, const void* const* gptrs, cudaStream_t st) 
     long long grid = P.nitems;
     if (grid < 1) return WS_OK;
     if (grid > 0x7fffffffLL) grid = 0x7fffffffLL;
-    // programmatic dependent launch: the kernel may start while the previous kernel of the stream drains
-    // (it reads only the plan and pointer tables before it waits for that kernel)
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3(kBlock);
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, update_kernel<OPT, GBF, OUT, VEC, U, RB, NP, FUSED>, P, gp);
+    // (the kernel reads only the plan and pointer tables before it waits for the kernel in front)
+    launch_pdl(update_kernel<OPT, GBF, OUT, VEC, U, RB, NP, FUSED>, grid, st, P, gp);
     return ws_check_launch(FUSED ? "ws_fused_update" : "ws_shard_update");
 }
 
@@ -438,10 +419,10 @@ ws_status prepare(const ws_plan* p, int32_t r, const ws_grads* g, const ws_state
     P.gtab = nullptr;
     P.wtab = nullptr;
     P.nw = 1;
-    // Norm pairs on all shards of a model small enough that a good part of what phase 2 reads again fits
-    // the L2: phase 1 leaves those lines in L2 (its gradient loads are evict-first) and phase 2 walks the
-    // items back to front, starting where phase 1 ended.  ResNet-50 set under LARS, 8 copies: 0.249 ms ->
-    // 0.241 ms; on models many times the L2 it costs 1 - 2 %, hence the limit.
+    // Norm pairs as three launches on all shards of a model small enough that a good part of what phase 2
+    // reads again fits the L2: phase 1 leaves those lines in L2 (its gradient loads are evict-first) and phase 2
+    // walks the items back to front, starting where phase 1 ended.  ResNet-50 set under LARS, 8 copies, as three
+    // launches: 0.249 ms -> 0.241 ms; on models many times the L2 it costs 1 - 2 %, hence the limit.
     {
         const bool pair = phase == K_LAMB1 || phase == K_LAMB2 || phase == K_LARS1 || phase == K_LARS2;
         const long long again = (phase == K_LAMB1 || phase == K_LAMB2) ? 12 : 8;     // bytes per parameter read twice
