@@ -153,11 +153,10 @@ ws_status ws_plan_upload(ws_plan* plan, void* dev_buf, size_t bytes, void* strea
  * as ONE kernel instead: the two phases of every tensor are work items (one or several whole work
  * tiles, several up to 8192 shard positions) ordered so that a tensor's phase 2 follows its phase 1 at a
  * short distance, while other tensors' phase 1 streams from DRAM, and phase 2 finds part of its operands
- * in L2 (toward the
- * update of Section 2.2, where every operand crosses HBM once).  Results: bit for bit those of the
- * three-launch form (the partial norms are the tiles' and are summed in the same order).
+ * in L2 (toward the update of Section 2.2, where every operand crosses HBM once).  Results: bit for bit
+ * those of the three-launch form (the partial norms are the tiles' and are summed in the same order).
  *   ws_plan_schedule_bytes   device bytes of the schedule (0: this plan has none - more than
- *                            65535 shards or 2^30 work items)
+ *                            65535 shards, 2^30 work items or 2^47 elements in a shard)
  *   ws_plan_upload_schedule  builds the schedule on first use and copies it into the caller's
  *                            buffer (16-byte aligned, alive while the plan is in use) with
  *                            cudaMemcpyAsync on `stream`; call once, before the plan is shared
@@ -171,7 +170,8 @@ ws_status ws_plan_upload(ws_plan* plan, void* dev_buf, size_t bytes, void* strea
  * the workspace (ws_workspace_sync_status gives its byte offset; 0 = completed, also after the
  * separate launches) - a caller that wants to detect this reads the word after synchronising the stream.
  *   ws_plan_one_kernel       1 where the all-shard update of `opt` from `copies` gradient copies of
- *                            `grad_dtype` runs as one kernel once the schedule is uploaded, else 0 (host only)
+ *                            `grad_dtype` runs as one kernel once the schedule is uploaded, else 0 (host only;
+ *                            LAMB and LARS with bf16 gradients also want fp32 outputs on 32-byte boundaries)
  * ws_plan_schedule_view / ws_plan_schedule_item expose the order for inspection (host only):
  * entry i of `order` is item index * 2 + phase (0: phase 1, 1: phase 2). */
 size_t ws_plan_schedule_bytes(const ws_plan* plan);

@@ -675,7 +675,9 @@ ws_status try_one_launch(const ws_plan* plan, int pair, const ws_grads* grads, c
     if (pair == 0 && (!state->v || !ws_aligned16(state->v))) return state->v ? WS_ERR_ALIGNMENT : WS_ERR_INVALID_ARG;
     if ((s = check_ws(plan, workspace, workspace_bytes, pair == 0 ? WS_LAMB : WS_LARS)) != WS_OK) return s;
     const WsLambWs L = ws_lamb_layout(plan, workspace);
-    bool wide = aligned32(P.w) && aligned32(P.m) && aligned32(P.v) && aligned32(P.gathered);
+    // wide1, wide: what the separate launches' phase 1 and phase 2 look at
+    bool wide1 = aligned32(P.w) && aligned32(P.m) && aligned32(P.v);
+    bool wide = wide1 && aligned32(P.gathered);
     std::vector<const void*> gp;
     if (fused) {
         const bool master = state->w == nullptr;
@@ -687,15 +689,21 @@ ws_status try_one_launch(const ws_plan* plan, int pair, const ws_grads* grads, c
         P.wtab = (void* const*)wtab->dev;
         P.nw = 1;
         out_kind = master ? O_F32M : (wtab->dtype == WS_F32 ? O_F32 : O_BF16);
-        wide = wide && (gbf || gtab->min_align >= 32) && (wtab->dtype == WS_BF16 || wtab->min_align >= 32);
+        wide1 = wide1 && (gbf || gtab->min_align >= 32) && (!master || wtab->min_align >= 32);
+        wide = wide && wide1 && (wtab->dtype == WS_BF16 || wtab->min_align >= 32);
     } else {
         offset_grad_ptrs(plan, -1, grads, gp);
-        for (int k = 0; k < grads->R && wide; ++k) wide = aligned32(gp[k]);
+        for (int k = 0; k < grads->R && wide1; ++k) wide1 = aligned32(gp[k]);
+        wide = wide && wide1;
     }
     if (pair == 1) {
         P.ghat = L.ghat;
-        wide = wide && aligned32(P.ghat);
+        wide1 = wide1 && aligned32(P.ghat);
+        wide = wide && wide1;
     }
+    // with bf16 gradients the width of phase 1 orders the norm sums: an output that is only 16-byte aligned would
+    // narrow it here and not there
+    if (gbf && wide1 && !wide) return WS_OK;
     OneLaunch Q;
     Q.sched = plan->d_sched;
     Q.nsched = (unsigned)(2 * plan->n_items);

@@ -868,6 +868,31 @@ def test_status_word_is_valid_after_every_all_shard_update(opt, slots, R):
         assert int(ws[off:off + 4].view(torch.int32).item()) == 0
 
 
+@pytest.mark.parametrize("opt", ["lamb", "lars"])
+@pytest.mark.parametrize("fused", [False, True])
+def test_outputs_on_16_byte_boundaries_keep_the_bits(opt, fused):
+    # bf16 gradients: the width of phase 1 orders the norm sums, and the alignment of what phase 2 writes must not
+    # narrow it on one route only
+    R, shapes = 8, [(1500, 2200), (7,), (300, 301)]
+    wl, w, m, v, g = _model(shapes, R, torch.bfloat16, seed=6, gstd=1e-3)
+    h = B.make_hyper(opt, _lars_hyper() if opt == "lars" else _hyper("lamb"))
+    got = []
+    for one_launch in (True, False):
+        plan = B.Plan(shapes, R, 32, one_launch=one_launch)
+        pw, pm, pv, pg = _pack_all(plan, w, m, v, g)
+        if opt == "lars":
+            pv = None
+        ws = torch.zeros(plan.workspace_bytes(opt), dtype=torch.uint8, device=DEV)
+        if fused:
+            outs = [torch.zeros(n + 4, device=DEV)[4:] for n in wl.numels]
+            B.ws_fused_update(plan, -1, B.TensorTable(plan, g), pw, pm, pv, h, B.TensorTable(plan, [outs]), ws)
+        else:
+            outs = [torch.zeros(plan.G + 4, device=DEV)[4:]]
+            B.ws_shard_update(plan, -1, pg, pw, pm, pv, h, outs[0], ws)
+        got.append([pw, pm] + outs + [ws[:16 + 16 * plan.T]])        # (with the ratios and squared norms)
+    assert all(torch.equal(a, b) for a, b in zip(*got))
+
+
 def test_lars_poisoned_pads_and_error_codes():
     import ctypes as C
     R = 5
