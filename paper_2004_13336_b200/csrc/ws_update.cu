@@ -516,6 +516,7 @@ int finalize_reps(const ws_plan* p) { return p->layout == WS_LAYOUT_CONCAT ? 1 :
 // spills in both forms - but not with 4 copies, where the separate kernel has a variant of its own.  Device time one
 // kernel / three launches, state and gradients not in L2 (encoder-decoder and image sets of M parameters, us):
 //   LAMB fp32   8 copies   1.7 M 30.2/28.2   2.4 M 40.1/36.3   4.6 M 62.4/63.1   7.6 M 81.8/93.7     26 M 257/279
+//              12 copies   2.4 M 56.2/49.1   4.6 M 77.9/79.5   6.9 M 117/115     7.6 M 116/123  26 M 345/362
 //              16 copies   4.6 M 86.0/83.1   7.6 M 130/128     26 M 389/411      32 copies 7.6 M 227/204  26 M 644/686
 //        bf16   8 copies  0.37 M 16.2/14.0   1.7 M 42.4/48.9   7.6 M 120/181     32 copies 1.7 M 78.9/85.7
 //   LARS fp32   4 copies   4.6 M 44.1/45.8   6.9 M 58.9/53.3   26 M 178/190      8 copies 2.4 M 37.4/31.9  4.6 M 55.4/53.5
@@ -526,7 +527,7 @@ long long pair_min_params(bool lars, bool gbf, int copies) {
     constexpr long long M = 1 << 20;
     if (copies < (lars ? 4 : 8) || copies > 32) return -1;
     if (lars) return gbf ? (copies == 4 ? -1 : 3 * M) : (copies == 4 ? 8 * M : copies <= 8 ? 4 * M : 32 * M);
-    return gbf ? M : (copies <= 8 ? 4 * M : copies <= 16 ? 8 * M : 16 * M);
+    return gbf ? M : (copies <= 12 ? 4 * M : copies <= 16 ? 8 * M : 16 * M);
 }
 
 // Whether an all-shard update of `opt` runs as one kernel where the plan's schedule is on the device.

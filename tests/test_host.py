@@ -315,7 +315,7 @@ def test_adafactor_short_tensors_are_one_block(shape, blocks, chunks):
 
 
 @pytest.mark.parametrize("opt,gdtype,copies,least", [
-    ("lamb", torch.float32, 8, 4 << 20), ("lamb", torch.float32, 9, 8 << 20), ("lamb", torch.float32, 32, 16 << 20),
+    ("lamb", torch.float32, 8, 4 << 20), ("lamb", torch.float32, 12, 4 << 20), ("lamb", torch.float32, 13, 8 << 20), ("lamb", torch.float32, 32, 16 << 20),
     ("lamb", torch.bfloat16, 8, 1 << 20), ("lamb", torch.bfloat16, 7, None), ("lamb", torch.float32, 33, None),
     ("lars", torch.float32, 4, 8 << 20), ("lars", torch.float32, 5, 4 << 20), ("lars", torch.float32, 9, 32 << 20),
     ("lars", torch.bfloat16, 5, 3 << 20), ("lars", torch.bfloat16, 4, None), ("lars", torch.float32, 3, None),
