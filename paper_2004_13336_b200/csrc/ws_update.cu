@@ -514,7 +514,8 @@ int finalize_reps(const ws_plan* p) { return p->layout == WS_LAYOUT_CONCAT ? 1 :
 // two or three of them; what it saves, phase 2's second read, grows with the model.  More copies shorten that saving's
 // share, and fp32 gradients leave the three launches closer to the copy bandwidth than bf16 ones, whose wide phase 1
 // spills in both forms - but not with 4 copies, where the separate kernel has a variant of its own.  Device time one
-// kernel / three launches, state and gradients not in L2 (encoder-decoder and image sets of M parameters, us):
+// kernel / three launches, formatting fused in, state and gradients not in L2 (encoder-decoder and image sets of M
+// parameters, us):
 //   LAMB fp32   8 copies   1.7 M 30.2/28.2   2.4 M 40.1/36.3   4.6 M 62.4/63.1   7.6 M 81.8/93.7     26 M 257/279
 //              12 copies   2.4 M 56.2/49.1   4.6 M 77.9/79.5   6.9 M 117/115     7.6 M 116/123  26 M 345/362
 //              16 copies   4.6 M 86.0/83.1   7.6 M 130/128     26 M 389/411      32 copies 7.6 M 227/204  26 M 644/686
