@@ -12,8 +12,7 @@ namespace wsk {
 
 constexpr int kBlock = 256;
 // Resident CTAs per SM the compiler must allow for (register budget): 3 measured best (4 forces
-// spills, 2 leaves bandwidth unused); the bf16-gradient wide kernel on packed buffers and the
-// many-replica kernel are faster with the registers of 2.
+// spills, 2 leaves bandwidth unused); the many-replica kernel is faster with the registers of 2.
 constexpr int kMinBlocks = 3;
 constexpr int kMinBlocksWide = 2;
 constexpr int kTreeBlockLarge = 16;   // gradients per tree block when R > 32
@@ -218,6 +217,40 @@ __device__ __forceinline__ void store_bf16(unsigned short* p, const Fv<VEC>& x) 
     }
     if constexpr (VEC == 4) __stcs(reinterpret_cast<uint2*>(p), make_uint2(pk[0], pk[1]));
     else __stcs(reinterpret_cast<uint4*>(p), make_uint4(pk[0], pk[1], pk[2], pk[3]));
+}
+
+// Element i of a vector of gradients as fp32.
+template <bool GBF, int VEC>
+__device__ __forceinline__ float raw_elem(const GradRaw<GBF, VEC>& g, int i) {
+    if constexpr (GBF) {
+        unsigned w;
+        if constexpr (VEC == 8) w = i < 2 ? g.u.x : i < 4 ? g.u.y : i < 6 ? g.u.z : g.u.w;
+        else w = i < 2 ? g.u.x : g.u.y;
+        return __uint_as_float(i & 1 ? w & 0xffff0000u : w << 16);
+    } else {
+        return g.f[i];
+    }
+}
+// The sum of RB copies as a tree, one element after the other.  Widened all at once, 8 bf16 copies of 8 elements
+// are 64 registers: the kernels of 5 and more bf16 copies then spilled up to 500 bytes a thread, and local memory
+// shares the L1 with the stream.  25.6 M parameters, formatting fused in, us, before / now: SGD-M 8 copies 211 / 126,
+// 6 copies 204 / 113, 1 copy 90 / 79; Adam 8 copies 287 / 160; LAMB 8 copies 340 / 210; LARS 8 copies 245 / 173; on
+// packed buffers, where 128 registers had kept most of it out of memory, Adam with 8 copies and its formatting 378 / 314.
+template <bool GBF, int VEC, int RB>
+__device__ __forceinline__ Fv<VEC> tree_sum(const GradRaw<GBF, VEC> (&raw)[RB]) {
+    Fv<VEC> o;
+#pragma unroll
+    for (int i = 0; i < VEC; ++i) {
+        float t[RB];
+#pragma unroll
+        for (int j = 0; j < RB; ++j) t[j] = raw_elem<GBF, VEC>(raw[j], i);
+#pragma unroll
+        for (int s = 1; s < RB; s <<= 1)
+#pragma unroll
+            for (int j = 0; j + s < RB; j += 2 * s) t[j] += t[j + s];
+        o.f[i] = t[0];
+    }
+    return o;
 }
 
 // Kahan step: (sum, comp) += x
@@ -567,13 +600,14 @@ __device__ __forceinline__ void process_item(const UpdParams& P, const GradPtrs<
         if (READS_G) {
             for (int k0 = 0; k0 < (LOOPK ? P.R : 1); k0 += RB) {
                 GradRaw<GBF, VEC> raw[U][RB];
-                bool have[RB];
 #pragma unroll
                 for (int j = 0; j < RB; ++j) {
-                    have[j] = (RB == 1) || (k0 + j < P.R);
+#pragma unroll
+                    for (int u = 0; u < U; ++u) raw[u][j] = {};          // (an absent copy adds +0)
+                    if (RB > 1 && k0 + j >= P.R) continue;
 #pragma unroll
                     for (int u = 0; u < U; ++u)
-                        if (have[j] && nv[u] > 0) {
+                        if (nv[u] > 0) {
                             if constexpr (FUSED) {
                                 const void* gk = sgp[k0 + j];
                                 if (nv[u] == VEC) raw[u][j] = load_grad<GBF, VEC>(gk, toff + e0[u]);
@@ -591,27 +625,12 @@ __device__ __forceinline__ void process_item(const UpdParams& P, const GradPtrs<
                 }
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
-                    Fv<VEC> gb[RB];
-#pragma unroll
-                    for (int j = 0; j < RB; ++j) {
-                        if (have[j] && nv[u] > 0) {
-                            gb[j] = widen<GBF, VEC>(raw[u][j]);
-                        } else {
-#pragma unroll
-                            for (int i = 0; i < VEC; ++i) gb[j].f[i] = 0.f;
-                        }
-                    }
-#pragma unroll
-                    for (int s = 1; s < RB; s <<= 1)
-#pragma unroll
-                        for (int j = 0; j + s < RB; j += 2 * s)
-#pragma unroll
-                            for (int i = 0; i < VEC; ++i) gb[j].f[i] += gb[j + s].f[i];
+                    const Fv<VEC> gb = tree_sum<GBF, VEC, RB>(raw[u]);
                     if (!LOOPK || k0 == 0) {
-                        gv[u] = gb[0];
+                        gv[u] = gb;
                     } else {
 #pragma unroll
-                        for (int i = 0; i < VEC; ++i) kahan1(gv[u].f[i], gc[u].f[i], gb[0].f[i]);
+                        for (int i = 0; i < VEC; ++i) kahan1(gv[u].f[i], gc[u].f[i], gb.f[i]);
                     }
                 }
             }

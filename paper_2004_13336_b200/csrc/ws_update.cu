@@ -34,7 +34,7 @@ using namespace wsk;
 // One CTA handles one (shard, tile) work item; the grid is the item count, so the
 // hardware CTA scheduler walks the buffers front to back.
 template <int OPT, bool GBF, int OUT, int VEC, int U, int RB, int NP, bool FUSED>
-__global__ void __launch_bounds__(kBlock, ((VEC == 8 && GBF && !FUSED) || RB > 8) ? kMinBlocksWide : kMinBlocks) update_kernel(const UpdParams P, const __grid_constant__ GradPtrs<NP> gp) {
+__global__ void __launch_bounds__(kBlock, (RB > 8) ? kMinBlocksWide : kMinBlocks) update_kernel(const UpdParams P, const __grid_constant__ GradPtrs<NP> gp) {
     constexpr bool READS_G = !is_phase2(OPT);
     constexpr bool NEEDS_WT = FUSED && (OUT != O_NONE);
     __shared__ float2 red[kBlock / 32];
