@@ -442,6 +442,17 @@ __device__ __forceinline__ Fv<VEC> load_f32_partial(const float* p, int n) {
     return o;
 }
 
+// 9 to 32 bf16 copies: two tree blocks of 8 at a time.  A thread's 4 elements of 16 copies are the 128 bytes in flight
+// that 8 elements of 8 copies are, with half the state and sums in registers (no spills), no idle half of a CTA on
+// tiles of 1024, and half the waits for memory.  Formatting fused in, us, 8 elements of 8 copies / these: Adam, 12,
+// 16, 32 copies, 4.1 M parameters (tiles of 1024) 59 / 43, 67 / 51, 125 / 92, 25.6 M 235 / 209, 248 / 234, 479 / 386;
+// SGD-M 16 and 32 copies, 25.6 M 198 / 197, 405 / 343; LAMB 16 copies 317 / 295.  LARS, whose phase 1 holds no slots,
+// is the exception and keeps 8 elements: 25.6 M, 12 and 16 copies 216 / 227, 245 / 255.
+template <int OPT, bool GBF, int VEC, int RB, int NP>
+__host__ __device__ constexpr int many_blocks() {
+    return GBF && VEC == 4 && RB == 8 && NP > RB && !is_af(OPT) && OPT != K_LARS1 ? 2 : 1;
+}
+
 // OPT: optimizer / phase.  GBF: gradients are bf16.  OUT: where the updated weights go.
 // VEC: elements per thread access.  U: accesses per thread per pass.
 // RB: gradients summed per tree block.  NP: capacity of the by-value pointer table.
@@ -471,6 +482,7 @@ __device__ __forceinline__ void process_item(const UpdParams& P, const GradPtrs<
     constexpr bool WRITES_M = (OPT != K_LAMB2 && OPT != K_LARS1 && !is_af(OPT));
     constexpr bool WRITES_GHAT = (OPT == K_LARS1 || OPT == K_AF1);
     constexpr bool LOOPK = (NP > RB);   // R may exceed one tree block: loop and compensate
+    constexpr int NBLK = many_blocks<OPT, GBF, VEC, RB, NP>();   // tree blocks whose loads are in flight together
     constexpr bool WMASTER = FUSED && OUT == O_F32M;   // w lives in the weight tensors only
     const int nvalid = it.nvalid;
     const long long gbase = it.gbase, sbase = it.sbase, obase = it.obase, toff = it.toff;
@@ -598,22 +610,22 @@ __device__ __forceinline__ void process_item(const UpdParams& P, const GradPtrs<
             }
         }
         if (READS_G) {
-            for (int k0 = 0; k0 < (LOOPK ? P.R : 1); k0 += RB) {
-                GradRaw<GBF, VEC> raw[U][RB];
+            for (int k0 = 0; k0 < (LOOPK ? P.R : 1); k0 += RB * NBLK) {
+                GradRaw<GBF, VEC> raw[U][NBLK][RB];
 #pragma unroll
-                for (int j = 0; j < RB; ++j) {
+                for (int j = 0; j < RB * NBLK; ++j) {
 #pragma unroll
-                    for (int u = 0; u < U; ++u) raw[u][j] = {};          // (an absent copy adds +0)
+                    for (int u = 0; u < U; ++u) raw[u][j / RB][j % RB] = {};          // (an absent copy adds +0)
                     if (RB > 1 && k0 + j >= P.R) continue;
 #pragma unroll
                     for (int u = 0; u < U; ++u)
                         if (nv[u] > 0) {
                             if constexpr (FUSED) {
                                 const void* gk = sgp[k0 + j];
-                                if (nv[u] == VEC) raw[u][j] = load_grad<GBF, VEC>(gk, toff + e0[u]);
-                                else raw[u][j] = load_grad_partial<GBF, VEC>(gk, toff + e0[u], nv[u]);
+                                if (nv[u] == VEC) raw[u][j / RB][j % RB] = load_grad<GBF, VEC>(gk, toff + e0[u]);
+                                else raw[u][j / RB][j % RB] = load_grad_partial<GBF, VEC>(gk, toff + e0[u], nv[u]);
                             } else {
-                                raw[u][j] = load_grad<GBF, VEC>(gp.p[k0 + j], gbase + e0[u]);
+                                raw[u][j / RB][j % RB] = load_grad<GBF, VEC>(gp.p[k0 + j], gbase + e0[u]);
                             }
                         }
                 }
@@ -625,12 +637,16 @@ __device__ __forceinline__ void process_item(const UpdParams& P, const GradPtrs<
                 }
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
-                    const Fv<VEC> gb = tree_sum<GBF, VEC, RB>(raw[u]);
-                    if (!LOOPK || k0 == 0) {
-                        gv[u] = gb;
-                    } else {
 #pragma unroll
-                        for (int i = 0; i < VEC; ++i) kahan1(gv[u].f[i], gc[u].f[i], gb.f[i]);
+                    for (int b = 0; b < NBLK; ++b) {
+                        if (b > 0 && k0 + b * RB >= P.R) break;
+                        const Fv<VEC> gb = tree_sum<GBF, VEC, RB>(raw[u][b]);
+                        if (!LOOPK || k0 + b == 0) {
+                            gv[u] = gb;
+                        } else {
+#pragma unroll
+                            for (int i = 0; i < VEC; ++i) kahan1(gv[u].f[i], gc[u].f[i], gb.f[i]);
+                        }
                     }
                 }
             }

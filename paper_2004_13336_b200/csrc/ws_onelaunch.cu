@@ -197,7 +197,7 @@ ws_status launch_r(const UpdParams& P, const void* const* gptrs, const OneLaunch
         return launch<PAIR, GBF, OUT, 4, 1, 8, 8, 4, FUSED>(P, gptrs, Q, st);
     }
     if (P.R <= 32) {
-        if (wide) return launch<PAIR, GBF, OUT, GBF ? 8 : 4, 1, 8, 32, 8, FUSED>(P, gptrs, Q, st);
+        if (wide) return launch<PAIR, GBF, OUT, GBF && PAIR == 1 ? 8 : 4, 1, 8, 32, 8, FUSED>(P, gptrs, Q, st);
         return launch<PAIR, GBF, OUT, 4, 1, 8, 32, 4, FUSED>(P, gptrs, Q, st);
     }
     return WS_ERR_TOO_LARGE;      // (more copies: the caller runs the separate launches)

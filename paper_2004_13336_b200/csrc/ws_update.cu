@@ -331,7 +331,7 @@ ws_status launch_r(const UpdParams& P, const void* const* gptrs, bool wide_ok, c
             return launch<OPT, GBF, OUT, 4, OPT == K_AF1 ? kUAf8 : 1, 8, 8, FUSED>(P, gptrs, st);
         }
         if (P.R <= 32) {
-            if constexpr (GBF && OPT != K_AF1) if (wide_ok) return launch<OPT, GBF, OUT, 8, 1, 8, 32, FUSED>(P, gptrs, st);
+            if constexpr (GBF && OPT == K_LARS1) if (wide_ok) return launch<OPT, GBF, OUT, 8, 1, 8, 32, FUSED>(P, gptrs, st);
             return launch<OPT, GBF, OUT, 4, 1, 8, 32, FUSED>(P, gptrs, st);
         }
         // many replicas make small shards and few CTAs: more loads in flight per thread
