@@ -50,6 +50,7 @@ struct UpdParams {
     long long g_stride;     // per-shard element stride inside a gradient buffer (S, or 0 in slice mode)
     long long st_stride;    // per-shard element stride inside w/m/v (S for [R][S] state, 0 for one shard)
     int R;
+    int tile;               // elements of a full tile
     int r0;                 // first shard of this launch
     int concat;             // concatenated layout: tiles [tile_lo, tile_lo + nitems), each names its shard
     long long tile_lo;
@@ -481,6 +482,7 @@ __device__ __forceinline__ void process_item(const UpdParams& P, const GradPtrs<
     constexpr bool WRITES_W = writes_weights(OPT);   // phase 1 only zeroes the pads of w
     constexpr bool WRITES_M = (OPT != K_LAMB2 && OPT != K_LARS1 && !is_af(OPT));
     constexpr bool WRITES_GHAT = (OPT == K_LARS1 || OPT == K_AF1);
+    constexpr bool ELEMENTWISE = OPT == K_SGDM || OPT == K_ADAM;   // nothing is summed over the CTA: any block size
     constexpr bool LOOPK = (NP > RB);   // R may exceed one tree block: loop and compensate
     constexpr int NBLK = many_blocks<OPT, GBF, VEC, RB, NP>();   // tree blocks whose loads are in flight together
     constexpr bool WMASTER = FUSED && OUT == O_F32M;   // w lives in the weight tensors only
@@ -571,7 +573,8 @@ __device__ __forceinline__ void process_item(const UpdParams& P, const GradPtrs<
 #pragma unroll
     for (int j = 0; j < (OPT == K_AF1 ? VEC : 1); ++j) cacc[j] = 0.f;
 
-    for (int q0 = 0; q0 < nvec; q0 += U * kBlock) {
+    const int nt = ELEMENTWISE ? (int)blockDim.x : kBlock;
+    for (int q0 = 0; q0 < nvec; q0 += U * nt) {
         int e0[U];
         int nv[U];
         Fv<VEC> wv[U], mv[U], vv[U], gv[U], gc[U];
@@ -579,7 +582,7 @@ __device__ __forceinline__ void process_item(const UpdParams& P, const GradPtrs<
         long long col0[is_af(OPT) ? U : 1];    // column of each vector's first element
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const int q = q0 + u * kBlock + threadIdx.x;
+            const int q = q0 + u * nt + threadIdx.x;
             e0[u] = q * VEC;
             if constexpr (is_af(OPT)) {
                 // this vector's row and column, then on to the thread's next vector
@@ -875,10 +878,10 @@ __device__ __forceinline__ void process_item(const UpdParams& P, const GradPtrs<
 // Programmatic dependent launch: the grid may become resident while the previous kernel of the stream drains;
 // a kernel launched this way touches nothing that kernel may write before its griddepcontrol.wait.
 template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(void (*kernel)(KArgs...), long long grid, cudaStream_t st, const Args&... args) {
+cudaError_t launch_pdl_as(void (*kernel)(KArgs...), long long grid, int threads, cudaStream_t st, const Args&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3(kBlock);
+    cfg.blockDim = dim3((unsigned)threads);
     cfg.stream = st;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -886,6 +889,10 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), long long grid, cudaStream_t st
     cfg.attrs = at;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+}
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl(void (*kernel)(KArgs...), long long grid, cudaStream_t st, const Args&... args) {
+    return launch_pdl_as(kernel, grid, kBlock, st, args...);
 }
 // Clears the counters and words of a one-kernel update (a 16-byte aligned range, a multiple of 16 bytes) and its
 // status word.  A kernel and not a memset, so that it and the update chain by programmatic dependent launch.

@@ -72,10 +72,10 @@ __global__ void __launch_bounds__(kBlock, (RB > 8) ? kMinBlocksWide : kMinBlocks
             if constexpr (READS_G) {
                 const void* const* gt = P.gtab + (long long)tl.seg * P.R;
                 __syncthreads();   // the previous item's readers are done with sgp
-                for (int k = threadIdx.x; k < P.R; k += kBlock) sgp[k] = gt[k];
+                for (int k = threadIdx.x; k < P.R; k += (int)blockDim.x) sgp[k] = gt[k];
                 if constexpr (writes_weights(OPT)) {
                     if (OUT != O_NONE)
-                        for (int k = threadIdx.x; k < P.nw; k += kBlock) swp[k] = P.wtab[(long long)tl.seg * P.nw + k];
+                        for (int k = threadIdx.x; k < P.nw; k += (int)blockDim.x) swp[k] = P.wtab[(long long)tl.seg * P.nw + k];
                 }
                 __syncthreads();
             }
@@ -305,7 +305,12 @@ ws_status launch(const UpdParams& P, const void* const* gptrs, cudaStream_t st) 
     if (grid < 1) return WS_OK;
     if (grid > 0x7fffffffLL) grid = 0x7fffffffLL;
     // (the kernel reads only the plan and pointer tables before it waits for the kernel in front)
-    launch_pdl(update_kernel<OPT, GBF, OUT, VEC, U, RB, NP, FUSED>, grid, st, P, gp);
+    // A tile of 1024 elements is 128 vectors of 8: half of 256 threads would have nothing, and six CTAs per SM wait for
+    // their tables side by side where three did.  Tiles of 1024, us, 256 / 128 threads: 4.1 M parameters, bf16 copies,
+    // SGD-M 8 copies 28.7 / 18.4, 4 copies 21.9 / 13.1, Adam 8 copies 36.2 / 24.2; 1.2 M, Adam, 4 bf16 copies 11.1 / 7.3,
+    // 2 fp32 copies 10.1 / 6.6.
+    const int threads = (OPT == K_SGDM || OPT == K_ADAM) && VEC == 8 && P.tile <= 1024 ? 128 : kBlock;
+    launch_pdl_as(update_kernel<OPT, GBF, OUT, VEC, U, RB, NP, FUSED>, grid, threads, st, P, gp);
     return ws_check_launch(FUSED ? "ws_fused_update" : "ws_shard_update");
 }
 
@@ -454,6 +459,7 @@ ws_status prepare(const ws_plan* p, int32_t r, const ws_grads* g, const ws_state
     }
     P.tiles = p->d_tiles;
     P.ntiles = p->ntiles;
+    P.tile = p->K;
     P.S = p->S;
     P.R = g ? g->R : p->R;
     const int nshards = (r < 0) ? p->R : 1;
