@@ -50,7 +50,7 @@ struct UpdParams {
     long long g_stride;     // per-shard element stride inside a gradient buffer (S, or 0 in slice mode)
     long long st_stride;    // per-shard element stride inside w/m/v (S for [R][S] state, 0 for one shard)
     int R;
-    int tile;               // elements of a full tile
+    int tile;               // elements of a tile on average
     int r0;                 // first shard of this launch
     int concat;             // concatenated layout: tiles [tile_lo, tile_lo + nitems), each names its shard
     long long tile_lo;
@@ -575,6 +575,8 @@ __device__ __forceinline__ void process_item(const UpdParams& P, const GradPtrs<
 
     const int nt = ELEMENTWISE ? (int)blockDim.x : kBlock;
     for (int q0 = 0; q0 < nvec; q0 += U * nt) {
+        // (a warp without a vector of a short tile has nothing to do; the norm pairs' warps meet again at their sums)
+        if (ELEMENTWISE && FUSED && q0 + (int)threadIdx.x >= nvec) break;
         int e0[U];
         int nv[U];
         Fv<VEC> wv[U], mv[U], vv[U], gv[U], gc[U];

@@ -305,11 +305,16 @@ ws_status launch(const UpdParams& P, const void* const* gptrs, cudaStream_t st) 
     if (grid < 1) return WS_OK;
     if (grid > 0x7fffffffLL) grid = 0x7fffffffLL;
     // (the kernel reads only the plan and pointer tables before it waits for the kernel in front)
-    // A tile of 1024 elements is 128 vectors of 8: half of 256 threads would have nothing, and six CTAs per SM wait for
-    // their tables side by side where three did.  Tiles of 1024, us, 256 / 128 threads: 4.1 M parameters, bf16 copies,
-    // SGD-M 8 copies 28.7 / 18.4, 4 copies 21.9 / 13.1, Adam 8 copies 36.2 / 24.2; 1.2 M, Adam, 4 bf16 copies 11.1 / 7.3,
-    // 2 fp32 copies 10.1 / 6.6.
-    const int threads = (OPT == K_SGDM || OPT == K_ADAM) && VEC == 8 && P.tile <= 1024 ? 128 : kBlock;
+    // Elementwise updates take the CTA that their tiles fill: a tile of 1024 elements is 128 vectors of 8, and a model of
+    // many small tensors cut into many shards has tiles of 32 to a few hundred elements.  The registers of the threads
+    // without a vector then hold further CTAs, and a CTA's chain of table reads is what small models wait for.  From
+    // more than three CTAs per SM on: a small launch has room for all its CTAs, and many copies (a thread of a CTA of 64
+    // passes over a full tile 4 times) want the threads.  us, 256 threads / this rule, formatting fused in: tiles of
+    // 1024, 4.1 M parameters, SGD-M 8 bf16 copies 28.7 / 17.9, 4 copies 21.9 / 12.7, Adam 8 copies 36.2 / 24.5;
+    // 1.2 M parameters in 161 tensors, Adam, 16 copies fp32 27.7 / 19.6, bf16 26.4 / 15.5, 32 copies bf16 57 / 34.
+    int threads = kBlock;
+    if ((OPT == K_SGDM || OPT == K_ADAM) && NP <= 32 && P.nitems > 444)
+        while (threads > 64 && P.tile <= VEC * threads / 2) threads /= 2;
     launch_pdl_as(update_kernel<OPT, GBF, OUT, VEC, U, RB, NP, FUSED>, grid, threads, st, P, gp);
     return ws_check_launch(FUSED ? "ws_fused_update" : "ws_shard_update");
 }
@@ -459,7 +464,7 @@ ws_status prepare(const ws_plan* p, int32_t r, const ws_grads* g, const ws_state
     }
     P.tiles = p->d_tiles;
     P.ntiles = p->ntiles;
-    P.tile = p->K;
+    P.tile = p->ntiles > 0 ? (int)((p->layout == WS_LAYOUT_CONCAT ? p->S * p->R : p->S) / p->ntiles) : p->K;
     P.S = p->S;
     P.R = g ? g->R : p->R;
     const int nshards = (r < 0) ? p->R : 1;
