@@ -50,7 +50,7 @@ struct UpdParams {
     long long g_stride;     // per-shard element stride inside a gradient buffer (S, or 0 in slice mode)
     long long st_stride;    // per-shard element stride inside w/m/v (S for [R][S] state, 0 for one shard)
     int R;
-    int tile;               // elements of a tile on average
+    int tile, tile_max;     // elements of a tile on average, and of a full one
     int r0;                 // first shard of this launch
     int concat;             // concatenated layout: tiles [tile_lo, tile_lo + nitems), each names its shard
     long long tile_lo;
@@ -260,6 +260,20 @@ __device__ __forceinline__ void kahan1(float& s, float& c, float x) {
     const float t = s + y;
     c = (t - s) - y;
     s = t;
+}
+
+// The order of the sum of more than 32 copies.  Blocks of kTreeBlockLarge copies are trees; consecutive blocks form up
+// to kManyGroups groups; a group's blocks are added with compensation, and so are the groups (sum and compensation).
+// Up to 128 copies a group is one block.  One thread can do it all (process_item), or the warps of a CTA a group each
+// (split_kernel): the bits are the same.  (The norm pairs and Adafactor have no such split and no groups.)
+constexpr int kManyGroups = 8;
+__host__ __device__ constexpr int many_blocks_per_group(int copies) {
+    return ((copies + kTreeBlockLarge - 1) / kTreeBlockLarge + kManyGroups - 1) / kManyGroups;
+}
+// Adds a group of several blocks, (s, c), to the groups before it.
+__device__ __forceinline__ void add_group(float& sum, float& comp, float s, float c) {
+    kahan1(sum, comp, s);
+    kahan1(sum, comp, -c);
 }
 
 // ------------------------------------------------------------------ math ---
@@ -485,6 +499,7 @@ __device__ __forceinline__ void process_item(const UpdParams& P, const GradPtrs<
     constexpr bool ELEMENTWISE = OPT == K_SGDM || OPT == K_ADAM;   // nothing is summed over the CTA: any block size
     constexpr bool LOOPK = (NP > RB);   // R may exceed one tree block: loop and compensate
     constexpr int NBLK = many_blocks<OPT, GBF, VEC, RB, NP>();   // tree blocks whose loads are in flight together
+    constexpr bool MANY = ELEMENTWISE && NP > kManyGroups * kTreeBlockLarge;   // groups of several blocks
     constexpr bool WMASTER = FUSED && OUT == O_F32M;   // w lives in the weight tensors only
     const int nvalid = it.nvalid;
     const long long gbase = it.gbase, sbase = it.sbase, obase = it.obase, toff = it.toff;
@@ -615,6 +630,10 @@ __device__ __forceinline__ void process_item(const UpdParams& P, const GradPtrs<
             }
         }
         if (READS_G) {
+            Fv<VEC> gs[MANY ? U : 1], gsc[MANY ? U : 1];       // the groups before this one
+            bool first = true;
+            const int group_blocks = MANY ? many_blocks_per_group(P.R) : 0;
+            int in_group = group_blocks > 1 ? 0 : 1;           // blocks of this group so far (a group of one: all blocks are one sum)
             for (int k0 = 0; k0 < (LOOPK ? P.R : 1); k0 += RB * NBLK) {
                 GradRaw<GBF, VEC> raw[U][NBLK][RB];
 #pragma unroll
@@ -646,7 +665,7 @@ __device__ __forceinline__ void process_item(const UpdParams& P, const GradPtrs<
                     for (int b = 0; b < NBLK; ++b) {
                         if (b > 0 && k0 + b * RB >= P.R) break;
                         const Fv<VEC> gb = tree_sum<GBF, VEC, RB>(raw[u][b]);
-                        if (!LOOPK || k0 + b == 0) {
+                        if (!LOOPK || k0 + b == 0 || (MANY && in_group == 0)) {
                             gv[u] = gb;
                         } else {
 #pragma unroll
@@ -654,6 +673,29 @@ __device__ __forceinline__ void process_item(const UpdParams& P, const GradPtrs<
                         }
                     }
                 }
+                if constexpr (MANY) {
+                    if (group_blocks > 1 && (++in_group == group_blocks || k0 + RB >= P.R)) {       // a group is complete
+#pragma unroll
+                        for (int u = 0; u < U; ++u)
+#pragma unroll
+                            for (int i = 0; i < VEC; ++i) {
+                                if (first) {
+                                    gs[u].f[i] = gv[u].f[i];
+                                    gsc[u].f[i] = gc[u].f[i];
+                                } else {
+                                    add_group(gs[u].f[i], gsc[u].f[i], gv[u].f[i], gc[u].f[i]);
+                                }
+                                gc[u].f[i] = 0.f;
+                            }
+                        first = false;
+                        in_group = 0;
+                    }
+                }
+            }
+            if constexpr (MANY) {
+                if (group_blocks > 1)
+#pragma unroll
+                    for (int u = 0; u < U; ++u) gv[u] = gs[u];
             }
         }
         if constexpr (OPT == K_AF1) {

@@ -31,10 +31,17 @@ namespace {
 constexpr long long kKeepReverseBytes = 256ll << 20;   // twice the L2: at least half of phase 2's re-reads can hit
 using namespace wsk;
 
+// (129 and more bf16 copies: 16 of 4 elements are 32 registers, and the third CTA per SM is worth a few spills - 512
+// copies of 346 K elements, Adam 98 -> 67 us, SGD-M 95 -> 64; 64 copies of 2.8 M, SGD-M, would go from 66 to 76)
+template <int OPT, bool GBF, int RB, int NP>
+constexpr int min_blocks() {
+    return RB > 8 && !(GBF && NP > 128 && (OPT == K_SGDM || OPT == K_ADAM)) ? kMinBlocksWide : kMinBlocks;
+}
+
 // One CTA handles one (shard, tile) work item; the grid is the item count, so the
 // hardware CTA scheduler walks the buffers front to back.
 template <int OPT, bool GBF, int OUT, int VEC, int U, int RB, int NP, bool FUSED>
-__global__ void __launch_bounds__(kBlock, (RB > 8) ? kMinBlocksWide : kMinBlocks) update_kernel(const UpdParams P, const __grid_constant__ GradPtrs<NP> gp) {
+__global__ void __launch_bounds__(kBlock, min_blocks<OPT, GBF, RB, NP>()) update_kernel(const UpdParams P, const __grid_constant__ GradPtrs<NP> gp) {
     constexpr bool READS_G = !is_phase2(OPT);
     constexpr bool NEEDS_WT = FUSED && (OUT != O_NONE);
     __shared__ float2 red[kBlock / 32];
@@ -88,6 +95,100 @@ __global__ void __launch_bounds__(kBlock, (RB > 8) ? kMinBlocksWide : kMinBlocks
         if (OPT == K_AF3) lr_rho = P.rho[tl.seg];         // alpha_t / max(1, RMS(U_t)/d)
         process_item<OPT, GBF, OUT, VEC, U, RB, NP, FUSED, HINT>(P, gp, it, sgp, swp, wt, lr_rho, red);
     }
+}
+
+// More than 32 packed copies of a shard too small to fill the chip: the warps of a CTA share 128 (bf16: 256) elements
+// and take a group of the copies each, so that a thread waits for memory once per block of its group and not once per
+// block of all copies.  The groups meet in shared memory with their compensations.  What bounds it: up to 64 K elements
+// those waits, one to eight in a row; beyond, DRAM pages of 512 bytes a copy and CTA.  Adam, us, one thread per element /
+// this, slices of one shard: 512 copies of 22 K elements fp32 32 / 10, bf16 40 / 10, of 87 K 41 / 37, 45 / 20; 1024
+// copies of 11 K 61 / 13, 76 / 16, of 43 K 74 / 40, 86 / 19 (10 us of each are the host's).
+template <int OPT, bool GBF, int OUT>
+__global__ void __launch_bounds__(kBlock, kMinBlocksWide) split_kernel(const UpdParams P, const __grid_constant__ GradPtrs<1024> gp, int nsub) {
+    constexpr int VEC = GBF ? 8 : 4, E = 32 * VEC, RB = kTreeBlockLarge;
+    static_assert(kBlock / 32 == kManyGroups, "a warp per group");
+    __shared__ float2 part[kManyGroups][E];             // a group's sum and its compensation
+    asm volatile("griddepcontrol.launch_dependents;");
+    const unsigned item = blockIdx.x / (unsigned)nsub;
+    const int e0 = (int)(blockIdx.x - item * (unsigned)nsub) * E;
+    long long rs = P.concat ? 0 : item / (unsigned)P.ntiles;
+    const WsTile tl = P.tiles[P.concat ? P.tile_lo + item : item - rs * P.ntiles];
+    if (e0 >= tl.len) return;
+    if (P.concat) rs = tl.shard - P.r0;
+    const long long r = P.r0 + rs;
+    const long long nvl = tl.vt - r * tl.piece;
+    const int nvalid = nvl < 0 ? 0 : (nvl > tl.len ? tl.len : (int)nvl);
+    const long long gbase = rs * P.g_stride + tl.pos, sbase = rs * P.st_stride + tl.pos, obase = r * P.S + tl.pos;
+#ifdef WS_DEBUG_BOUNDS
+    {
+        unsigned bits = 0;
+        if (sbase < 0 || sbase + tl.len > P.state_elems) bits |= WS_BOUNDS_STATE;
+        if (gbase < 0 || gbase + tl.len > P.grad_elems) bits |= WS_BOUNDS_GRAD;
+        if (OUT != O_NONE && (obase < 0 || obase + tl.len > P.out_elems)) bits |= WS_BOUNDS_OUT;
+        if (bits) {
+            if (threadIdx.x == 0 && P.bounds) atomicOr(P.bounds, bits);
+            return;
+        }
+    }
+#endif
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    // the thread's 4 elements of the update
+    const int x0 = 4 * (int)threadIdx.x, at = e0 + x0;
+    const bool mine = x0 < E && at < tl.len;
+    Fv<4> w = {}, m = {}, v = {};
+    if (mine && at < nvalid) {
+        w = load_f32<4>(P.w + sbase + at);
+        m = load_f32<4>(P.m + sbase + at);
+        if (OPT == K_ADAM) v = load_f32<4>(P.v + sbase + at);
+    }
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int blocks = (P.R + RB - 1) / RB, per = many_blocks_per_group(P.R), groups = (blocks + per - 1) / per;
+    const int eg = e0 + lane * VEC;
+    if (warp < groups) {
+        Fv<VEC> s = {}, c = {};
+        const int last = (warp + 1) * per < blocks ? (warp + 1) * per : blocks;
+        if (eg < nvalid)
+            for (int b = warp * per; b < last; ++b) {
+                GradRaw<GBF, VEC> raw[RB];
+#pragma unroll
+                for (int j = 0; j < RB; ++j) {
+                    raw[j] = {};
+                    if (b * RB + j < P.R) raw[j] = load_grad<GBF, VEC>(gp.p[b * RB + j], gbase + eg);
+                }
+                const Fv<VEC> t = tree_sum<GBF, VEC, RB>(raw);
+                if (b == warp * per) {
+                    s = t;
+                } else {
+#pragma unroll
+                    for (int i = 0; i < VEC; ++i) kahan1(s.f[i], c.f[i], t.f[i]);
+                }
+            }
+#pragma unroll
+        for (int i = 0; i < VEC; i += 2)
+            *reinterpret_cast<float4*>(&part[warp][lane * VEC + i]) = make_float4(s.f[i], c.f[i], s.f[i + 1], c.f[i + 1]);
+    }
+    __syncthreads();
+    if (!mine) return;
+    float none = 0.f;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        if (at + j < nvalid) {
+            float2 t = part[0][x0 + j];
+            for (int g = 1; g < groups; ++g) {
+                const float2 o = part[g][x0 + j];
+                if (per > 1) add_group(t.x, t.y, o.x, o.y);
+                else kahan1(t.x, t.y, o.x);
+            }
+            update_elem<OPT>(P.c, t.x * P.c.gscale, w.f[j], m.f[j], v.f[j], 0.f, none, none);
+        } else {
+            w.f[j] = m.f[j] = v.f[j] = 0.f;       // pad: +0 for every output
+        }
+    }
+    store_f32<4>(P.w + sbase + at, w);
+    store_f32<4>(P.m + sbase + at, m);
+    if (OPT == K_ADAM) store_f32<4>(P.v + sbase + at, v);
+    if (OUT == O_F32) store_f32<4>(reinterpret_cast<float*>(P.gathered) + obase + at, w);
+    if (OUT == O_BF16) store_bf16<4>(reinterpret_cast<unsigned short*>(P.gathered) + obase + at, w);
 }
 
 // Sum every shard's per-tile partials of tensor t (sum_partials), then rho_t = sqrt(a)/sqrt(b).
@@ -319,6 +420,17 @@ ws_status launch(const UpdParams& P, const void* const* gptrs, cudaStream_t st) 
     return ws_check_launch(FUSED ? "ws_fused_update" : "ws_shard_update");
 }
 
+// Elements of a launch up to which split_kernel is the faster one.  One thread per element costs about 1.2 us for every
+// 16 copies whatever the size, the split kernel half of the copy bandwidth once the chip is full.  us, one thread / split:
+// fp32, 128 copies of 88 K 9.7 / 12.6; 200 of 56 K 14.4 / 12.4, of 223 K 34 / 45; 512 of 87 K 41 / 37, of 162 K 53 / 65;
+// 1024 of 81 K 78 / 64, of 173 K 107 / 118; bf16, 128 of 88 K 12.9 / 9.6, of 349 K 16 / 23 (SGD-M); 200 of 223 K 32 / 25;
+// 512 of 162 K 61 / 39, of 346 K 67 / 69; 1024 of 81 K 108 / 41.
+long long split_elems(bool gbf, int copies) {
+    constexpr long long K = 1 << 10;
+    if (gbf) return (copies > 128 ? 256 : 128) * K;
+    return (copies >= 512 ? 128 : copies > 128 ? 64 : 32) * K;
+}
+
 // Wide (256-bit) accesses need 32-byte aligned buffers; they pay off when the
 // gradients are bf16 (a 128-bit gradient load then covers 8 elements) and for
 // small R, where the fp32 streams dominate.
@@ -345,7 +457,21 @@ ws_status launch_r(const UpdParams& P, const void* const* gptrs, bool wide_ok, c
             return launch<OPT, GBF, OUT, 4, 1, 8, 32, FUSED>(P, gptrs, st);
         }
         // many replicas make small shards and few CTAs: more loads in flight per thread
-        if (P.R <= 1024) return launch<OPT, GBF, OUT, 4, 1, kTreeBlockLarge, 1024, FUSED>(P, gptrs, st);
+        if (P.R <= 1024) {
+            if constexpr (!FUSED && (OPT == K_SGDM || OPT == K_ADAM)) {
+                // (full tiles far longer than the average would leave most of the grid empty)
+                const int nsub = (P.tile_max + (GBF ? 255 : 127)) / (GBF ? 256 : 128);
+                if (P.nitems >= 1 && P.nitems * P.tile <= split_elems(GBF, P.R) && P.nitems * nsub <= 65536) {
+                    GradPtrs<1024> gp;
+                    for (int k = 0; k < 1024; ++k) gp.p[k] = k < P.R ? gptrs[k] : nullptr;
+                    launch_pdl(split_kernel<OPT, GBF, OUT>, P.nitems * nsub, st, P, gp, nsub);
+                    return ws_check_launch("ws_shard_update");
+                }
+            }
+            if constexpr (OPT == K_SGDM || OPT == K_ADAM)
+                if (P.R <= 128) return launch<OPT, GBF, OUT, 4, 1, kTreeBlockLarge, 128, FUSED>(P, gptrs, st);
+            return launch<OPT, GBF, OUT, 4, 1, kTreeBlockLarge, 1024, FUSED>(P, gptrs, st);
+        }
         return WS_ERR_TOO_LARGE;
     }
 }
@@ -464,6 +590,7 @@ ws_status prepare(const ws_plan* p, int32_t r, const ws_grads* g, const ws_state
     }
     P.tiles = p->d_tiles;
     P.ntiles = p->ntiles;
+    P.tile_max = p->K;
     P.tile = p->ntiles > 0 ? (int)((p->layout == WS_LAYOUT_CONCAT ? p->S * p->R : p->S) / p->ntiles) : p->K;
     P.S = p->S;
     P.R = g ? g->R : p->R;

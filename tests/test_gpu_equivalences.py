@@ -123,3 +123,54 @@ def test_entry_points_agree(case):
         for k in range(R):
             for a, b in zip(lists[k], ref):
                 assert torch.equal(a, b), "replica kernels: weights"
+
+
+@pytest.mark.parametrize("layout", ["per_tensor", "concat"])
+@pytest.mark.parametrize("gdtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("opt", ["sgdm", "adam"])
+@pytest.mark.parametrize("R", [33, 64, 128, 129, 257, 1024])
+def test_many_copies_one_thread_or_a_group_per_warp(R, opt, gdtype, layout):
+    # one shard's slices (small: the groups of copies go to the warps of a CTA) against the same sums in one thread per
+    # element (the formatting-fused form): a last block, a last group and a last vector that are not full, shards of
+    # padding only; the sums against 64 bits
+    shapes = [(1031,), (3,), (257, 9), (0,), (128,), (41, 100)]
+    numel = [int(np.prod(s)) for s in shapes]
+    M = 3
+    plan = B.Plan(shapes, M, 8, layout=layout)
+    gen = torch.Generator(device=DEV).manual_seed(R)
+    def draw(std):
+        return [torch.randn(n, generator=gen, device=DEV) * std for n in numel]
+    w, m, v = draw(0.02), draw(1e-3), [x.abs() for x in draw(1e-5)]
+    g = [[x.to(gdtype) for x in draw(1e-3)] for _ in range(R)]
+    hy = B.make_hyper(opt, dict(lr=1.0 if opt == "sgdm" else 1e-3, beta1=0.9, beta2=0.999, eps=1e-8, weight_decay=0.0,
+                                momentum=0.0, grad_scale=1.0, step=3))
+
+    def packed(lst, dt=torch.float32):
+        b = torch.full((plan.G,), float("nan"), dtype=dt, device=DEV)
+        B.ws_pack(plan, lst, b)
+        return b
+
+    state = [packed(x) for x in (w, m, v)]
+    if opt == "sgdm":
+        state[2] = None
+    one = [None if x is None else x.clone() for x in state]
+    wt = [torch.empty(n, device=DEV) for n in numel]
+    B.ws_fused_update(plan, -1, B.TensorTable(plan, g), *one, hy, B.TensorTable(plan, [wt]))
+    pg = [packed(x, gdtype) for x in g]
+    S = plan.S
+    gathered = torch.full((plan.G,), 7.0, dtype=torch.bfloat16, device=DEV)
+    for r in range(M):
+        cut = [None if x is None else x[r * S:(r + 1) * S].clone() for x in state]
+        B.ws_shard_update(plan, r, [x[r * S:(r + 1) * S].clone() for x in pg], *cut, hy, gathered, None, slice_mode=1)
+        for a, b in zip(cut, one):
+            assert a is None or torch.equal(a, b[r * S:(r + 1) * S])
+    assert torch.equal(gathered, one[0].to(torch.bfloat16))
+    if opt == "sgdm":                              # m' is the sum itself: two roundings of compensated sums of trees of 16
+        for t, n in enumerate(numel):
+            exact = sum(gk[t].double() for gk in g)
+            lst = [torch.empty(k, device=DEV) for k in numel]
+            B.ws_unpack(plan, one[1], lst)
+            got = lst[t].double()
+            # a tree of 16 has 4 levels, each at most 2^-24 of its partial sums, which 16 sum |g| / R bound
+            bound = 6 * 2.0 ** -24 * sum(gk[t].double().abs() for gk in g)
+            assert bool(((got - exact).abs() <= bound).all())
