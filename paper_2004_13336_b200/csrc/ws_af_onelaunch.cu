@@ -27,7 +27,11 @@
 // word -> data, then the arrival): hence large blocks and one record per entry.
 // Measured against the six launches it replaces (us): Transformer set (211 M), fp32, R = 1 1148 -> 877, R = 4 1376 ->
 // 1245, R = 8 1862 -> 1760; ResNet-50 set (25.6 M), R = 4 269 -> 164; 22.7 M parameters in ragged tensors, R = 2:
-// 749 -> 172 (there a scalar reduction per element went to memory); 45 792 parameters, called from the host, 27 -> 17.
+// 749 -> 166 (there a scalar reduction per element went to memory); 45 792 parameters, called from the host, 27 -> 15.5.
+// The hand-over between the passes is a tiny model's whole time (P1 2.4, M 2.4, P2 2.0, its sum and step size 2.8, P3
+// 1 us): a counter's fences are one, the step size is published before anything else is stored, its two roots are
+// formed side by side, M reads the old state while it waits, and the rows in parallel are folded four at a time
+// (24 K parameters 16.6 -> 15.1 us, 0.7 M 20.8 -> 19.0, 4.1 M 38.3 -> 36.8; ragged 172 -> 166).
 //
 // Tickets, waits and their progress argument are those of ws_onelaunch.cu: an entry waits only for entries with
 // smaller tickets, which belong to CTAs that are running or have finished; every wait has an iteration limit.
@@ -404,16 +408,19 @@ __device__ __forceinline__ void sums_block(const AfLaunch& P, const WsAfTensor& 
                 }
             }
             const int quads = width / 4;
-            for (; rows > 1; rows = (rows + 1) / 2) {     // fold the upper rows onto the lower ones
-                const int half = (rows + 1) / 2;
+            while (rows > 1) {                            // fold the upper three quarters of the rows onto the lowest
+                const int part = (rows + 3) / 4;
                 __syncthreads();
-                for (int i = threadIdx.x; i < (rows - half) * quads; i += kBlock) {
+                for (int i = threadIdx.x; i < part * quads; i += kBlock) {
                     float4* a = reinterpret_cast<float4*>(colsum) + i;
-                    const float4 b = a[half * quads];
-                    float4 s = *a;
-                    s.x += b.x; s.y += b.y; s.z += b.z; s.w += b.w;
-                    *a = s;
+                    float4 s[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        s[j] = i + j * part * quads < rows * quads ? a[j * part * quads] : make_float4(0.f, 0.f, 0.f, 0.f);
+                    *a = make_float4((s[0].x + s[1].x) + (s[2].x + s[3].x), (s[0].y + s[1].y) + (s[2].y + s[3].y),
+                                     (s[0].z + s[1].z) + (s[2].z + s[3].z), (s[0].w + s[1].w) + (s[2].w + s[3].w));
                 }
+                rows = part;
             }
             __syncthreads();
             if (k.rr == 0 && k.nv > 0) {
@@ -613,17 +620,24 @@ __global__ void __launch_bounds__(kBlock, kMinBlocks) af_kernel(const AfLaunch P
     if (kind == 1) {
         // moments of one chunk of a tensor's factored state
         const long long begin = (long long)(((unsigned long long)(unsigned)it.col0 << 32) | (unsigned)it.row0);
+        constexpr int N = kWsAfChunk / kBlock;
+        float old[N];                              // (does not depend on P1)
+#pragma unroll
+        for (int j = 0; j < N; ++j) old[j] = tid + j * kBlock < (int)it.goff32 ? P.state[T.foff + begin + tid + j * kBlock] : 0.f;
         if (tid == 0) s_last = wait_count(P, P.count1 + it.seg, T.item_count);
         __syncthreads();
         if (!s_last) return;
         double rs = 0.0;
-        for (int i = tid; i < (int)it.goff32; i += kBlock) {
+#pragma unroll
+        for (int j = 0; j < N; ++j) {
+            const int i = tid + j * kBlock;
+            if (i >= (int)it.goff32) break;
             const long long e = begin + i;
             const bool isrow = e < T.nrow;
             const long long k = isrow ? T.irow + e : T.icol + (e - T.nrow);
-            const double v = P.beta * (double)P.state[T.foff + e] + (1.0 - P.beta) * (double)__ldcg(P.acc + k);
+            const double v = P.beta * (double)old[j] + (1.0 - P.beta) * (double)__ldcg(P.acc + k);
             P.state[T.foff + e] = (float)v;
-            const double f = 1.0 / sqrt((double)(float)v);
+            const double f = rsqrt((double)(float)v);
             if (isrow) P.rfac[T.rfac + e] = f;
             else P.fac[k] = (float)f;
             if (isrow) rs += v;
@@ -635,9 +649,7 @@ __global__ void __launch_bounds__(kBlock, kMinBlocks) af_kernel(const AfLaunch P
         if (tid == 0) {
             for (int i = 1; i < kBlock / 32; ++i) rs += da[i];
             if (rs != 0.0) atomicAdd(P.rsum + it.seg, rs);
-            __threadfence();
-            if (atomicAdd(P.countm + it.seg, 1) + 1 == T.chunk_count) {
-                __threadfence();
+            if (arrive(P.countm + it.seg) == T.chunk_count) {
                 // the row factors still lack sqrt(sum(Rv')), which goes with the word
                 // (its bits inverted: no square root gives the word 0)
                 const double r = sqrt(__ldcg(P.rsum + it.seg));
@@ -705,12 +717,10 @@ __global__ void __launch_bounds__(kBlock, kMinBlocks) af_kernel(const AfLaunch P
     sum_block(a, b, da, db);
     if (tid == 0) {
         P.ipart[it.item] = make_double2(a, b);
-        __threadfence();
-        s_last = (atomicAdd(P.count2 + it.seg, 1) + 1 == T.item_count) ? 1 : 0;
+        s_last = arrive(P.count2 + it.seg) == T.item_count ? 1 : 0;
     }
     __syncthreads();
     if (!s_last) return;
-    __threadfence();
     a = 0.0;
     b = 0.0;
     for (int i = tid; i < T.item_count; i += kBlock) {     // fixed order
@@ -719,17 +729,20 @@ __global__ void __launch_bounds__(kBlock, kMinBlocks) af_kernel(const AfLaunch P
         b += p.y;
     }
     sum_block(a, b, da, db);
-    if (tid == 0) {
-        const double rms_w = sqrt(a / (double)T.numel), rms_u = sqrt(b / (double)T.numel);
-        const double al = (P.eps2 > rms_w ? P.eps2 : rms_w) * P.rho_step;
-        const double clip = rms_u / P.clip > 1.0 ? rms_u / P.clip : 1.0;
-        const float rate = (float)(al / clip);
-        P.norms[2 * it.seg] = a;
-        P.norms[2 * it.seg + 1] = b;
-        P.alpha[it.seg] = (float)al;
-        P.rho[it.seg] = rate;
-        __threadfence();
-        st_release64(P.flag2 + it.seg, ((unsigned long long)__float_as_uint(rate) << 32) | 1ULL);
+    if (tid < 32) {
+        // (two lanes: a 64-bit root and quotient take longer than the exchange)
+        const double b0 = __shfl_sync(0xffffffffu, b, 0), mine = tid == 0 ? a : b0;
+        const double rms = sqrt(mine / (double)T.numel), rms_u = __shfl_down_sync(0xffffffffu, rms, 1);
+        if (tid == 0) {
+            const double al = (P.eps2 > rms ? P.eps2 : rms) * P.rho_step, d = rms_u / P.clip;
+            const float rate = (float)(d > 1.0 ? al / d : al);
+            // the word first: it is what the other CTAs wait for
+            st_release64(P.flag2 + it.seg, ((unsigned long long)__float_as_uint(rate) << 32) | 1ULL);
+            P.norms[2 * it.seg] = a;
+            P.norms[2 * it.seg + 1] = b;
+            P.alpha[it.seg] = (float)al;
+            P.rho[it.seg] = rate;
+        }
     }
     if (!P.master) zero_pads(P, T);
 }

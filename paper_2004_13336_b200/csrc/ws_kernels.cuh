@@ -324,6 +324,14 @@ __device__ __forceinline__ void red_add_vec(float* p, const float* x) {
                      :: "l"(p + j), "f"(x[j]), "f"(x[j + 1]), "f"(x[j + 2]), "f"(x[j + 3]) : "memory");
 }
 
+// Counts an arrival: what the CTA wrote before (its other threads' writes lie before a barrier) is visible to whoever
+// counts after it, and the other way round.  One fence where a plain atomic add has one before and one after it.
+__device__ __forceinline__ int arrive(int* p) {
+    int v;
+    asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;" : "=r"(v) : "l"(p) : "memory");
+    return v + 1;
+}
+
 // ---------------------------------------------------------------- kernel ---
 // One work item: a run of `len` consecutive shard positions inside one tensor's piece.
 struct ItemCtx {

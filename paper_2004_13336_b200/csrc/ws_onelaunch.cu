@@ -127,24 +127,20 @@ two_phase_kernel(const UpdParams P, const __grid_constant__ GradPtrs<NP> gp, con
         // warp 0 has stored the partial sums of the item's tiles; count the item, and the CTA that counts a
         // tensor's last one forms the ratio
         const uint4 sg = ld_u128(Q.segs + it.seg);
-        if (tid == 0) {
-            __threadfence();
-            s_last = (atomicAdd(Q.count + it.seg, 1) + 1 == (int)sg.y) ? 1 : 0;
-        }
+        if (tid == 0) s_last = arrive(Q.count + it.seg) == (int)sg.y ? 1 : 0;
         __syncthreads();
         if (!s_last) return;
-        __threadfence();
         double a, b;
         sum_partials(WsSegTiles{(int)sg.z, (int)sg.w}, P.partials, P.ntiles, Q.reps, fin_a, fin_b, a, b);
         if (tid == 0) {
-            Q.norms[2 * it.seg] = a;
-            Q.norms[2 * it.seg + 1] = b;
             float ratio = 1.0f;
             if (a > 0.0 && b > 0.0)
                 ratio = PAIR == 1 ? (float)(Q.eta * sqrt(a) / (sqrt(b) + Q.beta * sqrt(a))) : (float)(sqrt(a) / sqrt(b));
-            Q.rho[it.seg] = ratio;
-            __threadfence();
+            // the word first: it is what the other CTAs wait for
             st_release(Q.flag + it.seg, ((unsigned long long)__float_as_uint(ratio) << 32) | 1ULL);
+            Q.rho[it.seg] = ratio;
+            Q.norms[2 * it.seg] = a;
+            Q.norms[2 * it.seg + 1] = b;
         }
         return;
     }
