@@ -346,7 +346,7 @@ ws_status ws_workspace_partials(const ws_plan* plan, size_t* offset_bytes, size_
  * memory bound - read gradient, weight, auxiliaries; write weight,
  * auxiliaries).  With opt == WS_LAMB or WS_LARS only r == -1 is accepted here
  * (phase 1 over all shards, finalize, phase 2 over all shards, as three
- * launches or one kernel with the same bits): the per-tensor
+ * launches - two on small models - or one kernel, with the same bits): the per-tensor
  * ratio needs every shard's partial norms before any shard can apply
  * (Section 4.1).
  * WS_ADAFACTOR (r == -1 only) runs three passes, as one kernel or as stages: (1) reduce the gradients, keep

@@ -42,6 +42,16 @@ struct GradPtrs {
     const void* p[N];
 };
 
+// What the finalize step of a norm pair reads and writes.
+struct OwnRatio {
+    const WsSegTiles* segtiles;
+    float* rho;
+    double* norms;
+    int* status;
+    int T, reps, lars;
+    double eta, beta;
+};
+
 struct UpdParams {
     const WsTile* tiles;
     long long ntiles;
@@ -65,6 +75,7 @@ struct UpdParams {
     int reverse;             // norm pairs, phase 2: walk the items back to front (phase 1's last items are still in L2)
     float2* partials;       // phase 1: [R][ntiles] partial sums of the two norms
     const float* rho;       // phase 2: [T] trust ratio (LAMB) / local rate (LARS)
+    OwnRatio own;           // phase 2 of a small model: every CTA forms its tensor's ratio itself (segtiles not null)
     float* ghat;            // LARS, Adafactor: [R][S] summed gradients, written by phase 1, read afterwards
     const WsSegAf* segaf;   // Adafactor: [T] matrix view of every tensor
     float* af_acc;          // Adafactor pass 1: [F] row / column sums of g^2 + eps1 (atomic adds)

@@ -31,6 +31,44 @@ namespace {
 constexpr long long kKeepReverseBytes = 256ll << 20;   // twice the L2: at least half of phase 2's re-reads can hit
 using namespace wsk;
 
+// The ratio of tensor t's norms, as both forms of the norm pairs make it.
+__device__ __forceinline__ float norm_ratio(double a, double b, int lars, double eta, double beta) {
+    if (!(a > 0.0 && b > 0.0)) return 1.0f;
+    return lars ? (float)(eta * sqrt(a) / (sqrt(b) + beta * sqrt(a))) : (float)(sqrt(a) / sqrt(b));
+}
+
+// Phase 2 of a small model does lamb_finalize_kernel's work: the CTA sums its tensor's partial norms itself (the same
+// function, the same bits); the one with the tensor's first tile stores what the finalize step stores, and the grid's
+// first one the rest.  A launch less: 3 us of the host, which is what a tiny model's three launches are bound by, against
+// 2 us more in every CTA (24 to 374 K parameters, LAMB and LARS 11.4 -> 9.1 us).
+__device__ __forceinline__ float own_ratio(const UpdParams& P, int seg, bool first, bool rest) {
+    __shared__ double sa[kBlock / 32], sb[kBlock / 32];
+    __shared__ float s_rho;
+    const OwnRatio& F = P.own;
+    double a, b;
+    __syncthreads();                                   // (an earlier item's readers are done with s_rho)
+    sum_partials(F.segtiles[seg], P.partials, P.ntiles, F.reps, sa, sb, a, b);
+    if (threadIdx.x == 0) {
+        const float rho = norm_ratio(a, b, F.lars, F.eta, F.beta);
+        s_rho = rho;
+        if (first) {
+            F.rho[seg] = rho;
+            F.norms[2 * seg] = a;
+            F.norms[2 * seg + 1] = b;
+        }
+        if (rest) *F.status = 0;
+    }
+    if (rest)
+        for (int t = threadIdx.x; t < F.T; t += kBlock)
+            if (F.segtiles[t].tile_count == 0) {       // no element, no tile
+                F.rho[t] = 1.0f;
+                F.norms[2 * t] = 0.0;
+                F.norms[2 * t + 1] = 0.0;
+            }
+    __syncthreads();
+    return s_rho;
+}
+
 // (129 and more bf16 copies: 16 of 4 elements are 32 registers, and the third CTA per SM is worth a few spills - 512
 // copies of 346 K elements, Adam 98 -> 67 us, SGD-M 95 -> 64; 64 copies of 2.8 M, SGD-M, would go from 66 to 76)
 template <int OPT, bool GBF, int RB, int NP>
@@ -91,7 +129,14 @@ __global__ void __launch_bounds__(kBlock, min_blocks<OPT, GBF, RB, NP>()) update
         // stream; everything read from here on may
         asm volatile("griddepcontrol.wait;" ::: "memory");
         float lr_rho = 0.f;
-        if (OPT == K_LAMB2 || OPT == K_LARS2) lr_rho = P.c.lr * P.rho[tl.seg];
+        if constexpr (OPT == K_LAMB2 || OPT == K_LARS2) {
+            if (P.own.segtiles) {
+                const bool first = ti == P.own.segtiles[tl.seg].tile_begin && r == (P.concat ? r : 0);
+                lr_rho = P.c.lr * own_ratio(P, tl.seg, first, item0 == 0);
+            } else {
+                lr_rho = P.c.lr * P.rho[tl.seg];
+            }
+        }
         if (OPT == K_AF3) lr_rho = P.rho[tl.seg];         // alpha_t / max(1, RMS(U_t)/d)
         process_item<OPT, GBF, OUT, VEC, U, RB, NP, FUSED, HINT>(P, gp, it, sgp, swp, wt, lr_rho, red);
     }
@@ -208,9 +253,7 @@ __global__ void __launch_bounds__(kBlock) lamb_finalize_kernel(const WsSegTiles*
         if (t == 0) *status = 0;      // (nothing waits in this form: the update is complete)
         norms[2 * t] = a;
         norms[2 * t + 1] = b;
-        if (!(a > 0.0 && b > 0.0)) rho[t] = 1.0f;
-        else if (lars) rho[t] = (float)(eta * sqrt(a) / (sqrt(b) + beta * sqrt(a)));
-        else rho[t] = (float)(sqrt(a) / sqrt(b));
+        rho[t] = norm_ratio(a, b, lars, eta, beta);
     }
 }
 
@@ -619,6 +662,7 @@ ws_status prepare(const ws_plan* p, int32_t r, const ws_grads* g, const ws_state
     P.gathered = (out_kind != O_NONE) ? out->gathered : nullptr;
     P.partials = nullptr;
     P.rho = nullptr;
+    P.own.segtiles = nullptr;
     P.ghat = nullptr;
     P.c = make_consts(h);
 #ifdef WS_DEBUG_BOUNDS
@@ -686,6 +730,28 @@ bool one_kernel(const ws_plan* p, int opt, int copies, bool gbf) {
     return p->af_scalar <= p->N / 8 || copies <= (gbf ? 16 : 32) / (p->N > (24LL << 20) ? 2 : 1);
 }
 
+// Whether phase 2 of an all-shard norm pair forms the ratios itself, in place of a finalize launch between the phases.
+// Up to two waves of CTAs, measured in work items (us, finalize launch / own ratios): LAMB, 2 bf16 copies, 0.4 M in 103
+// tensors (620 items) 16.2 / 12.4, LARS 12.3 / 9.1; 1.2 M with 1 and 3 copies (1300, 1700 items) LAMB 19.6 / 20.5, 17.8 /
+// 19.6, LARS 14.2 / 15.9, 15.2 / 18.2; 4.1 M, 1 copy, LARS 24.0 / 28.4.
+constexpr long long kOwnRatioItems = 888;
+bool forms_own_ratios(const ws_plan* p) {
+    const long long items = p->layout == WS_LAYOUT_CONCAT ? p->ntiles : p->ntiles * p->R;
+    return items >= 1 && items <= kOwnRatioItems;
+}
+void set_own_ratios(const ws_plan* p, const WsLambWs& L, const ws_hyper* h, UpdParams& P) {
+    P.partials = L.partials;
+    P.own.segtiles = p->d_segtiles;
+    P.own.rho = L.rho;
+    P.own.norms = L.norms;
+    P.own.status = L.status;
+    P.own.T = p->T;
+    P.own.reps = finalize_reps(p);
+    P.own.lars = h->opt == WS_LARS;
+    P.own.eta = h->trust_coeff;
+    P.own.beta = h->weight_decay;
+}
+
 ws_status check_ws(const ws_plan* p, void* workspace, size_t bytes, ws_opt opt = WS_LAMB) {
     if (!workspace || bytes < ws_workspace_bytes(p, opt)) return WS_ERR_WORKSPACE;
     if (!ws_aligned16(workspace)) return WS_ERR_ALIGNMENT;
@@ -738,6 +804,20 @@ extern "C" ws_status ws_lamb_apply(const ws_plan* plan, int32_t r, const ws_stat
     if ((s = check_ws(plan, workspace, workspace_bytes)) != WS_OK) return s;
     P.rho = ws_lamb_layout(plan, workspace).rho;
     return launch_any(K_LAMB2, false, ok, P, nullptr, (cudaStream_t)stream);
+}
+
+// Phase 2 of all shards on packed buffers, with the ratios formed by its CTAs.
+static ws_status apply_with_ratios(const ws_plan* plan, int phase, const ws_state* state, const ws_hyper* hyper, const ws_out* out,
+                                   void* workspace, cudaStream_t st) {
+    UpdParams P;
+    int ok;
+    bool gbf;
+    const ws_status s = prepare(plan, -1, nullptr, state, hyper, out, phase, P, ok, gbf);
+    if (s != WS_OK) return s;
+    const WsLambWs L = ws_lamb_layout(plan, workspace);
+    if (phase == K_LARS2) P.ghat = L.ghat;
+    set_own_ratios(plan, L, hyper, P);
+    return launch_any(phase, false, ok, P, nullptr, st);
 }
 
 extern "C" ws_status ws_lars_partial(const ws_plan* plan, int32_t r, const ws_grads* grads, const ws_state* state,
@@ -898,6 +978,7 @@ extern "C" ws_status ws_shard_update(const ws_plan* plan, int32_t r, const ws_gr
         s = try_one_launch(plan, 0, grads, nullptr, state, hyper, out, nullptr, workspace, workspace_bytes, (cudaStream_t)stream, done);
         if (s != WS_OK || done) return s;
         if ((s = ws_lamb_partial(plan, -1, grads, state, hyper, workspace, workspace_bytes, stream)) != WS_OK) return s;
+        if (forms_own_ratios(plan)) return apply_with_ratios(plan, K_LAMB2, state, hyper, out, workspace, (cudaStream_t)stream);
         if ((s = ws_lamb_finalize(plan, workspace, workspace_bytes, stream)) != WS_OK) return s;
         return ws_lamb_apply(plan, -1, state, hyper, out, workspace, workspace_bytes, stream);
     }
@@ -912,6 +993,7 @@ extern "C" ws_status ws_shard_update(const ws_plan* plan, int32_t r, const ws_gr
         s = try_one_launch(plan, 1, grads, nullptr, state, hyper, out, nullptr, workspace, workspace_bytes, (cudaStream_t)stream, done);
         if (s != WS_OK || done) return s;
         if ((s = ws_lars_partial(plan, -1, grads, state, hyper, workspace, workspace_bytes, stream)) != WS_OK) return s;
+        if (forms_own_ratios(plan)) return apply_with_ratios(plan, K_LARS2, state, hyper, out, workspace, (cudaStream_t)stream);
         if ((s = ws_lars_finalize(plan, hyper, workspace, workspace_bytes, stream)) != WS_OK) return s;
         return ws_lars_apply(plan, -1, state, hyper, out, workspace, workspace_bytes, stream);
     }
@@ -996,6 +1078,7 @@ ws_status fused_phase(const ws_plan* plan, int32_t r, const ws_tensor_table* gra
         P.partials = L.partials;
         P.rho = L.rho;
         P.ghat = L.ghat;
+        if ((phase == K_LAMB2 || phase == K_LARS2) && forms_own_ratios(plan)) set_own_ratios(plan, L, hyper, P);
         if (is_af(phase)) {
             P.af_acc = L.acc;
             P.af_fac = L.fac;
@@ -1223,7 +1306,7 @@ extern "C" ws_status ws_fused_update(const ws_plan* plan, int32_t r, const ws_te
         s = try_one_launch(plan, 0, nullptr, grads, state, hyper, nullptr, weights, workspace, workspace_bytes, st, done);
         if (s != WS_OK || done) return s;
         if ((s = fused_phase(plan, -1, grads, state, hyper, weights, K_LAMB1, workspace, st)) != WS_OK) return s;
-        if ((s = ws_lamb_finalize(plan, workspace, workspace_bytes, stream)) != WS_OK) return s;
+        if (!forms_own_ratios(plan) && (s = ws_lamb_finalize(plan, workspace, workspace_bytes, stream)) != WS_OK) return s;
         return fused_phase(plan, -1, grads, state, hyper, weights, K_LAMB2, workspace, st);
     }
     if (hyper->opt == WS_LARS) {
@@ -1234,10 +1317,12 @@ extern "C" ws_status ws_fused_update(const ws_plan* plan, int32_t r, const ws_te
         s = try_one_launch(plan, 1, nullptr, grads, state, hyper, nullptr, weights, workspace, workspace_bytes, st, done);
         if (s != WS_OK || done) return s;
         if ((s = fused_phase(plan, -1, grads, state, hyper, weights, K_LARS1, workspace, st)) != WS_OK) return s;
-        const WsLambWs L = ws_lamb_layout(plan, workspace);
-        launch_lamb_finalize(plan->T, st, plan->d_segtiles, L.partials, plan->ntiles, finalize_reps(plan), L.rho,
-                                                        L.norms, 1, hyper->trust_coeff, hyper->weight_decay, L.status);
-        if ((s = ws_check_launch("ws_fused_update(LARS finalize)")) != WS_OK) return s;
+        if (!forms_own_ratios(plan)) {
+            const WsLambWs L = ws_lamb_layout(plan, workspace);
+            launch_lamb_finalize(plan->T, st, plan->d_segtiles, L.partials, plan->ntiles, finalize_reps(plan), L.rho, L.norms, 1,
+                                 hyper->trust_coeff, hyper->weight_decay, L.status);
+            if ((s = ws_check_launch("ws_fused_update(LARS finalize)")) != WS_OK) return s;
+        }
         return fused_phase(plan, -1, grads, state, hyper, weights, K_LARS2, workspace, st);
     }
     if (hyper->opt != WS_SGDM && hyper->opt != WS_ADAM) return WS_ERR_INVALID_ARG;
