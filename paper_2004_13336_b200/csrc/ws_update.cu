@@ -148,8 +148,8 @@ __global__ void __launch_bounds__(kBlock, min_blocks<OPT, GBF, RB, NP>()) update
 // those waits, one to eight in a row; beyond, DRAM pages of 512 bytes a copy and CTA.  Adam, us, one thread per element /
 // this, slices of one shard: 512 copies of 22 K elements fp32 32 / 10, bf16 40 / 10, of 87 K 41 / 37, 45 / 20; 1024
 // copies of 11 K 61 / 13, 76 / 16, of 43 K 74 / 40, 86 / 19 (10 us of each are the host's).
-template <int OPT, bool GBF, int OUT>
-__global__ void __launch_bounds__(kBlock, kMinBlocksWide) split_kernel(const UpdParams P, const __grid_constant__ GradPtrs<1024> gp, int nsub) {
+template <int OPT, bool GBF, int OUT, int NP>
+__global__ void __launch_bounds__(kBlock, kMinBlocksWide) split_kernel(const UpdParams P, const __grid_constant__ GradPtrs<NP> gp, int nsub) {
     constexpr int VEC = GBF ? 8 : 4, E = 32 * VEC, RB = kTreeBlockLarge;
     static_assert(kBlock / 32 == kManyGroups, "a warp per group");
     __shared__ float2 part[kManyGroups][E];             // a group's sum and its compensation
@@ -463,6 +463,14 @@ ws_status launch(const UpdParams& P, const void* const* gptrs, cudaStream_t st) 
     return ws_check_launch(FUSED ? "ws_fused_update" : "ws_shard_update");
 }
 
+template <int OPT, bool GBF, int OUT, int NP>
+ws_status launch_split(const UpdParams& P, const void* const* gptrs, int nsub, cudaStream_t st) {
+    GradPtrs<NP> gp;
+    for (int k = 0; k < NP; ++k) gp.p[k] = k < P.R ? gptrs[k] : nullptr;
+    launch_pdl(split_kernel<OPT, GBF, OUT, NP>, P.nitems * nsub, st, P, gp, nsub);
+    return ws_check_launch("ws_shard_update");
+}
+
 // Elements of a launch up to which split_kernel is the faster one.  One thread per element costs about 1.2 us for every
 // 16 copies whatever the size, the split kernel half of the copy bandwidth once the chip is full.  us, one thread / split:
 // fp32, 128 copies of 88 K 9.7 / 12.6; 200 of 56 K 14.4 / 12.4, of 223 K 34 / 45; 512 of 87 K 41 / 37, of 162 K 53 / 65;
@@ -505,10 +513,8 @@ ws_status launch_r(const UpdParams& P, const void* const* gptrs, bool wide_ok, c
                 // (full tiles far longer than the average would leave most of the grid empty)
                 const int nsub = (P.tile_max + (GBF ? 255 : 127)) / (GBF ? 256 : 128);
                 if (P.nitems >= 1 && P.nitems * P.tile <= split_elems(GBF, P.R) && P.nitems * nsub <= 65536) {
-                    GradPtrs<1024> gp;
-                    for (int k = 0; k < 1024; ++k) gp.p[k] = k < P.R ? gptrs[k] : nullptr;
-                    launch_pdl(split_kernel<OPT, GBF, OUT>, P.nitems * nsub, st, P, gp, nsub);
-                    return ws_check_launch("ws_shard_update");
+                    if (P.R <= 128) return launch_split<OPT, GBF, OUT, 128>(P, gptrs, nsub, st);
+                    return launch_split<OPT, GBF, OUT, 1024>(P, gptrs, nsub, st);
                 }
             }
             if constexpr (OPT == K_SGDM || OPT == K_ADAM)
