@@ -10,6 +10,7 @@ from __future__ import annotations
 import ctypes as C
 import os
 import struct
+from array import array
 from typing import List, Optional, Sequence
 
 import torch
@@ -277,6 +278,7 @@ class PtrList:
     def __init__(self, tensors: Sequence[torch.Tensor]):
         self.tensors = list(tensors)
         self.arr = _ptr_array(self.tensors)
+        self.addr = C.addressof(self.arr)
         self.dtype = self.tensors[0].dtype if self.tensors else torch.float32
 
     def __len__(self):
@@ -293,6 +295,16 @@ def _ptr_array(tensors):
     for i, t in enumerate(tensors):
         arr[i] = t.data_ptr()
     return arr
+
+
+def _ptr_table(tensors):
+    """(address of the tensors' pointers, their owner) for the plain-address prototypes."""
+    if type(tensors) is PtrList:
+        return tensors.addr, tensors
+    if isinstance(tensors, PtrList):
+        return C.addressof(tensors.arr), tensors
+    own = array("Q", [t.data_ptr() for t in tensors] or (0,))
+    return own.buffer_info()[0], own
 
 
 _HYPER = struct.Struct("@i4x7dq4d")          # ws_hyper as the C compiler lays it out
@@ -430,15 +442,15 @@ class Plan:
 
 
 def ws_pack(plan: Plan, tensors: Sequence[torch.Tensor], flat: torch.Tensor):
-    dt = _dtype_code(flat.dtype)
-    st = _step().ws_pack(plan.handle, _ptr_array(tensors), dt, flat.data_ptr(), _stream())
+    addr, own = _ptr_table(tensors)
+    st = _step().ws_pack(plan._h, addr, _dtype_code(flat.dtype), flat.data_ptr(), _stream())
     if st:
         raise WsError(st, "ws_pack")
 
 
 def ws_unpack(plan: Plan, flat: torch.Tensor, tensors: Sequence[torch.Tensor]):
-    dt = _dtype_code(flat.dtype)
-    st = _step().ws_unpack(plan.handle, flat.data_ptr(), dt, _ptr_array(tensors), _stream())
+    addr, own = _ptr_table(tensors)
+    st = _step().ws_unpack(plan._h, flat.data_ptr(), _dtype_code(flat.dtype), addr, _stream())
     if st:
         raise WsError(st, "ws_unpack")
 
@@ -455,10 +467,11 @@ def _state(w, m, v):
                     v.data_ptr() if v is not None else None)
 
 
-# ws_state and ws_out as the C compiler lays them out; a bytes object is passed by its address
+# ws_grads, ws_state and ws_out as the C compiler lays them out; a bytes object is passed by its address
+_GRADS = struct.Struct("@Piii4x")
 _STATE = struct.Struct("@PPP")
 _OUT = struct.Struct("@Pi4x")
-assert _STATE.size == C.sizeof(ws_state) and _OUT.size == C.sizeof(ws_out)
+assert _GRADS.size == C.sizeof(ws_grads) and _STATE.size == C.sizeof(ws_state) and _OUT.size == C.sizeof(ws_out)
 
 
 def _refuse(x, cls):
@@ -485,12 +498,12 @@ def ws_shard_update(plan: Plan, r: int, gbufs: Sequence[torch.Tensor], w, m, v, 
                     slice_mode: int = 0):
     if type(hyper) is not ws_hyper:
         _refuse(hyper, ws_hyper)
-    g = _grads(gbufs, slice_mode)
+    addr, own = _ptr_table(gbufs)
     st = _step().ws_shard_update(
-        plan.handle, r, C.addressof(g), _state_bytes(w, m, v), C.addressof(hyper),
+        plan._h, r, _GRADS.pack(addr, len(gbufs), _dtype_code(gbufs[0].dtype), slice_mode), _state_bytes(w, m, v), C.addressof(hyper),
         _OUT.pack(gathered.data_ptr(), _dtype_code(gathered.dtype)) if gathered is not None else None,
         workspace.data_ptr() if workspace is not None else None,
-        workspace.numel() * workspace.element_size() if workspace is not None else 0, _stream())
+        workspace.nbytes if workspace is not None else 0, _stream())
     if st:
         raise WsError(st, "ws_shard_update")
 
@@ -638,9 +651,9 @@ def ws_fused_update(plan: Plan, r: int, grads: TensorTable, w, m, v, hyper: ws_h
         for x, cls in ((gc, ws_tensor_table), (hyper, ws_hyper), (wc, ws_tensor_table)):
             _refuse(x, cls)
     st = _step().ws_fused_update(
-        plan.handle, r, C.addressof(gc), _state_bytes(w, m, v), C.addressof(hyper), C.addressof(wc),
+        plan._h, r, C.addressof(gc), _state_bytes(w, m, v), C.addressof(hyper), C.addressof(wc),
         workspace.data_ptr() if workspace is not None else None,
-        workspace.numel() * workspace.element_size() if workspace is not None else 0, _stream())
+        workspace.nbytes if workspace is not None else 0, _stream())
     if st:
         raise WsError(st, "ws_fused_update")
 
@@ -649,6 +662,7 @@ def ws_pack_sets(plan: Plan, table: TensorTable, flats):
     """All sets of a tensor table packed in one launch (set k -> flats[k])."""
     if type(table.c) is not ws_tensor_table:
         _refuse(table.c, ws_tensor_table)
-    st = _step().ws_pack_sets(plan.handle, C.addressof(table.c), _ptr_array(flats), _stream())
+    addr, own = _ptr_table(flats)
+    st = _step().ws_pack_sets(plan._h, C.addressof(table.c), addr, _stream())
     if st:
         raise WsError(st, "ws_pack_sets")
