@@ -89,14 +89,20 @@ static void launch_pdl(void (*kernel)(KArgs...), long long grid, int block, cuda
     cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
 }
 
+// A model of many small tensors cut into many shards has tiles of 32 to a few hundred elements, and the launch of a CTA
+// takes longer than one of them.  SHORT: a warp per tile, kShortBlock threads a CTA.
+constexpr int kShortBlock = 128;
+
 // EB = element bytes (4 or 2); PACK = true: tensors -> flat, false: flat -> tensors; VB = vector bytes
-template <int EB, bool PACK, int VB, int NP>
+template <int EB, bool PACK, int VB, int NP, bool SHORT>
 __global__ void __launch_bounds__(kBlock) pack_kernel(PackParams P, const __grid_constant__ PtrChunk<NP> tab,
                                                       char* __restrict__ flat) {
     constexpr int EPV = VB / EB;  // elements per vector
     // the next kernel of the stream may start its prologue while this grid's last CTAs run
     asm volatile("griddepcontrol.launch_dependents;");
-    for (long long item = blockIdx.x; item < P.nitems; item += gridDim.x) {
+    const long long item0 = SHORT ? (long long)blockIdx.x * (kShortBlock / 32) + (threadIdx.x >> 5) : blockIdx.x;
+    const int first = SHORT ? threadIdx.x & 31 : threadIdx.x, step = SHORT ? 32 : blockDim.x;
+    for (long long item = item0; item < P.nitems; item += (long long)gridDim.x * (SHORT ? kShortBlock / 32 : 1)) {
         long long r = P.concat ? 0 : item / P.ntl;
         const WsTile tl = P.tiles[P.tile_lo + (item - r * P.ntl)];
         if (P.concat) r = tl.shard;
@@ -108,7 +114,7 @@ __global__ void __launch_bounds__(kBlock) pack_kernel(PackParams P, const __grid
         nv = nv < 0 ? 0 : (nv > tl.len ? (long long)tl.len : nv);
 #ifdef WS_DEBUG_BOUNDS
         if (r * P.S + tl.pos < 0 || r * P.S + tl.pos + tl.len > P.flat_elems) {
-            if (threadIdx.x == 0 && P.bounds) atomicOr(P.bounds, (unsigned)WS_BOUNDS_FLAT);
+            if (first == 0 && P.bounds) atomicOr(P.bounds, (unsigned)WS_BOUNDS_FLAT);
             continue;
         }
 #endif
@@ -116,7 +122,7 @@ __global__ void __launch_bounds__(kBlock) pack_kernel(PackParams P, const __grid
         char* tn = tensor + src0 * EB;
         const int nvec = tl.len / EPV;
 #pragma unroll 4
-        for (int i = threadIdx.x; i < nvec; i += blockDim.x) {
+        for (int i = first; i < nvec; i += step) {
             const long long e0 = (long long)i * EPV;
             if (e0 + EPV <= nv) {
                 if (PACK) st_stream<VB>(fl + (long long)i * VB, ld_stream<VB>(tn + (long long)i * VB));
@@ -148,13 +154,15 @@ __global__ void __launch_bounds__(kBlock) pack_kernel(PackParams P, const __grid
 
 // All gradient lists of a step in one launch: set k's tensors (found through the device table
 // [T][nsets]) go to flats.p[k].  Work items are set-major, so each set is walked front to back.
-template <int EB, int VB, int NP>
+template <int EB, int VB, int NP, bool SHORT>
 __global__ void __launch_bounds__(kBlock) pack_sets_kernel(PackParams P, const void* const* __restrict__ table, int nsets,
                                                            const __grid_constant__ PtrChunk<NP> flats) {
     constexpr int EPV = VB / EB;
     const long long total = P.nitems * nsets;
     asm volatile("griddepcontrol.launch_dependents;");
-    for (long long gi = blockIdx.x; gi < total; gi += gridDim.x) {
+    const long long item0 = SHORT ? (long long)blockIdx.x * (kShortBlock / 32) + (threadIdx.x >> 5) : blockIdx.x;
+    const int first = SHORT ? threadIdx.x & 31 : threadIdx.x, step = SHORT ? 32 : blockDim.x;
+    for (long long gi = item0; gi < total; gi += (long long)gridDim.x * (SHORT ? kShortBlock / 32 : 1)) {
         const int k = (int)(gi / P.nitems);
         const long long item = gi - (long long)k * P.nitems;
         long long r = P.concat ? 0 : item / P.ntl;
@@ -167,14 +175,14 @@ __global__ void __launch_bounds__(kBlock) pack_sets_kernel(PackParams P, const v
         nv = nv < 0 ? 0 : (nv > tl.len ? (long long)tl.len : nv);
 #ifdef WS_DEBUG_BOUNDS
         if (r * P.S + tl.pos < 0 || r * P.S + tl.pos + tl.len > P.flat_elems) {
-            if (threadIdx.x == 0 && P.bounds) atomicOr(P.bounds, (unsigned)WS_BOUNDS_FLAT);
+            if (first == 0 && P.bounds) atomicOr(P.bounds, (unsigned)WS_BOUNDS_FLAT);
             continue;
         }
 #endif
         char* fl = (char*)flats.p[k] + (r * P.S + tl.pos) * EB;
         const int nvec = tl.len / EPV;
 #pragma unroll 4
-        for (int i = threadIdx.x; i < nvec; i += blockDim.x) {
+        for (int i = first; i < nvec; i += step) {
             const long long e0 = (long long)i * EPV;
             if (e0 + EPV <= nv) {
                 st_stream<VB>(fl + (long long)i * VB, ld_stream<VB>(tn + (long long)i * VB));
@@ -200,38 +208,61 @@ __global__ void __launch_bounds__(kBlock) pack_sets_kernel(PackParams P, const v
 // one vector behind ~100 instructions of tile bookkeeping.  Two or more vectors per thread measured
 // best (ResNet-50 set: pack of the 8 lists 0.90 -> 0.99 of the copy bandwidth with 128 threads), while
 // 8192-element tiles keep 256 threads.
-int pack_block(const ws_plan* p, int eb, int vb) {
+//
+// Short tiles (SHORT above) are those of 3 KB or less on average, from 32 CTAs per SM on; us, a CTA / a warp per
+// tile: a replica's pack, update and unpack, 64 shards, bf16, 25.6 M parameters in 161 tensors 71 / 42, 47 M in 400
+// tensors 140 / 70; pack of 8 lists, update and unpack of 1.2 M in 161 tensors fp32 35 / 28, bf16 32 / 22, of 4.1 M bf16
+// 72 / 59.  With 3.7 KB (16
+// shards of the 25.6 M) it is 43 / 45, and below 4736 tiles (4.1 M, one list) 27.7 / 29.3.
+struct PackShape {
+    bool is_short;
+    int threads;
+    long long grid;
+};
+PackShape pack_shape(const ws_plan* p, int eb, int vb, long long items) {
+    PackShape s;
+    const long long tile = p->ntiles > 0 ? (p->layout == WS_LAYOUT_CONCAT ? p->S * p->R : p->S) / p->ntiles : p->K;
+    s.is_short = items > 4736 && tile * eb <= 3072;
+    s.threads = s.is_short ? kShortBlock : 256;
     const long long vecs = (long long)p->K * eb / vb;     // vectors per full tile
-    int b = 256;
-    while (b > 64 && vecs < 2LL * b) b >>= 1;
-    return b;
+    while (!s.is_short && s.threads > 64 && vecs < 2LL * s.threads) s.threads >>= 1;
+    const int per_cta = s.is_short ? kShortBlock / 32 : 1;
+    s.grid = (items + per_cta - 1) / per_cta;
+    if (s.grid > 0x7fffffffLL) s.grid = 0x7fffffffLL;
+    return s;
 }
 
 // `n` pointers starting at tensor (set) 0 of `ptrs`, to the kernel with the smallest table that holds them.
-template <bool PACK, int NP>
-void launch_pack(int n, void* const* ptrs, bool wide, ws_dtype dtype, long long grid, int nb, cudaStream_t st, const PackParams& P, char* flat) {
+template <bool PACK, int NP, bool SHORT>
+void launch_pack(int n, void* const* ptrs, bool wide, ws_dtype dtype, const PackShape& s, cudaStream_t st, const PackParams& P, char* flat) {
     PtrChunk<NP> tab;
     for (int t = 0; t < NP; ++t) tab.p[t] = t < n ? ptrs[t] : nullptr;
     if (wide) {
-        if (dtype == WS_F32) launch_pdl(pack_kernel<4, PACK, 32, NP>, grid, nb, st, P, tab, flat);
-        else                 launch_pdl(pack_kernel<2, PACK, 32, NP>, grid, nb, st, P, tab, flat);
+        if (dtype == WS_F32) launch_pdl(pack_kernel<4, PACK, 32, NP, SHORT>, s.grid, s.threads, st, P, tab, flat);
+        else                 launch_pdl(pack_kernel<2, PACK, 32, NP, SHORT>, s.grid, s.threads, st, P, tab, flat);
     } else {
-        if (dtype == WS_F32) launch_pdl(pack_kernel<4, PACK, 16, NP>, grid, nb, st, P, tab, flat);
-        else                 launch_pdl(pack_kernel<2, PACK, 16, NP>, grid, nb, st, P, tab, flat);
+        if (dtype == WS_F32) launch_pdl(pack_kernel<4, PACK, 16, NP, SHORT>, s.grid, s.threads, st, P, tab, flat);
+        else                 launch_pdl(pack_kernel<2, PACK, 16, NP, SHORT>, s.grid, s.threads, st, P, tab, flat);
     }
 }
-template <int NP>
-void launch_sets(const ws_tensor_table* table, void* const* flats, bool wide, long long grid, int nb, cudaStream_t st, const PackParams& P) {
+template <bool PACK, bool SHORT>
+void launch_pack_n(int n, void* const* ptrs, bool wide, ws_dtype dtype, const PackShape& s, cudaStream_t st, const PackParams& P, char* flat) {
+    if (n <= 32) launch_pack<PACK, 32, SHORT>(n, ptrs, wide, dtype, s, st, P, flat);
+    else if (n <= 256) launch_pack<PACK, 256, SHORT>(n, ptrs, wide, dtype, s, st, P, flat);
+    else launch_pack<PACK, kPtrChunk, SHORT>(n, ptrs, wide, dtype, s, st, P, flat);
+}
+template <int NP, bool SHORT>
+void launch_sets(const ws_tensor_table* table, void* const* flats, bool wide, const PackShape& s, cudaStream_t st, const PackParams& P) {
     PtrChunk<NP> fp;
     const int ns = table->nsets;
     for (int k = 0; k < NP; ++k) fp.p[k] = k < ns ? flats[k] : nullptr;
     const void* const* tb = (const void* const*)table->dev;
     if (wide) {
-        if (table->dtype == WS_F32) launch_pdl(pack_sets_kernel<4, 32, NP>, grid, nb, st, P, tb, ns, fp);
-        else                        launch_pdl(pack_sets_kernel<2, 32, NP>, grid, nb, st, P, tb, ns, fp);
+        if (table->dtype == WS_F32) launch_pdl(pack_sets_kernel<4, 32, NP, SHORT>, s.grid, s.threads, st, P, tb, ns, fp);
+        else                        launch_pdl(pack_sets_kernel<2, 32, NP, SHORT>, s.grid, s.threads, st, P, tb, ns, fp);
     } else {
-        if (table->dtype == WS_F32) launch_pdl(pack_sets_kernel<4, 16, NP>, grid, nb, st, P, tb, ns, fp);
-        else                        launch_pdl(pack_sets_kernel<2, 16, NP>, grid, nb, st, P, tb, ns, fp);
+        if (table->dtype == WS_F32) launch_pdl(pack_sets_kernel<4, 16, NP, SHORT>, s.grid, s.threads, st, P, tb, ns, fp);
+        else                        launch_pdl(pack_sets_kernel<2, 16, NP, SHORT>, s.grid, s.threads, st, P, tb, ns, fp);
     }
 }
 
@@ -266,14 +297,10 @@ ws_status run(const ws_plan* p, void* const* tensor_ptrs, ws_dtype dtype, void* 
         P.bounds = ws_bounds_word();
         P.flat_elems = (long long)p->R * p->S;
 #endif
-        long long grid = P.nitems;   // one CTA per (shard, tile): the CTA scheduler walks the buffers in order
-        if (grid > 0x7fffffffLL) grid = 0x7fffffffLL;
-        if (grid < 1) continue;
-        const int nb = pack_block(p, eb, wide ? 32 : 16);
-        const int n = seg_hi - seg_lo;
-        if (n <= 32) launch_pack<PACK, 32>(n, tensor_ptrs + seg_lo, wide, dtype, grid, nb, st, P, (char*)flat);
-        else if (n <= 256) launch_pack<PACK, 256>(n, tensor_ptrs + seg_lo, wide, dtype, grid, nb, st, P, (char*)flat);
-        else launch_pack<PACK, kPtrChunk>(n, tensor_ptrs + seg_lo, wide, dtype, grid, nb, st, P, (char*)flat);
+        if (P.nitems < 1) continue;
+        const PackShape shape = pack_shape(p, eb, wide ? 32 : 16, P.nitems);   // (the CTA scheduler walks the buffers in order)
+        (shape.is_short ? launch_pack_n<PACK, true> : launch_pack_n<PACK, false>)(seg_hi - seg_lo, tensor_ptrs + seg_lo, wide, dtype, shape,
+                                                                                  st, P, (char*)flat);
         ws_status s = ws_check_launch(PACK ? "ws_pack" : "ws_unpack");
         if (s != WS_OK) return s;
     }
@@ -316,15 +343,13 @@ extern "C" ws_status ws_pack_sets(const ws_plan* p, const ws_tensor_table* table
     P.bounds = ws_bounds_word();
     P.flat_elems = (long long)p->R * p->S;
 #endif
-    long long grid = P.nitems * table->nsets;
-    if (grid < 1) return WS_OK;
-    if (grid > 0x7fffffffLL) grid = 0x7fffffffLL;
+    if (P.nitems < 1) return WS_OK;
     cudaStream_t st = (cudaStream_t)stream;
     const int eb = table->dtype == WS_BF16 ? 2 : 4;
     bool wide = table->min_align >= 32 && (p->A * eb) % 32 == 0;
     for (int k = 0; k < table->nsets; ++k) wide = wide && (reinterpret_cast<uintptr_t>(flats[k]) & 31u) == 0;
-    const int nb = pack_block(p, eb, wide ? 32 : 16);
-    if (table->nsets <= 32) launch_sets<32>(table, flats, wide, grid, nb, st, P);
-    else launch_sets<kPtrChunk>(table, flats, wide, grid, nb, st, P);
+    const PackShape shape = pack_shape(p, eb, wide ? 32 : 16, P.nitems * table->nsets);
+    if (table->nsets <= 32) (shape.is_short ? launch_sets<32, true> : launch_sets<32, false>)(table, flats, wide, shape, st, P);
+    else (shape.is_short ? launch_sets<kPtrChunk, true> : launch_sets<kPtrChunk, false>)(table, flats, wide, shape, st, P);
     return ws_check_launch("ws_pack_sets");
 }
