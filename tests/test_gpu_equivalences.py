@@ -174,3 +174,52 @@ def test_many_copies_one_thread_or_a_group_per_warp(R, opt, gdtype, layout):
             # a tree of 16 has 4 levels, each at most 2^-24 of its partial sums, which 16 sum |g| / R bound
             bound = 6 * 2.0 ** -24 * sum(gk[t].double().abs() for gk in g)
             assert bool(((got - exact).abs() <= bound).all())
+
+
+@pytest.mark.parametrize("gdtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("R,shift", [(3, 0), (8, 8), (12, 0), (16, 8), (32, 0)])
+def test_many_short_tiles(R, gdtype, shift):
+    # 700 tensors of 0 to 900 elements cut into R shards: pieces of 8 to a few hundred elements, where pack and unpack
+    # give a warp to a tile and an update has CTAs of 64 threads; tensors 32 bytes aligned, or 16 (`shift`)
+    rng = np.random.default_rng(R)
+    numel = [int(x) for x in rng.integers(0, 900, 700)] + [1, 7, 8, 9, 1024, 2049]
+    plan = B.Plan([(n,) for n in numel], R, 8)
+    assert plan.ntiles * R > 4736 or R == 3
+    gen = torch.Generator(device=DEV).manual_seed(R)
+    views = lambda t: [t[o:o + n] for o, n in zip(offs, numel)]  # noqa: E731
+    offs, at = [], shift
+    for n in numel:
+        offs.append(at)
+        at += (n + 15) // 16 * 16 + shift
+    draw = lambda std, dt=torch.float32: (torch.randn(at + 16, generator=gen, device=DEV) * std).to(dt)  # noqa: E731
+    w, m, v, g = draw(0.02), draw(1e-3), draw(1e-5).abs(), [draw(1e-3, gdtype) for _ in range(R)]
+    segs = plan.segments()
+
+    def placed(t):                                  # [R][S] by the definition of the layout
+        flat = torch.zeros(R, plan.S, dtype=t.dtype, device=DEV)
+        for s, o, n in zip(segs, offs, numel):
+            if n:
+                full = torch.zeros(R * s.piece, dtype=t.dtype, device=DEV)
+                full[:n] = t[o:o + n]
+                flat[:, s.shard_off:s.shard_off + s.piece] = full.view(R, s.piece)
+        return flat.view(-1)
+
+    state = []
+    for t in (w, m, v):
+        flat = torch.full((plan.G,), float("nan"), device=DEV)
+        B.ws_pack(plan, views(t), flat)
+        assert torch.equal(flat, placed(t))
+        state.append(flat)
+    packed = [torch.full((plan.G,), float("nan"), dtype=gdtype, device=DEV) for _ in range(R)]
+    table = B.TensorTable(plan, [views(t) for t in g])
+    B.ws_pack_sets(plan, table, packed)
+    assert all(torch.equal(a, placed(b)) for a, b in zip(packed, g))
+    hy = B.make_hyper("adam", dict(lr=1e-3, beta1=0.9, beta2=0.999, eps=1e-8, weight_decay=0.0, momentum=0.0, grad_scale=1.0, step=10))
+    master = w.clone()
+    pm, pv = state[1].clone(), state[2].clone()
+    B.ws_fused_update(plan, -1, table, None, pm, pv, hy, B.TensorTable(plan, [views(master)]))
+    B.ws_shard_update(plan, -1, packed, *state, hy)
+    back = torch.zeros_like(w)
+    B.ws_unpack(plan, state[0], views(back))
+    assert torch.equal(state[1], pm) and torch.equal(state[2], pv)
+    assert all(torch.equal(a, b) for a, b in zip(views(master), views(back)))
