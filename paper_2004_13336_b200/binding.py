@@ -443,14 +443,14 @@ class Plan:
 
 def ws_pack(plan: Plan, tensors: Sequence[torch.Tensor], flat: torch.Tensor):
     addr, own = _ptr_table(tensors)
-    st = _step().ws_pack(plan._h, addr, _dtype_code(flat.dtype), flat.data_ptr(), _stream())
+    st = _step().ws_pack(plan.handle, addr, _dtype_code(flat.dtype), flat.data_ptr(), _stream())
     if st:
         raise WsError(st, "ws_pack")
 
 
 def ws_unpack(plan: Plan, flat: torch.Tensor, tensors: Sequence[torch.Tensor]):
     addr, own = _ptr_table(tensors)
-    st = _step().ws_unpack(plan._h, flat.data_ptr(), _dtype_code(flat.dtype), addr, _stream())
+    st = _step().ws_unpack(plan.handle, flat.data_ptr(), _dtype_code(flat.dtype), addr, _stream())
     if st:
         raise WsError(st, "ws_unpack")
 
@@ -500,7 +500,7 @@ def ws_shard_update(plan: Plan, r: int, gbufs: Sequence[torch.Tensor], w, m, v, 
         _refuse(hyper, ws_hyper)
     addr, own = _ptr_table(gbufs)
     st = _step().ws_shard_update(
-        plan._h, r, _GRADS.pack(addr, len(gbufs), _dtype_code(gbufs[0].dtype), slice_mode), _state_bytes(w, m, v), C.addressof(hyper),
+        plan.handle, r, _GRADS.pack(addr, len(gbufs), _dtype_code(gbufs[0].dtype), slice_mode), _state_bytes(w, m, v), C.addressof(hyper),
         _OUT.pack(gathered.data_ptr(), _dtype_code(gathered.dtype)) if gathered is not None else None,
         workspace.data_ptr() if workspace is not None else None,
         workspace.nbytes if workspace is not None else 0, _stream())
@@ -651,7 +651,7 @@ def ws_fused_update(plan: Plan, r: int, grads: TensorTable, w, m, v, hyper: ws_h
         for x, cls in ((gc, ws_tensor_table), (hyper, ws_hyper), (wc, ws_tensor_table)):
             _refuse(x, cls)
     st = _step().ws_fused_update(
-        plan._h, r, C.addressof(gc), _state_bytes(w, m, v), C.addressof(hyper), C.addressof(wc),
+        plan.handle, r, C.addressof(gc), _state_bytes(w, m, v), C.addressof(hyper), C.addressof(wc),
         workspace.data_ptr() if workspace is not None else None,
         workspace.nbytes if workspace is not None else 0, _stream())
     if st:
@@ -663,6 +663,6 @@ def ws_pack_sets(plan: Plan, table: TensorTable, flats):
     if type(table.c) is not ws_tensor_table:
         _refuse(table.c, ws_tensor_table)
     addr, own = _ptr_table(flats)
-    st = _step().ws_pack_sets(plan._h, C.addressof(table.c), addr, _stream())
+    st = _step().ws_pack_sets(plan.handle, C.addressof(table.c), addr, _stream())
     if st:
         raise WsError(st, "ws_pack_sets")

@@ -190,6 +190,34 @@ def test_step_calls_refuse_another_struct():
         B.ws_pack_sets(plan, Other, B.PtrList([torch.zeros(1)]))
 
 
+def _host_call(monkeypatch):
+    """A host plan and operands of a step call that reaches the library and ends there with status 5 (not uploaded)."""
+    monkeypatch.setattr(B, "_stream", lambda: 0)
+    plan = B.Plan([(64,)], 2, 8, upload=False)
+    flat = torch.zeros(plan.G + 8)
+    flat = flat[(-flat.data_ptr() // 4) % 4:][:plan.G]
+    hy = B.make_hyper("adam", W.tiny().hyper)
+    calls = [lambda p, l: B.ws_pack(p, l, flat), lambda p, l: B.ws_unpack(p, flat, l),
+             lambda p, l, mode=1: B.ws_shard_update(p, 0, l, flat, flat, flat, hy, slice_mode=mode)]
+    return plan, [torch.zeros(72)], calls
+
+
+def _status(call, *args, **kw):
+    with pytest.raises(B.WsError) as e:
+        call(*args, **kw)
+    return e.value.status
+
+
+def test_step_calls_take_any_object_with_the_plan_handle(monkeypatch):
+    plan, x, calls = _host_call(monkeypatch)
+
+    class Handle:
+        handle = plan.handle
+
+    for call in calls:
+        assert _status(call, plan, x) == _status(call, Handle, x) == 5
+
+
 def test_make_hyper_takes_what_ctypes_takes():
     base = dict(lr=1, beta1=0.9, beta2=np.float32(0.5), eps=1e-8, weight_decay=torch.tensor(0.25), momentum=0,
                 grad_scale=1, step=np.int64(7), trust_coeff="0.5", decay_exponent="0.75")
