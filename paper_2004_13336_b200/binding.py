@@ -303,7 +303,8 @@ def _ptr_table(tensors):
         return tensors.addr, tensors
     if isinstance(tensors, PtrList):
         return C.addressof(tensors.arr), tensors
-    own = array("Q", [t.data_ptr() for t in tensors] or (0,))
+    # (a list and no iterator: the tensors of one may be gone when the call reads their pointers)
+    own = array("Q", [t.data_ptr() for t in tensors] if len(tensors) else (0,))
     return own.buffer_info()[0], own
 
 

@@ -218,6 +218,14 @@ def test_step_calls_take_any_object_with_the_plan_handle(monkeypatch):
         assert _status(call, plan, x) == _status(call, Handle, x) == 5
 
 
+def test_step_calls_refuse_an_iterator(monkeypatch):
+    # its tensors would be gone when the library reads their addresses
+    plan, x, calls = _host_call(monkeypatch)
+    for call in calls:
+        with pytest.raises(TypeError):
+            call(plan, (t for t in x))
+
+
 def test_make_hyper_takes_what_ctypes_takes():
     base = dict(lr=1, beta1=0.9, beta2=np.float32(0.5), eps=1e-8, weight_decay=torch.tensor(0.25), momentum=0,
                 grad_scale=1, step=np.int64(7), trust_coeff="0.5", decay_exponent="0.75")
