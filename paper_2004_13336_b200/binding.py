@@ -499,9 +499,14 @@ def ws_shard_update(plan: Plan, r: int, gbufs: Sequence[torch.Tensor], w, m, v, 
                     slice_mode: int = 0):
     if type(hyper) is not ws_hyper:
         _refuse(hyper, ws_hyper)
-    addr, own = _ptr_table(gbufs)
+    if type(slice_mode) is int and 0 <= slice_mode <= 1:
+        addr, own = _ptr_table(gbufs)
+        g = _GRADS.pack(addr, len(gbufs), _dtype_code(gbufs[0].dtype), slice_mode)
+    else:                        # by ctypes' rules
+        own = _grads(gbufs, slice_mode)
+        g = C.addressof(own)
     st = _step().ws_shard_update(
-        plan.handle, r, _GRADS.pack(addr, len(gbufs), _dtype_code(gbufs[0].dtype), slice_mode), _state_bytes(w, m, v), C.addressof(hyper),
+        plan.handle, r, g, _state_bytes(w, m, v), C.addressof(hyper),
         _OUT.pack(gathered.data_ptr(), _dtype_code(gathered.dtype)) if gathered is not None else None,
         workspace.data_ptr() if workspace is not None else None,
         workspace.nbytes if workspace is not None else 0, _stream())

@@ -226,6 +226,15 @@ def test_step_calls_refuse_an_iterator(monkeypatch):
             call(plan, (t for t in x))
 
 
+def test_slice_mode_by_ctypes_rules(monkeypatch):
+    plan, x, calls = _host_call(monkeypatch)
+    for mode in (None, 1.0, "1"):
+        with pytest.raises(TypeError):
+            calls[2](plan, x, mode=mode)
+    for mode in (0, 1, True, np.int64(1), 2 ** 32, -2 ** 32 + 1):       # a ctypes integer wraps
+        assert _status(calls[2], plan, x, mode=mode) == 5
+
+
 def test_make_hyper_takes_what_ctypes_takes():
     base = dict(lr=1, beta1=0.9, beta2=np.float32(0.5), eps=1e-8, weight_decay=torch.tensor(0.25), momentum=0,
                 grad_scale=1, step=np.int64(7), trust_coeff="0.5", decay_exponent="0.75")
