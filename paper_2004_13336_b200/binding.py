@@ -278,7 +278,6 @@ class PtrList:
     def __init__(self, tensors: Sequence[torch.Tensor]):
         self.tensors = list(tensors)
         self.arr = _ptr_array(self.tensors)
-        self.addr = C.addressof(self.arr)
         self.dtype = self.tensors[0].dtype if self.tensors else torch.float32
 
     def __len__(self):
@@ -299,10 +298,8 @@ def _ptr_array(tensors):
 
 def _ptr_table(tensors):
     """(address of the tensors' pointers, their owner) for the plain-address prototypes."""
-    if type(tensors) is PtrList:
-        return tensors.addr, tensors
     if isinstance(tensors, PtrList):
-        return C.addressof(tensors.arr), tensors
+        return C.addressof(tensors.arr), tensors.arr
     # (a list and no iterator: the tensors of one may be gone when the call reads their pointers)
     own = array("Q", [t.data_ptr() for t in tensors] if len(tensors) else (0,))
     return own.buffer_info()[0], own

@@ -235,6 +235,13 @@ def test_slice_mode_by_ctypes_rules(monkeypatch):
         assert _status(calls[2], plan, x, mode=mode) == 5
 
 
+def test_pointer_list_follows_its_array(monkeypatch):
+    lst, other = B.PtrList([torch.zeros(8)]), [torch.zeros(8)]
+    lst.arr = B._ptr_array(other)
+    addr, own = B._ptr_table(lst)
+    assert addr == C.addressof(lst.arr) and C.cast(addr, C.POINTER(C.c_uint64))[0] == other[0].data_ptr()
+
+
 def test_make_hyper_takes_what_ctypes_takes():
     base = dict(lr=1, beta1=0.9, beta2=np.float32(0.5), eps=1e-8, weight_decay=torch.tensor(0.25), momentum=0,
                 grad_scale=1, step=np.int64(7), trust_coeff="0.5", decay_exponent="0.75")
