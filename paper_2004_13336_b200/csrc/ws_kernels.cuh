@@ -281,10 +281,12 @@ constexpr int kManyGroups = 8;
 __host__ __device__ constexpr int many_blocks_per_group(int copies) {
     return ((copies + kTreeBlockLarge - 1) / kTreeBlockLarge + kManyGroups - 1) / kManyGroups;
 }
-// Adds a group of several blocks, (s, c), to the groups before it.
+// Adds a group of several blocks, (s, c), to the groups before it.  A sum that became infinite with this group has no
+// compensation to add (c is then a difference of infinities): an infinite copy in the last block leaves +-inf, as it
+// does with 9 to 128 copies, and in an earlier block NaN or the infinity.
 __device__ __forceinline__ void add_group(float& sum, float& comp, float s, float c) {
     kahan1(sum, comp, s);
-    kahan1(sum, comp, -c);
+    if (fabsf(sum) < INFINITY) kahan1(sum, comp, -c);
 }
 
 // ------------------------------------------------------------------ math ---

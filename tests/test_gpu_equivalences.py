@@ -177,6 +177,40 @@ def test_many_copies_one_thread_or_a_group_per_warp(R, opt, gdtype, layout):
 
 
 @pytest.mark.parametrize("gdtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("S,form", [(2048, "slices"), (1 << 19, "slices"), (2048, "fused")])   # a group per warp, one thread, one thread
+@pytest.mark.parametrize("R", [129, 250, 256])       # a last group of one copy, of two blocks (the last not full), of two full ones
+def test_an_infinite_copy_among_many(R, S, form, gdtype):
+    # in the last tree block it leaves the sum +-inf, elsewhere nothing finite, and no other element changes
+    plan = B.Plan([(S,)], 1, 8)
+    gen = torch.Generator(device=DEV).manual_seed(R)
+    g = [(torch.randn(S, generator=gen, device=DEV) * 1e-3).to(gdtype) for _ in range(R)]
+    hy = B.make_hyper("sgdm", dict(lr=0.0, beta1=0.9, beta2=0.999, eps=1e-8, weight_decay=0.0, momentum=0.0, grad_scale=1.0, step=1))
+
+    def summed():                                    # m' without momentum and decay is the sum
+        w, m = torch.zeros(S, device=DEV), torch.zeros(S, device=DEV)
+        if form == "slices":
+            B.ws_shard_update(plan, 0, g, w, m, None, hy, slice_mode=1)
+        else:
+            B.ws_fused_update(plan, -1, B.TensorTable(plan, [[x] for x in g]), None, m, None, hy, B.TensorTable(plan, [[w]]))
+        return m
+
+    clean = summed()
+    inf = float("inf")
+    last = (R - 1) // 16 * 16
+    placed = {3: (R - 1, inf), 4: (R - 1, -inf), 5: (last, inf), 701: (last, -inf), 900: (0, inf), 901: (40, -inf)}
+    for e, (k, x) in placed.items():
+        g[k][e] = x
+    got = summed()
+    for e, (k, x) in placed.items():
+        if k >= last:
+            assert got[e].item() == x, e
+        assert not torch.isfinite(got[e]), e
+    rest = torch.ones(S, dtype=torch.bool, device=DEV)
+    rest[list(placed)] = False
+    assert torch.isfinite(clean).all() and torch.equal(got[rest], clean[rest])
+
+
+@pytest.mark.parametrize("gdtype", [torch.float32, torch.bfloat16])
 @pytest.mark.parametrize("R,shift", [(3, 0), (8, 8), (12, 0), (16, 8), (32, 0)])
 def test_many_short_tiles(R, gdtype, shift):
     # 700 tensors of 0 to 900 elements cut into R shards: pieces of 8 to a few hundred elements, where pack and unpack
