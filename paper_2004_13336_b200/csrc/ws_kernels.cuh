@@ -42,9 +42,15 @@ struct GradPtrs {
     const void* p[N];
 };
 
-// What the finalize step of a norm pair reads and writes.
+// Phase 2 of a norm pair: the finalize step has formed the ratios ...
+struct ReadRatio {};
+// ... or every CTA forms its tensor's itself: what the finalize step reads and writes.  Kernels of their own: with both
+// in one, the sums in front of the update took the registers of the larger models' phase 2 (LARS, fp32 master: 72
+// against 52, 3 CTAs per SM against 4; 25.6 M parameters, 2 fp32 copies 167 us against 157, 3 bf16 copies 159 against 151).
 struct OwnRatio {
     const WsSegTiles* segtiles;
+    const float2* partials;
+    long long ntiles;
     float* rho;
     double* norms;
     int* status;
@@ -75,7 +81,6 @@ struct UpdParams {
     int reverse;             // norm pairs, phase 2: walk the items back to front (phase 1's last items are still in L2)
     float2* partials;       // phase 1: [R][ntiles] partial sums of the two norms
     const float* rho;       // phase 2: [T] trust ratio (LAMB) / local rate (LARS)
-    OwnRatio own;           // phase 2 of a small model: every CTA forms its tensor's ratio itself (segtiles not null)
     float* ghat;            // LARS, Adafactor: [R][S] summed gradients, written by phase 1, read afterwards
     const WsSegAf* segaf;   // Adafactor: [T] matrix view of every tensor
     float* af_acc;          // Adafactor pass 1: [F] row / column sums of g^2 + eps1 (atomic adds)

@@ -27,6 +27,8 @@
 // The k* constants below are the values measured best on a B200.
 #include "ws_kernels.cuh"
 
+#include <type_traits>
+
 namespace {
 constexpr long long kKeepReverseBytes = 256ll << 20;   // twice the L2: at least half of phase 2's re-reads can hit
 using namespace wsk;
@@ -41,13 +43,12 @@ __device__ __forceinline__ float norm_ratio(double a, double b, int lars, double
 // function, the same bits); the one with the tensor's first tile stores what the finalize step stores, and the grid's
 // first one the rest.  A launch less: 3 us of the host, which is what a tiny model's three launches are bound by, against
 // 2 us more in every CTA (24 to 374 K parameters, LAMB and LARS 11.4 -> 9.1 us).
-__device__ __forceinline__ float own_ratio(const UpdParams& P, int seg, bool first, bool rest) {
+__device__ __forceinline__ float own_ratio(const OwnRatio& F, int seg, bool first, bool rest) {
     __shared__ double sa[kBlock / 32], sb[kBlock / 32];
     __shared__ float s_rho;
-    const OwnRatio& F = P.own;
     double a, b;
     __syncthreads();                                   // (an earlier item's readers are done with s_rho)
-    sum_partials(F.segtiles[seg], P.partials, P.ntiles, F.reps, sa, sb, a, b);
+    sum_partials(F.segtiles[seg], F.partials, F.ntiles, F.reps, sa, sb, a, b);
     if (threadIdx.x == 0) {
         const float rho = norm_ratio(a, b, F.lars, F.eta, F.beta);
         s_rho = rho;
@@ -78,8 +79,9 @@ constexpr int min_blocks() {
 
 // One CTA handles one (shard, tile) work item; the grid is the item count, so the
 // hardware CTA scheduler walks the buffers front to back.
-template <int OPT, bool GBF, int OUT, int VEC, int U, int RB, int NP, bool FUSED>
-__global__ void __launch_bounds__(kBlock, min_blocks<OPT, GBF, RB, NP>()) update_kernel(const UpdParams P, const __grid_constant__ GradPtrs<NP> gp) {
+template <int OPT, bool GBF, int OUT, int VEC, int U, int RB, int NP, bool FUSED, typename RATIO>
+__global__ void __launch_bounds__(kBlock, min_blocks<OPT, GBF, RB, NP>()) update_kernel(const UpdParams P, const __grid_constant__ GradPtrs<NP> gp,
+                                                                                        const RATIO ratio) {
     constexpr bool READS_G = !is_phase2(OPT);
     constexpr bool NEEDS_WT = FUSED && (OUT != O_NONE);
     __shared__ float2 red[kBlock / 32];
@@ -130,9 +132,9 @@ __global__ void __launch_bounds__(kBlock, min_blocks<OPT, GBF, RB, NP>()) update
         asm volatile("griddepcontrol.wait;" ::: "memory");
         float lr_rho = 0.f;
         if constexpr (OPT == K_LAMB2 || OPT == K_LARS2) {
-            if (P.own.segtiles) {
-                const bool first = ti == P.own.segtiles[tl.seg].tile_begin && r == (P.concat ? r : 0);
-                lr_rho = P.c.lr * own_ratio(P, tl.seg, first, item0 == 0);
+            if constexpr (std::is_same_v<RATIO, OwnRatio>) {
+                const bool first = ti == ratio.segtiles[tl.seg].tile_begin && r == (P.concat ? r : 0);
+                lr_rho = P.c.lr * own_ratio(ratio, tl.seg, first, item0 == 0);
             } else {
                 lr_rho = P.c.lr * P.rho[tl.seg];
             }
@@ -441,8 +443,8 @@ void launch_lamb_finalize(int T, cudaStream_t st, const WsSegTiles* segtiles, co
     launch_pdl(lamb_finalize_kernel, T, st, segtiles, partials, ntiles, R, rho, norms, lars, eta, beta, status);
 }
 
-template <int OPT, bool GBF, int OUT, int VEC, int U, int RB, int NP, bool FUSED>
-ws_status launch(const UpdParams& P, const void* const* gptrs, cudaStream_t st) {
+template <int OPT, bool GBF, int OUT, int VEC, int U, int RB, int NP, bool FUSED, typename RATIO = ReadRatio>
+ws_status launch(const UpdParams& P, const void* const* gptrs, cudaStream_t st, const RATIO& ratio = {}) {
     GradPtrs<NP> gp;
     for (int k = 0; k < NP; ++k) gp.p[k] = (!FUSED && gptrs && k < P.R) ? gptrs[k] : nullptr;
     long long grid = P.nitems;
@@ -459,7 +461,7 @@ ws_status launch(const UpdParams& P, const void* const* gptrs, cudaStream_t st) 
     int threads = kBlock;
     if ((OPT == K_SGDM || OPT == K_ADAM) && NP <= 32 && P.nitems > 444)
         while (threads > 64 && P.tile <= VEC * threads / 2) threads /= 2;
-    launch_pdl_as(update_kernel<OPT, GBF, OUT, VEC, U, RB, NP, FUSED>, grid, threads, st, P, gp);
+    launch_pdl_as(update_kernel<OPT, GBF, OUT, VEC, U, RB, NP, FUSED, RATIO>, grid, threads, st, P, gp, ratio);
     return ws_check_launch(FUSED ? "ws_fused_update" : "ws_shard_update");
 }
 
@@ -486,8 +488,10 @@ long long split_elems(bool gbf, int copies) {
 // gradients are bf16 (a 128-bit gradient load then covers 8 elements) and for
 // small R, where the fp32 streams dominate.
 template <int OPT, bool GBF, int OUT, bool FUSED>
-ws_status launch_r(const UpdParams& P, const void* const* gptrs, bool wide_ok, cudaStream_t st) {
+ws_status launch_r(const UpdParams& P, const void* const* gptrs, bool wide_ok, cudaStream_t st, const OwnRatio* own) {
     if constexpr (is_phase2(OPT)) {
+        if constexpr (OPT == K_LAMB2 || OPT == K_LARS2)
+            if (own) return wide_ok ? launch<OPT, GBF, OUT, 8, 1, 1, 1, FUSED>(P, gptrs, st, *own) : launch<OPT, GBF, OUT, 4, 1, 1, 1, FUSED>(P, gptrs, st, *own);
         if (wide_ok) return launch<OPT, GBF, OUT, 8, 1, 1, 1, FUSED>(P, gptrs, st);
         return launch<OPT, GBF, OUT, 4, 1, 1, 1, FUSED>(P, gptrs, st);
     } else {
@@ -529,40 +533,41 @@ bool aligned32(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 31u) ==
 
 // `wide` on entry: whether the caller-side tensors (fused formatting) allow 256-bit accesses.
 template <int OPT, bool GBF, bool FUSED>
-ws_status launch_o(const UpdParams& P, const void* const* gptrs, int out, bool wide, cudaStream_t st) {
+ws_status launch_o(const UpdParams& P, const void* const* gptrs, int out, bool wide, cudaStream_t st, const OwnRatio* own = nullptr) {
     wide = wide && aligned32(P.w) && aligned32(P.m) && aligned32(P.v) && aligned32(P.gathered);
     if (!FUSED && !is_phase2(OPT))
         for (int k = 0; k < P.R && wide; ++k) wide = aligned32(gptrs[k]);
     if (OPT == K_LARS1 || OPT == K_LARS2 || is_af(OPT)) wide = wide && aligned32(P.ghat);
     if (OPT == K_AF1) wide = false;   // pass 1 is instruction-heavy: 128-bit vectors measured faster at every R
     if constexpr (is_phase1(OPT)) {
-        if constexpr (FUSED) if (out == O_F32M) return launch_r<OPT, GBF, O_F32M, FUSED>(P, gptrs, wide, st);
-        return launch_r<OPT, GBF, O_NONE, FUSED>(P, gptrs, wide, st);
+        if constexpr (FUSED) if (out == O_F32M) return launch_r<OPT, GBF, O_F32M, FUSED>(P, gptrs, wide, st, own);
+        return launch_r<OPT, GBF, O_NONE, FUSED>(P, gptrs, wide, st, own);
     } else {
         switch (out) {
             case O_NONE:
                 if constexpr (FUSED) return WS_ERR_INVALID_ARG;
-                else return launch_r<OPT, GBF, O_NONE, FUSED>(P, gptrs, wide, st);
-            case O_F32: return launch_r<OPT, GBF, O_F32, FUSED>(P, gptrs, wide, st);
+                else return launch_r<OPT, GBF, O_NONE, FUSED>(P, gptrs, wide, st, own);
+            case O_F32: return launch_r<OPT, GBF, O_F32, FUSED>(P, gptrs, wide, st, own);
             case O_F32M:
-                if constexpr (FUSED) return launch_r<OPT, GBF, O_F32M, FUSED>(P, gptrs, wide, st);
+                if constexpr (FUSED) return launch_r<OPT, GBF, O_F32M, FUSED>(P, gptrs, wide, st, own);
                 else return WS_ERR_INVALID_ARG;
-            default: return launch_r<OPT, GBF, O_BF16, FUSED>(P, gptrs, wide, st);
+            default: return launch_r<OPT, GBF, O_BF16, FUSED>(P, gptrs, wide, st, own);
         }
     }
 }
 
 template <bool FUSED>
-ws_status launch_f(int opt, bool gbf, int out, const UpdParams& P, const void* const* gptrs, bool wide, cudaStream_t st) {
+ws_status launch_f(int opt, bool gbf, int out, const UpdParams& P, const void* const* gptrs, bool wide, cudaStream_t st,
+                   const OwnRatio* own = nullptr) {
     switch (opt) {
         case K_SGDM: return gbf ? launch_o<K_SGDM, true, FUSED>(P, gptrs, out, wide, st) : launch_o<K_SGDM, false, FUSED>(P, gptrs, out, wide, st);
         case K_ADAM: return gbf ? launch_o<K_ADAM, true, FUSED>(P, gptrs, out, wide, st) : launch_o<K_ADAM, false, FUSED>(P, gptrs, out, wide, st);
         case K_LAMB1: return gbf ? launch_o<K_LAMB1, true, FUSED>(P, gptrs, out, wide, st) : launch_o<K_LAMB1, false, FUSED>(P, gptrs, out, wide, st);
         case K_LARS1: return gbf ? launch_o<K_LARS1, true, FUSED>(P, gptrs, out, wide, st) : launch_o<K_LARS1, false, FUSED>(P, gptrs, out, wide, st);
-        case K_LARS2: return launch_o<K_LARS2, false, FUSED>(P, gptrs, out, wide, st);
+        case K_LARS2: return launch_o<K_LARS2, false, FUSED>(P, gptrs, out, wide, st, own);
         case K_AF1: return gbf ? launch_o<K_AF1, true, FUSED>(P, gptrs, out, wide, st) : launch_o<K_AF1, false, FUSED>(P, gptrs, out, wide, st);
         case K_AF3: return launch_o<K_AF3, false, FUSED>(P, gptrs, out, wide, st);
-        default: return launch_o<K_LAMB2, false, FUSED>(P, gptrs, out, wide, st);
+        default: return launch_o<K_LAMB2, false, FUSED>(P, gptrs, out, wide, st, own);
     }
 }
 
@@ -668,7 +673,6 @@ ws_status prepare(const ws_plan* p, int32_t r, const ws_grads* g, const ws_state
     P.gathered = (out_kind != O_NONE) ? out->gathered : nullptr;
     P.partials = nullptr;
     P.rho = nullptr;
-    P.own.segtiles = nullptr;
     P.ghat = nullptr;
     P.c = make_consts(h);
 #ifdef WS_DEBUG_BOUNDS
@@ -745,17 +749,8 @@ bool forms_own_ratios(const ws_plan* p) {
     const long long items = p->layout == WS_LAYOUT_CONCAT ? p->ntiles : p->ntiles * p->R;
     return items >= 1 && items <= kOwnRatioItems;
 }
-void set_own_ratios(const ws_plan* p, const WsLambWs& L, const ws_hyper* h, UpdParams& P) {
-    P.partials = L.partials;
-    P.own.segtiles = p->d_segtiles;
-    P.own.rho = L.rho;
-    P.own.norms = L.norms;
-    P.own.status = L.status;
-    P.own.T = p->T;
-    P.own.reps = finalize_reps(p);
-    P.own.lars = h->opt == WS_LARS;
-    P.own.eta = h->trust_coeff;
-    P.own.beta = h->weight_decay;
+OwnRatio own_ratios(const ws_plan* p, const WsLambWs& L, const ws_hyper* h) {
+    return {p->d_segtiles, L.partials, p->ntiles, L.rho, L.norms, L.status, p->T, finalize_reps(p), h->opt == WS_LARS, h->trust_coeff, h->weight_decay};
 }
 
 ws_status check_ws(const ws_plan* p, void* workspace, size_t bytes, ws_opt opt = WS_LAMB) {
@@ -822,8 +817,8 @@ static ws_status apply_with_ratios(const ws_plan* plan, int phase, const ws_stat
     if (s != WS_OK) return s;
     const WsLambWs L = ws_lamb_layout(plan, workspace);
     if (phase == K_LARS2) P.ghat = L.ghat;
-    set_own_ratios(plan, L, hyper, P);
-    return launch_any(phase, false, ok, P, nullptr, st);
+    const OwnRatio own = own_ratios(plan, L, hyper);
+    return launch_f<false>(phase, false, ok, P, nullptr, true, st, &own);
 }
 
 extern "C" ws_status ws_lars_partial(const ws_plan* plan, int32_t r, const ws_grads* grads, const ws_state* state,
@@ -1084,7 +1079,10 @@ ws_status fused_phase(const ws_plan* plan, int32_t r, const ws_tensor_table* gra
         P.partials = L.partials;
         P.rho = L.rho;
         P.ghat = L.ghat;
-        if ((phase == K_LAMB2 || phase == K_LARS2) && forms_own_ratios(plan)) set_own_ratios(plan, L, hyper, P);
+        if ((phase == K_LAMB2 || phase == K_LARS2) && forms_own_ratios(plan)) {
+            const OwnRatio own = own_ratios(plan, L, hyper);
+            return launch_f<true>(phase, gbf, out_kind, P, nullptr, wide, st, &own);
+        }
         if (is_af(phase)) {
             P.af_acc = L.acc;
             P.af_fac = L.fac;

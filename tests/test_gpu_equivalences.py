@@ -210,6 +210,52 @@ def test_an_infinite_copy_among_many(R, S, form, gdtype):
     assert torch.isfinite(clean).all() and torch.equal(got[rest], clean[rest])
 
 
+@pytest.mark.parametrize("layout", ["per_tensor", "concat"])
+@pytest.mark.parametrize("opt", ["lamb", "lars"])
+@pytest.mark.parametrize("R,items", [(1, "few"), (3, "few"), (3, "many")])
+def test_ratios_formed_in_phase_two(R, items, opt, layout):
+    # small models form the ratios in phase 2 ("few"), larger ones in a launch of their own: ratios and norms (also those
+    # of a tensor without elements), state and weights are bit for bit those of the calls shard by shard
+    shapes = [(0,), (257, 33), (1,), (0, 5), (40, 1031), (64,), (0,)] + ([(700, 3000)] if items == "many" else [])
+    wl = W.Workload("f", shapes, R=R, opt=opt, hyper={}, grad_dtype=torch.float32, grad_std=1e-3, seed=R)
+    plan = B.Plan(shapes, R, 32, 1024, layout=layout, one_launch=False)
+    assert (plan.ntiles * (R if layout == "per_tensor" else 1) <= 888) == (items == "few")
+    h = dict(lr=1e-3, beta1=0.9, beta2=0.999, eps=1e-6, weight_decay=0.01, momentum=0.9, grad_scale=1.0, step=4, trust_coeff=0.001)
+    hy = B.make_hyper(opt, h)
+    w, m, v = W.make_state(wl, DEV)
+    g = W.make_grads(wl, DEV)
+
+    def packed(lst):
+        b = torch.empty(plan.G, device=DEV)
+        B.ws_pack(plan, lst, b)
+        return b
+
+    state = [packed(w), packed(m), packed(v) if opt == "lamb" else None]
+    pg = [packed(x) for x in g]
+    per = [None if x is None else x.clone() for x in state]
+    one, fused = ([None if x is None else x.clone() for x in state] for _ in range(2))
+    wsp, wso, wsf = (torch.full((plan.workspace_bytes(opt),), x, dtype=torch.uint8, device=DEV) for x in (0, 0xA5, 0x5A))
+    go, gp = (torch.zeros(plan.G, dtype=torch.bfloat16, device=DEV) for _ in range(2))
+    B.ws_shard_update(plan, -1, pg, *one, hy, go, wso)
+    cut = lambda r: [None if x is None else x[r * plan.S:(r + 1) * plan.S] for x in per]  # noqa: E731
+    for r in range(R):
+        sw, sm, sv = cut(r)
+        B.ws_lamb_partial(plan, r, pg, sw, sm, sv, hy, wsp) if opt == "lamb" else B.ws_lars_partial(plan, r, pg, sw, sm, hy, wsp)
+    B.ws_lamb_finalize(plan, wsp) if opt == "lamb" else B.ws_lars_finalize(plan, hy, wsp)
+    for r in range(R):
+        sw, sm, sv = cut(r)
+        B.ws_lamb_apply(plan, r, sw, sm, sv, hy, wsp, gp) if opt == "lamb" else B.ws_lars_apply(plan, r, sw, sm, hy, wsp, gp)
+    wt = [torch.zeros(x.numel(), device=DEV) for x in w]
+    B.ws_fused_update(plan, -1, B.TensorTable(plan, g), *fused, hy, B.TensorTable(plan, [wt]), wsf)
+    head = (4 * plan.T + 15) // 16 * 16 + 16 * plan.T           # ratios and squared norms
+    off = plan.sync_status_offset()
+    for ws, st in ((wso, one), (wsf, fused)):
+        assert torch.equal(ws[:4 * plan.T], wsp[:4 * plan.T]) and torch.equal(ws[head - 16 * plan.T:head], wsp[head - 16 * plan.T:head])
+        assert int(ws[off:off + 4].view(torch.int32).item()) == 0
+        assert all(a is None or torch.equal(a, b) for a, b in zip(st, per))
+    assert torch.equal(go, gp)
+
+
 @pytest.mark.parametrize("gdtype", [torch.float32, torch.bfloat16])
 @pytest.mark.parametrize("R,shift", [(3, 0), (8, 8), (12, 0), (16, 8), (32, 0)])
 def test_many_short_tiles(R, gdtype, shift):
