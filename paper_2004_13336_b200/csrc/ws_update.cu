@@ -154,7 +154,7 @@ template <int OPT, bool GBF, int OUT, int NP>
 __global__ void __launch_bounds__(kBlock, kMinBlocksWide) split_kernel(const UpdParams P, const __grid_constant__ GradPtrs<NP> gp, int nsub) {
     constexpr int VEC = GBF ? 8 : 4, E = 32 * VEC, RB = kTreeBlockLarge;
     static_assert(kBlock / 32 == kManyGroups, "a warp per group");
-    __shared__ float2 part[kManyGroups][E];             // a group's sum and its compensation
+    __shared__ __align__(16) float2 part[kManyGroups][E];     // a group's sum and its compensation, stored two at a time
     asm volatile("griddepcontrol.launch_dependents;");
     const unsigned item = blockIdx.x / (unsigned)nsub;
     const int e0 = (int)(blockIdx.x - item * (unsigned)nsub) * E;
