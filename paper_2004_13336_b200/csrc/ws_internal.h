@@ -132,6 +132,7 @@ struct ws_plan {
     int layout = 0;                           // ws_layout
     long long S = 0, N = 0;
     long long ntiles = 0;                     // per-tensor layout: tiles per shard; concatenated: all tiles
+    int longest = 0;                          // elements of the longest tile (at most K)
     std::vector<long long> shard_tile_begin;  // concatenated layout: [R+1] first tile of every shard
     std::vector<ws_segment> segs;
     std::vector<WsTile> tiles;

@@ -209,11 +209,12 @@ __global__ void __launch_bounds__(kBlock) pack_sets_kernel(PackParams P, const v
 // best (ResNet-50 set: pack of the 8 lists 0.90 -> 0.99 of the copy bandwidth with 128 threads), while
 // 8192-element tiles keep 256 threads.
 //
-// Short tiles (SHORT above) are those of 3 KB or less on average, from 32 CTAs per SM on; us, a CTA / a warp per
-// tile: a replica's pack, update and unpack, 64 shards, bf16, 25.6 M parameters in 161 tensors 71 / 42, 47 M in 400
-// tensors 140 / 70; pack of 8 lists, update and unpack of 1.2 M in 161 tensors fp32 35 / 28, bf16 32 / 22, of 4.1 M bf16
-// 72 / 59.  With 3.7 KB (16
-// shards of the 25.6 M) it is 43 / 45, and below 4736 tiles (4.1 M, one list) 27.7 / 29.3.
+// Short tiles (SHORT above) are those of 3 KB or less on average, from 32 CTAs per SM on.  us, a CTA / a warp per tile: a
+// replica's pack, update and unpack, 64 shards, bf16, 25.6 M parameters in 161 tensors 71 / 42, 47 M in 400 tensors 140 / 70;
+// pack of 8 lists, update and unpack of 1.2 M in 161 tensors fp32 35 / 28, bf16 32 / 22, of 4.1 M bf16 72 / 59.  With tiles
+// of 3.7 KB (16 shards of the 25.6 M) it is 43 / 45, and below 4736 tiles (4.1 M, one list) 27.7 / 29.3.  A long tile
+// (a caller's own length) may have 512 KB: the pack of 8 lists with a few such tiles among 24 000 of 32 elements takes 312 / 315,
+// with tiles of 4 MB 845 / 2179.
 struct PackShape {
     bool is_short;
     int threads;
@@ -222,7 +223,7 @@ struct PackShape {
 PackShape pack_shape(const ws_plan* p, int eb, int vb, long long items) {
     PackShape s;
     const long long tile = p->ntiles > 0 ? (p->layout == WS_LAYOUT_CONCAT ? p->S * p->R : p->S) / p->ntiles : p->K;
-    s.is_short = items > 4736 && tile * eb <= 3072;
+    s.is_short = items > 4736 && tile * eb <= 3072 && (long long)p->longest * eb <= 512 << 10;
     s.threads = s.is_short ? kShortBlock : 256;
     const long long vecs = (long long)p->K * eb / vb;     // vectors per full tile
     while (!s.is_short && s.threads > 64 && vecs < 2LL * s.threads) s.threads >>= 1;

@@ -280,6 +280,7 @@ extern "C" ws_status ws_plan_create_layout(const ws_tensor_desc* descs, int32_t 
                     if (!seen[t]) { seen[t] = 1; p->segtiles[t].tile_begin = (int)p->tiles.size(); }
                     p->segtiles[t].tile_count += 1;
                     p->tiles.push_back(tl);
+                    if (tl.len > p->longest) p->longest = tl.len;
                     pos += len;
                 }
             }
@@ -328,6 +329,7 @@ extern "C" ws_status ws_plan_create_layout(const ws_tensor_desc* descs, int32_t 
                 tl.len = (int)(len < tile_elems ? len : tile_elems);
                 tl.seg = t;
                 p->tiles.push_back(tl);
+                if (tl.len > p->longest) p->longest = tl.len;
             }
             off += piece;
         }

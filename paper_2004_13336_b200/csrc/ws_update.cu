@@ -454,13 +454,15 @@ ws_status launch(const UpdParams& P, const void* const* gptrs, cudaStream_t st, 
     // Elementwise updates take the CTA that their tiles fill: a tile of 1024 elements is 128 vectors of 8, and a model of
     // many small tensors cut into many shards has tiles of 32 to a few hundred elements.  The registers of the threads
     // without a vector then hold further CTAs, and a CTA's chain of table reads is what small models wait for.  From
-    // more than three CTAs per SM on: a small launch has room for all its CTAs, and many copies (a thread of a CTA of 64
-    // passes over a full tile 4 times) want the threads.  us, 256 threads / this rule, formatting fused in: tiles of
-    // 1024, 4.1 M parameters, SGD-M 8 bf16 copies 28.7 / 17.9, 4 copies 21.9 / 12.7, Adam 8 copies 36.2 / 24.5;
+    // more than three CTAs per SM on (a small launch has room for all its CTAs) and up to 32 copies (more want the threads).
+    // A few long tiles (a caller's own tile length) among many short ones: the fewer threads, the longer the last of them
+    // takes alone, at most 64 passes.  us, 256 threads / the average alone / this rule, Adam, 24 000 tiles of 32 elements and, of
+    // 125 K each, 8 tiles: fp32 338 / 757 / 328, bf16 494 / 528 / 264; with 16 of 16 K: fp32 184 / 136 / 136.
+    // us, 256 threads / this rule, formatting fused in: tiles of 1024, 4.1 M parameters, SGD-M 8 bf16 copies 28.7 / 17.9, 4 copies 21.9 / 12.7, Adam 8 copies 36.2 / 24.5;
     // 1.2 M parameters in 161 tensors, Adam, 16 copies fp32 27.7 / 19.6, bf16 26.4 / 15.5, 32 copies bf16 57 / 34.
     int threads = kBlock;
     if ((OPT == K_SGDM || OPT == K_ADAM) && NP <= 32 && P.nitems > 444)
-        while (threads > 64 && P.tile <= VEC * threads / 2) threads /= 2;
+        while (threads > 64 && P.tile <= VEC * threads / 2 && P.tile_max <= 32 * VEC * threads) threads /= 2;
     launch_pdl_as(update_kernel<OPT, GBF, OUT, VEC, U, RB, NP, FUSED, RATIO>, grid, threads, st, P, gp, ratio);
     return ws_check_launch(FUSED ? "ws_fused_update" : "ws_shard_update");
 }
@@ -514,7 +516,7 @@ ws_status launch_r(const UpdParams& P, const void* const* gptrs, bool wide_ok, c
         // many replicas make small shards and few CTAs: more loads in flight per thread
         if (P.R <= 1024) {
             if constexpr (!FUSED && (OPT == K_SGDM || OPT == K_ADAM)) {
-                // (full tiles far longer than the average would leave most of the grid empty)
+                // (tiles far longer than the average would leave most of the grid empty)
                 const int nsub = (P.tile_max + (GBF ? 255 : 127)) / (GBF ? 256 : 128);
                 if (P.nitems >= 1 && P.nitems * P.tile <= split_elems(GBF, P.R) && P.nitems * nsub <= 65536) {
                     if (P.R <= 128) return launch_split<OPT, GBF, OUT, 128>(P, gptrs, nsub, st);
@@ -644,7 +646,7 @@ ws_status prepare(const ws_plan* p, int32_t r, const ws_grads* g, const ws_state
     }
     P.tiles = p->d_tiles;
     P.ntiles = p->ntiles;
-    P.tile_max = p->K;
+    P.tile_max = p->longest;
     P.tile = p->ntiles > 0 ? (int)((p->layout == WS_LAYOUT_CONCAT ? p->S * p->R : p->S) / p->ntiles) : p->K;
     P.S = p->S;
     P.R = g ? g->R : p->R;

@@ -257,6 +257,33 @@ def test_ratios_formed_in_phase_two(R, items, opt, layout):
 
 
 @pytest.mark.parametrize("gdtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("tile", [1 << 15, 1 << 17, 1 << 20])
+def test_few_long_tiles_among_short_ones(tile, gdtype):
+    # the average tile is short, the longest is not: packed buffers, state and weights are those of a plan with tiles of 1024
+    numel, R = [40] * 2500 + [700_001] + [17] * 100, 2
+    got = []
+    for t in (1024, tile):
+        plan = B.Plan([(n,) for n in numel], R, 8, t)
+        gen = torch.Generator(device=DEV).manual_seed(3)
+        offs = [plan.arena_offsets()[i] for i in range(plan.T)]
+        arena = lambda std, dt=torch.float32: (torch.randn(plan.arena_elems, generator=gen, device=DEV) * std).to(dt)  # noqa: E731,B023
+        views = lambda x: [x[o:o + n] for o, n in zip(offs, numel)]  # noqa: E731,B023
+        w, g = arena(0.02), [arena(1e-3, gdtype) for _ in range(R)]
+        m, v = torch.zeros(plan.G, device=DEV), torch.zeros(plan.G, device=DEV)
+        packed = [torch.empty(plan.G, dtype=gdtype, device=DEV) for _ in range(R)]
+        table = B.TensorTable(plan, [views(x) for x in g])
+        B.ws_pack_sets(plan, table, packed)
+        hy = B.make_hyper("adam", dict(lr=1e-3, beta1=0.9, beta2=0.999, eps=1e-8, weight_decay=0.0, momentum=0.0, grad_scale=1.0, step=1))
+        B.ws_fused_update(plan, -1, table, None, m, v, hy, B.TensorTable(plan, [views(w)]))
+        flat, back = torch.empty(plan.G, device=DEV), torch.zeros_like(w)
+        B.ws_pack(plan, views(w), flat)
+        B.ws_unpack(plan, flat, views(back))
+        assert all(torch.equal(a, b) for a, b in zip(views(w), views(back)))
+        got.append([w, m, v, flat] + packed)
+    assert all(torch.equal(a, b) for a, b in zip(*got))
+
+
+@pytest.mark.parametrize("gdtype", [torch.float32, torch.bfloat16])
 @pytest.mark.parametrize("R,shift", [(3, 0), (8, 8), (12, 0), (16, 8), (32, 0)])
 def test_many_short_tiles(R, gdtype, shift):
     # 700 tensors of 0 to 900 elements cut into R shards: pieces of 8 to a few hundred elements, where pack and unpack
