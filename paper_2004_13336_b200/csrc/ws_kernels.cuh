@@ -57,6 +57,9 @@ struct OwnRatio {
     int T, reps, lars;
     double eta, beta;
 };
+// CTAS: resident CTAs per SM that its registers allow for (forms_own_ratios says why there are two)
+template <int CTAS>
+struct OwnRatioAt : OwnRatio {};
 
 struct UpdParams {
     const WsTile* tiles;
@@ -390,12 +393,13 @@ __device__ __forceinline__ void sum_block(double& a, double& b, double* sa, doub
 // per-replica reduce results with one batched scalar all-reduce, Section 4.1 / 5.2); the totals are valid in
 // thread 0.  One function for the finalize step and for the one-kernel routes, so that both give the same bits.
 // R: strided repetitions of the tensor's tile run; sa, sb: kBlock/32 doubles of shared memory each.
+// U: loads in flight per thread (no part of the order).
+template <int U = 8>
 __device__ __forceinline__ void sum_partials(const WsSegTiles st, const float2* partials, long long ntiles, int R,
                                              double* sa, double* sb, double& a, double& b) {
     const long long n = (long long)R * st.tile_count;
     a = 0.0;
     b = 0.0;
-    constexpr int U = 8;                                  // loads in flight per thread
     // partial i is tile i % tile_count of repetition i / tile_count; a thread takes every kBlock-th one
     const int tc = st.tile_count > 0 ? st.tile_count : 1, dr = kBlock / tc, dk = kBlock - dr * tc;
     int r = (int)threadIdx.x / tc, k = (int)threadIdx.x - r * tc;

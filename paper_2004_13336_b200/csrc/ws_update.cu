@@ -27,8 +27,6 @@
 // The k* constants below are the values measured best on a B200.
 #include "ws_kernels.cuh"
 
-#include <type_traits>
-
 namespace {
 constexpr long long kKeepReverseBytes = 256ll << 20;   // twice the L2: at least half of phase 2's re-reads can hit
 using namespace wsk;
@@ -43,12 +41,13 @@ __device__ __forceinline__ float norm_ratio(double a, double b, int lars, double
 // function, the same bits); the one with the tensor's first tile stores what the finalize step stores, and the grid's
 // first one the rest.  A launch less: 3 us of the host, which is what a tiny model's three launches are bound by, against
 // 2 us more in every CTA (24 to 374 K parameters, LAMB and LARS 11.4 -> 9.1 us).
+template <int U>
 __device__ __forceinline__ float own_ratio(const OwnRatio& F, int seg, bool first, bool rest) {
     __shared__ double sa[kBlock / 32], sb[kBlock / 32];
     __shared__ float s_rho;
     double a, b;
     __syncthreads();                                   // (an earlier item's readers are done with s_rho)
-    sum_partials(F.segtiles[seg], F.partials, F.ntiles, F.reps, sa, sb, a, b);
+    sum_partials<U>(F.segtiles[seg], F.partials, F.ntiles, F.reps, sa, sb, a, b);
     if (threadIdx.x == 0) {
         const float rho = norm_ratio(a, b, F.lars, F.eta, F.beta);
         s_rho = rho;
@@ -77,11 +76,15 @@ constexpr int min_blocks() {
     return RB > 8 && !(GBF && NP > 128 && (OPT == K_SGDM || OPT == K_ADAM)) ? kMinBlocksWide : kMinBlocks;
 }
 
+// Resident CTAs per SM of a phase 2 that forms its own ratios, 0 for every other kernel.
+template <typename RATIO> constexpr int own_ctas = 0;
+template <int CTAS> constexpr int own_ctas<OwnRatioAt<CTAS>> = CTAS;
+
 // One CTA handles one (shard, tile) work item; the grid is the item count, so the
 // hardware CTA scheduler walks the buffers front to back.
 template <int OPT, bool GBF, int OUT, int VEC, int U, int RB, int NP, bool FUSED, typename RATIO>
-__global__ void __launch_bounds__(kBlock, min_blocks<OPT, GBF, RB, NP>()) update_kernel(const UpdParams P, const __grid_constant__ GradPtrs<NP> gp,
-                                                                                        const RATIO ratio) {
+__global__ void __launch_bounds__(kBlock, own_ctas<RATIO> ? own_ctas<RATIO> : min_blocks<OPT, GBF, RB, NP>())
+update_kernel(const UpdParams P, const __grid_constant__ GradPtrs<NP> gp, const RATIO ratio) {
     constexpr bool READS_G = !is_phase2(OPT);
     constexpr bool NEEDS_WT = FUSED && (OUT != O_NONE);
     __shared__ float2 red[kBlock / 32];
@@ -132,9 +135,9 @@ __global__ void __launch_bounds__(kBlock, min_blocks<OPT, GBF, RB, NP>()) update
         asm volatile("griddepcontrol.wait;" ::: "memory");
         float lr_rho = 0.f;
         if constexpr (OPT == K_LAMB2 || OPT == K_LARS2) {
-            if constexpr (std::is_same_v<RATIO, OwnRatio>) {
+            if constexpr (own_ctas<RATIO> != 0) {
                 const bool first = ti == ratio.segtiles[tl.seg].tile_begin && r == (P.concat ? r : 0);
-                lr_rho = P.c.lr * own_ratio(ratio, tl.seg, first, item0 == 0);
+                lr_rho = P.c.lr * own_ratio<own_ctas<RATIO> == 3 ? 4 : 2>(ratio, tl.seg, first, item0 == 0);
             } else {
                 lr_rho = P.c.lr * P.rho[tl.seg];
             }
@@ -486,14 +489,24 @@ long long split_elems(bool gbf, int copies) {
     return (copies >= 512 ? 128 : copies > 128 ? 64 : 32) * K;
 }
 
+constexpr long long kOwnRatioItems3 = 444, kOwnRatioItems4 = 592;      // (see forms_own_ratios)
+
 // Wide (256-bit) accesses need 32-byte aligned buffers; they pay off when the
 // gradients are bf16 (a 128-bit gradient load then covers 8 elements) and for
 // small R, where the fp32 streams dominate.
 template <int OPT, bool GBF, int OUT, bool FUSED>
 ws_status launch_r(const UpdParams& P, const void* const* gptrs, bool wide_ok, cudaStream_t st, const OwnRatio* own) {
     if constexpr (is_phase2(OPT)) {
-        if constexpr (OPT == K_LAMB2 || OPT == K_LARS2)
-            if (own) return wide_ok ? launch<OPT, GBF, OUT, 8, 1, 1, 1, FUSED>(P, gptrs, st, *own) : launch<OPT, GBF, OUT, 4, 1, 1, 1, FUSED>(P, gptrs, st, *own);
+        if constexpr (OPT == K_LAMB2 || OPT == K_LARS2) {
+            if (own && P.nitems > kOwnRatioItems3) {
+                const OwnRatioAt<4> f = {*own};
+                return wide_ok ? launch<OPT, GBF, OUT, 8, 1, 1, 1, FUSED>(P, gptrs, st, f) : launch<OPT, GBF, OUT, 4, 1, 1, 1, FUSED>(P, gptrs, st, f);
+            }
+            if (own) {
+                const OwnRatioAt<3> f = {*own};
+                return wide_ok ? launch<OPT, GBF, OUT, 8, 1, 1, 1, FUSED>(P, gptrs, st, f) : launch<OPT, GBF, OUT, 4, 1, 1, 1, FUSED>(P, gptrs, st, f);
+            }
+        }
         if (wide_ok) return launch<OPT, GBF, OUT, 8, 1, 1, 1, FUSED>(P, gptrs, st);
         return launch<OPT, GBF, OUT, 4, 1, 1, 1, FUSED>(P, gptrs, st);
     } else {
@@ -742,14 +755,14 @@ bool one_kernel(const ws_plan* p, int opt, int copies, bool gbf) {
     return p->af_scalar <= p->N / 8 || copies <= (gbf ? 16 : 32) / (p->N > (24LL << 20) ? 2 : 1);
 }
 
-// Whether phase 2 of an all-shard norm pair forms the ratios itself, in place of a finalize launch between the phases.
-// Up to two waves of CTAs, measured in work items (us, finalize launch / own ratios): LAMB, 2 bf16 copies, 0.4 M in 103
-// tensors (620 items) 16.2 / 12.4, LARS 12.3 / 9.1; 1.2 M with 1 and 3 copies (1300, 1700 items) LAMB 19.6 / 20.5, 17.8 /
-// 19.6, LARS 14.2 / 15.9, 15.2 / 18.2; 4.1 M, 1 copy, LARS 24.0 / 28.4.
-constexpr long long kOwnRatioItems = 888;
+// Whether phase 2 of an all-shard norm pair forms the ratios itself, in place of a finalize launch between the phases: as
+// long as its CTAs are all resident at once, with the registers of 3 per SM (phase 2 then keeps more loads in flight) or
+// of 4.  us, calls back to back, finalize launch / own ratios with 3 / with 4: LARS, 0.37 M parameters (359 items) 7.0 / 5.7 /
+// 6.2, LAMB 8.8 / 7.5 / 8.0; 0.4 M (502 items) LARS 7.1 / 7.8 / 5.8, LAMB 11.1 / 12.5 / 9.9; 0.7 M (719 items) LARS 10.0 / 10.3 /
+// 10.2, LAMB 13.4 / 14.0 / 13.7.
 bool forms_own_ratios(const ws_plan* p) {
     const long long items = p->layout == WS_LAYOUT_CONCAT ? p->ntiles : p->ntiles * p->R;
-    return items >= 1 && items <= kOwnRatioItems;
+    return items >= 1 && items <= kOwnRatioItems4;
 }
 OwnRatio own_ratios(const ws_plan* p, const WsLambWs& L, const ws_hyper* h) {
     return {p->d_segtiles, L.partials, p->ntiles, L.rho, L.norms, L.status, p->T, finalize_reps(p), h->opt == WS_LARS, h->trust_coeff, h->weight_decay};

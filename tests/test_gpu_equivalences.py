@@ -212,14 +212,15 @@ def test_an_infinite_copy_among_many(R, S, form, gdtype):
 
 @pytest.mark.parametrize("layout", ["per_tensor", "concat"])
 @pytest.mark.parametrize("opt", ["lamb", "lars"])
-@pytest.mark.parametrize("R,items", [(1, "few"), (3, "few"), (3, "many")])
+@pytest.mark.parametrize("R,items", [(1, "few"), (3, "few"), (1, "some"), (3, "some"), (3, "many")])
 def test_ratios_formed_in_phase_two(R, items, opt, layout):
-    # small models form the ratios in phase 2 ("few"), larger ones in a launch of their own: ratios and norms (also those
+    # small models form the ratios in phase 2 ("few" and, with other registers, "some"), larger ones in a launch of their own: ratios and norms (also those
     # of a tensor without elements), state and weights are bit for bit those of the calls shard by shard
-    shapes = [(0,), (257, 33), (1,), (0, 5), (40, 1031), (64,), (0,)] + ([(700, 3000)] if items == "many" else [])
+    shapes = [(0,), (257, 33), (1,), (0, 5), (40, 1031), (64,), (0,)] + {"few": [], "some": [(490, 1000)], "many": [(700, 3000)]}[items]
     wl = W.Workload("f", shapes, R=R, opt=opt, hyper={}, grad_dtype=torch.float32, grad_std=1e-3, seed=R)
     plan = B.Plan(shapes, R, 32, 1024, layout=layout, one_launch=False)
-    assert (plan.ntiles * (R if layout == "per_tensor" else 1) <= 888) == (items == "few")
+    n = plan.ntiles * (R if layout == "per_tensor" else 1)
+    assert {"few": n <= 444, "some": 444 < n <= 592, "many": n > 592}[items]
     h = dict(lr=1e-3, beta1=0.9, beta2=0.999, eps=1e-6, weight_decay=0.01, momentum=0.9, grad_scale=1.0, step=4, trust_coeff=0.001)
     hy = B.make_hyper(opt, h)
     w, m, v = W.make_state(wl, DEV)
