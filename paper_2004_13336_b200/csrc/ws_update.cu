@@ -719,23 +719,33 @@ int finalize_reps(const ws_plan* p) { return p->layout == WS_LAYOUT_CONCAT ? 1 :
 // Parameters from which the one kernel of LAMB / LARS is not slower than the three launches (-1: never); both give
 // the same bits.  Its two phases are the waves of one grid, each behind a chain of table reads, and a small model has
 // two or three of them; what it saves, phase 2's second read, grows with the model.  More copies shorten that saving's
-// share, and fp32 gradients leave the three launches closer to the copy bandwidth than bf16 ones, whose wide phase 1
-// spills in both forms - but not with 4 copies, where the separate kernel has a variant of its own.  Device time one
-// kernel / three launches, formatting fused in, state and gradients not in L2 (encoder-decoder and image sets of M
-// parameters, us):
-//   LAMB fp32   8 copies   1.7 M 30.2/28.2   2.4 M 40.1/36.3   4.6 M 62.4/63.1   7.6 M 81.8/93.7     26 M 257/279
-//              12 copies   2.4 M 56.2/49.1   4.6 M 77.9/79.5   6.9 M 117/115     7.6 M 116/123  26 M 345/362
-//              16 copies   4.6 M 86.0/83.1   7.6 M 130/128     26 M 389/411      32 copies 7.6 M 227/204  26 M 644/686
-//        bf16   8 copies  0.37 M 16.2/14.0   1.7 M 42.4/48.9   7.6 M 120/181     32 copies 1.7 M 78.9/85.7
-//   LARS fp32   4 copies   4.6 M 44.1/45.8   6.9 M 58.9/53.3   26 M 178/190      8 copies 2.4 M 37.4/31.9  4.6 M 55.4/53.5
-//               8 copies   6.9 M 76.9/77.4   7.6 M 75.6/81.7   26 M 229/234     16 copies 26 M 359/356  56 M 748/772
-//        bf16   4 copies   7.6 M 76.0/47.9   56 M 459/350        8 copies 2.0 M 50.5/46.6  4.1 M 67.9/78.5  26 M 243/299
-// LAMB with 2 to 7 copies and LARS with 2 or 3 run as three launches (211 M, LAMB: 4 copies 1.64 ms against 1.67).
+// share, and with them the line moves up.  Device time three launches / one kernel, us, formatting fused in, state and
+// gradients not in L2 (encoder-decoder and image sets of M parameters); on packed buffers the lines lie where these do:
+//   LAMB bf16   8 copies  1.1 M 31.7/39.9   1.7 M 35.8/35.8   2.6 M 48.4/48.2   4.1 M 72.7/64.6   9.4 M 132/93   26 M 232/214
+//              12 copies  1.7 M 39.9/44.1   2.6 M 56.3/62.5   4.1 M 76.8/82.9   5.7 M 89.1/87.1   9.4 M 140/122  26 M 290/271
+//              16 copies  4.1 M 85.0/97.3   5.7 M 99.3/105    9.4 M 144/136     26 M 312/300      56 M 658/616
+//              32 copies  4.1 M 132/171     9.4 M 196/222     26 M 499/480      56 M 961/960
+//        fp32   8 copies  2.6 M 48.1/52.2   4.1 M 68.8/68.6   5.7 M 85.0/83.0   6.9 M 101/93
+//              12 copies  4.1 M 85.0/91.2   5.7 M 103/102     6.9 M 128/128     9.4 M 163/151
+//              16 copies  6.9 M 140/144     9.4 M 169/167     26 M 419/394      32 copies 9.4 M 259/286  26 M 679/667
+//   LARS bf16   6 copies  2.6 M 39.9/42.2   4.1 M 54.2/48.1   8 copies 2.6 M 39.9/42.0  4.1 M 58.3/54.3  26 M 187/175
+//              12 copies  1.7 M 39.8/37.9   4.1 M 74.8/70.8   9.4 M 136/97      26 M 236/220
+//              16 copies  2.6 M 54.2/64.5   3.2 M 60.4/54.3   4.1 M 85.0/85.0   5.7 M 97.3/87.1   9.4 M 138/108  26 M 253/249
+//              32 copies  2.6 M 97.3/114    3.2 M 99.3/89.1   4.1 M 151/161     5.7 M 169/157   26 M 540/415  56 M 812/835
+//        fp32   4 copies  6.9 M 56.4/62.6   9.4 M 70.8/74.9   26 M 179/181      52 M 367/351
+//               8 copies  2.6 M 39.9/46.1   4.1 M 60.4/60.5   5.7 M 71.6/72.7   6.9 M 85.0/81.1   9.4 M 107/95
+//              12 copies  9.4 M 136/132     26 M 308/308      39 M 484/474      16 copies 26 M 357/364   39 M 581/568
+// LAMB with 2 to 7 copies, LARS with 2 or 3 and with 4 bf16 ones run as three launches: those are the faster form on small
+// models and on the largest (211 M, bf16: LAMB 2 copies 1262/1365, 4 1376/1445, LARS 2 1011/1079, 4 1130/1164).  Between
+// about 16 M and 60 M the one kernel is 3 to 15 % faster there, too (26 M: LAMB 6 fp32 copies 263/237, LARS 4 bf16 153/148;
+// 52 M: LAMB 4 bf16 417/363): a line with two ends, which this rule does not have.
 long long pair_min_params(bool lars, bool gbf, int copies) {
     constexpr long long M = 1 << 20;
     if (copies < (lars ? 4 : 8) || copies > 32) return -1;
-    if (lars) return gbf ? (copies == 4 ? -1 : 3 * M) : (copies == 4 ? 8 * M : copies <= 8 ? 4 * M : 32 * M);
-    return gbf ? M : (copies <= 12 ? 4 * M : copies <= 16 ? 8 * M : 16 * M);
+    if (lars && gbf) return copies == 4 ? -1 : 3 * M;
+    if (lars) return copies == 4 ? 8 * M : copies <= 8 ? 4 * M : 32 * M;
+    if (gbf) return copies <= 8 ? 2 * M : copies <= 12 ? 5 * M : copies <= 16 ? 8 * M : 16 * M;
+    return copies <= 12 ? 4 * M : copies <= 16 ? 8 * M : 16 * M;
 }
 
 // Whether an all-shard update of `opt` runs as one kernel where the plan's schedule is on the device.

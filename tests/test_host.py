@@ -368,9 +368,10 @@ def test_adafactor_short_tensors_are_one_block(shape, blocks, chunks):
 
 @pytest.mark.parametrize("opt,gdtype,copies,least", [
     ("lamb", torch.float32, 8, 4 << 20), ("lamb", torch.float32, 12, 4 << 20), ("lamb", torch.float32, 13, 8 << 20), ("lamb", torch.float32, 32, 16 << 20),
-    ("lamb", torch.bfloat16, 8, 1 << 20), ("lamb", torch.bfloat16, 7, None), ("lamb", torch.float32, 33, None),
+    ("lamb", torch.bfloat16, 8, 2 << 20), ("lamb", torch.bfloat16, 9, 5 << 20), ("lamb", torch.bfloat16, 13, 8 << 20),
+    ("lamb", torch.bfloat16, 32, 16 << 20), ("lamb", torch.bfloat16, 7, None), ("lamb", torch.float32, 33, None),
     ("lars", torch.float32, 4, 8 << 20), ("lars", torch.float32, 5, 4 << 20), ("lars", torch.float32, 9, 32 << 20),
-    ("lars", torch.bfloat16, 5, 3 << 20), ("lars", torch.bfloat16, 4, None), ("lars", torch.float32, 3, None),
+    ("lars", torch.bfloat16, 5, 3 << 20), ("lars", torch.bfloat16, 32, 3 << 20), ("lars", torch.bfloat16, 4, None), ("lars", torch.float32, 3, None),
     ("lars", torch.bfloat16, 33, None), ("sgdm", torch.float32, 8, None), ("adam", torch.float32, 8, None)])
 def test_one_kernel_route_by_size_and_copies(opt, gdtype, copies, least):
     route = lambda n: B.lib().ws_plan_one_kernel(  # noqa: E731
