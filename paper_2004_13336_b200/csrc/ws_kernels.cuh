@@ -425,6 +425,13 @@ __device__ __forceinline__ void sum_partials(const WsSegTiles st, const float2* 
     sum_block(a, b, sa, sb);
 }
 
+// The ratio of a tensor's norms from their squares: LAMB's trust ratio or LARS's local rate.  One function for all forms,
+// so that they give the same bits.
+__device__ __forceinline__ float norm_ratio(double a, double b, int lars, double eta, double beta) {
+    if (!(a > 0.0 && b > 0.0)) return 1.0f;
+    return lars ? (float)(eta * sqrt(a) / (sqrt(b) + beta * sqrt(a))) : (float)(sqrt(a) / sqrt(b));
+}
+
 // Sums two values over the CTA at once (one pair of barriers for both); the totals are valid in
 // thread 0.  The order of the additions is fixed, so the result is run-to-run bit-stable.
 __device__ __forceinline__ float2 block_sum2(float x, float y, float2* smem /* kBlock/32 entries */) {

@@ -133,9 +133,7 @@ two_phase_kernel(const UpdParams P, const __grid_constant__ GradPtrs<NP> gp, con
         double a, b;
         sum_partials(WsSegTiles{(int)sg.z, (int)sg.w}, P.partials, P.ntiles, Q.reps, fin_a, fin_b, a, b);
         if (tid == 0) {
-            float ratio = 1.0f;
-            if (a > 0.0 && b > 0.0)
-                ratio = PAIR == 1 ? (float)(Q.eta * sqrt(a) / (sqrt(b) + Q.beta * sqrt(a))) : (float)(sqrt(a) / sqrt(b));
+            const float ratio = norm_ratio(a, b, PAIR, Q.eta, Q.beta);
             // the word first: it is what the other CTAs wait for
             st_release(Q.flag + it.seg, ((unsigned long long)__float_as_uint(ratio) << 32) | 1ULL);
             Q.rho[it.seg] = ratio;

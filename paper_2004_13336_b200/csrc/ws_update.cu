@@ -31,12 +31,6 @@ namespace {
 constexpr long long kKeepReverseBytes = 256ll << 20;   // twice the L2: at least half of phase 2's re-reads can hit
 using namespace wsk;
 
-// The ratio of tensor t's norms, as both forms of the norm pairs make it.
-__device__ __forceinline__ float norm_ratio(double a, double b, int lars, double eta, double beta) {
-    if (!(a > 0.0 && b > 0.0)) return 1.0f;
-    return lars ? (float)(eta * sqrt(a) / (sqrt(b) + beta * sqrt(a))) : (float)(sqrt(a) / sqrt(b));
-}
-
 // Phase 2 of a small model does lamb_finalize_kernel's work: the CTA sums its tensor's partial norms itself (the same
 // function, the same bits); the one with the tensor's first tile stores what the finalize step stores, and the grid's
 // first one the rest.  A launch less: 3 us of the host, which is what a tiny model's three launches are bound by, against
