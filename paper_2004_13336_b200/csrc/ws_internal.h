@@ -143,6 +143,7 @@ struct ws_plan {
     // images of small uploads; they live as long as the plan, since a captured copy reads its source at every replay
     std::vector<char> table_image, sched_image;
     // device copies (caller-owned memory, set by ws_plan_upload)
+    int sms = 148;                            // multiprocessors of the device of the upload
     const WsTile* d_tiles = nullptr;
     const WsSegTiles* d_segtiles = nullptr;
     std::vector<WsSegAf> segaf;

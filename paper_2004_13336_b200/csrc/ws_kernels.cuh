@@ -70,6 +70,7 @@ struct UpdParams {
     long long st_stride;    // per-shard element stride inside w/m/v (S for [R][S] state, 0 for one shard)
     int R;
     int tile, tile_max;     // elements of a tile on average, and of the longest
+    int sms;                // multiprocessors of the device
     int r0;                 // first shard of this launch
     int concat;             // concatenated layout: tiles [tile_lo, tile_lo + nitems), each names its shard
     long long tile_lo;

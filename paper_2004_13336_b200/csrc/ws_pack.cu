@@ -223,7 +223,7 @@ struct PackShape {
 PackShape pack_shape(const ws_plan* p, int eb, int vb, long long items) {
     PackShape s;
     const long long tile = p->ntiles > 0 ? (p->layout == WS_LAYOUT_CONCAT ? p->S * p->R : p->S) / p->ntiles : p->K;
-    s.is_short = items > 4736 && tile * eb <= 3072 && (long long)p->longest * eb <= 512 << 10;
+    s.is_short = items > 32LL * p->sms && tile * eb <= 3072 && (long long)p->longest * eb <= 512 << 10;
     s.threads = s.is_short ? kShortBlock : 256;
     const long long vecs = (long long)p->K * eb / vb;     // vectors per full tile
     while (!s.is_short && s.threads > 64 && vecs < 2LL * s.threads) s.threads >>= 1;

@@ -418,6 +418,9 @@ extern "C" ws_status ws_plan_upload(ws_plan* p, void* dev_buf, size_t bytes, voi
     for (int i = 0; i < 4; ++i) { o[i] = at; at += round16(nb[i]); }
     const ws_status s = upload_image(base, src, nb, o, 4, at, p->table_image, (cudaStream_t)stream, "ws_plan_upload");
     if (s != WS_OK) return s;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&p->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        p->sms = 148;
     p->d_tiles = (const WsTile*)(base + o[0]);
     p->d_segtiles = (const WsSegTiles*)(base + o[1]);
     p->d_segaf = (const WsSegAf*)(base + o[2]);

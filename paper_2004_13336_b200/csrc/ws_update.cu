@@ -458,7 +458,7 @@ ws_status launch(const UpdParams& P, const void* const* gptrs, cudaStream_t st, 
     // us, 256 threads / this rule, formatting fused in: tiles of 1024, 4.1 M parameters, SGD-M 8 bf16 copies 28.7 / 17.9, 4 copies 21.9 / 12.7, Adam 8 copies 36.2 / 24.5;
     // 1.2 M parameters in 161 tensors, Adam, 16 copies fp32 27.7 / 19.6, bf16 26.4 / 15.5, 32 copies bf16 57 / 34.
     int threads = kBlock;
-    if ((OPT == K_SGDM || OPT == K_ADAM) && NP <= 32 && P.nitems > 444)
+    if ((OPT == K_SGDM || OPT == K_ADAM) && NP <= 32 && P.nitems > 3LL * P.sms)
         while (threads > 64 && P.tile <= VEC * threads / 2 && P.tile_max <= 32 * VEC * threads) threads /= 2;
     launch_pdl_as(update_kernel<OPT, GBF, OUT, VEC, U, RB, NP, FUSED, RATIO>, grid, threads, st, P, gp, ratio);
     return ws_check_launch(FUSED ? "ws_fused_update" : "ws_shard_update");
@@ -483,8 +483,6 @@ long long split_elems(bool gbf, int copies) {
     return (copies >= 512 ? 128 : copies > 128 ? 64 : 32) * K;
 }
 
-constexpr long long kOwnRatioItems3 = 444, kOwnRatioItems4 = 592;      // (see forms_own_ratios)
-
 // Wide (256-bit) accesses need 32-byte aligned buffers; they pay off when the
 // gradients are bf16 (a 128-bit gradient load then covers 8 elements) and for
 // small R, where the fp32 streams dominate.
@@ -492,7 +490,7 @@ template <int OPT, bool GBF, int OUT, bool FUSED>
 ws_status launch_r(const UpdParams& P, const void* const* gptrs, bool wide_ok, cudaStream_t st, const OwnRatio* own) {
     if constexpr (is_phase2(OPT)) {
         if constexpr (OPT == K_LAMB2 || OPT == K_LARS2) {
-            if (own && P.nitems > kOwnRatioItems3) {
+            if (own && P.nitems > 3LL * P.sms) {            // (see forms_own_ratios)
                 const OwnRatioAt<4> f = {*own};
                 return wide_ok ? launch<OPT, GBF, OUT, 8, 1, 1, 1, FUSED>(P, gptrs, st, f) : launch<OPT, GBF, OUT, 4, 1, 1, 1, FUSED>(P, gptrs, st, f);
             }
@@ -654,6 +652,7 @@ ws_status prepare(const ws_plan* p, int32_t r, const ws_grads* g, const ws_state
     P.tiles = p->d_tiles;
     P.ntiles = p->ntiles;
     P.tile_max = p->longest;
+    P.sms = p->sms;
     P.tile = p->ntiles > 0 ? (int)((p->layout == WS_LAYOUT_CONCAT ? p->S * p->R : p->S) / p->ntiles) : p->K;
     P.S = p->S;
     P.R = g ? g->R : p->R;
@@ -766,7 +765,7 @@ bool one_kernel(const ws_plan* p, int opt, int copies, bool gbf) {
 // 10.2, LAMB 13.4 / 14.0 / 13.7.
 bool forms_own_ratios(const ws_plan* p) {
     const long long items = p->layout == WS_LAYOUT_CONCAT ? p->ntiles : p->ntiles * p->R;
-    return items >= 1 && items <= kOwnRatioItems4;
+    return items >= 1 && items <= 4LL * p->sms;
 }
 OwnRatio own_ratios(const ws_plan* p, const WsLambWs& L, const ws_hyper* h) {
     return {p->d_segtiles, L.partials, p->ntiles, L.rho, L.norms, L.status, p->T, finalize_reps(p), h->opt == WS_LARS, h->trust_coeff, h->weight_decay};
@@ -1173,10 +1172,7 @@ ws_status af_stage(const ws_plan* plan, int stage, int32_t r, const ws_grads* gr
             P.ghat = L.ghat;
             P.af_fac = L.fac;
             if (P.nitems < 1) return WS_OK;
-            int dev = 0, sms = 148;
-            cudaGetDevice(&dev);
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-            const long long cap = (long long)sms * kAf2Ctas;
+            const long long cap = (long long)plan->sms * kAf2Ctas;
             af_sumsq_kernel<<<(unsigned)(P.nitems < cap ? P.nitems : cap), kBlock, 0, st>>>(P);
             return ws_check_launch("adafactor(pass 2)");
         }
