@@ -10,6 +10,7 @@ import torch
 
 from paper_2004_13336_b200 import binding as B
 from paper_2004_13336_b200 import workloads as W
+from tests._util import TOL_FP32
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda"
@@ -285,49 +286,86 @@ def test_few_long_tiles_among_short_ones(tile, gdtype):
 
 
 @pytest.mark.parametrize("gdtype", [torch.float32, torch.bfloat16])
-@pytest.mark.parametrize("R,shift", [(3, 0), (8, 8), (12, 0), (16, 8), (32, 0)])
-def test_many_short_tiles(R, gdtype, shift):
-    # 700 tensors of 0 to 900 elements cut into R shards: pieces of 8 to a few hundred elements, where pack and unpack
-    # give a warp to a tile and an update has CTAs of 64 threads; tensors 32 bytes aligned, or 16 (`shift`)
-    rng = np.random.default_rng(R)
-    numel = [int(x) for x in rng.integers(0, 900, 700)] + [1, 7, 8, 9, 1024, 2049]
-    plan = B.Plan([(n,) for n in numel], R, 8)
-    assert plan.ntiles * R > 4736 or R == 3
-    gen = torch.Generator(device=DEV).manual_seed(R)
-    views = lambda t: [t[o:o + n] for o, n in zip(offs, numel)]  # noqa: E731
-    offs, at = [], shift
+@pytest.mark.parametrize("shards,copies,align,layout,shift", [(3, 3, 8, "per_tensor", 0), (8, 8, 8, "per_tensor", 16), (8, 12, 32, "concat", 16),
+                                                              (12, 4, 32, "per_tensor", 0), (5000, 2, 8, "concat", 0), (5000, 16, 32, "concat", 0),
+                                                              (5000, 1, 32, "concat", 16), (16, 32, 32, "per_tensor", 16), (32, 32, 8, "per_tensor", 0)])
+def test_many_short_tiles(shards, copies, align, layout, shift, gdtype):
+    # 1200 tensors of 0 to 900 elements (two tables of tensor pointers) cut into shards: pieces of 8 to a few hundred
+    # elements, where pack and unpack give a warp to a tile and an update has CTAs of 64 or 128 threads; tensors on
+    # 32-byte boundaries, or 16 bytes beside one (`shift`), and with `align` 32 vectors of 32 bytes in bf16 too
+    rng = np.random.default_rng(shards + align)
+    numel = [int(x) for x in rng.integers(0, 900, 1200)] + [1, 7, 8, 9, 1024, 2049]
+    plan = B.Plan([(n,) for n in numel], shards, align, layout=layout)
+    assert plan.ntiles * (1 if layout == "concat" else shards) > 444
+    gen = torch.Generator(device=DEV).manual_seed(shards + copies)
+    offs, at = [], 0
     for n in numel:
         offs.append(at)
-        at += (n + 15) // 16 * 16 + shift
-    draw = lambda std, dt=torch.float32: (torch.randn(at + 16, generator=gen, device=DEV) * std).to(dt)  # noqa: E731
-    w, m, v, g = draw(0.02), draw(1e-3), draw(1e-5).abs(), [draw(1e-3, gdtype) for _ in range(R)]
-    segs = plan.segments()
+        at += (n + 15) // 16 * 16 + 16
 
-    def placed(t):                                  # [R][S] by the definition of the layout
-        flat = torch.zeros(R, plan.S, dtype=t.dtype, device=DEV)
-        for s, o, n in zip(segs, offs, numel):
-            if n:
-                full = torch.zeros(R * s.piece, dtype=t.dtype, device=DEV)
-                full[:n] = t[o:o + n]
-                flat[:, s.shard_off:s.shard_off + s.piece] = full.view(R, s.piece)
-        return flat.view(-1)
+    def arena(std, dt=torch.float32):
+        return (torch.randn(at + 16, generator=gen, device=DEV) * std).to(dt)
 
+    def views(t, size=None):
+        k = shift // (size or t.element_size())
+        return [t[o + k:o + k + n] for o, n in zip(offs, numel)]
+
+    def placed(lst):                                # [R][S] by the definition of the layout
+        flat = torch.zeros(plan.G, dtype=lst[0].dtype, device=DEV)
+        for s, x in zip(plan.segments(), lst):
+            if x.numel() == 0:
+                continue
+            if layout == "concat":
+                flat[s.shard_off:s.shard_off + x.numel()] = x
+            else:
+                full = torch.zeros(shards * s.piece, dtype=x.dtype, device=DEV)
+                full[:x.numel()] = x
+                flat.view(shards, plan.S)[:, s.shard_off:s.shard_off + s.piece] = full.view(shards, s.piece)
+        return flat
+
+    w, m, v, g = arena(0.02), arena(1e-3), arena(1e-5).abs(), [arena(1e-3, gdtype) for _ in range(copies)]
     state = []
-    for t in (w, m, v):
-        flat = torch.full((plan.G,), float("nan"), device=DEV)
+    for t in (w, m, v, g[0]):
+        flat = torch.full((plan.G,), float("nan"), dtype=t.dtype, device=DEV)
         B.ws_pack(plan, views(t), flat)
-        assert torch.equal(flat, placed(t))
+        assert torch.equal(flat, placed(views(t)))
+        back, expect = torch.full_like(t, 7.0), torch.full_like(t, 7.0)
+        B.ws_unpack(plan, flat, views(back))
+        for a, b in zip(views(expect), views(t)):
+            a.copy_(b)
+        assert torch.equal(back, expect)            # (and nothing between the tensors)
         state.append(flat)
-    packed = [torch.full((plan.G,), float("nan"), dtype=gdtype, device=DEV) for _ in range(R)]
+    packed = [torch.full((plan.G,), float("nan"), dtype=gdtype, device=DEV) for _ in range(copies)]
     table = B.TensorTable(plan, [views(t) for t in g])
     B.ws_pack_sets(plan, table, packed)
-    assert all(torch.equal(a, placed(b)) for a, b in zip(packed, g))
-    hy = B.make_hyper("adam", dict(lr=1e-3, beta1=0.9, beta2=0.999, eps=1e-8, weight_decay=0.0, momentum=0.0, grad_scale=1.0, step=10))
-    master = w.clone()
-    pm, pv = state[1].clone(), state[2].clone()
-    B.ws_fused_update(plan, -1, table, None, pm, pv, hy, B.TensorTable(plan, [views(master)]))
-    B.ws_shard_update(plan, -1, packed, *state, hy)
-    back = torch.zeros_like(w)
-    B.ws_unpack(plan, state[0], views(back))
-    assert torch.equal(state[1], pm) and torch.equal(state[2], pv)
-    assert all(torch.equal(a, b) for a, b in zip(views(master), views(back)))
+    assert all(torch.equal(a, placed(views(b))) for a, b in zip(packed, g))
+
+    def close(x, ref):
+        # a chain of fewer than 16 fp32 roundings of 2^-24 (tree, compensated sum, moments, root, quotient) is below 1e-6 of
+        # the operands' scale, the measure that every output of these optimizers is held to
+        rms = ref.square().mean().sqrt()
+        return bool(((x.double() - ref).abs() <= TOL_FP32 * torch.maximum(ref.abs(), rms)).all())
+
+    # both elementwise optimizers against 64 bits; several weight lists, the packed form and the master form against the first
+    gs = sum(t.double() for t in g).roll(shift // 4 - shift // g[0].element_size())      # at the places of the fp32 tensors
+    for opt in ("adam", "sgdm"):
+        hy = B.make_hyper(opt, dict(lr=1e-3, beta1=0.9, beta2=0.999, eps=1e-8, weight_decay=0.0, momentum=0.9, grad_scale=1.0, step=10))
+        s = [x.clone() for x in state[:3]]
+        outs = [torch.zeros_like(w) for _ in range(min(copies, 3))]
+        B.ws_fused_update(plan, -1, table, *s, hy, B.TensorTable(plan, [views(x) for x in outs]))
+        if opt == "adam":
+            m1, v1 = 0.9 * m.double() + 0.1 * gs, 0.999 * v.double() + 0.001 * gs * gs
+            w1 = w.double() - 1e-3 * (m1 / (1 - 0.9 ** 10)) / ((v1 / (1 - 0.999 ** 10)).sqrt() + 1e-8)
+        else:
+            m1, v1 = 0.9 * m.double() + gs, v.double()
+            w1 = w.double() - 1e-3 * m1
+        assert all(close(got, placed(views(ref, 4))) for got, ref in zip(s, (w1, m1, v1)))
+        one = [x.clone() for x in state[:3]]
+        B.ws_shard_update(plan, -1, packed, *one, hy)
+        mm, mv, master = state[1].clone(), state[2].clone(), w.clone()
+        B.ws_fused_update(plan, -1, table, None, mm, mv, hy, B.TensorTable(plan, [views(master)]))
+        assert all(torch.equal(a, b) for a, b in zip(one, s)) and torch.equal(mm, s[1]) and torch.equal(mv, s[2])
+        back = torch.zeros_like(w)
+        B.ws_unpack(plan, s[0], views(back))
+        for o in outs + [master]:
+            assert all(torch.equal(a, b) for a, b in zip(views(o), views(back)))
