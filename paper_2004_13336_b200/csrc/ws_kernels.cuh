@@ -12,7 +12,8 @@ namespace wsk {
 
 constexpr int kBlock = 256;
 // Resident CTAs per SM the compiler must allow for (register budget): 3 measured best (4 forces
-// spills, 2 leaves bandwidth unused); the many-replica kernel is faster with the registers of 2.
+// spills, 2 leaves bandwidth unused); the many-replica kernel is faster with the registers of 2
+// (min_blocks and own_ctas in ws_update.cu name the exceptions).
 constexpr int kMinBlocks = 3;
 constexpr int kMinBlocksWide = 2;
 constexpr int kTreeBlockLarge = 16;   // gradients per tree block when R > 32
@@ -253,10 +254,9 @@ __device__ __forceinline__ float raw_elem(const GradRaw<GBF, VEC>& g, int i) {
     }
 }
 // The sum of RB copies as a tree, one element after the other.  Widened all at once, 8 bf16 copies of 8 elements
-// are 64 registers: the kernels of 5 and more bf16 copies then spilled up to 500 bytes a thread, and local memory
-// shares the L1 with the stream.  25.6 M parameters, formatting fused in, us, before / now: SGD-M 8 copies 211 / 126,
-// 6 copies 204 / 113, 1 copy 90 / 79; Adam 8 copies 287 / 160; LAMB 8 copies 340 / 210; LARS 8 copies 245 / 173; on
-// packed buffers, where 128 registers had kept most of it out of memory, Adam with 8 copies and its formatting 378 / 314.
+// are 64 registers: the kernels of 5 and more bf16 copies then spill up to 500 bytes a thread, and local memory
+// shares the L1 with the stream.  25.6 M parameters, formatting fused in, us, all at once / one after the other: SGD-M 8
+// copies 211 / 126, 6 copies 204 / 113, 1 copy 90 / 79; Adam 8 copies 287 / 160; LAMB 340 / 210; LARS 245 / 173.
 template <bool GBF, int VEC, int RB>
 __device__ __forceinline__ Fv<VEC> tree_sum(const GradRaw<GBF, VEC> (&raw)[RB]) {
     Fv<VEC> o;
@@ -496,7 +496,7 @@ __device__ __forceinline__ Fv<VEC> load_f32_partial(const float* p, int n) {
 }
 
 // 9 to 32 bf16 copies: two tree blocks of 8 at a time.  A thread's 4 elements of 16 copies are the 128 bytes in flight
-// that 8 elements of 8 copies are, with half the state and sums in registers (no spills), no idle half of a CTA on
+// that 8 elements of 8 copies are, with half the state and sums in registers, no idle half of a CTA on
 // tiles of 1024, and half the waits for memory.  Formatting fused in, us, 8 elements of 8 copies / these: Adam, 12,
 // 16, 32 copies, 4.1 M parameters (tiles of 1024) 59 / 43, 67 / 51, 125 / 92, 25.6 M 235 / 209, 248 / 234, 479 / 386;
 // SGD-M 16 and 32 copies, 25.6 M 198 / 197, 405 / 343; LAMB 16 copies 317 / 295.  LARS, whose phase 1 holds no slots,
@@ -537,7 +537,7 @@ __device__ __forceinline__ void process_item(const UpdParams& P, const GradPtrs<
     constexpr bool ELEMENTWISE = OPT == K_SGDM || OPT == K_ADAM;   // nothing is summed over the CTA: any block size
     constexpr bool LOOPK = (NP > RB);   // R may exceed one tree block: loop and compensate
     constexpr int NBLK = many_blocks<OPT, GBF, VEC, RB, NP>();   // tree blocks whose loads are in flight together
-    constexpr bool MANY = ELEMENTWISE && NP > kManyGroups * kTreeBlockLarge;   // groups of several blocks
+    constexpr bool MANY = ELEMENTWISE && NP > kManyGroups * kTreeBlockLarge;   // (the table of more than 128 copies: groups of several blocks)
     constexpr bool WMASTER = FUSED && OUT == O_F32M;   // w lives in the weight tensors only
     const int nvalid = it.nvalid;
     const long long gbase = it.gbase, sbase = it.sbase, obase = it.obase, toff = it.toff;
@@ -671,7 +671,7 @@ __device__ __forceinline__ void process_item(const UpdParams& P, const GradPtrs<
             Fv<VEC> gs[MANY ? U : 1], gsc[MANY ? U : 1];       // the groups before this one
             bool first = true;
             const int group_blocks = MANY ? many_blocks_per_group(P.R) : 0;
-            int in_group = group_blocks > 1 ? 0 : 1;           // blocks of this group so far (a group of one: all blocks are one sum)
+            int in_group = 0;                                  // blocks of this group so far
             for (int k0 = 0; k0 < (LOOPK ? P.R : 1); k0 += RB * NBLK) {
                 GradRaw<GBF, VEC> raw[U][NBLK][RB];
                 // (fp32 slices of more than 32 copies: a full block's loads without a condition each, in the order of the copies.
@@ -719,7 +719,7 @@ __device__ __forceinline__ void process_item(const UpdParams& P, const GradPtrs<
                     }
                 }
                 if constexpr (MANY) {
-                    if (group_blocks > 1 && (++in_group == group_blocks || k0 + RB >= P.R)) {       // a group is complete
+                    if (++in_group == group_blocks || k0 + RB >= P.R) {       // a group is complete
 #pragma unroll
                         for (int u = 0; u < U; ++u)
 #pragma unroll
@@ -738,9 +738,8 @@ __device__ __forceinline__ void process_item(const UpdParams& P, const GradPtrs<
                 }
             }
             if constexpr (MANY) {
-                if (group_blocks > 1)
 #pragma unroll
-                    for (int u = 0; u < U; ++u) gv[u] = gs[u];
+                for (int u = 0; u < U; ++u) gv[u] = gs[u];
             }
         }
         if constexpr (OPT == K_AF1) {

@@ -33,8 +33,7 @@ using namespace wsk;
 
 // Phase 2 of a small model does lamb_finalize_kernel's work: the CTA sums its tensor's partial norms itself (the same
 // function, the same bits); the one with the tensor's first tile stores what the finalize step stores, and the grid's
-// first one the rest.  A launch less: 3 us of the host, which is what a tiny model's three launches are bound by, against
-// 2 us more in every CTA (24 to 374 K parameters, LAMB and LARS 11.4 -> 9.1 us).
+// first one the rest.  A launch less against 2 us more in every CTA; forms_own_ratios says where that is the faster form.
 template <int U>
 __device__ __forceinline__ float own_ratio(const OwnRatio& F, int seg, bool first, bool rest) {
     __shared__ double sa[kBlock / 32], sb[kBlock / 32];
@@ -63,8 +62,9 @@ __device__ __forceinline__ float own_ratio(const OwnRatio& F, int seg, bool firs
     return s_rho;
 }
 
-// (129 and more bf16 copies: 16 of 4 elements are 32 registers, and the third CTA per SM is worth a few spills - 512
-// copies of 346 K elements, Adam 98 -> 67 us, SGD-M 95 -> 64; 64 copies of 2.8 M, SGD-M, would go from 66 to 76)
+// (129 and more bf16 copies: 16 of 4 elements are 32 registers, and the third CTA per SM is worth a few spills.  us, two
+// CTAs / three: slices, 512 copies of 346 K elements, Adam 98 / 67, SGD-M 95 / 64; formatting fused in, 2 M parameters, Adam,
+// 160 copies 546 / 358, 256 copies 1038 / 723.  64 copies of 2.8 M, SGD-M, would go from 66 to 76)
 template <int OPT, bool GBF, int RB, int NP>
 constexpr int min_blocks() {
     return RB > 8 && !(GBF && NP > 128 && (OPT == K_SGDM || OPT == K_ADAM)) ? kMinBlocksWide : kMinBlocks;
@@ -146,7 +146,7 @@ update_kernel(const UpdParams P, const __grid_constant__ GradPtrs<NP> gp, const 
 // block of all copies.  The groups meet in shared memory with their compensations.  What bounds it: up to 64 K elements
 // those waits, one to eight in a row; beyond, DRAM pages of 512 bytes a copy and CTA.  Adam, us, one thread per element /
 // this, slices of one shard: 512 copies of 22 K elements fp32 32 / 10, bf16 40 / 10, of 87 K 41 / 37, 45 / 20; 1024
-// copies of 11 K 61 / 13, 76 / 16, of 43 K 74 / 40, 86 / 19 (10 us of each are the host's).
+// copies of 11 K 61 / 13, 76 / 16, of 43 K 74 / 40, 86 / 19 (6 to 8 us of each are the host's).
 template <int OPT, bool GBF, int OUT, int NP>
 __global__ void __launch_bounds__(kBlock, kMinBlocksWide) split_kernel(const UpdParams P, const __grid_constant__ GradPtrs<NP> gp, int nsub) {
     constexpr int VEC = GBF ? 8 : 4, E = 32 * VEC, RB = kTreeBlockLarge;
