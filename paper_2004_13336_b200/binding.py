@@ -280,6 +280,15 @@ class PtrList:
         self.arr = _ptr_array(self.tensors)
         self.dtype = self.tensors[0].dtype if self.tensors else torch.float32
 
+    @property
+    def arr(self):
+        return self._arr
+
+    @arr.setter
+    def arr(self, arr):
+        self._arr = arr
+        self.addr = C.addressof(arr)
+
     def __len__(self):
         return len(self.tensors)
 
@@ -298,6 +307,8 @@ def _ptr_array(tensors):
 
 def _ptr_table(tensors):
     """(address of the tensors' pointers, their owner) for the plain-address prototypes."""
+    if type(tensors) is PtrList:
+        return tensors.addr, tensors._arr
     if isinstance(tensors, PtrList):
         return C.addressof(tensors.arr), tensors.arr
     # (a list and no iterator: the tensors of one may be gone when the call reads their pointers)
@@ -344,6 +355,7 @@ class Plan:
         self.layout = layout
         _check(lib().ws_plan_create_layout(descs, T, R, align_elems, tile_elems, LAYOUT_CODE[layout],
                                            C.byref(self._h)), "ws_plan_create_layout")
+        vars(self)["handle"] = self._h
         L = lib()
         self.T, self.R, self.A = L.ws_plan_num_tensors(self._h), L.ws_plan_num_shards(self._h), L.ws_plan_align(self._h)
         self.S, self.N = L.ws_plan_shard_elems(self._h), L.ws_plan_valid_elems(self._h)
@@ -356,9 +368,7 @@ class Plan:
             if one_launch:
                 self.upload_schedule(device)
 
-    @property
-    def handle(self):
-        return self._h
+    # `handle`, the plan's address, is an attribute of the instance (a property costs a call more in every step call)
 
     def segments(self) -> List[ws_segment]:
         segs, T = C.POINTER(ws_segment)(), C.c_int32()
@@ -434,7 +444,7 @@ class Plan:
         try:
             if self._h:
                 lib().ws_plan_destroy(self._h)
-                self._h = None
+                self._h = vars(self)["handle"] = None
         except Exception:
             pass
 
@@ -496,10 +506,10 @@ def ws_shard_update(plan: Plan, r: int, gbufs: Sequence[torch.Tensor], w, m, v, 
                     slice_mode: int = 0):
     if type(hyper) is not ws_hyper:
         _refuse(hyper, ws_hyper)
-    if type(slice_mode) is int and 0 <= slice_mode <= 1:
-        addr, own = _ptr_table(gbufs)
-        g = _GRADS.pack(addr, len(gbufs), _dtype_code(gbufs[0].dtype), slice_mode)
-    else:                        # by ctypes' rules
+    addr, own = _ptr_table(gbufs)
+    try:
+        g = _GRADS.pack(addr, len(gbufs), _dtype_code(gbufs[0].dtype), slice_mode if type(slice_mode) is int else None)
+    except struct.error:         # what struct refuses goes by ctypes' rules
         own = _grads(gbufs, slice_mode)
         g = C.addressof(own)
     st = _step().ws_shard_update(
