@@ -65,8 +65,12 @@ __device__ __forceinline__ float own_ratio(const OwnRatio& F, int seg, bool firs
 // (129 and more bf16 copies: 16 of 4 elements are 32 registers, and the third CTA per SM is worth a few spills.  us, two
 // CTAs / three: slices, 512 copies of 346 K elements, Adam 98 / 67, SGD-M 95 / 64; formatting fused in, 2 M parameters, Adam,
 // 160 copies 546 / 358, 256 copies 1038 / 723.  64 copies of 2.8 M, SGD-M, would go from 66 to 76)
+// (LARS' phase 2, three streams of loads: 4 CTAs per SM, up to 64 registers in place of 78 where fp32 master
+// weights, which take 52, do not have them anyway.  us, 3 / 4, bf16 weights: 1 copy, 25.6 M parameters 157 / 148; 3 copies,
+// 7.1 M 49.3 / 47.2; 12 copies, 7.1 M 110 / 105)
 template <int OPT, bool GBF, int RB, int NP>
 constexpr int min_blocks() {
+    if (OPT == K_LARS2) return 4;
     return RB > 8 && !(GBF && NP > 128 && (OPT == K_SGDM || OPT == K_ADAM)) ? kMinBlocksWide : kMinBlocks;
 }
 
