@@ -295,7 +295,11 @@ __host__ __device__ constexpr int many_blocks_per_group(int copies) {
 // does with 9 to 128 copies, and in an earlier block NaN or the infinity.
 __device__ __forceinline__ void add_group(float& sum, float& comp, float s, float c) {
     kahan1(sum, comp, s);
-    if (fabsf(sum) < INFINITY) kahan1(sum, comp, -c);
+    float sum_c = sum, comp_c = comp;          // (both ways and a choice: a branch would stand in the chain of the groups)
+    kahan1(sum_c, comp_c, -c);
+    const bool finite = fabsf(sum) < INFINITY;
+    sum = finite ? sum_c : sum;
+    comp = finite ? comp_c : comp;
 }
 
 // ------------------------------------------------------------------ math ---
